@@ -20,8 +20,7 @@
 #include "simt_gemm.cuh"
 #include "small_solvers.cuh"
 #include "block_jacobi.cuh"
-#include "cluster_jacobi.cuh"
-#include "eig_presolve.cuh"
+#include "eig_tridiag.cuh"
 #include "tc_orth.cuh"
 #include "rope.cuh"
 #include "attend.cuh"
@@ -31,14 +30,13 @@ using namespace jolt;
 namespace jolt {
 thread_local std::string g_err;
 std::atomic<long long> g_launches{0};
-std::atomic<int> g_eig_smem{1};
 #ifdef JOLT_DEBUG
 long long *g_dbg_stamps = nullptr;   // device buffer for kernel cycle stamps (profiling aid)
 #endif
 std::atomic<int> g_n_cell_groups{4};        // concurrent cell groups of jolt_compress (jolt_set_stream_groups)
 std::atomic<int> g_dec_tail_pct{0}, g_dec_tail_chunk{8};   // test switch: chunked tail of the persistent decode (off)
 std::atomic<int> g_fast{255};  // bit 0: fused backbone kernels, bit 1: factor sweeps, bit 2: Gram on tensor cores,
-                              // bit 3: rotary embedding inside the decode kernel, bit 4: cluster-resident eigen-solver,
+                              // bit 3: rotary embedding inside the decode kernel, bit 4: tridiagonal eigen-solver,
                               // bit 5: CholeskyQR on tensor cores, bit 6: two output tiles per CTA in the factor sweeps,
                               // bit 7: persistent decode kernel
 
@@ -392,103 +390,35 @@ void add_gemm(Program &P, int stage, const std::vector<GemmTask> &all_tasks, boo
 
 void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sweeps) {
   if (tasks.empty()) return;
-  // problems that fit one CTA's shared memory take the resident kernel, the rest the global-memory one
-  std::vector<EigTask> small64, small32, big;
+  std::vector<TdTask> td[2];               // tridiagonal solver: one CTA per matrix (n <= kTdSmallMaxN) / a cluster per matrix
+  std::vector<EigTask> small;              // portable: Jacobi in one CTA's shared memory (n <= 32) / block Jacobi
   std::vector<BJTask> bj;
-  std::vector<CholFactorTask> cf;          // Cholesky factor for the cluster solver: work matrix in global memory (n > 152)
-  std::vector<tc::CholInvTask> cfs;        // ... in shared memory
-  std::vector<CJTask> cj;                  // one launch: rows per lane follow the largest matrix
-  std::vector<PresolveTask> pre;           // block-solver problems that start from a single-precision basis
   for (auto &t : tasks) {
-    // singular values of B (w_sqrt): single-precision cluster solver; the mode-3 Gram, whose spectrum spans 1e6 and more
-    // when the cache has outlier channels, stays on the fp64 block solver
-    if (t.bjA && t.w_sqrt && t.n > 32 && t.n <= kCJMaxN && (g_fast.load() & 16)) {
-      // Cholesky factor in the block solver's scratch, then the cluster-resident one-sided Jacobi on its columns
-      if (t.n <= tc::kCholInvMaxN) cfs.push_back({nullptr, 0, 0, t.A, t.n, nullptr, nullptr, nullptr, t.bjA, t.status, 1e-13});
-      else cf.push_back({t.A, t.bjA, t.n, t.status});
-      CJTask c; memset(&c, 0, sizeof c);
-      c.L = t.bjA; c.n = t.n; c.U_out = t.U_out; c.ld_out = t.ld_out; c.r_out = t.r_out; c.w_out = t.w_out; c.w_sqrt = t.w_sqrt;
-      c.status = t.status; c.sweeps_out = t.bjDone;
-      cj.push_back(c);
-      continue;
-    }
-    if (t.bjA && t.n > 32 && g_eig_smem.load() != 2) {
+    if (t.td) {
+      TdTask q; memset(&q, 0, sizeof q);
+      q.A = t.A; q.n = t.n; q.U_out = t.U_out; q.ld_out = t.ld_out; q.r_out = t.r_out; q.w_out = t.w_out; q.w_sqrt = t.w_sqrt; q.status = t.status;
+      td_set_scratch(q, t.td);
+      td[t.n > kTdSmallMaxN].push_back(q);
+    } else if (t.n <= kEigSmemMaxN) {
+      small.push_back(t);
+    } else {
       BJTask b; memset(&b, 0, sizeof b);
-      const bool presolve = t.preL && !t.w_sqrt && t.n <= tc::kCholInvMaxN && (g_fast.load() & 16);
-      if (presolve) {
-        // A + shift -> Cholesky factor -> single-precision one-sided Jacobi: U; then A' = U^T A U, block solver from V = U
-        pre.push_back({t.A, t.preA, t.preU, t.preT, t.n});
-        cfs.push_back({nullptr, 0, 0, t.preA, t.n, nullptr, nullptr, nullptr, t.preL, nullptr, 0.0});
-        CJTask c; memset(&c, 0, sizeof c);
-        c.L = t.preL; c.n = t.n; c.U_out = t.preU; c.ld_out = t.n; c.r_out = t.n;
-        c.status = nullptr;      // only a starting basis: if this iteration stops short, the block solver sweeps more
-        cj.push_back(c);
-        b.V0 = t.preU;
-      }
-      b.A_in = presolve ? t.preA : t.A; b.A = t.bjA; b.V = t.bjV; b.J = t.bjJ; b.off = t.bjOff; b.done = t.bjDone; b.ticket = (unsigned *)(t.bjDone + 1);
+      b.A_in = t.A; b.A = t.bjA; b.V = t.bjV; b.J = t.bjJ; b.off = t.bjOff; b.done = t.bjDone; b.ticket = (unsigned *)(t.bjDone + 1);
       b.n = t.n; b.nbe = (((t.n + kBJBlock - 1) / kBJBlock) + 1) & ~1; b.nP = b.nbe * kBJBlock;
       b.w = t.w; b.U_out = t.U_out; b.ld_out = t.ld_out; b.r_out = t.r_out; b.w_out = t.w_out; b.w_sqrt = t.w_sqrt; b.status = t.status;
       b.tol = kBJTol;
       bj.push_back(b);
-      continue;
-    }
-    if (!g_eig_smem.load() || t.n > kEigSmemMaxN) big.push_back(t);
-    else if (eig_smem_bytes(t.n, 8) <= kSmemOptIn - 1024) small64.push_back(t);   // fp64 eigenvector accumulator fits
-    else if (eig_smem_bytes(t.n, 4) <= kSmemOptIn - 1024) small32.push_back(t);
-    else big.push_back(t);
-  }
-  const size_t o_pre = P.push(pre);
-  const int n_pre = (int)pre.size();
-  int pre_n = 0;
-  for (auto &q : pre) pre_n = std::max(pre_n, q.n);
-  if (n_pre) P.add(stage, [=](char *dev, cudaStream_t s) {
-    presolve_shift_kernel<<<dim3(16, n_pre), 256, 0, s>>>((const PresolveTask *)(dev + o_pre)); LAUNCHED();
-  });
-  if (!cfs.empty()) {
-    const size_t off = P.push(cfs);
-    const int n = (int)cfs.size();
-    int cmn = 0;
-    for (auto &c : cfs) cmn = std::max(cmn, c.k);
-    const size_t cshm = tc::cholinv_smem_bytes(cmn);
-    static bool cattr = false;
-    if (!cattr) { cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN)); cattr = true; }
-    P.add(stage, [=](char *dev, cudaStream_t s) {
-      tc::cholinv_kernel<<<n, tc::kCholInvThreads, cshm, s>>>((const tc::CholInvTask *)(dev + off)); LAUNCHED();
-    });
-  }
-  if (!cf.empty()) {
-    const size_t off = P.push(cf);
-    const int n = (int)cf.size();
-    int cmn = 0;
-    for (auto &c : cf) cmn = std::max(cmn, c.n);
-    const size_t cshm = std::max(chol_factor_smem_bytes(kCholFactorSmemN), chol_factor_smem_bytes(cmn));
-    static bool cattr = false;
-    if (!cattr) { cudaFuncSetAttribute(chol_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 2048)); cattr = true; }
-    P.add(stage, [=](char *dev, cudaStream_t s) {
-      chol_factor_kernel<<<n, kCholFactorThreads, cshm, s>>>((const CholFactorTask *)(dev + off)); LAUNCHED();
-    });
-  }
-  if (!cj.empty()) {
-    static bool cjattr = false;
-    if (!cjattr) { cj_opt_in_smem(); cjattr = true; }
-    {
-      int mn = 0;
-      for (auto &c : cj) mn = std::max(mn, c.n);
-      const int nr = cj_rows_per_lane(mn), nt = (int)cj.size();
-      const size_t o2 = P.push(cj);
-      P.add(stage, [=](char *dev, cudaStream_t s) { cj_launch((const CJTask *)(dev + o2), nt, mn, nr, s); LAUNCHED(); });
     }
   }
-  if (n_pre) P.add(stage, [=](char *dev, cudaStream_t s) {
-    const dim3 grid((pre_n + 15) / 16, n_pre);
-    presolve_mul_kernel<false><<<grid, 256, 0, s>>>((const PresolveTask *)(dev + o_pre)); LAUNCHED();
-    presolve_mul_kernel<true><<<grid, 256, 0, s>>>((const PresolveTask *)(dev + o_pre)); LAUNCHED();
-  });
+  for (auto &q : td) {
+    if (q.empty()) continue;
+    int mn = 0, mr = 0;
+    for (auto &t : q) { mn = std::max(mn, t.n); if (t.U_out) mr = std::max(mr, t.r_out); }
+    const size_t off = P.push(q);
+    const int n = (int)q.size();
+    P.add(stage, [=](char *dev, cudaStream_t s) { g_launches += td_launch((const TdTask *)(dev + off), n, mn, mr, s); });
+  }
   if (!bj.empty()) {
-    // with a single-precision starting basis for every problem one sweep converges (measured: relative off-diagonal
-    // mass 1e-12 .. 1e-13 before it, rank-deficient matrices included); four are allowed, and the launches after
-    // convergence are no-ops of a few microseconds each
-    if (n_pre == (int)bj.size()) bj_sweeps = std::min(bj_sweeps, 4);
     int max_nbe = 0, max_nP = 0;
     for (auto &b : bj) { max_nbe = std::max(max_nbe, b.nbe); max_nP = std::max(max_nP, b.nP); }
     const size_t off = P.push(bj);
@@ -508,35 +438,14 @@ void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sw
       bj_finish_kernel<<<n, 256, 0, s>>>(d, n_steps & 1); LAUNCHED();
     });
   }
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaFuncSetAttribute(jacobi_eig_smem_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024));
-    cudaFuncSetAttribute(jacobi_eig_smem_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024));
-    attr_done = true;
-  }
-  for (int pass = 0; pass < 2; ++pass) {
-    const std::vector<EigTask> &small = pass == 0 ? small64 : small32;
-    if (small.empty()) continue;
+  if (!small.empty()) {
     int mn = 0;
     for (auto &t : small) mn = std::max(mn, t.n);
-    const size_t shm = eig_smem_bytes(mn, pass == 0 ? 8 : 4);
+    const size_t shm = eig_smem_bytes(mn);
     const size_t off = P.push(small);
     const int n = (int)small.size();
-    const bool dbl = pass == 0;
     P.add(stage, [=](char *dev, cudaStream_t s) {
-      if (dbl) jacobi_eig_smem_kernel<double><<<n, kEigThreads, shm, s>>>((const EigTask *)(dev + off));
-      else jacobi_eig_smem_kernel<float><<<n, kEigThreads, shm, s>>>((const EigTask *)(dev + off));
-      LAUNCHED();
-    });
-  }
-  if (!big.empty()) {
-    int mn = 0;
-    for (auto &t : big) mn = std::max(mn, t.n);
-    const size_t off = P.push(big);
-    const int n = (int)big.size();
-    const size_t shm = (size_t)(2 * ((mn + 1) / 2) + 32) * sizeof(double);
-    P.add(stage, [=](char *dev, cudaStream_t s) {
-      jacobi_eig_kernel<<<n, kEigThreads, shm, s>>>((const EigTask *)(dev + off));
+      jacobi_eig_smem_kernel<<<n, kEigThreads, shm, s>>>((const EigTask *)(dev + off));
       LAUNCHED();
     });
   }
@@ -560,7 +469,7 @@ struct CellWork {      // device scratch of one cell
   double *bjA = nullptr, *bjV = nullptr, *bjJ = nullptr, *bjOff = nullptr; int *bjDone = nullptr;
   // eigen-solver scratch of the feature stage: its own, since the probe runs that stage concurrently with the token stage
   double *bjfA = nullptr, *bjfV = nullptr, *bjfJ = nullptr, *bjfOff = nullptr; int *bjfDone = nullptr;
-  double *preL = nullptr, *preT = nullptr, *preA = nullptr; float *preU = nullptr;      // pre-solve of the feature eigenproblem
+  double *td = nullptr, *tdf = nullptr;        // tridiagonal solver's scratch: token stage, feature stage
   double *BBt = nullptr, *BBv = nullptr, *BBw = nullptr;
   float *Ut = nullptr, *sigma = nullptr;
   float *UT32 = nullptr, *G32 = nullptr;
@@ -572,6 +481,7 @@ struct CellWork {      // device scratch of one cell
   float *pmax = nullptr;     // partial maxima of |G| for the core exponent
   float *rho = nullptr;      // where the residual of the converged-subspace check goes (exact mode at large T)
   int n_sigma = 0;
+  bool tridiag = false;      // eigen-solves take the tridiagonal solver
   // tensor-core sweeps
   bool tc = false;           // sketch / projection sweeps run on tcgen05
   bool tc_gram = false;      // mode-3 Gram runs on tcgen05
@@ -603,18 +513,19 @@ void carve(Bump &b, CellWork &w, int mode, bool need_backbone_scratch) {
     w.pmax = b.take<float>(32);
     w.Zp = b.take<float>((size_t)c.m * kD * std::max<size_t>(k, c.r_t));
     if (mode != FM_INJECTED) {
-      {
-        const size_t nmax = std::max<size_t>(kD, mode == FM_EXACT ? T : k);
-        const size_t nbe = (((nmax + kBJBlock - 1) / kBJBlock) + 1) & ~(size_t)1, nP = nbe * kBJBlock;
+      // the feature stage has a scratch of its own: the probe runs it concurrently with the token stage
+      const int n_eig = mode == FM_EXACT ? c.T : c.k;
+      if (w.tridiag && n_eig <= kTdMaxN) w.td = b.take<double>(td_scratch_doubles(n_eig, c.r_t));
+      else {
+        const size_t nbe = (((n_eig + kBJBlock - 1) / kBJBlock) + 1) & ~(size_t)1, nP = nbe * kBJBlock;
         w.bjA = b.take<double>(2 * nP * nP); w.bjV = b.take<double>(nP * nP); w.bjJ = b.take<double>(2 * (nbe / 2) * 1024);
         w.bjOff = b.take<double>(4); w.bjDone = b.take<int>(4);
       }
-      {
+      if (w.tridiag) w.tdf = b.take<double>(td_scratch_doubles(kD, kD));
+      else {
         const size_t nbe = (((kD + kBJBlock - 1) / kBJBlock) + 1) & ~(size_t)1, nP = nbe * kBJBlock;
         w.bjfA = b.take<double>(2 * nP * nP); w.bjfV = b.take<double>(nP * nP); w.bjfJ = b.take<double>(2 * (nbe / 2) * 1024);
         w.bjfOff = b.take<double>(4); w.bjfDone = b.take<int>(4);
-        w.preL = b.take<double>(kD * kD + 8); w.preT = b.take<double>(kD * kD); w.preA = b.take<double>(kD * kD);
-        w.preU = b.take<float>(kD * kD);
       }
       w.gram_part = b.take<double>((size_t)c.m * kD * kD * std::max(1, (tok_segments(c.T) + 1) / 2));
       w.C = b.take<double>(kD * kD); w.Cv = b.take<double>(kD * kD); w.Cw = b.take<double>(kD);
@@ -927,7 +838,7 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
       EigTask e; memset(&e, 0, sizeof e);
       e.bjA = w.bjfA; e.bjV = w.bjfV; e.bjJ = w.bjfJ; e.bjOff = w.bjfOff; e.bjDone = w.bjfDone;
       e.A = w.C; e.Vt = w.Cv; e.w = w.Cw; e.n = kD; e.status = w.status; e.w_out = w.lam; e.w_sqrt = 0;
-      e.preL = w.preL; e.preU = w.preU; e.preT = w.preT; e.preA = w.preA;
+      e.td = w.tdf;
       if (!probe) { e.U_out = w.UF32; e.ld_out = c.r_f; e.r_out = c.r_f; }
       eg.push_back(e);
     }
@@ -969,7 +880,7 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
       const CellDesc &c = w.c;
       tgb.push_back({w.Z, c.N, c.k, w.gpart, w.BBt});
       EigTask e; memset(&e, 0, sizeof e);
-      e.bjA = w.bjA; e.bjV = w.bjV; e.bjJ = w.bjJ; e.bjOff = w.bjOff; e.bjDone = w.bjDone;
+      e.bjA = w.bjA; e.bjV = w.bjV; e.bjJ = w.bjJ; e.bjOff = w.bjOff; e.bjDone = w.bjDone; e.td = w.td;
       e.A = w.BBt; e.Vt = w.BBv; e.w = w.BBw; e.n = c.k; e.status = w.status; e.w_out = w.sigma; e.w_sqrt = 1;
       if (!probe) { e.U_out = w.Ut; e.ld_out = c.r_t; e.r_out = c.r_t; }
       eg.push_back(e);
@@ -1016,7 +927,7 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
       t.nseg = c.m; t.seg_inner = c.m; t.a_si = (long long)c.T * c.r_f; t.b_si = (long long)c.T * c.r_f;
       g2.push_back(t);
       EigTask e; memset(&e, 0, sizeof e);
-      e.bjA = w.bjA; e.bjV = w.bjV; e.bjJ = w.bjJ; e.bjOff = w.bjOff; e.bjDone = w.bjDone;
+      e.bjA = w.bjA; e.bjV = w.bjV; e.bjJ = w.bjJ; e.bjOff = w.bjOff; e.bjDone = w.bjDone; e.td = w.td;
       e.A = w.Gt; e.Vt = w.Gtv; e.w = w.Gtw; e.n = c.T; e.status = w.status; e.w_out = w.sigma; e.w_sqrt = 1;
       if (!probe) { e.U_out = w.UT32; e.ld_out = c.r_t; e.r_out = c.r_t; }
       eg.push_back(e);
@@ -1414,6 +1325,7 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
       w.tc = (fmask & 2) && w.active && mode == FM_RANDOMIZED && tc_sweep_ok(cells[i], L->mem_space == JOLT_MEM_HOST);
       w.tc_gram = (fmask & 4) && w.active && mode != FM_INJECTED && tc_sweep_ok(cells[i], L->mem_space == JOLT_MEM_HOST);
       w.ufI = w.active && cells[i].r_f == kD;
+      w.tridiag = (fmask & 16) != 0;
       if (pass == 1) { w.lam = H->cells[i].lam; w.sigma = H->cells[i].n_sigma ? H->cells[i].sigma : nullptr; w.status = d_status + 4 * i; w.rho = (float *)(H->cells[i].e + 1); }
       carve(b, w, mode, true);
       if (pass == 1 && !w.n_sigma) w.n_sigma = H->cells[i].n_sigma;
@@ -2262,6 +2174,7 @@ extern "C" int jolt_probe(const jolt_layout *L, const void *K, const void *V, do
       ws[i].tc = (fmask & 2) && mode == FM_RANDOMIZED && tc_sweep_ok(cells[i], L->mem_space == JOLT_MEM_HOST);
       ws[i].tc_gram = (fmask & 4) && tc_sweep_ok(cells[i], L->mem_space == JOLT_MEM_HOST);
       ws[i].ufI = true;
+      ws[i].tridiag = (fmask & 16) != 0;
       carve(b, ws[i], mode, false);
     }
     if (pass == 0) { pack_floats = 0; for (int i = 0; i < nc; ++i) pack_floats += kD + (size_t)ws[i].n_sigma; }

@@ -18,9 +18,7 @@ struct EigTask {
   int *status;      // set to 1 if not converged
   // optional scratch of the multi-launch block solver (null: single-CTA kernels)
   double *bjA, *bjV, *bjJ, *bjOff; int *bjDone;
-  // optional scratch of the single-precision pre-solve that gives the block solver its starting basis (null: start
-  // from the identity): preL n*n+8 doubles, preU n*n floats, preT and preA n*n doubles each
-  double *preL; float *preU; double *preT, *preA;
+  double *td;       // scratch of the tridiagonal solver (eig_tridiag.cuh); null: Jacobi
 };
 
 constexpr int kEigThreads = 1024;
@@ -70,135 +68,25 @@ __device__ __forceinline__ void rr_pair(int r, int i, int ne, int &p, int &q) {
   if (p > q) { const int tmp = p; p = q; q = tmp; }
 }
 
-__global__ void __launch_bounds__(kEigThreads) jacobi_eig_kernel(const EigTask *__restrict__ tasks) {
-  const EigTask t = tasks[blockIdx.x];
-  const int n = t.n;
-  if (n <= 0) return;
-  double *A = t.A, *Vt = t.Vt;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int ne = (n + 1) & ~1;          // padded to even; index n (if present) is a bye
-  const int np = ne / 2;
-  extern __shared__ double sh[];        // c[np], s[np], red[32]
-  double *cs_c = sh, *cs_s = sh + np, *red = sh + 2 * np;
-  __shared__ int pp[1024], qq[1024];    // np <= 1024 (n <= 2048)
-  __shared__ int rk[2048];
-  __shared__ double s_total, s_off;
-
-  for (int i = tid; i < n * n; i += nt) Vt[i] = ((i / n) == (i % n)) ? 1.0 : 0.0;
-  // ||A||_F^2
-  double loc = 0;
-  for (int i = tid; i < n * n; i += nt) loc += A[i] * A[i];
-  for (int o = 16; o; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
-  if ((tid & 31) == 0) red[tid >> 5] = loc;
-  __syncthreads();
-  if (tid == 0) { double s = 0; for (int i = 0; i < nt / 32; ++i) s += red[i]; s_total = s; }
-  __syncthreads();
-  const double total = s_total;
-  bool converged = (total == 0.0);
-  int sweep = 0;
-  for (; sweep < kEigMaxSweeps && !converged; ++sweep) {
-    for (int r = 0; r < ne - 1; ++r) {
-      for (int i = tid; i < np; i += nt) {
-        int p, q; rr_pair(r, i, ne, p, q);
-        double c = 1.0, s = 0.0;
-        if (q < n) {
-          const double apq = A[(size_t)p * n + q];
-          const double app = A[(size_t)p * n + p], aqq = A[(size_t)q * n + q];
-          if (fabs(apq) > 1e-300 && fabs(apq) > 1e-17 * sqrt(fabs(app * aqq))) {
-            const double tau = (aqq - app) / (2.0 * apq);
-            const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + tt * tt);
-            s = tt * c;
-          }
-        } else { q = p; }
-        pp[i] = p; qq[i] = q; cs_c[i] = c; cs_s[i] = s;
-      }
-      __syncthreads();
-      // rows of A and of Vt:  row_p' = c row_p - s row_q ; row_q' = s row_p + c row_q
-      for (int it = tid; it < np * n; it += nt) {
-        const int i = it / n, j = it - i * n;
-        const int p = pp[i], q = qq[i];
-        if (p == q) continue;
-        const double c = cs_c[i], s = cs_s[i];
-        if (s == 0.0) continue;
-        double ap = A[(size_t)p * n + j], aq = A[(size_t)q * n + j];
-        A[(size_t)p * n + j] = c * ap - s * aq;
-        A[(size_t)q * n + j] = s * ap + c * aq;
-        double vp = Vt[(size_t)p * n + j], vq = Vt[(size_t)q * n + j];
-        Vt[(size_t)p * n + j] = c * vp - s * vq;
-        Vt[(size_t)q * n + j] = s * vp + c * vq;
-      }
-      __syncthreads();
-      // columns of A
-      for (int it = tid; it < np * n; it += nt) {
-        const int row = it / np, i = it - row * np;
-        const int p = pp[i], q = qq[i];
-        if (p == q) continue;
-        const double c = cs_c[i], s = cs_s[i];
-        if (s == 0.0) continue;
-        double ap = A[(size_t)row * n + p], aq = A[(size_t)row * n + q];
-        A[(size_t)row * n + p] = c * ap - s * aq;
-        A[(size_t)row * n + q] = s * ap + c * aq;
-      }
-      __syncthreads();
-    }
-    // off-diagonal mass
-    double off = 0;
-    for (int i = tid; i < n * n; i += nt) { if ((i / n) != (i % n)) off += A[i] * A[i]; }
-    for (int o = 16; o; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
-    if ((tid & 31) == 0) red[tid >> 5] = off;
-    __syncthreads();
-    if (tid == 0) { double s = 0; for (int i = 0; i < nt / 32; ++i) s += red[i]; s_off = s; }
-    __syncthreads();
-    converged = (s_off <= 1e-26 * total);
-    __syncthreads();
-  }
-  if (!converged && tid == 0 && t.status) *t.status = 1;
-  for (int i = tid; i < n; i += nt) t.w[i] = A[(size_t)i * n + i];
-  __syncthreads();
-  // rank sort (descending, ties by index) and scatter
-  for (int i = tid; i < n; i += nt) {
-    const double wi = t.w[i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) { const double wj = t.w[j]; rank += (wj > wi) || (wj == wi && j < i); }
-    if (t.w_out) { const double v = wi > 0 ? wi : 0.0; t.w_out[rank] = (float)(t.w_sqrt ? sqrt(v) : v); }
-    if (n <= 2048) rk[i] = rank;
-  }
-  __syncthreads();
-  if (t.U_out) {
-    for (int it = tid; it < n * n; it += nt) {
-      const int i = it / n, j = it - i * n;   // eigenvector i, component j
-      int rank;
-      if (n <= 2048) rank = rk[i];
-      else {
-        const double wi = t.w[i]; rank = 0;
-        for (int jj = 0; jj < n; ++jj) { const double wj = t.w[jj]; rank += (wj > wi) || (wj == wi && jj < i); }
-      }
-      if (rank < t.r_out) t.U_out[(size_t)j * t.ld_out + rank] = (float)Vt[(size_t)i * n + j];
-    }
-  }
-}
-
-// Shared-memory variant for n <= kEigSmemMaxN: the symmetric matrix lives as a packed lower triangle in
-// fp64, the eigenvector accumulator as fp32 rows.  One round = rotation parameters for n/2 disjoint pairs,
+// Portable solver for n <= kEigSmemMaxN: the symmetric matrix lives as a packed lower triangle in fp64, the eigenvector
+// accumulator as fp64 rows.  One round = rotation parameters for n/2 disjoint pairs,
 // then ONE fused update: every 2x2 block A[{p_a,q_a}][{p_b,q_b}] (a <= b) becomes J_a^T blk J_b, and rows
 // p, q of V^T rotate.  Two barriers per round, no global traffic.
-constexpr int kEigSmemMaxN = 168;
+constexpr int kEigSmemMaxN = 32;
 constexpr size_t kSmemOptIn = 232448;    // 227 KB of dynamic shared memory per CTA
 
-__host__ __device__ inline size_t eig_smem_bytes(int n, size_t vsize) {
+__host__ __device__ inline size_t eig_smem_bytes(int n) {
   const int np = (n + 1) / 2;
   size_t b = (size_t)n * (n + 1) / 2 * sizeof(double);       // packed A
   b += (size_t)np * 2 * sizeof(double);                       // c, s
   b += 40 * sizeof(double);                                   // reduction scratch
-  b += (size_t)n * n * vsize;                                 // V^T
+  b += (size_t)n * n * sizeof(double);                                 // V^T
   b += (size_t)np * 2 * sizeof(int) + (size_t)n * sizeof(int) + 64;
   return b;
 }
 
 __device__ __forceinline__ int tri_idx(int i, int j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
 
-template <typename VT>
 __global__ void __launch_bounds__(kEigThreads, 1) jacobi_eig_smem_kernel(const EigTask *__restrict__ tasks) {
   const EigTask t = tasks[blockIdx.x];
   const int n = t.n;
@@ -208,7 +96,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) jacobi_eig_smem_kernel(const E
   const int ntri = n * (n + 1) / 2;
   double *A = shd;
   double *cs_c = A + ntri, *cs_s = cs_c + np, *red = cs_s + np;
-  VT *Vt = (VT *)(red + 40);
+  double *Vt = (double *)(red + 40);
   int *pp = (int *)(Vt + (size_t)n * n), *qq = pp + np, *rk = qq + np;
   __shared__ double s_total, s_off;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -219,7 +107,7 @@ __global__ void __launch_bounds__(kEigThreads, 1) jacobi_eig_smem_kernel(const E
     const double v = t.A[e];
     loc += v * v;
     if (j <= i) A[i * (i + 1) / 2 + j] = (i == j) ? v : 0.5 * (v + t.A[(size_t)j * n + i]);
-    Vt[e] = (i == j) ? VT(1) : VT(0);
+    Vt[e] = (i == j) ? 1.0 : 0.0;
   }
   for (int o = 16; o; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
   if ((tid & 31) == 0) red[tid >> 5] = loc;
@@ -290,11 +178,11 @@ __global__ void __launch_bounds__(kEigThreads, 1) jacobi_eig_smem_kernel(const E
       if (vi0 < vcols) {
         for (int i = vi0; i < np; i += vcols) {
           const int q = qq[i];
-          const VT s = (VT)cs_s[i];
-          if (q < 0 || s == VT(0)) continue;
+          const double s = cs_s[i];
+          if (q < 0 || s == 0.0) continue;
           const int p = pp[i];
-          const VT c = (VT)cs_c[i];
-          const VT vp = Vt[p * n + vj], vq = Vt[q * n + vj];
+          const double c = cs_c[i];
+          const double vp = Vt[p * n + vj], vq = Vt[q * n + vj];
           Vt[p * n + vj] = c * vp - s * vq;
           Vt[q * n + vj] = s * vp + c * vq;
         }
@@ -343,15 +231,13 @@ __global__ void __launch_bounds__(kEigThreads, 1) jacobi_eig_smem_kernel(const E
 // (0 for a dead pivot).  trsm_rows_kernel then solves  dst_row * L^T = src_row  for 128 rows per CTA.
 constexpr int kCholSmemMaxN = 168;
 
-// 1 / sqrt(d) for d > 0: single-precision seed and two Newton steps in fp64 (full accuracy), the library routine
-// outside the single-precision range
+// 1 / sqrt(d) for d > 0: single-precision seed (relative error e below 2^-22) and one third-order step in fp64
+// (error of the order of e^3), the library routine outside the single-precision range
 __device__ __forceinline__ double rsqrt_pos(double d) {
   if (!(d > 1e-30 && d < 1e30)) return rsqrt(d);
-  const double h = 0.5 * d;
-  double y = (double)rsqrtf((float)d);
-  y = y * fma(-h * y, y, 1.5);
-  y = y * fma(-h * y, y, 1.5);
-  return y;
+  const double y = (double)rsqrtf((float)d);
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 

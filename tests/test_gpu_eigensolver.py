@@ -1,0 +1,67 @@
+"""The tridiagonal eigen-solver against the Jacobi solvers (the portable path, bit 4 of the kernel mask off) and against
+LAPACK, at the sizes where its kernels change: one CTA up to n = 160 (rows beyond 128 in shared memory), a cluster beyond."""
+import numpy as np
+import pytest
+import torch
+
+import __graft_entry__ as entry
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    entry.build()
+    import paper_2607_12550_b200 as pkg
+    return pkg.load()
+
+
+def _cache(T, m, rank, noise, seed):
+    g = torch.Generator().manual_seed(seed)
+    P = torch.randn(T, rank, generator=g) / torch.arange(1, rank + 1)
+    X = torch.einsum("tr,mfr->mtf", P, torch.randn(m, 128, rank, generator=g)) + noise * torch.randn(m, T, 128, generator=g)
+    return X.view(1, m, T, 128).float().cuda()
+
+
+def _solve(B, K, V, plan, mask, **opt):
+    prev = B.set_fast_path(mask)
+    try:
+        h = B.jolt_compress(K, V, [0, 1], plan, B.default_options(seed=3, power_iters=1, **opt))
+        sig = [h.component(c, 6).astype(np.float64) for c in range(2)]
+        UT = [h.component(c, 8).reshape(K.shape[2], -1).astype(np.float64) for c in range(2)]
+        h.free()
+    finally:
+        B.set_fast_path(prev)
+    return sig, UT
+
+
+# sketch width = rank + 10: both sides of 32 (portable solver), 128 (register block), 160 (one CTA), 288 and 544 (rows per lane)
+@pytest.mark.parametrize("r_t", [2, 22, 23, 54, 118, 119, 128, 150, 151, 278, 279, 534, 535])
+def test_small_svd_matches_jacobi(B, r_t):
+    T = 640
+    K, V = _cache(T, 6, 40, 0.05, 1), _cache(T, 6, 700, 0.3, 2)
+    plan = [(r_t, 128, 4), (r_t, 128, 4)]
+    sig, UT = _solve(B, K, V, plan, 0)
+    sig2, UT2 = _solve(B, K, V, plan, 16)
+    for c in range(2):
+        # both solvers return the fp32 rounding of an fp64 solution of the same matrix, up to the Jacobi threshold (1e-7 relative)
+        assert np.abs(sig2[c] - sig[c]).max() <= 3e-6 * sig[c][0]
+        assert np.abs(UT2[c].T @ UT2[c] - np.eye(r_t)).max() <= 1e-4        # single-precision products of two orthonormal factors
+        gap = sig[c][r_t - 1] ** 2 - sig[c][r_t] ** 2
+        if gap > 1e-3 * sig[c][0] ** 2:
+            assert np.linalg.norm(UT[c] @ UT[c].T - UT2[c] @ UT2[c].T) <= 1e-3
+
+
+@pytest.mark.parametrize("T", [128, 256, 640, 1024])
+def test_exact_token_factor_matches_lapack(B, T):
+    m = 2
+    K, V = _cache(T, m, 24, 0.02, 5), _cache(T, m, 12, 0.0, 6)              # V: exactly rank 12, a null space of T - 12 (T x T)
+    sig, UT = _solve(B, K, V, [(24, 128, 4), (16, 128, 4)], 255, token_mode=B.TOKEN_EXACT)
+    for c, X in enumerate((K, V)):
+        A = X[0].permute(1, 0, 2).reshape(T, -1).double().cpu().numpy()
+        U, s, _ = np.linalg.svd(A, full_matrices=False)
+        n = min(T, len(s))
+        assert np.abs(sig[c][:n] ** 2 - s[:n] ** 2).max() <= 1e-6 * s[0] ** 2    # fp32 input products, fp64 solve
+        r = 24 if c == 0 else 12
+        assert np.linalg.norm(UT[c][:, :r] @ UT[c][:, :r].T - U[:, :r] @ U[:, :r].T) <= 1e-4
+        assert np.abs(UT[c].T @ UT[c] - np.eye(UT[c].shape[1])).max() <= 1e-5   # a full basis, null directions included
