@@ -7,6 +7,8 @@
 #include "tc_decode_p.cuh"
 #include "tc_gemm.cuh"
 #include "tc_orth.cuh"
+#include "tc_orth_wide.cuh"
+#include "chol_cluster.cuh"
 
 namespace {
 
@@ -443,11 +445,116 @@ inline void add_sketch_gen_tc(Program &P, int stage, std::vector<CellWork> &ws, 
 }
 
 // ------------------------------------------------------------------ CholeskyQR on tensor cores
-// Cells whose basis is already kept as the hi + lo operand of the sweeps (tensor-core cells with r_f = d, sketch
-// width up to OR_MAX_K) orthonormalise it there: Gram and Q = R L^-T are tcgen05 GEMMs, the Cholesky factor and its
-// inverse one fp64 CTA per cell.
+// Cells whose basis is already kept as the hi + lo operand of the sweeps (tensor-core cells with r_f = d) orthonormalise
+// it there: Gram and Q = R L^-T are tcgen05 GEMMs, the Cholesky factor and its inverse one fp64 CTA per cell up to
+// OR_MAX_K columns (one accumulator, one shared memory), a cluster per cell beyond.
 inline bool orth_tc_ok(const CellWork &w) {
-  return w.active && w.tc && w.ufI && w.c.k <= tc::OR_MAX_K && w.kp <= tc::OR_MAX_KP && w.c.T % 128 == 0 && w.orthPart != nullptr;
+  return w.active && w.tc && w.ufI && w.c.T % 128 == 0 && w.orthPart != nullptr;
+}
+inline bool orth_is_wide(const CellWork &w) { return w.c.k > tc::OR_MAX_K || w.kp > tc::OR_MAX_KP; }
+
+// The sweep left the raw basis as fp32 rows: measure its magnitude (unless the sweep's epilogue did), split it into the
+// operand layout.
+inline void add_orth_split(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side) {
+  std::vector<tc::AbsMaxJob> am;
+  std::vector<tc::SplitJob> sp;
+  for (int i : idx) {
+    CellWork &w = ws[i];
+    const CellDesc &c = w.c;
+    const int rpp = token_side ? c.T : kD, panels = token_side ? 1 : c.m;
+    float *src = token_side ? w.S : w.Z;
+    unsigned *slot = w.orthMax + (w.orthMaxUsed++ % kOrthMaxSlots);
+    if (!w.absmax_ready) am.push_back({src, (long long)rpp * panels * c.k, slot});
+    w.absmax_ready = false;
+    tc::SplitJob j;
+    j.in = src; j.hi = w.Bhi; j.lo = w.Blo; j.batch = panels; j.rows = rpp; j.cols = c.k; j.ld_in = c.k; j.kp = w.kp; j.scale_exp = 0;
+    j.absmax = slot;
+    sp.push_back(j);
+  }
+  const size_t o_am = P.push(am), o_sp = P.push(sp);
+  const int n = (int)idx.size(), n_am = (int)am.size();
+  P.add(stage, [=](char *dev_t, cudaStream_t s) {
+    if (n_am) { tc::absmax_kernel<<<dim3(32, n_am), 256, 0, s>>>((const tc::AbsMaxJob *)(dev_t + o_am)); LAUNCHED(); }
+    tc::split_transpose_kernel<<<dim3(148, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + o_sp)); LAUNCHED();
+  });
+}
+
+// Wide sketches (k > OR_MAX_K): blocked Gram and apply, cluster Cholesky.
+constexpr double kOrthRedoRel = 5e-7;      // about eight times the error of a single-precision Gram relative to its diagonal
+inline void add_orth_wide(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side, int passes,
+                          bool want_fp32) {
+  if (idx.empty()) return;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(tc::orthw_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OW_GRAM_SMEM);
+    cudaFuncSetAttribute(tc::orthw_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OW_APPLY_SMEM);
+  });
+  add_orth_split(P, stage, ws, idx, token_side);
+  std::vector<tc::OrthWCell> oc, oc_last;
+  std::vector<CholTask> ct, ct_redo;
+  std::vector<TallGram> tg;
+  int max_chunks = 0, max_tiles = 0, max_pairs = 0, max_k = 0;
+  for (int i : idx) {
+    CellWork &w = ws[i];
+    const CellDesc &c = w.c;
+    const int rpp = token_side ? c.T : kD, panels = token_side ? 1 : c.m;
+    tc::OrthWCell o;
+    memset(&o, 0, sizeof o);
+    {
+      const uint64_t dims[3] = {(uint64_t)rpp, (uint64_t)w.kp, (uint64_t)panels};
+      const uint64_t str[2] = {(uint64_t)rpp * 2, (uint64_t)w.kp * rpp * 2};
+      const uint32_t box[3] = {64, 128, 1}, boxa[3] = {64, 64, 1};
+      make_tmap_f16(&o.tmHi, w.Bhi, 3, dims, str, box);
+      make_tmap_f16(&o.tmLo, w.Blo, 3, dims, str, box);
+      make_tmap_f16(&o.tmAhi, w.Bhi, 3, dims, str, boxa);
+      make_tmap_f16(&o.tmAlo, w.Blo, 3, dims, str, boxa);
+    }
+    {
+      const uint64_t dims[2] = {(uint64_t)w.kp, (uint64_t)w.kp};
+      const uint64_t str[1] = {(uint64_t)w.kp * 2};
+      const uint32_t box[2] = {64, 128};
+      make_tmap_f16(&o.tmLhi, w.orthLhi, 2, dims, str, box);
+      make_tmap_f16(&o.tmLlo, w.orthLlo, 2, dims, str, box);
+    }
+    const int steps = panels * (rpp / 64), nb = (w.kp + 127) / 128;
+    o.part = w.orthPart; o.l_exp = w.orthExp; o.out32 = nullptr; o.ld = c.k; o.k = c.k; o.kp = w.kp; o.rpp = rpp; o.panels = panels;
+    o.n_chunks = (steps + tc::OW_GRAM_STEPS - 1) / tc::OW_GRAM_STEPS;
+    o.out_exp = ilog2_floor((long long)rpp * panels) / 2;
+    o.status = w.status;
+    oc.push_back(o);
+    o.out32 = want_fp32 ? (token_side ? w.S : w.Z) : nullptr;
+    oc_last.push_back(o);
+    ct.push_back({w.orthPart, o.n_chunks, c.k, w.kp, w.cholW, w.cholW + (size_t)c.k * c.k, w.orthLhi, w.orthLlo, w.orthExp, w.status, 1e-10, nullptr, 0.0, nullptr, nullptr});
+    {
+      // the raw basis may be as ill-conditioned as the cache: where the single-precision Gram is too coarse for a pivot, the
+      // Gram is taken again in fp64 from the fp32 rows the sweep left (the second pass starts from a conditioned basis)
+      CholTask r = ct.back();
+      ct.back().redo = w.orthExp + 1; ct.back().redo_rel = kOrthRedoRel;
+      r.only = w.orthExp + 1; r.A64 = w.Gs;
+      ct_redo.push_back(r);
+      tg.push_back({token_side ? w.S : w.Z, rpp * panels, c.k, w.gpart, w.Gs, w.orthExp + 1});
+    }
+    max_chunks = std::max(max_chunks, o.n_chunks);
+    max_tiles = std::max(max_tiles, panels * (rpp / 128));
+    max_pairs = std::max(max_pairs, nb * (nb + 1) / 2); max_k = std::max(max_k, c.k);
+    w.split_ready = token_side ? 1 : 2;
+  }
+  const size_t o_oc = P.push(oc), o_ocl = P.push(oc_last), o_ct = P.push(ct), o_ctr = P.push(ct_redo);
+  const int n = (int)idx.size();
+  for (int pass = 0; pass < passes; ++pass) {
+    const size_t o_app = pass + 1 == passes ? o_ocl : o_oc;
+    P.add(stage, [=](char *dev_t, cudaStream_t s) {
+      tc::orthw_gram_kernel<<<dim3(max_chunks, max_pairs, n), tc::OW_THREADS, tc::OW_GRAM_SMEM, s>>>((const tc::OrthWCell *)(dev_t + o_oc)); LAUNCHED();
+      chol_cluster_launch((const CholTask *)(dev_t + o_ct), n, max_k, s); g_launches += 2;
+    });
+    if (pass == 0) {
+      add_tall_gram(P, stage, tg);
+      P.add(stage, [=](char *dev_t, cudaStream_t s) { chol_cluster_launch((const CholTask *)(dev_t + o_ctr), n, max_k, s); g_launches += 2; });
+    }
+    P.add(stage, [=](char *dev_t, cudaStream_t s) {
+      tc::orthw_apply_kernel<<<dim3(max_tiles, n), tc::OW_THREADS, tc::OW_APPLY_SMEM, s>>>((const tc::OrthWCell *)(dev_t + o_app)); LAUNCHED();
+    });
+  }
 }
 
 inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side, int passes,
@@ -460,9 +567,7 @@ inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const 
     cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN));
     attr_done = true;
   }
-  // the sweep left the raw basis as fp32 rows: measure its magnitude, split it into the operand layout
-  std::vector<tc::AbsMaxJob> am;
-  std::vector<tc::SplitJob> sp;
+  add_orth_split(P, stage, ws, idx, token_side);
   std::vector<tc::OrthCell> oc, oc_last;      // the fp32 rows of Q are only written by the last pass, and only if someone reads them
   std::vector<tc::CholInvTask> ci;
   int max_chunks = 0, max_tiles = 0, max_kp = 0, max_k = 0;
@@ -471,13 +576,6 @@ inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const 
     const CellDesc &c = w.c;
     const int rpp = token_side ? c.T : kD, panels = token_side ? 1 : c.m;
     float *src = token_side ? w.S : w.Z;
-    unsigned *slot = w.orthMax + (w.orthMaxUsed++ % kOrthMaxSlots);
-    if (!w.absmax_ready) am.push_back({src, (long long)rpp * panels * c.k, slot});      // else the sweep's epilogue measured it
-    w.absmax_ready = false;
-    tc::SplitJob j;
-    j.in = src; j.hi = w.Bhi; j.lo = w.Blo; j.batch = panels; j.rows = rpp; j.cols = c.k; j.ld_in = c.k; j.kp = w.kp; j.scale_exp = 0;
-    j.absmax = slot;
-    sp.push_back(j);
     tc::OrthCell o;
     memset(&o, 0, sizeof o);
     {
@@ -509,15 +607,8 @@ inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const 
     max_kp = std::max(max_kp, w.kp); max_k = std::max(max_k, c.k);
     w.split_ready = token_side ? 1 : 2;
   }
-  const size_t o_am = P.push(am), o_oc = P.push(oc), o_ocl = P.push(oc_last), o_ci = P.push(ci);
-  const int n = (int)idx.size(), n_am = (int)am.size();
-  {
-    const size_t o_sp = P.push(sp);
-    P.add(stage, [=](char *dev_t, cudaStream_t s) {
-      if (n_am) { tc::absmax_kernel<<<dim3(32, n_am), 256, 0, s>>>((const tc::AbsMaxJob *)(dev_t + o_am)); LAUNCHED(); }
-      tc::split_transpose_kernel<<<dim3(148, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + o_sp)); LAUNCHED();
-    });
-  }
+  const size_t o_oc = P.push(oc), o_ocl = P.push(oc_last), o_ci = P.push(ci);
+  const int n = (int)idx.size();
   const uint32_t tile = (uint32_t)max_kp * 128u;
   const int g_stages = std::max(2, std::min(6, (int)((tc::OR_SMEM_LIMIT - 16384 - 2048) / (2 * tile))));
   const size_t g_smem = (size_t)g_stages * 2 * tile + 16384 + 1024 + 1024;

@@ -22,6 +22,8 @@
 #include "block_jacobi.cuh"
 #include "eig_tridiag.cuh"
 #include "tc_orth.cuh"
+#include "tc_orth_wide.cuh"
+#include "chol_cluster.cuh"
 #include "rope.cuh"
 #include "attend.cuh"
 
@@ -491,6 +493,7 @@ struct CellWork {      // device scratch of one cell
   __half *Bhi = nullptr, *Blo = nullptr;
   // CholeskyQR on tensor cores: Gram partials, L^-1 as fp16 hi + lo, its exponent, slots for measured magnitudes
   float *orthPart = nullptr; __half *orthLhi = nullptr, *orthLlo = nullptr; int *orthExp = nullptr;
+  double *cholW = nullptr;                     // cluster Cholesky of wide sketches: work matrix and panels
   unsigned *orthMax = nullptr; int orthMaxUsed = 0; bool absmax_ready = false;
   int split_ready = 0;       // 1 / 2: Bhi, Blo already hold the split of S / Z (written by the last triangular solve)
 };
@@ -541,9 +544,11 @@ void carve(Bump &b, CellWork &w, int mode, bool need_backbone_scratch) {
         const size_t nb = std::max((size_t)c.m * w.kp * kD, (size_t)w.kp * T);
         w.Bhi = b.take<__half>(nb); w.Blo = b.take<__half>(nb);
         if (tok_segments(c.T) > 1) w.Zpart = b.take<float>((size_t)tok_segments(c.T) * c.m * kD * k);
-        if (w.ufI && k <= 152 && w.kp <= 160) {
-          const size_t steps = std::max((size_t)T / 64, (size_t)c.m * 2);
-          w.orthPart = b.take<float>(((steps + 7) / 8) * w.kp * w.kp);
+        if (w.ufI && k <= kCholClMaxN) {
+          const bool wide = k > tc::OR_MAX_K || w.kp > tc::OR_MAX_KP;
+          const size_t steps = std::max((size_t)T / 64, (size_t)c.m * 2), per = wide ? tc::OW_GRAM_STEPS : tc::OR_STEPS_PER_CTA;
+          w.orthPart = b.take<float>(((steps + per - 1) / per) * w.kp * w.kp);
+          if (wide) w.cholW = b.take<double>(chol_scratch_doubles((int)k));
           w.orthLhi = b.take<__half>((size_t)w.kp * w.kp); w.orthLlo = b.take<__half>((size_t)w.kp * w.kp);
           w.orthExp = b.take<int>(4); w.orthMax = b.take<unsigned>(kOrthMaxSlots);
         }
@@ -567,13 +572,15 @@ void carve(Bump &b, CellWork &w, int mode, bool need_backbone_scratch) {
   }
 }
 
+struct TallGram { const float *M; int rows, k; double *part, *out; const int *only = nullptr; };
+void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs);
+
 }  // namespace
 #include "fast_path.cuh"
 namespace {
 
 // G = M^T M (k x k, fp64) of tall fp32 matrices, split over row chunks so that the grid fills the GPU;
 // the partials are summed in a fixed order.
-struct TallGram { const float *M; int rows, k; double *part, *out; };
 void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs) {
   std::vector<ReduceJob> rj;
   std::vector<TallGramJob> fastj[6];        // register-tiled kernel, column blocks of width <= 48 / 96 / 144; +3: off-diagonal blocks
@@ -586,9 +593,9 @@ void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs) {
     const int cls = bw <= 48 ? 0 : (bw <= 96 ? 1 : 2);
     for (int bi = 0; bi < nb; ++bi)
       for (int bj = 0; bj <= bi; ++bj)
-        fastj[cls + (bi == bj ? 0 : 3)].push_back({j.M, j.rows, j.k, chunk, j.part, bi * bw, std::min(bw, j.k - bi * bw), bj * bw, std::min(bw, j.k - bj * bw)});
+        fastj[cls + (bi == bj ? 0 : 3)].push_back({j.M, j.rows, j.k, chunk, j.part, bi * bw, std::min(bw, j.k - bi * bw), bj * bw, std::min(bw, j.k - bj * bw), j.only});
     fast_chunks[cls] = std::max(fast_chunks[cls], n);
-    rj.push_back({j.part, j.out, n, j.k * j.k});
+    rj.push_back({j.part, j.out, n, j.k * j.k, j.only});
   }
   for (int q = 0; q < 6; ++q) {
     if (fastj[q].empty()) continue;
@@ -616,10 +623,11 @@ void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs) {
 // orth(S) for every active cell by CholeskyQR2: twice {Gs = S^T S (fp64), Gs = L L^T, S <- S L^-T}.
 // token_side selects S (T rows) or Z (N rows); the result is left in the source buffer.
 void add_orth(Program &P, int stage, std::vector<CellWork> &ws, bool token_side, int passes, bool final_basis = false) {
-  std::vector<int> on_tc;
+  std::vector<int> on_tc[2];
   if (g_fast.load() & 32)
-    for (size_t i = 0; i < ws.size(); ++i) if (orth_tc_ok(ws[i])) on_tc.push_back((int)i);
-  add_orth_tc(P, stage, ws, on_tc, token_side, passes, final_basis);
+    for (size_t i = 0; i < ws.size(); ++i) if (orth_tc_ok(ws[i])) on_tc[orth_is_wide(ws[i])].push_back((int)i);
+  add_orth_tc(P, stage, ws, on_tc[0], token_side, passes, final_basis);
+  add_orth_wide(P, stage, ws, on_tc[1], token_side, passes, final_basis);
   for (int pass = 0; pass < 2; ++pass) {
     // cls 0: Cholesky work matrix and L^T resident in shared memory (k <= kCholSmemMaxN); cls 1: both in global memory
     std::vector<TallGram> tg;

@@ -493,9 +493,10 @@ __global__ void __launch_bounds__(RB / 2) trsm_rows_kernel(const TrsmJob *__rest
 }
 
 // sum of fp64 partials with a per-job element count
-struct ReduceJob { const double *parts; double *out; int count, n_elems; };
+struct ReduceJob { const double *parts; double *out; int count, n_elems; const int *only; };      // only: nothing is done unless *only (null: always)
 __global__ void reduce_partials_var_kernel(const ReduceJob *__restrict__ jobs) {
   const ReduceJob j = jobs[blockIdx.y];
+  if (j.only && !*j.only) return;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < j.n_elems; e += gridDim.x * blockDim.x) {
     double s = 0;
     for (int h = 0; h < j.count; ++h) s += j.parts[(size_t)h * j.n_elems + e];
@@ -509,11 +510,12 @@ __global__ void reduce_partials_var_kernel(const ReduceJob *__restrict__ jobs) {
 // through shared memory 16 at a time (converted to fp64 once, on the way in).
 // One job = one block (columns [ca, ca+wa) x [cb, cb+wb)) of the k x k Gram; k <= 16 TI takes a single block,
 // wider matrices the lower-triangular blocks, whose results are also written mirrored.
-struct TallGramJob { const float *M; int rows, k, chunk; double *part; int ca, wa, cb, wb; };
+struct TallGramJob { const float *M; int rows, k, chunk; double *part; int ca, wa, cb, wb; const int *only; };
 
 template <int TI, bool SAME>      // SAME: diagonal block (ca == cb), one staged tile serves both operands
 __global__ void __launch_bounds__(256, 1) tall_gram_kernel(const TallGramJob *__restrict__ jobs) {
   const TallGramJob t = jobs[blockIdx.y];
+  if (t.only && !*t.only) return;
   const int r_begin = blockIdx.x * t.chunk;
   if (r_begin >= t.rows) return;
   const int r_end = min(t.rows, r_begin + t.chunk);

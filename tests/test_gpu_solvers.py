@@ -65,3 +65,24 @@ def test_exact_token_factor_matches_lapack(B, T):
         r = 24 if c == 0 else 12
         assert np.linalg.norm(UT[c][:, :r] @ UT[c][:, :r].T - U[:, :r] @ U[:, :r].T) <= 1e-4
         assert np.abs(UT[c].T @ UT[c] - np.eye(UT[c].shape[1])).max() <= 1e-5   # a full basis, null directions included
+
+
+# sketch width = rank + 10: one accumulator up to 152, blocks of 128 columns beyond (edges of the blocks), panels of 32 in the Cholesky
+@pytest.mark.parametrize("r_t", [142, 143, 150, 246, 247, 256, 374, 375, 502, 503])
+def test_wide_choleskyqr_matches_cuda_core_path(B, r_t):
+    T = 768
+    K, V = _cache(T, 6, 40, 0.05, 1).half(), _cache(T, 6, 700, 0.3, 2).half()
+    K[:, :, :, 64:] = 0          # rank deficient beyond 384 directions: dead pivots in the Gram of the token basis
+    plan = [(r_t // 16 * 16 if r_t > 374 else r_t, 128, 4), (r_t, 128, 4)]
+    sig, UT = _solve(B, K, V, plan, 255 - 32)
+    sig2, UT2 = _solve(B, K, V, plan, 255)
+    for c in range(2):
+        r = plan[c][0] if c else min(plan[c][0], 384)
+        # the flat tail of a sketch with the width of the rank depends on the test matrix; compare down to the widest gap
+        # both bases are single precision (hi + lo 22 bits, fp32 accumulation): 2^-20 of the square root of the contraction
+        assert np.abs(UT2[c][:, :r].T @ UT2[c][:, :r] - np.eye(r)).max() <= 2e-5
+        n = int((sig[c][4:r - 1] / sig[c][5:r]).argmax()) + 5                      # the widest relative gap behind the first
+        assert np.abs(sig2[c] - sig[c])[:n].max() <= 1e-5 * sig[c][0]
+        energy = (sig[c][:r] ** 2).sum()
+        assert abs((sig2[c][:r] ** 2).sum() - energy) <= 1e-6 * energy             # no direction of the range is lost
+        assert np.linalg.norm(UT[c][:, :n] @ UT[c][:, :n].T - UT2[c][:, :n] @ UT2[c][:, :n].T) <= 1e-3
