@@ -227,8 +227,9 @@ int jolt_serialize(const jolt_handle *h, void *host_dst, int64_t cap, void *stre
 int jolt_deserialize(const void *host_src, int64_t bytes, void *stream, jolt_handle **out);
 
 /* Release a handle and all buffers it owns.  NULL is accepted.  The compressed buffers are returned to the
- * stream-ordered pool after the last call that read them (ordered on that call's stream; if that stream no longer
- * exists, after the device has gone idle), so a decode that is still running keeps its data. */
+ * library after the last call that read them (ordered on that call's stream; if that stream no longer
+ * exists, after the device has gone idle), so a decode that is still running keeps its data.  The library keeps the memory
+ * of at most three freed handles per device for the next ones (jolt_release_workspace frees it). */
 int jolt_free(jolt_handle *h);
 
 /* Stored bytes of the compressed cache: factors + core + packed codes + scales, i.e. Eq. (1) plus
@@ -273,7 +274,8 @@ int jolt_eps2_table(double out[9]);
 int jolt_sketch_host(uint64_t seed, int32_t cell, int32_t stream_id, int64_t n_rows, int32_t n_cols, float *out);
 int jolt_signs_host(uint64_t seed, int32_t cell, float out[128]);
 
-/* Free cached device workspace held by the library for the current device. */
+/* Free what the library keeps for the current device between calls: the workspace, the argument tables and the memory of
+ * up to three freed handles that jolt_compress / jolt_deserialize would use again. */
 int jolt_release_workspace(void);
 
 /* Number of kernel launches the library has issued since load (all streams). */

@@ -103,6 +103,7 @@ extern "C" int jolt_decompress_static(const jolt_handle *H, const jolt_layout *L
   // words (the handle's) start at zero.
   H->last_stream = st;
   CU(cudaMemsetAsync(d_status, 0, sizeof(int) * 4 * nc, st));
+  H->status_epoch = 0;
   if (!P.host.empty()) CU(cudaMemcpyAsync(d_tab, P.host.data(), P.host.size(), cudaMemcpyHostToDevice, st));
   for (auto &s : P.steps) s.run(d_tab, st);
   CU(cudaGetLastError());

@@ -86,73 +86,6 @@ inline void add_backbone_tc(Program &P, int stage, const std::vector<tc::BBCell>
   });
 }
 
-inline void add_decode_tc(Program &P, int stage, std::vector<tc::BBCell> cells, uint64_t seed) {
-  if (cells.empty()) return;
-  using LY = tc::DecLayout;
-  static bool attr_done = false;
-  static int n_sm = 0;
-  if (!attr_done) {
-    cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<false, 0x11Fu>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x11Fu>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x110u>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x010u>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x100u>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x014u>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    cudaFuncSetAttribute(tc::decode_persistent_kernel<true, 0x018u>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    attr_done = true;
-  }
-  // persistent form: every cell with r_t <= 128, the same sequence length and no rotation of keys at decode.  It is
-  // instantiated per output mode and per set of bit widths: with at most two tile loops compiled in (and fp16 output
-  // through bulk tensor stores only) ptxas keeps the whole epilogue in registers; with three or more it spills 50-60
-  // bytes, and a spill reload inside the tile loop costs several per cent of the launch.
-  bool persistent = (g_fast.load() & 128) != 0 && n_sm > 0, tma_only = true;
-  unsigned bitmask = 0;
-  long long total = 0;
-  for (auto &c : cells) {
-    if (c.r_t > 128 || c.T != cells[0].T) persistent = false;
-    if (c.rope) persistent = false;
-    if (!(c.tma_out != 0 && c.out_dtype == DT_F16)) tma_only = false;
-    bitmask |= 1u << c.bits;
-    c.tile_base = (int)total;
-    total += (long long)c.m * (c.T / 128);
-  }
-  if (total >= (1ll << 30)) persistent = false;
-  int gx = 0;
-  for (auto &c : cells) gx = std::max(gx, c.m * c.items_per_head);
-  const int nt = cells[0].T / 128, tot = (int)total;
-  const size_t off = P.push(cells);
-  const int n = (int)cells.size();
-  const int grid_p = (int)std::min<long long>(n_sm, total);
-  // The persistent kernel takes a fixed contiguous share per CTA and can hand a tail of the list out in chunks through
-  // a counter (zero at every launch: it travels in the argument table).  The tail is empty unless a test asks for one: measured on the
-  // benchmark mix, a 5 % tail in 8-tile chunks made the launch slower (0.199 against 0.192 ms), because every chunk
-  // reloads its head's projected core into the single P buffer and restarts the unpack -> rotation pipeline.
-  const size_t off_cnt = P.push(std::vector<int>(4, 0));
-  std::vector<int2> run0(std::max(grid_p, 1), make_int2(tot, tot));
-  const int pool = (int)((long long)tot * (100 - g_dec_tail_pct.load()) / 100), chunk = std::max(1, g_dec_tail_chunk.load());
-  for (int i = 0; i < grid_p; ++i) run0[i] = make_int2((int)((long long)pool * i / grid_p), (int)((long long)pool * (i + 1) / grid_p));
-  const size_t off_run0 = P.push(run0);
-  P.add(stage, [=](char *dev_t, cudaStream_t s) {
-    if (persistent) {
-      tc::DecPArgs a{(const tc::BBCell *)(dev_t + off), n, nt, tot, seed, (const int2 *)(dev_t + off_run0), pool, chunk, (int *)(dev_t + off_cnt)};
-      if (tma_only && bitmask == 0x010u) tc::decode_persistent_kernel<true, 0x010u><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else if (tma_only && bitmask == 0x100u) tc::decode_persistent_kernel<true, 0x100u><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else if (tma_only && (bitmask & ~0x110u) == 0) tc::decode_persistent_kernel<true, 0x110u><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else if (tma_only && (bitmask & ~0x014u) == 0) tc::decode_persistent_kernel<true, 0x014u><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else if (tma_only && (bitmask & ~0x018u) == 0) tc::decode_persistent_kernel<true, 0x018u><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else if (tma_only) tc::decode_persistent_kernel<true, 0x11Fu><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-      else tc::decode_persistent_kernel<false, 0x11Fu><<<grid_p, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
-    } else {
-      tc::decode_kernel<<<dim3(gx, n), LY::THREADS, LY::SMEM_BYTES, s>>>((const tc::BBCell *)(dev_t + off), seed);
-    }
-    LAUNCHED();
-  });
-}
-
 inline void fill_bb_common(tc::BBCell &b, const CellStore &cs, int *status) {
   memset(&b, 0, sizeof b);
   b.tmUT = cs.tmUT; b.tmP = cs.tmP;
@@ -162,6 +95,78 @@ inline void fill_bb_common(tc::BBCell &b, const CellStore &cs, int *status) {
   b.status = status;
 }
 
+
+// Per-item decode kernel: cells of r_t > 128, keys rotated at decode, and every cell when the persistent kernel is off.
+inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, cudaStream_t s) {
+  using LY = tc::DecLayout;
+  static std::once_flag once;
+  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  tc::DecIArgs a;
+  memset(&a, 0, sizeof a);
+  a.out = out; a.cells = (const tc::BBCell *)H->d_dec + first; a.rope = rope; a.seed = H->seed;
+#ifdef JOLT_DEBUG
+  a.dbg = dbg;
+#else
+  (void)dbg;
+#endif
+  int heads = 0, m_max = 0;
+  for (int i = first; i < first + n; ++i) { heads += H->dec.m[i]; m_max = std::max(m_max, H->dec.m[i]); }
+  bb_split(heads, H->T / 128, a.tiles_per_item, a.items_per_head);
+  tc::decode_kernel<<<dim3(m_max * a.items_per_head, n), LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+  LAUNCHED();
+}
+
+template <bool TMA_ONLY, unsigned BITMASK>
+inline void launch_decode_p(const tc::DecPArgs &a, int grid, cudaStream_t s) {
+  using LY = tc::DecLayout;
+  static std::once_flag once;
+  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  tc::decode_persistent_kernel<TMA_ONLY, BITMASK><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+}
+
+// The persistent kernel is instantiated per output mode and per set of bit widths: with at most two tile loops compiled
+// in (and fp16 output through bulk tensor stores only) ptxas keeps the whole epilogue in registers; with three or more
+// it spills 50-60 bytes, and a spill reload inside the tile loop costs several per cent of the launch.
+inline void launch_decode_widths(const tc::DecPArgs &a, unsigned bitmask, int grid, cudaStream_t s) {
+  const bool tma_only = a.out.tma_out != 0 && a.out.out_dtype == DT_F16;
+  if (!tma_only) launch_decode_p<false, 0x11Fu>(a, grid, s);
+  else if (bitmask == 0x010u) launch_decode_p<true, 0x010u>(a, grid, s);
+  else if (bitmask == 0x100u) launch_decode_p<true, 0x100u>(a, grid, s);
+  else if ((bitmask & ~0x110u) == 0) launch_decode_p<true, 0x110u>(a, grid, s);
+  else if ((bitmask & ~0x014u) == 0) launch_decode_p<true, 0x014u>(a, grid, s);
+  else if ((bitmask & ~0x018u) == 0) launch_decode_p<true, 0x018u>(a, grid, s);
+  else launch_decode_p<true, 0x11Fu>(a, grid, s);
+}
+
+// Descriptors of the cells that take the tensor-core decode, in the order [values, r_t <= 128][keys, r_t <= 128][r_t > 128]
+// and in each class the costliest first (most residual bits, then largest r_t: the last wave of per-item CTAs is then the
+// cheapest).  The persistent kernel takes the first two classes in one launch, or only the first when keys are rotated.
+inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
+  table.clear();
+  H.dec = jolt_handle::DecTable();
+  long long total = 0;
+  for (int cls = 0; cls < 3; ++cls) {
+    std::vector<tc::BBCell> v;
+    for (size_t i = 0; i < H.cells.size(); ++i) {
+      const CellStore &cs = H.cells[i];
+      if (!cs.tc_ok || cls != (cs.c.r_t > 128 ? 2 : (i % 2 == 0 ? 1 : 0))) continue;
+      tc::BBCell b;
+      fill_bb_common(b, cs, H.d_status + 4 * i);
+      b.layer0 = H.group_start[i / 2];
+      v.push_back(b);
+    }
+    std::stable_sort(v.begin(), v.end(), [](const tc::BBCell &x, const tc::BBCell &y) { return x.bits != y.bits ? x.bits > y.bits : x.r_t > y.r_t; });
+    for (auto &b : v) {
+      b.tile_base = (int)std::min<long long>(total, 1 << 30);
+      total += (long long)b.m * (b.T / 128);
+      for (int q = cls; q < 2; ++q) H.dec.bitmask[q] |= 1u << b.bits;
+      H.dec.m.push_back(b.m);
+    }
+    table.insert(table.end(), v.begin(), v.end());
+    H.dec.end[cls] = (int)table.size();
+    H.dec.tiles[cls] = total;
+  }
+}
 
 // ------------------------------------------------------------------ tensor-core sweeps of the factor stage
 

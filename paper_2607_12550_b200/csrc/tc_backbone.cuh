@@ -28,9 +28,7 @@ struct alignas(64) BBCell {
   CUtensorMap tmUT;     // fp16 [T][r_t]           dims {r_t, T},       box {64, 128}
   CUtensorMap tmP;      // fp16 [m*r_t][128]       dims {128, m*r_t},   box {64, r_t}
   CUtensorMap tmX;      // fp16 [L][n_h][T][128]   dims {128, T, n_h, L}, box {64, 128, 1, 1}   (RESIDUAL)
-  CUtensorMap tmOut;    // same shape over the output tensor (DECODE, fp16 destinations TMA can address)
-  CUtensorMap tmOutW;   // the output tensor again with box {64, 32, 1, 1}: the 32 rows one warp stages and stores
-  int tma_out;
+  int tma_out;          // DECODE: filled in from the launch's destination (DecOut)
   long long *dbg;       // optional: cycle stamps of CTA 0 (profiling aid), 8 per tile per warpgroup
   uint32_t *words;      // [m][T][4*bits]
   __half *scales;       // [m][T][4]
@@ -41,6 +39,7 @@ struct alignas(64) BBCell {
   int m, n_heads, T, r_t, r_f, bits, cell;
   int tiles_per_item, items_per_head;
   int tile_base;        // persistent decode: first tile of this cell in the launch's linear (cell, head, tile) order
+  int layer0;           // DECODE: first layer of the cell in the destination
   int *status;
   const float2 *rope;   // DECODE of key cells: (cos, sin) of feature pair j at token t in rope[j * T + t]; null = no rotation
 };

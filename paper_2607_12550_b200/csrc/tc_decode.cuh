@@ -45,6 +45,20 @@ struct DecLayout {
   static constexpr int PROD_REGS = 56;
 };
 
+// where a decode writes: one destination for the keys, one for the values of all cells
+struct DecOut {
+  CUtensorMap tm[2];   // [L][n_h][T][128] fp16, box {64, 32, 1, 1}: the 32 rows one warp stages and stores (tma_out)
+  char *base[2];
+  long long osl, osh, ost;
+  int out_dtype, tma_out;
+};
+
+__device__ __forceinline__ void dec_fill_out(BBCell &c, const DecOut &o) {      // the destination's part of a staged descriptor
+  c.out = o.base[c.cell & 1] + (long long)c.layer0 * o.osl * (o.out_dtype == DT_F16 ? 2 : 4);
+  c.osl = o.osl; c.osh = o.osh; c.ost = o.ost;
+  c.out_dtype = o.out_dtype; c.tma_out = o.tma_out;
+}
+
 template <int BITS>
 struct DecCodesRow { uint32_t words[BITS > 0 ? 4 * BITS : 1]; uint2 sc; };
 
@@ -298,7 +312,7 @@ __device__ __forceinline__ void dec_build_rotation(unsigned char *smH, uint64_t 
 struct DecCtx {
   uint32_t bTfull, bTempty, bRready, bHready, t_acc, s_obuf;
   unsigned char *rbuf, *obuf, *smH;
-  const BBCell *cg;       // the descriptor in global memory: tensor maps are addressed there
+  const DecOut *out;      // kernel argument: the destination
   volatile int *abort_flag;
   int wg, nwg, rit, h, tile0, n_tiles, l, hd;
   int ex;                 // core exponent: loaded at kernel start, first USED after the rotation operand is built
@@ -314,6 +328,8 @@ __device__ __forceinline__ bool dec_tile_loop(const BBCell &c, const DecCtx &x) 
   DecCodes<BITS> cur, nxt;
   bool ok = true;
   const bool tma_out = c.tma_out != 0;
+  const int lane = x.rit & 31, wrow0 = x.rit & ~31;
+  const uint32_t s_wrows = x.s_obuf + (uint32_t)wrow0 * 128u;
   if (x.wg < x.n_tiles) dec_load_codes<BITS>(c, (long long)x.h * c.T + (x.tile0 + x.wg) * 128 + x.rit, cur);
   dec_build_rotation(x.smH, x.seed, c.cell, x.wg * 128 + x.rit, x.bHready);     // the first codes are in flight meanwhile
   const DecScales sc = dec_scales(x.ex);
@@ -323,9 +339,9 @@ __device__ __forceinline__ bool dec_tile_loop(const BBCell &c, const DecCtx &x) 
     const int token = tt * 128 + x.rit;
     JOLT_DBG(long long *dbg = stamp ? c.dbg + (size_t)i * 8 : nullptr;)
     JOLT_DBG(if (dbg) dbg[0] = clock64();)
-    if (tma_out) {   // the operand tile doubles as staging buffer: the previous store must have read it first
-      if (x.rit == 0) tma_store_wait_read();
-      named_bar_sync(1 + x.wg, 128);
+    if (tma_out) {   // the warp's rows of the operand tile double as its staging rows: the previous store must have read them
+      if (lane == 0) tma_store_wait_read();
+      __syncwarp();
     }
     JOLT_DBG(if (dbg) dbg[1] = clock64();)
     if constexpr (BITS > 0) {
@@ -377,18 +393,18 @@ __device__ __forceinline__ bool dec_tile_loop(const BBCell &c, const DecCtx &x) 
     JOLT_DBG(if (dbg) dbg[5] = clock64();)
     if (tma_out) {
       fence_proxy_async();
-      named_bar_sync(1 + x.wg, 128);
+      __syncwarp();
       JOLT_DBG(if (dbg) dbg[6] = clock64();)
-      if (x.rit == 0 && ok) {
-        tma_store_4d(&x.cg->tmOut, x.s_obuf, 0, tt * 128, x.hd, x.l);
-        tma_store_4d(&x.cg->tmOut, x.s_obuf + 16384, 64, tt * 128, x.hd, x.l);
+      if (lane == 0 && ok) {
+        tma_store_4d(&x.out->tm[c.cell & 1], s_wrows, 0, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
+        tma_store_4d(&x.out->tm[c.cell & 1], s_wrows + 16384, 64, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
         tma_store_commit();
       }
     }
     JOLT_DBG(if (dbg) dbg[7] = clock64();)
     if constexpr (BITS > 0) cur = nxt;
   }
-  if (tma_out && x.rit == 0) tma_store_wait_all();
+  if (tma_out && lane == 0) tma_store_wait_all();
   return ok;
 }
 
@@ -467,8 +483,8 @@ __device__ __forceinline__ bool dec_tile_loop_acc4(const BBCell &c, const DecCtx
           __syncwarp();
           JOLT_DBG(if (dbg) dbg[5] = clock64();)
           if (lane == 0) {
-            tma_store_4d(&x.cg->tmOutW, s_wrows, 0, tt * 128 + wrow0, x.hd, x.l);
-            tma_store_4d(&x.cg->tmOutW, s_wrows + 16384, 64, tt * 128 + wrow0, x.hd, x.l);
+            tma_store_4d(&x.out->tm[c.cell & 1], s_wrows, 0, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
+            tma_store_4d(&x.out->tm[c.cell & 1], s_wrows + 16384, 64, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
             tma_store_commit();
           }
         } else {
@@ -598,8 +614,8 @@ __device__ __forceinline__ bool dec_tile_loop_acc4_rope(const BBCell &c, const D
       __syncwarp();
       JOLT_DBG(if (dbg) dbg[5] = clock64();)
       if (lane == 0) {
-        tma_store_4d(&x.cg->tmOutW, s_wrows, 0, tt * 128 + wrow0, x.hd, x.l);
-        tma_store_4d(&x.cg->tmOutW, s_wrows + 16384, 64, tt * 128 + wrow0, x.hd, x.l);
+        tma_store_4d(&x.out->tm[c.cell & 1], s_wrows, 0, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
+        tma_store_4d(&x.out->tm[c.cell & 1], s_wrows + 16384, 64, tt * 128 + wrow0, x.hd, c.layer0 + x.l);
         tma_store_commit();
       }
     } else if (ok && c.out_dtype == DT_F16) {
@@ -622,7 +638,18 @@ __device__ __forceinline__ bool dec_tile_loop_acc4_rope(const BBCell &c, const D
   return ok;
 }
 
-__global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const BBCell *__restrict__ cells, uint64_t seed) {
+struct DecIArgs {
+  DecOut out;
+  const BBCell *cells;                        // grid.y of them
+  const float2 *rope;                         // (cos, sin) table of the key cells, or null (BBCell::rope)
+  uint64_t seed;
+  int tiles_per_item, items_per_head;
+#ifdef JOLT_DEBUG
+  long long *dbg;
+#endif
+};
+
+__global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __grid_constant__ DecIArgs a) {
   using LY = DecLayout;
   constexpr int NWG = DEC_NWG;
   constexpr int DEC_P_BYTES = LY::P_BYTES, DEC_BIG_BYTES = LY::BIG_BYTES, DEC_NS = LY::NS;
@@ -630,8 +657,9 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const BBC
   // The cell's descriptor is read from global memory ONCE, cooperatively, into shared memory: the scalar fields are
   // used all over the kernel and each first touch from global would be a dependent L2 round trip on the critical
   // path of the CTA's start.  Only the tensor maps are addressed in global memory (the copy engine requires that).
-  const BBCell &cg = cells[blockIdx.y];
-  const int items_per_head = cg.items_per_head, tiles_per_item = cg.tiles_per_item, n_tok_tiles = cg.T / 128;
+  const BBCell &cg = a.cells[blockIdx.y];
+  const uint64_t seed = a.seed;
+  const int items_per_head = a.items_per_head, tiles_per_item = a.tiles_per_item, n_tok_tiles = cg.T / 128;
   if ((int)blockIdx.x >= cg.m * items_per_head) return;
   const int h = blockIdx.x / items_per_head;
   const int item = blockIdx.x - h * items_per_head;
@@ -658,7 +686,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const BBC
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wg = warp >> 2;
-  JOLT_DBG(long long *kdbg = (cg.dbg && blockIdx.x == 0 && blockIdx.y == gridDim.y / 2 && threadIdx.x == 0) ? cg.dbg + 16 * 8 : nullptr;)
+  JOLT_DBG(long long *kdbg = (a.dbg && blockIdx.x == 0 && blockIdx.y == gridDim.y / 2 && threadIdx.x == 0) ? a.dbg + 16 * 8 : nullptr;)
   JOLT_DBG(if (kdbg) { kdbg[0] = clock64(); long long gt; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(gt)); kdbg[6] = gt; })
   BBCell *sc_cell = (BBCell *)(sm + DEC_P_BYTES + DEC_H_BYTES + DEC_BIG_BYTES + 512);
   for (int i = threadIdx.x; i < (int)(sizeof(BBCell) / 16); i += LY::THREADS) ((uint4 *)sc_cell)[i] = __ldg((const uint4 *)&cg + i);
@@ -674,6 +702,11 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const BBC
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (threadIdx.x == 0) {      // read by the epilogue warpgroups after their own named barrier
+    dec_fill_out(*sc_cell, a.out);
+    sc_cell->rope = (sc_cell->cell & 1) == 0 && sc_cell->r_t <= 128 ? a.rope : nullptr;
+    JOLT_DBG(sc_cell->dbg = a.dbg;)
+  }
   const uint32_t tmem_base = *tmem_slot;
   JOLT_DBG(if (kdbg) kdbg[1] = clock64();)
   const BBCell &c = *sc_cell;            // scalar fields from here on; tensor maps through cg
@@ -781,9 +814,10 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const BBC
     const int q = warp & 3;
     const int rit = q * 32 + lane;                 // row in tile
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
+    named_bar_sync(1, NWG * 128);                  // the destination's part of the descriptor is in
     {
       DecCtx x;
-      x.cg = &cg;
+      x.out = &a.out;
       x.ex = *c.e;             // requested now, first used after the rotation operand is built
       x.bTfull = bTfull(wg); x.bTempty = bTempty(wg); x.bRready = bRready(wg); x.bHready = bHready;
       x.t_acc = t_lane + wg * 128; x.rbuf = smR + wg * 32768; x.smH = smH; x.seed = seed;

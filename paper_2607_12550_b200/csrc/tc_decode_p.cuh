@@ -17,7 +17,7 @@
 // then converts and stores the second 64 features of tile i while the rotation of i + 2 runs.
 //
 // What changes at a boundary:
-//   head   the projected core P_h (one 32 KB buffer; the 32 KB next to it is the staging region): a thread of its own
+//   head   the projected core P_h (one buffer): a thread of its own
 //          requests the next head's block once the backbone thread has released the buffer (a commit barrier) and
 //          asks for the block after that to be brought into L2.  The backbone thread runs up to two tiles ahead of the
 //          rotation, which absorbs most of the reload; the U_T ring (four stages) is indifferent to heads.
@@ -25,8 +25,9 @@
 //          rotation MMAs of the old cell are complete by then: each warpgroup has read its last accumulator), copy
 //          the new descriptor, rebuild the rotation operand and re-enter the tile loop compiled for the new bit
 //          width.  A CTA's share touches two cells at most once in a while; cells are never interleaved.
-// Launches with a cell of r_t > 128 (its P block needs the whole P region), with keys rotated at decode, or with
-// mixed sequence lengths take the per-item kernel.
+// Cells of r_t > 128 (their P block needs the whole P region) and keys rotated at decode take the per-item kernel.  A
+// layout with 64 KB for P and a ring of two U_T stages was tried for r_t > 128: the ring of two cannot cover the loads
+// (0.345 ms against 0.29 ms per-item for the eleven such cells of a 8192-token cache).
 #pragma once
 #include "tc_decode.cuh"
 
@@ -34,15 +35,19 @@ namespace jolt {
 namespace tc {
 
 struct DecPArgs {
+  DecOut out;
   const BBCell *cells;
   int n_cells;
-  int nt;              // 128-token tiles per head (all cells of a launch share T)
+  int nt;              // 128-token tiles per head (all cells of a handle share T)
   int total;           // tiles of the launch
   uint64_t seed;
-  const int2 *run0;    // per CTA: [first, end) of its fixed share
-  int pool;            // tiles from here on are handed out in chunks ...
+  int pool;            // tiles [0, pool) are dealt out in equal shares; from here on in chunks ...
   int chunk;           // ... of this many tiles
-  int *counter;        // chunks handed out so far (zero at launch)
+  int *counter;        // chunks handed out so far (zero at launch when pool < total; not read otherwise)
+  int epoch;           // a failed wait writes (epoch << 8 | 8) into the status word of the first cell
+#ifdef JOLT_DEBUG
+  long long *dbg;
+#endif
 };
 
 // linear tile p of the launch -> (cell, head, tile in head); cells[].tile_base is the first linear tile of a cell
@@ -66,12 +71,14 @@ __device__ __forceinline__ void dec_acc_of(int j, int &b, int &nb) {
 }
 
 struct DecPCtx {
-  uint32_t bTfull, bTempty, bRready;      // of accumulator 0 of this warpgroup; accumulator 1 sixteen bytes further
-  uint32_t t_acc, s_stg;
+  uint32_t bTfull;                        // of accumulator 0 of this warpgroup; accumulator 1 sixteen bytes further
+  __device__ __forceinline__ uint32_t bTempty() const { return bTfull + 32; }       // (a live register each would spill)
+  __device__ __forceinline__ uint32_t bRready() const { return bTfull + 64; }
+  uint32_t t_acc;
   unsigned char *rbuf, *stg;              // the warpgroup's operand tile; the warp's 32 staging rows (128 bytes each)
-  const BBCell *cg;                       // the cell's descriptor in global memory (tensor maps)
+  const DecOut *out;                      // kernel argument: the destination
   volatile int *abort_flag;
-  int wg, rit;
+  int rit;
   int nt, base;                           // tiles per head; first linear tile of the cell
   int joff;                               // tile p of the current run is the CTA's tile number j = p + joff
   int ex;
@@ -110,7 +117,7 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
       fence_proxy_async();
     }
     // (a cell without residual arrives all the same: the barrier's phases then count tiles, whatever the cells hold)
-    mbar_arrive(x.bRready + 16 * (((p0 + x.joff) >> 1) & 1));
+    mbar_arrive(x.bRready() + 16 * (((p0 + x.joff) >> 1) & 1));
     if constexpr (BITS > 0) {
       if (p0 + 2 < p_end) { dec_load_codes<BITS>(c, (long long)hl * c.T + tl * 128 + x.rit, cur); advance(hl, tl); }
     }
@@ -131,7 +138,7 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
       tmem_ld32(t_acc + half * 64, va[0]);
       tmem_ld32(t_acc + half * 64 + 32, va[1]);
       tmem_wait_ld();
-      if (half == 1) { tc_fence_before(); mbar_arrive(x.bTempty + 16 * acc); }
+      if (half == 1) { tc_fence_before(); mbar_arrive(x.bTempty() + 16 * acc); }
       if (!f16) {
         float4 *pf = (float4 *)((float *)c.out + (long long)l * c.osl + (long long)hd * c.osh + (long long)(tt * 128 + x.rit) * c.ost) + half * 16;
 #pragma unroll
@@ -159,7 +166,7 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) {
-          tma_store_4d(&x.cg->tmOutW, x.s_stg, half * 64, tt * 128 + wrow0, hd, l);
+          tma_store_4d(&x.out->tm[c.cell & 1], smem_u32(x.stg), half * 64, tt * 128 + wrow0, hd, c.layer0 + l);
           tma_store_commit();
         }
         pending = true;
@@ -185,7 +192,7 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
             dec_unpack_row<BITS>(cur, sc.pre, x.rbuf, x.rit);
             fence_proxy_async();
           }
-          mbar_arrive(x.bRready + 16 * (acc ^ 1));
+          mbar_arrive(x.bRready() + 16 * (acc ^ 1));
           if constexpr (BITS > 0) {
             if (p + 4 < p_end) { dec_load_codes<BITS>(c, (long long)hl * c.T + tl * 128 + x.rit, cur); advance(hl, tl); }
           }
@@ -234,27 +241,27 @@ struct DecRunQ {
 // BITMASK: bit b set = the tile loop for b-bit cells is compiled in (a launch takes the smallest instantiated superset
 // of its cells' bit widths: fewer tile loops, a smaller instruction footprint)
 template <bool TMA_ONLY, unsigned BITMASK>
-__global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kernel(const DecPArgs a) {
+__global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kernel(const __grid_constant__ DecPArgs a) {
   using LY = DecLayout;
   constexpr int NWG = DEC_NWG, NS = LY::NS;
   extern __shared__ unsigned char smem_raw[];
   const BBCell *cells = a.cells;
   const int nt = a.nt, total = a.total;
-  const int2 my_run0 = a.run0[blockIdx.x];
-  const int run0_first = my_run0.x, run0_end = my_run0.y;
   const int pool = a.pool;
-  JOLT_DBG(long long *cta_dbg = cells[0].dbg ? cells[0].dbg + 128 + blockIdx.x * 4 : nullptr;)
+  const int run0_first = (int)((long long)pool * blockIdx.x / gridDim.x), run0_end = (int)((long long)pool * (blockIdx.x + 1) / gridDim.x);
+  JOLT_DBG(long long *cta_dbg = a.dbg ? a.dbg + 128 + blockIdx.x * 4 : nullptr;)
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; unsigned sm; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)); cta_dbg[0] = g; cta_dbg[2] = sm; })
 
   // shared memory: P block (32 KB) | output staging (2 x 16 KB) | rotation operand H | U_T ring | operand tiles | barriers
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char *sm = smem_raw + (base - raw);
-  const uint32_t sP = base, sStg = base + 32768u, sH = base + LY::P_BYTES, sBig = sH + DEC_H_BYTES;
-  const uint32_t sRing = sBig, sR = sBig + NS * BB_STAGE_BYTES;
-  const uint32_t sBar = sBig + LY::BIG_BYTES;
-  unsigned char *smStg = sm + 32768, *smH = sm + LY::P_BYTES, *smR = sm + LY::P_BYTES + DEC_H_BYTES + NS * BB_STAGE_BYTES;
-  unsigned char *smBar = sm + LY::P_BYTES + DEC_H_BYTES + LY::BIG_BYTES;
+  constexpr uint32_t OFF_STG = 32768u, OFF_H = OFF_STG + 32768u, OFF_RING = OFF_H + DEC_H_BYTES, OFF_R = OFF_RING + NS * BB_STAGE_BYTES, OFF_BAR = OFF_R + 65536u;
+  const uint32_t sP = base, sH = base + OFF_H;
+  const uint32_t sRing = base + OFF_RING, sR = base + OFF_R;
+  const uint32_t sBar = base + OFF_BAR;
+  unsigned char *smStg = sm + OFF_STG, *smH = sm + OFF_H, *smR = sm + OFF_R;
+  unsigned char *smBar = sm + OFF_BAR;
   volatile int *abort_flag = (volatile int *)(smBar + 256);
   uint32_t *tmem_slot = (uint32_t *)(smBar + 264);
   DecRunQ runq{(volatile int *)(smBar + 272), total, abort_flag};      // 8 slots of 16 bytes
@@ -297,7 +304,9 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
       int cnt = 0, ci = 0;
       bool ok = true;
       int first = run0_first, end = run0_end;
-      int next_chunk = atomicAdd(a.counter, 1);      // asked for one run ahead; read when the run starts
+      // asked for one run ahead, read when the run starts; without a tail the counter is not touched (nobody cleared it)
+      auto take_chunk = [&] { return pool < total ? atomicAdd(a.counter, 1) : 1 << 30; };
+      int next_chunk = take_chunk();
       int k = 0;
       for (;; ++k) {
         if (k >= 1) {
@@ -305,7 +314,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           end = min(total, first + a.chunk);
           runq.publish(k, first, end);
           if (first >= total) break;
-          next_chunk = atomicAdd(a.counter, 1);
+          next_chunk = take_chunk();
         }
         int left = end - first;
         if (left <= 0) continue;
@@ -481,6 +490,11 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           named_bar_sync(1, NWG * 128);
           for (int i = et; i < (int)(sizeof(BBCell) / 16); i += NWG * 128) ((uint4 *)sc_cell)[i] = __ldg((const uint4 *)&cg + i);
           named_bar_sync(1, NWG * 128);
+          if (et == 0) {
+            dec_fill_out(*sc_cell, a.out);
+            JOLT_DBG(sc_cell->dbg = a.dbg;)
+          }
+          named_bar_sync(1, NWG * 128);
           dec_build_rotation(smH, a.seed, sc_cell->cell, et, bHready);
           cur_ci = ci;
         }
@@ -489,12 +503,12 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
         const int cell_end = min(end, cell_last);
         if (ok) {
           DecPCtx x;
-          x.cg = &cg;
+          x.out = &a.out;
           x.ex = *c.e;
-          x.bTfull = bTfull(wg); x.bTempty = bTempty(wg); x.bRready = bRready(wg);
+          x.bTfull = bTfull(wg);
           x.t_acc = t_lane + wg * 128; x.rbuf = smR + wg * 32768;
-          x.s_stg = sStg + (uint32_t)(wg * 16384 + qd * 4096); x.stg = smStg + wg * 16384 + qd * 4096;
-          x.abort_flag = abort_flag; x.wg = wg; x.rit = rit; x.nt = nt; x.base = c.tile_base; x.joff = j - p;
+          x.stg = smStg + wg * 16384 + qd * 4096;
+          x.abort_flag = abort_flag; x.rit = rit; x.nt = nt; x.base = c.tile_base; x.joff = j - p;
           const int p0 = p + (((j & 1) == wg) ? 0 : 1);      // this warpgroup's first tile of the piece
           int rcode = pending ? 2 : 0;      // a bit width that is not compiled in: reported as a failed launch
           const int bits = c.bits;
@@ -518,7 +532,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   __syncthreads();
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); cta_dbg[1] = g; cta_dbg[3] = 0; })
   if (*abort_flag) {
-    if (threadIdx.x == 0) atomicOr(cells[0].status, 8);
+    if (threadIdx.x == 0) atomicMax(cells[0].status, a.epoch << 8 | 8);
     const long long t0 = clock64();
     while (clock64() - t0 < 2000000) {}      // let copies still in flight land before the CTA's memory is reused
     __syncthreads();

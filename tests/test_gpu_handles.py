@@ -1,0 +1,90 @@
+"""Decode of caches whose cells fall into different kernel classes, and the memory of freed handles used again."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    entry.build()
+    import paper_2607_12550_b200 as pkg
+    return pkg.load()
+
+
+def _cache(layers, heads, T, seed, dtype=torch.float16):
+    g = torch.Generator().manual_seed(seed)
+    P = torch.randn(T, 24, generator=g) / torch.arange(1, 25)
+    mk = lambda: (torch.einsum("tr,lhfr->lhtf", P, torch.randn(layers, heads, 128, 24, generator=g)) + 0.1 * torch.randn(layers, heads, T, 128, generator=g)).to(dtype).cuda()
+    return mk(), mk()
+
+
+# keys / values of r_t <= 128, above 128, and ranks the tensor-core kernels do not take, in one call
+@pytest.mark.parametrize("plans", [
+    [(64, 128, 4), (144, 128, 2), (160, 96, 8), (128, 128, 3)],
+    [(48, 64, 2), (32, 128, 4), (50, 128, 4), (176, 128, 1)],
+    [(144, 128, 4), (256, 128, 0), (256, 128, 4), (160, 128, 8)],
+    [(16, 16, 1), (0, 0, 4), (64, 128, 2), (0, 0, 2)],
+])
+@pytest.mark.parametrize("rope", [False, True])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
+def test_mixed_cells_decode_like_the_portable_kernels(B, plans, rope, dtype):
+    K, V = _cache(3, 2, 384, 5)
+    gs = [0, 2, 3]
+    h = B.jolt_compress(K, V, gs, plans, B.default_options(seed=4))
+    outs = []
+    for mask in (0, 255, 255 - 128):
+        prev = B.set_fast_path(mask)
+        try:
+            Ko, Vo = (torch.full(K.shape, float("nan"), dtype=dtype, device="cuda") for _ in range(2))
+            for _ in range(2):
+                if rope:
+                    B.jolt_decompress_rope(h, Ko, Vo, gs, base=10000.0, pos0=17)
+                else:
+                    B.jolt_decompress(h, Ko, Vo, gs)
+                B.check_status(h)
+            outs.append((Ko.float(), Vo.float()))
+        finally:
+            B.set_fast_path(prev)
+    # fp16 rounding of the output (twice where keys are rotated by the separate pass) and of the residual operand
+    for a, b in zip(outs[0], outs[1]):
+        assert float((a - b).norm() / a.norm()) <= 1e-3
+    for a, b in zip(outs[1], outs[2]):
+        assert float((a - b).norm() / a.norm()) <= 5e-4
+    h.free()
+
+
+def test_memory_of_freed_handles_is_used_again_in_order(B):
+    """Handles made, decoded and freed in turn on two streams without a host wait between: every decode sees its own cache."""
+    gs = [0, 2, 4]
+    plans = [(64, 128, 4), (32, 128, 4)] * 2
+    caches = [_cache(4, 4, 1024, 20 + i) for i in range(4)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    opts = B.default_options(seed=4)
+    want = []
+    for K, V in caches:
+        h = B.jolt_compress(K, V, gs, plans, opts)
+        o = torch.empty_like(K), torch.empty_like(V)
+        B.jolt_decompress(h, *o, gs)
+        torch.cuda.synchronize()
+        want.append(o)
+        h.free()
+    got = []
+    for i in range(12):
+        st = streams[i % 2]
+        h = B.jolt_compress(*caches[i % 4], gs, plans, opts, stream=st)
+        o = torch.empty_like(caches[0][0]), torch.empty_like(caches[0][1])
+        B.jolt_decompress(h, *o, gs, stream=st)
+        h.free()                                   # the decode may still be running
+        got.append(o)
+    torch.cuda.synchronize()
+    for i, o in enumerate(got):
+        assert torch.equal(o[0], want[i % 4][0]) and torch.equal(o[1], want[i % 4][1]), i
+    B.release_workspace()
+    h = B.jolt_compress(*caches[1], gs, plans, opts)
+    B.jolt_decompress(h, *got[0], gs)
+    torch.cuda.synchronize()
+    assert torch.equal(got[0][0], want[1][0])
+    h.free()
