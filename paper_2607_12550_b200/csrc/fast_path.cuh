@@ -323,20 +323,25 @@ inline void add_tok_tc(Program &P, int stage, std::vector<CellWork> &ws, const s
     }
     std::vector<std::pair<int, int>> ch;
     sketch_chunks(w.kp, ch);
-    if (ch.size() == 1 && (g_fast.load() & 64)) {
-      // one column chunk: two token tiles per CTA share every operand tile
-      tc::Gemm2Cell g;
-      memset(&g, 0, sizeof g);
-      const uint64_t dims[3] = {(uint64_t)kD, (uint64_t)w.kp, (uint64_t)c.m};
-      const uint64_t str[2] = {(uint64_t)kD * 2, (uint64_t)w.kp * kD * 2};
-      const uint32_t box[3] = {64, (uint32_t)w.kp, 1};
-      bool okm = make_x_map4(&g.tmX, c, 256, 1) && make_tmap_f16(&g.tmBhi, w.Bhi, 3, dims, str, box) &&
-                 make_tmap_f16(&g.tmBlo, w.Blo, 3, dims, str, box);
-      (void)okm;
-      g.C = w.S; g.ldc = c.k; g.ncols = c.k; g.kp = w.kp; g.has_lo = src[i] != 0; g.scale_exp = se;
-      g.m = c.m; g.n_heads = c.n_heads; g.T = c.T; g.status = w.status;
-      if (orth_tc_ok(w)) { g.absmax = w.orthMax + (w.orthMaxUsed % kOrthMaxSlots); w.absmax_ready = true; }
-      gc2.push_back(g);
+    if (g_fast.load() & 64) {
+      // two token tiles per CTA share every operand tile
+      if (orth_tc_ok(w)) w.absmax_ready = true;
+      for (auto &cc : ch) {
+        const int c0 = cc.first, kc = cc.second;
+        if (c0 >= c.k) break;
+        tc::Gemm2Cell g;
+        memset(&g, 0, sizeof g);
+        const uint64_t dims[3] = {(uint64_t)kD, (uint64_t)kc, (uint64_t)c.m};
+        const uint64_t str[2] = {(uint64_t)kD * 2, (uint64_t)w.kp * kD * 2};
+        const uint32_t box[3] = {64, (uint32_t)kc, 1};
+        bool okm = make_x_map4(&g.tmX, c, 256, 1) && make_tmap_f16(&g.tmBhi, w.Bhi + (size_t)c0 * kD, 3, dims, str, box) &&
+                   make_tmap_f16(&g.tmBlo, w.Blo + (size_t)c0 * kD, 3, dims, str, box);
+        (void)okm;
+        g.C = w.S + c0; g.ldc = c.k; g.ncols = std::min(kc, c.k - c0); g.kp = kc; g.has_lo = src[i] != 0; g.scale_exp = se;
+        g.m = c.m; g.n_heads = c.n_heads; g.T = c.T; g.status = w.status;
+        if (w.absmax_ready) g.absmax = w.orthMax + (w.orthMaxUsed % kOrthMaxSlots);
+        gc2.push_back(g);
+      }
       continue;
     }
     for (auto &cc : ch) {
@@ -378,26 +383,32 @@ inline void add_feat_tc(Program &P, int stage, std::vector<CellWork> &ws) {
     w.split_ready = 0;
     std::vector<std::pair<int, int>> ch;
     sketch_chunks(w.kp, ch);
-    if (ch.size() == 1 && c.n_heads % 2 == 0 && (g_fast.load() & 64)) {
-      // one column chunk: two heads of a layer per CTA share every tile of Q
-      tc::Gemm2Cell g;
-      memset(&g, 0, sizeof g);
-      const uint64_t dims[2] = {(uint64_t)c.T, (uint64_t)w.kp};
-      const uint64_t str[1] = {(uint64_t)c.T * 2};
-      const uint32_t box[2] = {64, (uint32_t)w.kp};
-      bool okm = make_x_map4(&g.tmX, c, 64, 2) && make_tmap_f16(&g.tmBhi, w.Bhi, 2, dims, str, box) &&
-                 make_tmap_f16(&g.tmBlo, w.Blo, 2, dims, str, box);
-      (void)okm;
-      g.ldc = c.k; g.ncols = c.k; g.kp = w.kp; g.has_lo = 1; g.scale_exp = se;
-      g.m = c.m; g.n_heads = c.n_heads; g.T = c.T; g.status = w.status;
+    if (c.n_heads % 2 == 0 && (g_fast.load() & 64)) {
+      // two heads of a layer per CTA share every tile of Q
       const int nseg = tok_segments(c.T);
-      if (nseg == 1 && orth_tc_ok(w)) { g.absmax = w.orthMax + (w.orthMaxUsed % kOrthMaxSlots); w.absmax_ready = true; }
-      for (int sg = 0; sg < nseg; ++sg) {
-        g.C = nseg > 1 ? w.Zpart + (size_t)sg * c.m * kD * c.k : w.Zp;
-        g.t0 = sg * kTokSegment; g.n_tok = std::min(kTokSegment, c.T - g.t0);
-        gc2.push_back(g);
+      if (orth_tc_ok(w)) w.absmax_ready = true;
+      unsigned *slot = w.absmax_ready ? w.orthMax + (w.orthMaxUsed % kOrthMaxSlots) : nullptr;
+      for (auto &cc : ch) {
+        const int c0 = cc.first, kc = cc.second;
+        if (c0 >= c.k) break;
+        tc::Gemm2Cell g;
+        memset(&g, 0, sizeof g);
+        const uint64_t dims[2] = {(uint64_t)c.T, (uint64_t)kc};
+        const uint64_t str[1] = {(uint64_t)c.T * 2};
+        const uint32_t box[2] = {64, (uint32_t)kc};
+        bool okm = make_x_map4(&g.tmX, c, 64, 2) && make_tmap_f16(&g.tmBhi, w.Bhi + (size_t)c0 * c.T, 2, dims, str, box) &&
+                   make_tmap_f16(&g.tmBlo, w.Blo + (size_t)c0 * c.T, 2, dims, str, box);
+        (void)okm;
+        g.ldc = c.k; g.ncols = std::min(kc, c.k - c0); g.kp = kc; g.has_lo = 1; g.scale_exp = se;
+        g.m = c.m; g.n_heads = c.n_heads; g.T = c.T; g.status = w.status;
+        g.absmax = nseg == 1 ? slot : nullptr;
+        for (int sg = 0; sg < nseg; ++sg) {
+          g.C = (nseg > 1 ? w.Zpart + (size_t)sg * c.m * kD * c.k : w.Zp) + c0;
+          g.t0 = sg * kTokSegment; g.n_tok = std::min(kTokSegment, c.T - g.t0);
+          gc2.push_back(g);
+        }
       }
-      if (nseg > 1) sums.push_back({w.Zpart, w.Zp, (long long)c.m * kD * c.k, (long long)c.m * kD * c.k, nseg});
+      if (nseg > 1) sums.push_back({w.Zpart, w.Zp, (long long)c.m * kD * c.k, (long long)c.m * kD * c.k, nseg, slot});
       continue;
     }
     for (auto &cc : ch) {
@@ -420,7 +431,7 @@ inline void add_feat_tc(Program &P, int stage, std::vector<CellWork> &ws) {
         gc.push_back(g);
       }
     }
-    if (tok_segments(c.T) > 1) sums.push_back({w.Zpart, w.Zp, (long long)c.m * kD * c.k, (long long)c.m * kD * c.k, tok_segments(c.T)});
+    if (tok_segments(c.T) > 1) sums.push_back({w.Zpart, w.Zp, (long long)c.m * kD * c.k, (long long)c.m * kD * c.k, tok_segments(c.T), nullptr});
   }
   launch_split(P, stage, sp);
   launch_tc_gemm<tc::GM_FEAT>(P, stage, gc);

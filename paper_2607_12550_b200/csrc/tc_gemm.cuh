@@ -182,7 +182,8 @@ struct alignas(64) Gemm2Cell {
   CUtensorMap tmBhi;    // as in GemmCell
   CUtensorMap tmBlo;
   float *C;             // TOK: S [T][ldc];  FEAT: Z' [m][128][ldc]
-  int ldc, ncols, kp, has_lo, scale_exp;
+  int ldc, ncols;       // row pitch and columns of this launch item (fewer than ldc: a column chunk of a wide sketch)
+  int kp, has_lo, scale_exp;
   int m, n_heads, T;
   int t0, n_tok;        // FEAT: token range
   unsigned *absmax;     // optional
@@ -289,7 +290,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm2_kernel(const Gemm2Cell
     const uint32_t t_lane = tmem_base + ((uint32_t)(warp * 32) << 16);
     const float scale = ldexpf(1.0f, -c.scale_exp);
     const int ncols = c.ncols, ldc = c.ldc;
-    float *stg = (float *)sm;                        // every stage has been consumed: [128][ldc] staging tile
+    float *stg = (float *)sm;                        // every stage has been consumed: [128][ncols] staging tile
     float amax = 0.f;
     for (int sub = 0; sub < n_sub; ++sub) {
       if (ok) {
@@ -299,15 +300,23 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm2_kernel(const Gemm2Cell
           tmem_wait_ld();
 #pragma unroll
           for (int j = 0; j < 32; ++j)
-            if (ch * 32 + j < ncols) { const float x = v[j] * scale; stg[row * ldc + ch * 32 + j] = x; amax = fmaxf(amax, fabsf(x)); }
+            if (ch * 32 + j < ncols) { const float x = v[j] * scale; stg[row * ncols + ch * 32 + j] = x; amax = fmaxf(amax, fabsf(x)); }
         }
       }
       named_bar_sync(1, 128);
       if (ok && !*abort_flag) {
-        // the tile's 128 rows are one contiguous block of the output (row pitch ldc = ncols)
         float *dst = c.C + (size_t)(2 * item + sub) * 128 * ldc;
-        const int total = 128 * ldc;
-        if (((((uintptr_t)dst) & 15) == 0) && (total & 3) == 0) {
+        const int total = 128 * ncols;
+        if (ldc != ncols) {            // a column chunk of a wider result: row by row, 8-byte pieces (the chunk starts at a multiple of 16)
+          if (((ldc | ncols) & 1) == 0 && (((uintptr_t)dst) & 7) == 0) {
+            const int n2 = ncols >> 1;
+            for (int r = warp; r < 128; r += 4)
+              for (int e = lane; e < n2; e += 32) ((float2 *)(dst + (size_t)r * ldc))[e] = ((const float2 *)(stg + r * ncols))[e];
+          } else {
+            for (int r = warp; r < 128; r += 4)
+              for (int e = lane; e < ncols; e += 32) dst[(size_t)r * ldc + e] = stg[r * ncols + e];
+          }
+        } else if (((((uintptr_t)dst) & 15) == 0) && (total & 3) == 0) {      // the 128 rows are one contiguous block of the output
           const float4 *s4 = (const float4 *)stg;
           float4 *d4 = (float4 *)dst;
           for (int e = threadIdx.x; e < total / 4; e += 128) d4[e] = s4[e];
@@ -402,13 +411,19 @@ __global__ void reduce_gram_partials_kernel(const float *const *partials, double
 }
 
 // out[e] = sum of `count` fp32 partials `stride` elements apart, added in fp64 in a fixed order
-struct SumJob { const float *part; float *out; long long n, stride; int count; };
+struct SumJob { const float *part; float *out; long long n, stride; int count; unsigned *absmax; };      // absmax: optional, largest |out|
 __global__ void sum_partials_f32_kernel(const SumJob *__restrict__ jobs) {
   const SumJob j = jobs[blockIdx.y];
+  float mx = 0.f;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < j.n; e += (long long)gridDim.x * blockDim.x) {
     double s = 0;
     for (int p = 0; p < j.count; ++p) s += (double)j.part[(size_t)p * j.stride + e];
     j.out[e] = (float)s;
+    mx = fmaxf(mx, fabsf((float)s));
+  }
+  if (j.absmax) {
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx > 0.f && isfinite(mx)) atomicMax(j.absmax, __float_as_uint(mx));
   }
 }
 
