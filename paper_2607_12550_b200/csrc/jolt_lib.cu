@@ -362,39 +362,50 @@ GemmTask mk(const void *A, int ta, long long a_rs, long long a_cs, const void *B
   memset(&t, 0, sizeof t);
   t.A = A; t.B = B; t.C = C; t.M = M; t.N = N; t.K = K; t.nseg = 1; t.seg_inner = 1;
   t.a_rs = a_rs; t.a_cs = a_cs; t.b_rs = b_rs; t.b_cs = b_cs; t.c_rs = c_rs; t.c_cs = 1;
-  t.ta = ta; t.tb = tb; t.tc = tc; t.alpha = 1.f; t.alpha_exp = nullptr; t.accumulate = 0;
+  t.ta = ta; t.tb = tb; t.tc = tc; t.alpha = 1.f; t.alpha_exp = nullptr; t.accumulate = 0; t.symmetric = 0;
   return t;
 }
 
 void add_gemm(Program &P, int stage, const std::vector<GemmTask> &all_tasks, bool f64) {
   if (all_tasks.empty()) return;
   // one launch per tile-count class: a grid sized for the largest task would start mostly empty CTAs for the rest.
-  // Plain fp32 tasks take the register-tiled kernel (128 x 64 tiles), everything else the generic one (64 x 64).
-  struct Bucket { long long key; bool fast; std::vector<GemmTask> tasks; };
+  // Plain fp32 tasks take the register-tiled kernel (128 x 64 tiles) when their tiles fill most of the machine; the rest
+  // take the generic one (64 x 64), whose clusters split K until about two CTAs per SM have work (at least four steps of
+  // 16 each: below that the exchange of the partial tiles costs more than it saves).
+  struct Bucket { long long key; bool fast; long long tiles; int steps; std::vector<GemmTask> tasks; };
   std::vector<Bucket> buckets;
+  long long sg_tiles = 0;
+  if (!f64)
+    for (auto &t : all_tasks)
+      if (t.M > 0 && t.N > 0 && sgemm_fast_ok(t)) sg_tiles += (long long)((t.M + 127) / 128) * ((t.N + 63) / 64);
   for (auto &t : all_tasks) {
     if (t.M <= 0 || t.N <= 0) continue;
-    const bool fastk = !f64 && sgemm_fast_ok(t);
+    const bool fastk = !f64 && sgemm_fast_ok(t) && (sg_tiles >= 100 || t.K < 128);
     const int bm = fastk ? 128 : 64;
-    const long long key = ((long long)((t.M + bm - 1) / bm) << 32) | (long long)((t.N + 63) / 64);
+    const long long tm = (t.M + bm - 1) / bm, tn = (t.N + 63) / 64;
+    const long long key = (tm << 32) | tn;
     size_t b = 0;
     for (; b < buckets.size(); ++b) if (buckets[b].key == key && buckets[b].fast == fastk) break;
-    if (b == buckets.size()) buckets.push_back({key, fastk, {}});
+    if (b == buckets.size()) buckets.push_back({key, fastk, 0, 1 << 30, {}});
     buckets[b].tasks.push_back(t);
+    buckets[b].tiles += t.symmetric ? tm * (tm + 1) / 2 : tm * tn;
+    buckets[b].steps = std::min(buckets[b].steps, t.nseg * ((t.K + 15) / 16));
   }
   for (auto &bk : buckets) {
     const std::vector<GemmTask> &tasks = bk.tasks;
     const int tm = (int)(bk.key >> 32), tn = (int)(bk.key & 0xffffffff);
     const bool fastk = bk.fast;
+    int S = 1;
+    while (S < 8 && bk.tiles * 2 * S <= 300 && bk.steps >= 8 * S) S *= 2;
     const size_t off = P.push(tasks);
     const int n = (int)tasks.size();
     P.add(stage, [=](char *dev, cudaStream_t s) {
       const GemmTask *d = (const GemmTask *)(dev + off);
       for (int z0 = 0; z0 < n; z0 += 32768) {
-        dim3 grid(tn, tm, std::min(32768, n - z0));
-        if (f64) simt_gemm_kernel<double><<<grid, 256, 0, s>>>(d + z0);
-        else if (fastk) simt_sgemm_kernel<<<grid, 256, 0, s>>>(d + z0);
-        else simt_gemm_kernel<float><<<grid, 256, 0, s>>>(d + z0);
+        const int nz = std::min(32768, n - z0);
+        if (f64) simt_gemm_launch<double>(d + z0, tn, tm, nz, S, s);
+        else if (fastk) simt_sgemm_kernel<<<dim3(tn, tm, nz), 256, 0, s>>>(d + z0);
+        else simt_gemm_launch<float>(d + z0, tn, tm, nz, S, s);
         LAUNCHED();
       }
     });
@@ -849,9 +860,11 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
       if (w.ufI) { idU.push_back(w.UF32); idLd.push_back(c.r_f); }
       if (w.ufI && !probe) { w.tc_gram = false; w.skip_feat = true; continue; }   // r_f = d: U_F = I, no Gram, no eigen-solve
       if (!w.tc_gram) {
-        for (int h = 0; h < c.m; ++h)
+        for (int h = 0; h < c.m; ++h) {
           g.push_back(mk(x_head(c, h), c.dtype, 1, c.st, x_head(c, h), c.dtype, c.st, 1, w.gram_part + (size_t)h * kD * kD,
                          DT_F64, kD, kD, kD, c.T));
+          g.back().symmetric = 1;
+        }
         parts.push_back(w.gram_part); outs.push_back(w.C); counts.push_back(c.m);
       }
       EigTask e; memset(&e, 0, sizeof e);
@@ -943,7 +956,7 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
         g1.push_back(mk(x_head(c, h), c.dtype, c.st, 1, w.UF32, DT_F32, c.r_f, 1, w.Y + (size_t)h * c.T * c.r_f, DT_F32,
                         c.r_f, c.T, c.r_f, kD));
       GemmTask t = mk(w.Y, DT_F32, c.r_f, 1, w.Y, DT_F32, 1, c.r_f, w.Gt, DT_F64, c.T, c.T, c.T, c.r_f);
-      t.nseg = c.m; t.seg_inner = c.m; t.a_si = (long long)c.T * c.r_f; t.b_si = (long long)c.T * c.r_f;
+      t.nseg = c.m; t.seg_inner = c.m; t.a_si = (long long)c.T * c.r_f; t.b_si = (long long)c.T * c.r_f; t.symmetric = 1;
       g2.push_back(t);
       EigTask e; memset(&e, 0, sizeof e);
       e.bjA = w.bjA; e.bjV = w.bjV; e.bjJ = w.bjJ; e.bjOff = w.bjOff; e.bjDone = w.bjDone; e.td = w.td;
