@@ -20,6 +20,7 @@
 #include "simt_gemm.cuh"
 #include "small_solvers.cuh"
 #include "block_jacobi.cuh"
+#include "cluster_jacobi.cuh"
 #include "eig_tridiag.cuh"
 #include "tc_orth.cuh"
 #include "tc_orth_wide.cuh"
@@ -417,8 +418,16 @@ void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sw
   std::vector<TdTask> td[2];               // tridiagonal solver: one CTA per matrix (n <= kTdSmallMaxN) / a cluster per matrix
   std::vector<EigTask> small;              // portable: Jacobi in one CTA's shared memory (n <= 32) / block Jacobi
   std::vector<BJTask> bj;
+  std::vector<CholFactorTask> cf;          // the probe's singular values: Cholesky factor (work matrix in global memory, n > 152) ...
+  std::vector<tc::CholInvTask> cfs;        // ... or in shared memory, then the cluster Jacobi on its columns
+  std::vector<CJTask> cj;
   for (auto &t : tasks) {
-    if (t.td) {
+    if (t.td && t.w_sqrt && !t.U_out && t.n > 32 && t.n <= kCJMaxN) {
+      double *L = t.td;                    // n * n + 1 doubles of the tridiagonal solver's scratch
+      if (t.n <= tc::kCholInvMaxN) cfs.push_back({nullptr, 0, 0, t.A, t.n, nullptr, nullptr, nullptr, L, t.status, 1e-13});
+      else cf.push_back({t.A, L, t.n, t.status});
+      cj.push_back({L, t.n, t.w_out, t.w_sqrt, t.status});
+    } else if (t.td) {
       TdTask q; memset(&q, 0, sizeof q);
       q.A = t.A; q.n = t.n; q.U_out = t.U_out; q.ld_out = t.ld_out; q.r_out = t.r_out; q.w_out = t.w_out; q.w_sqrt = t.w_sqrt; q.status = t.status;
       td_set_scratch(q, t.td);
@@ -433,6 +442,35 @@ void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sw
       b.tol = kBJTol;
       bj.push_back(b);
     }
+  }
+  if (!cfs.empty()) {
+    const size_t off = P.push(cfs);
+    const int n = (int)cfs.size();
+    int cmn = 0;
+    for (auto &c : cfs) cmn = std::max(cmn, c.k);
+    const size_t cshm = tc::cholinv_smem_bytes(cmn);
+    static std::once_flag once;
+    std::call_once(once, [] { cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN)); });
+    P.add(stage, [=](char *dev, cudaStream_t s) { tc::cholinv_kernel<<<n, tc::kCholInvThreads, cshm, s>>>((const tc::CholInvTask *)(dev + off)); LAUNCHED(); });
+  }
+  if (!cf.empty()) {
+    const size_t off = P.push(cf);
+    const int n = (int)cf.size();
+    int cmn = 0;
+    for (auto &c : cf) cmn = std::max(cmn, c.n);
+    const size_t cshm = std::max(chol_factor_smem_bytes(kCholFactorSmemN), chol_factor_smem_bytes(cmn));
+    static std::once_flag once;
+    std::call_once(once, [] { cudaFuncSetAttribute(chol_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 2048)); });
+    P.add(stage, [=](char *dev, cudaStream_t s) { chol_factor_kernel<<<n, kCholFactorThreads, cshm, s>>>((const CholFactorTask *)(dev + off)); LAUNCHED(); });
+  }
+  if (!cj.empty()) {
+    static std::once_flag once;
+    std::call_once(once, [] { cj_opt_in_smem(); });
+    int mn = 0;
+    for (auto &c : cj) mn = std::max(mn, c.n);
+    const int nr = cj_rows_per_lane(mn), nt = (int)cj.size();
+    const size_t off = P.push(cj);
+    P.add(stage, [=](char *dev, cudaStream_t s) { cj_launch((const CJTask *)(dev + off), nt, mn, nr, s); LAUNCHED(); });
   }
   for (auto &q : td) {
     if (q.empty()) continue;

@@ -86,3 +86,25 @@ def test_wide_choleskyqr_matches_cuda_core_path(B, r_t):
         energy = (sig[c][:r] ** 2).sum()
         assert abs((sig2[c][:r] ** 2).sum() - energy) <= 1e-6 * energy             # no direction of the range is lost
         assert np.linalg.norm(UT[c][:, :n] @ UT[c][:, :n].T - UT2[c][:, :n] @ UT2[c][:, :n].T) <= 1e-3
+
+
+# sketch width = cap + 10: portable up to 32, Cholesky in shared memory to 152, in global memory to 288, tridiagonal beyond
+@pytest.mark.parametrize("q_cap", [16, 32, 142, 144, 278, 279, 320])
+def test_probe_values_give_the_portable_plan(B, q_cap):
+    T = 640
+    K, V = _cache(T, 6, 40, 0.05, 1).half(), _cache(T, 6, 700, 0.3, 2).half()
+    raw = 2 * K.numel() * 2
+    opts = B.default_options(seed=3, power_iters=1, q_cap=q_cap)
+    got = []
+    for mask in (255 - 16, 255):
+        prev = B.set_fast_path(mask)
+        try:
+            sp = B.jolt_probe(K, V, [0, 1], 3.0, opts)
+            got.append([sp.plan(raw / r, opts) for r in (2.0, 3.0, 5.0)])
+            sp.free()
+        finally:
+            B.set_fast_path(prev)
+    for (p, a), (q, b) in zip(*got):
+        # values agree to some 1e-6 of the largest: a near-tie moves one cell by one step of the grid, and nothing else moves
+        assert sum(x != y for x, y in zip(p, q)) <= 1, (p, q)
+        assert all(abs(x[0] - y[0]) <= 16 and x[1] == y[1] and x[2] == y[2] for x, y in zip(p, q)), (p, q)
