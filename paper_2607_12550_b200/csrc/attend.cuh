@@ -11,20 +11,16 @@
 // so a call streams U_T and the packed codes once each (the compressed bytes) instead of the fp16 cache, and the
 // Hadamard rotation is applied to one query / one output row per head instead of every token.
 //
-// Kernels of a call (the contractions with a tensor-core shape are warp-level fp16 MMAs with fp32 accumulation, an fp32
+// Kernels of a call (contractions with a tensor-core shape are warp-level fp16 MMAs with fp32 accumulation, an fp32
 // operand entering as hi + lo fp16; the rest is CUDA-core fp32):
 //   (P_h = fp16(G_h U_F^T), the projected core the decoder also reads, is kept with the handle since compress)
 //   attend_prep_kernel     per (group, head, query): rotated scaled query (fp32, and scaled hi + lo fp16), w = P_h q
-//   attend_bscore_kernel   backbone scores U_T w of all heads of a cell as one dense product (U_T is shared by the heads)
-//   attend_scores_mma_kernel / attend_scores_kernel   per (group, head, 256-token chunk): residual scores added (codes
-//                          times rotated query: MMAs for 1-, 2-, 4- and 8-bit codes, CUDA cores for 3-bit codes and for
-//                          cells without a residual), chunk maximum, p = exp(s - max), chunk sum
-//   attend_values_mma_kernel / attend_values_kernel   per (group, head, chunk): sum_t p_t r^'_t (MMAs with M = features,
-//                          K = tokens over an fp16 tile of expanded codes for 1-, 2-, 4- and 8-bit codes; CUDA cores,
-//                          codes staged in shared memory and read feature-wise, for 3-bit codes)
-//   attend_bvalue_kernel   p^T U_T per chunk for all heads of a cell as one dense product
+//   attend_stream_kernel   per (group, head, 256-token chunk): scores, chunk maximum, p = exp(s - max), chunk sum,
+//                          sum_t p_t r^'_t and p^T U_T
 //   attend_combine_kernel  per (group, head, query): merges the chunks (running-maximum rescaling), applies P_h of the
 //                          value cell and the inverse rotation, divides by the softmax denominator
+// The portable path has four kernels in place of the streaming one: attend_bscore_kernel (U_T w of all heads of a cell as one
+// dense product), attend_scores_kernel, attend_values_kernel (codes on the CUDA cores), attend_bvalue_kernel (p^T U_T).
 // Keys compressed before a rotary embedding cannot use the first identity (the rotation differs per token).
 #pragma once
 #include <cuda_fp16.h>
@@ -58,23 +54,44 @@ struct AttendJob {                  // one per layer group
   float *qe;                        // [m][8]            2^E
   float *p;                         // [m][T][NQP]       exp(s - chunk maximum)
   float *ml;                        // [m][n_chunks][2][NQP]  chunk maximum, chunk sum
-  float *y;                         // [m][n_chunks][v.r_t][NQP]
-  float *a;                         // [m][n_chunks][128][NQP]
+  float *y;                         // [m][n_chunks][NQP][v.r_t]
+  float *a;                         // [m][n_chunks][NQP][128]
 };
 
-// 128-point Walsh-Hadamard transform of buf[0..127] by 128 threads (thread f owns element f on return).
-__device__ __forceinline__ float att_wht_smem(float *buf, int f) {
-  float v = buf[f];
+// 128-point Walsh-Hadamard transform by one warp: lane l holds elements 4 l .. 4 l + 3.
+__device__ __forceinline__ void att_wht_warp(float (&v)[4]) {
+  const int lane = threadIdx.x & 31;
+  float a = v[0] + v[1], b = v[0] - v[1], c = v[2] + v[3], d = v[2] - v[3];
+  v[0] = a + c; v[1] = b + d; v[2] = a - c; v[3] = b - d;
 #pragma unroll
-  for (int len = 1; len < 128; len <<= 1) {
-    const float o = buf[f ^ len];
-    __syncthreads();
-    v = (f & len) ? o - v : v + o;
-    buf[f] = v;
-    __syncthreads();
-  }
-  return v;
+  for (int len = 1; len < 32; len <<= 1)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float o = __shfl_xor_sync(0xffffffffu, v[j], len);
+      v[j] = lane & len ? o - v[j] : v[j] + o;
+    }
 }
+
+// Sums over the warp of N values a lane (4 or 8): the sum of value att_sum_index(lane) on return.
+template <int N>
+__device__ __forceinline__ float att_warp_sums(float (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = N; n > 1; n >>= 1, o >>= 1)
+#pragma unroll
+    for (int j = 0; j < n / 2; ++j) {
+      const float keep = lane & o ? v[j + n / 2] : v[j], give = lane & o ? v[j] : v[j + n / 2];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return v[0];
+}
+
+// A kernel launched while its predecessor still runs waits here before it reads what that one wrote.
+__device__ __forceinline__ void att_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void att_let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float att_sign(uint64_t seed, int cell, int f) {
   uint32_t sw[4];
@@ -82,85 +99,94 @@ __device__ __forceinline__ float att_sign(uint64_t seed, int cell, int f) {
   return ((sw[f >> 5] >> (f & 31)) & 1u) ? -1.f : 1.f;
 }
 
-// grid (m, groups, NQP), 128 threads (thread = feature), 128 floats of dynamic shared memory.  CTA z rotates query z
-// and forms every NQP-th group of four rows of w.
-__global__ void __launch_bounds__(128) attend_prep_kernel(const AttendJob *__restrict__ jobs, int n_q, int NQP, float scale,
-                                                          uint64_t seed) {
+// grid (m, groups), 256 threads: a warp per query rotates it (four features a lane), then a warp per row of P_h forms w with
+// four rows in flight.  Bound by the latency of its few loads: with a CTA per query, block-wide transforms and five shuffles
+// per value and row it took 19.6 us at 8 groups of 32 heads, rank 128; now 8.8.
+template <int NQ>
+__global__ void __launch_bounds__(256) attend_prep_kernel(const AttendJob *__restrict__ jobs, int n_q, float scale, uint64_t seed) {
   const AttendJob &jb = jobs[blockIdx.y];
-  const int h = blockIdx.x, f = threadIdx.x, i = blockIdx.z;
+  const int h = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (h >= jb.m) return;
-  extern __shared__ unsigned char att_smem[];
-  float *buf = (float *)att_smem;
-  if (jb.k.bits > 0) {
-    buf[f] = i < n_q ? att_sign(seed, jb.k.cell, f) * jb.q[((size_t)h * n_q + i) * 128 + f] : 0.f;
-    __syncthreads();
-    const float v = att_wht_smem(buf, f) * kInvSqrtD * scale;
-    jb.qt[((size_t)h * 128 + f) * NQP + i] = v;
+  att_let_successor_start();
+  const int kr = jb.k.r_t;
+  float q[NQ][4];
+#pragma unroll
+  for (int c = 0; c < NQ; ++c) {
+    const float4 v = c < n_q ? *(const float4 *)(jb.q + ((size_t)h * n_q + c) * 128 + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    q[c][0] = v.x; q[c][1] = v.y; q[c][2] = v.z; q[c][3] = v.w;
+  }
+  if (jb.k.bits > 0 && warp < NQ) {
+    const int i = warp;
+    float v[4];
+#pragma unroll
+    for (int c = 0; c < NQ; ++c)
+      if (c == i) { v[0] = q[c][0]; v[1] = q[c][1]; v[2] = q[c][2]; v[3] = q[c][3]; }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] *= att_sign(seed, jb.k.cell, lane * 4 + j);
+    att_wht_warp(v);
+    float mx = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[j] = v[j] * kInvSqrtD * scale;
+      jb.qt[((size_t)h * 128 + lane * 4 + j) * NQ + i] = v[j];
+      mx = fmaxf(mx, fabsf(v[j]));
+    }
     // the tensor-core form of the same row: scaled by a power of two so that hi + lo fp16 hold it (|entry| < 2^13)
-    __shared__ float wmax[4];
-    float mx = fabsf(v);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((f & 31) == 0) wmax[f >> 5] = mx;
-    __syncthreads();
-    mx = fmaxf(fmaxf(wmax[0], wmax[1]), fmaxf(wmax[2], wmax[3]));
     int ex = 0;
     if (mx > 0.f && mx < INFINITY) frexpf(mx, &ex);                  // mx < 2^ex
-    const float sv = ldexpf(v, 13 - ex);
-    const __half hi = __float2half_rn(sv);
-    jb.qh[((size_t)h * kAttMaxQ + i) * 128 + f] = hi;
-    jb.ql[((size_t)h * kAttMaxQ + i) * 128 + f] = __float2half_rn(sv - __half2float(hi));
-    if (f == 0) jb.qe[h * kAttMaxQ + i] = ldexpf(1.f, ex - 13);
+    const float up = ldexpf(1.f, 13 - ex);
+    __half hi[4], lo[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float sv = v[j] * up;
+      hi[j] = __float2half_rn(sv);
+      lo[j] = __float2half_rn(sv - __half2float(hi[j]));
+    }
+    *(uint2 *)(jb.qh + ((size_t)h * kAttMaxQ + i) * 128 + lane * 4) = *(const uint2 *)hi;
+    *(uint2 *)(jb.ql + ((size_t)h * kAttMaxQ + i) * 128 + lane * 4) = *(const uint2 *)lo;
+    if (lane == 0) jb.qe[h * kAttMaxQ + i] = ldexpf(1.f, ex - 13);
   }
-  if (jb.k.r_t > 0) {
+  if (kr > 0) {
     // w[n][k] = sum_f P_h[k][f] q[f] for column n = (head, query): a warp per row k, a lane per four features.  Stored as
     // hi + lo fp16 times 2^-E_n with 2^E_n > |q|_2: a row of P_h has norm below 2^14.52 (|G| 2^-e < 2^11, r_f <= 128, U_F
     // orthonormal, fp16 rounding), so every scaled entry is below 2^14.52 in magnitude and fits fp16.
-    const float se = scale * ldexpf(1.f, *jb.k.e);
-    const int warp = f >> 5, lane = f & 31;
-    float q[kAttMaxQ][4];
-    int ex[kAttMaxQ];
-    float inv[kAttMaxQ];
+    constexpr int RI = 4;                                              // rows in flight
+    const uint2 *pr = (const uint2 *)(jb.kP + (size_t)h * kr * 128) + lane;
+    uint2 p4[RI];
 #pragma unroll
-    for (int c = 0; c < kAttMaxQ; ++c) {
-      const float4 v = c < n_q ? *(const float4 *)(jb.q + ((size_t)h * n_q + c) * 128 + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      q[c][0] = v.x; q[c][1] = v.y; q[c][2] = v.z; q[c][3] = v.w;
-      float sq = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, v.w * v.w)));
+    for (int r = 0; r < RI; ++r) p4[r] = __ldg(pr + (size_t)min(warp * RI + r, kr - 1) * 32);
+    float sq[NQ];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-      const float nrm = sqrtf(sq);
-      ex[c] = 0;
-      if (nrm > 0.f && nrm < INFINITY) frexpf(nrm, &ex[c]);              // |q|_2 < 2^ex
-      ++ex[c];                                                          // headroom for the rounding of the norm itself
-      inv[c] = ldexpf(1.f, -ex[c]);
-    }
-    if (blockIdx.z == 0 && f < NQP) {
-      int e_f = 0;
+    for (int c = 0; c < NQ; ++c) sq[c] = fmaf(q[c][0], q[c][0], fmaf(q[c][1], q[c][1], fmaf(q[c][2], q[c][2], q[c][3] * q[c][3])));
+    const float nrm = sqrtf(att_warp_sums<NQ>(sq));
+    const int c = lane / (32 / NQ);                                    // this lane's query
+    int ex = 0;
+    if (nrm > 0.f && nrm < INFINITY) frexpf(nrm, &ex);                 // |q|_2 < 2^ex
+    ++ex;                                                              // headroom for the rounding of the norm itself
+    const float inv = ldexpf(1.f, -ex);
+    const bool first = lane % (32 / NQ) == 0;
+    if (warp == 0 && first) jb.we[h * NQ + c] = scale * ldexpf(1.f, *jb.k.e) * ldexpf(1.f, ex);
+    for (int k = warp * RI; k < kr; k += 8 * RI) {
+      uint2 pc[RI];
 #pragma unroll
-      for (int c = 0; c < kAttMaxQ; ++c)
-        if (c == f) e_f = ex[c];
-      jb.we[h * NQP + f] = se * ldexpf(1.f, e_f);
-    }
-    for (int k = warp + 4 * blockIdx.z; k < jb.k.r_t; k += 4 * gridDim.z) {
-      const uint2 p4 = __ldg((const uint2 *)(jb.kP + ((size_t)h * jb.k.r_t + k) * 128 + lane * 4));
-      const __half *ph = (const __half *)&p4;
-      const float p0 = __half2float(ph[0]), p1 = __half2float(ph[1]), p2 = __half2float(ph[2]), p3 = __half2float(ph[3]);
-      float v[kAttMaxQ];
+      for (int r = 0; r < RI; ++r) pc[r] = p4[r];
+      if (k + 8 * RI < kr)
 #pragma unroll
-      for (int c = 0; c < kAttMaxQ; ++c) v[c] = fmaf(p0, q[c][0], fmaf(p1, q[c][1], fmaf(p2, q[c][2], p3 * q[c][3])));
+        for (int r = 0; r < RI; ++r) p4[r] = __ldg(pr + (size_t)min(k + 8 * RI + r, kr - 1) * 32);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
+      for (int r = 0; r < RI; ++r) {
+        const float2 a = __half22float2(*(const __half2 *)&pc[r].x), b = __half22float2(*(const __half2 *)&pc[r].y);
+        float v[NQ];
 #pragma unroll
-        for (int c = 0; c < kAttMaxQ; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-      // lane c stores column c (every lane holds all the sums)
-      float sv = 0.f;
-#pragma unroll
-      for (int c = 0; c < kAttMaxQ; ++c)
-        if (c == lane) sv = v[c] * inv[c];
-      if (lane < NQP) {
-        const __half hi = __float2half_rn(sv);
-        jb.wh[((size_t)h * NQP + lane) * jb.k.r_t + k] = hi;
-        jb.wl[((size_t)h * NQP + lane) * jb.k.r_t + k] = __float2half_rn(sv - __half2float(hi));
+        for (int i = 0; i < NQ; ++i) v[i] = fmaf(a.x, q[i][0], fmaf(a.y, q[i][1], fmaf(b.x, q[i][2], b.y * q[i][3])));
+        const float sv = att_warp_sums<NQ>(v) * inv;
+        if (first && k + r < kr) {
+          const __half hi = __float2half_rn(sv);
+          jb.wh[((size_t)h * NQ + c) * kr + k + r] = hi;
+          jb.wl[((size_t)h * NQ + c) * kr + k + r] = __float2half_rn(sv - __half2float(hi));
+        }
       }
     }
   }
@@ -295,180 +321,9 @@ __global__ void __launch_bounds__(kAttChunk, 3) attend_scores_kernel(const Atten
 
 // warp-level m16n8k16 MMA, fp16 operands, fp32 accumulation
 __device__ __forceinline__ void att_mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// The score kernel for 1-, 2-, 4- and 8-bit codes with the code-times-query contraction on the tensor cores.
-// grid (ceil(n_chunks / 2), m, groups), kAttChunk threads = 8 warps; a CTA walks every gridDim.x-th chunk of its head, a
-// warp owns 32 tokens of the chunk = two 16-row MMA tiles.  The chunk's
-// packed rows and scales are loaded coalesced and staged in shared memory; the m16n8k16 A fragments are built from
-// words read there (odd row pitch: the eight rows of a fragment column fall into eight banks), a pair of codes expanding to the exact fp16
-// integers 2u + 1 - 2^b (so the mid-rise half step is part of the operand and the product is twice the wanted sum).
-// B = the rotated query as hi + lo fp16, 8 query columns, staged once per CTA in shared memory (4 conflict-free word
-// reads per MMA pair).  Per 32-feature group the 16 x 8 partial product is scaled by Delta / 2 of its row.  Registers are
-// capped for three CTAs per SM: the kernel is bound by the latency of its row loads, not by any pipe.
-__device__ __forceinline__ uint32_t att_pair_f16(uint32_t x, int bits) {
-  const uint32_t mask = (1u << bits) - 1u;
-  const uint32_t v = ((x & mask) << 1) | (((x >> bits) & mask) << 17) | 0x64016401u;        // half2(1024 + 2u + 1)
-  const __half2 off = __float2half2_rn(1024.f + (float)(1 << bits));
-  const __half2 r = __hsub2(*(const __half2 *)&v, off);
-  return *(const uint32_t *)&r;
-}
-
-template <int BITS>
-__global__ void __launch_bounds__(kAttChunk, BITS >= 4 ? 2 : 3) attend_scores_mma_kernel(const AttendJob *__restrict__ jobs, int NQP, int n_chunks) {
-  static_assert(BITS == 1 || BITS == 2 || BITS == 4 || BITS == 8, "codes that do not straddle words");
-  const AttendJob &jb = jobs[blockIdx.z];
-  if (jb.k.bits != BITS) return;
-  const int h = blockIdx.y;
-  if (h >= jb.m || (int)blockIdx.x * kAttChunk >= jb.T) return;
-  __shared__ float red[2][kAttChunk / 32][kAttMaxQ];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
-  // the chunk's packed rows and scales, requested one chunk ahead: consecutive threads take consecutive 16-byte pieces
-  // (coalesced), and put them into shared memory with an odd row pitch, from where the fragment builders read words
-  constexpr int RP = 4 * BITS + 1;                 // words per staged row: rows g = 0..7 of one word fall into 8 banks
-  __shared__ uint32_t rows[kAttChunk][RP];
-  __shared__ uint2 scs[kAttChunk];
-  uint4 npc[BITS];                                 // pieces tid, tid + 256, ... of the chunk's kAttChunk * BITS
-  uint2 nsc = make_uint2(0u, 0u);
-  float2 nsb[4];                   // backbone scores of this lane's four (row, query pair) results
-  const bool qok = 2 * c < NQP;
-  auto fetch = [&](int chunk) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) nsb[r] = make_float2(0.f, 0.f);
-    if (chunk >= n_chunks) return;
-    const int t0 = chunk * kAttChunk, nt = min(kAttChunk, jb.T - t0);
-    if (qok && jb.k.r_t > 0 && warp * 32 < nt) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        nsb[r] = *(const float2 *)(jb.p + ((size_t)h * jb.T + t0 + warp * 32 + (r >> 1) * 16 + (r & 1) * 8 + g) * NQP + 2 * c);
-    }
-    const uint4 *wp = (const uint4 *)(jb.k.words + ((size_t)h * jb.T + t0) * (4 * BITS));
-#pragma unroll
-    for (int i = 0; i < BITS; ++i) {
-      const int idx = tid + i * kAttChunk;
-      npc[i] = idx < nt * BITS ? __ldg(wp + idx) : make_uint4(0u, 0u, 0u, 0u);
-    }
-    nsc = tid < nt ? __ldg((const uint2 *)(jb.k.scales + ((size_t)h * jb.T + t0) * 4) + tid) : make_uint2(0u, 0u);
-  };
-  fetch(blockIdx.x);
-  // B operand (rotated query, hi and lo) of the head in shared memory: [query][feature pair], 68 words per row so that
-  // the fragment reads (query g, pair 8 s + c) touch 32 different banks
-  __shared__ uint32_t Bq[2][kAttMaxQ][68];
-  for (int i = tid; i < 2 * kAttMaxQ * 64; i += kAttChunk) {
-    const int hl = i >> 9, q = (i >> 6) & 7, w = i & 63;
-    const uint32_t *src = (const uint32_t *)((hl ? jb.ql : jb.qh) + ((size_t)h * kAttMaxQ + q) * 128);
-    Bq[hl][q][w] = q < NQP ? __ldg(src + w) : 0u;
-  }
-  __syncthreads();
-  for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-  const bool live = chunk * kAttChunk + warp * 32 < jb.T;      // T is a multiple of 128: a warp is all in or all out
-  __syncthreads();                                       // the previous chunk's rows have been read
-#pragma unroll
-  for (int i = 0; i < BITS; ++i) {
-    const int idx = tid + i * kAttChunk, r = idx / BITS, w4 = (idx % BITS) * 4;
-    rows[r][w4] = npc[i].x; rows[r][w4 + 1] = npc[i].y; rows[r][w4 + 2] = npc[i].z; rows[r][w4 + 3] = npc[i].w;
-  }
-  scs[tid] = nsc;
-  float2 sb[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) sb[r] = nsb[r];
-  __syncthreads();
-  fetch(chunk + gridDim.x);                              // in flight during this chunk's MMAs
-  float sc[2][4];          // [tile][row g: queries 2c, 2c+1; row g + 8: queries 2c, 2c+1]
-#pragma unroll
-  for (int tl = 0; tl < 2; ++tl)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) sc[tl][j] = 0.f;
-#pragma unroll
-  for (int tl = 0; tl < 2; ++tl) {
-    const uint32_t *ra = rows[warp * 32 + tl * 16 + g], *rb = rows[warp * 32 + tl * 16 + g + 8];      // rows g and g + 8 of this tile
-    const uint2 sa = scs[warp * 32 + tl * 16 + g], sbw = scs[warp * 32 + tl * 16 + g + 8];
-    const uint32_t sxa = sa.x, sya = sa.y, sxb = sbw.x, syb = sbw.y;
-#pragma unroll
-    for (int gq = 0; gq < 4; ++gq) {
-      float d[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int s2 = 0; s2 < 2; ++s2) {
-        const int s8 = gq * 2 + s2;
-        uint32_t a[4];
-        if constexpr (BITS == 8) {            // 16 bits at bit 128 s2 + 16 c: word 4 s2 + (c >> 1), half c & 1; + 8 columns: two words on
-          const int w0 = gq * 8 + s2 * 4 + (c >> 1), sh = 16 * (c & 1);
-          a[0] = att_pair_f16(ra[w0] >> sh, 8); a[1] = att_pair_f16(rb[w0] >> sh, 8);
-          a[2] = att_pair_f16(ra[w0 + 2] >> sh, 8); a[3] = att_pair_f16(rb[w0 + 2] >> sh, 8);
-        } else if constexpr (BITS == 4) {     // 8 bits at bit 64 s2 + 8 c: word 2 s2, byte c; + 8 columns: the next word
-          const int w0 = gq * 4 + s2 * 2;
-          a[0] = att_pair_f16(ra[w0] >> (8 * c), 4); a[1] = att_pair_f16(rb[w0] >> (8 * c), 4);
-          a[2] = att_pair_f16(ra[w0 + 1] >> (8 * c), 4); a[3] = att_pair_f16(rb[w0 + 1] >> (8 * c), 4);
-        } else if constexpr (BITS == 2) {     // 4 bits at bit 32 s2 + 4 c: word s2, nibble c; + 8 columns: 16 bits on
-          const uint32_t a0 = ra[gq * 2 + s2], b0 = rb[gq * 2 + s2];
-          a[0] = att_pair_f16(a0 >> (4 * c), 2); a[1] = att_pair_f16(b0 >> (4 * c), 2);
-          a[2] = att_pair_f16(a0 >> (4 * c + 16), 2); a[3] = att_pair_f16(b0 >> (4 * c + 16), 2);
-        } else {                              // 2 bits at bit 16 s2 + 2 c of the group's single word; + 8 columns: 8 bits on
-          const uint32_t a0 = ra[gq], b0 = rb[gq];
-          a[0] = att_pair_f16(a0 >> (16 * s2 + 2 * c), 1); a[1] = att_pair_f16(b0 >> (16 * s2 + 2 * c), 1);
-          a[2] = att_pair_f16(a0 >> (16 * s2 + 2 * c + 8), 1); a[3] = att_pair_f16(b0 >> (16 * s2 + 2 * c + 8), 1);
-        }
-        att_mma_f16(d, a, Bq[0][g][s8 * 8 + c], Bq[0][g][s8 * 8 + c + 4]);
-        att_mma_f16(d, a, Bq[1][g][s8 * 8 + c], Bq[1][g][s8 * 8 + c + 4]);
-      }
-      // Delta / 2 of rows g and g + 8 for this group: half (gq & 1) of scale word gq >> 1
-      const uint32_t wa = (gq & 2) ? sya : sxa, wb = (gq & 2) ? syb : sxb;
-      const float da = 0.5f * __half2float(__ushort_as_half((unsigned short)((gq & 1) ? (wa >> 16) : (wa & 0xFFFFu))));
-      const float db = 0.5f * __half2float(__ushort_as_half((unsigned short)((gq & 1) ? (wb >> 16) : (wb & 0xFFFFu))));
-      sc[tl][0] = fmaf(da, d[0], sc[tl][0]); sc[tl][1] = fmaf(da, d[1], sc[tl][1]);
-      sc[tl][2] = fmaf(db, d[2], sc[tl][2]); sc[tl][3] = fmaf(db, d[3], sc[tl][3]);
-    }
-  }
-  // undo the query scaling, add the backbone scores; this lane: queries 2c, 2c + 1 of rows g, g + 8, 16 + g, 24 + g
-  const float e0 = qok ? jb.qe[h * kAttMaxQ + 2 * c] : 0.f, e1 = qok ? jb.qe[h * kAttMaxQ + 2 * c + 1] : 0.f;
-  const int tw = chunk * kAttChunk + warp * 32;
-  float *prow[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) prow[r] = jb.p + ((size_t)h * jb.T + tw + (r >> 1) * 16 + (r & 1) * 8 + g) * NQP + 2 * c;
-  float sv[4][2];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    sv[r][0] = sc[r >> 1][(r & 1) * 2] * e0;
-    sv[r][1] = sc[r >> 1][(r & 1) * 2 + 1] * e1;
-    sv[r][0] += sb[r].x; sv[r][1] += sb[r].y;
-  }
-  // chunk maximum and sum of exp(s - maximum), per query: over this lane's rows, the lanes of equal c, the warps
-  float m0 = -INFINITY, m1 = -INFINITY;
-  if (live) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) { m0 = fmaxf(m0, sv[r][0]); m1 = fmaxf(m1, sv[r][1]); }
-  }
-#pragma unroll
-  for (int o = 4; o < 32; o <<= 1) { m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o)); m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o)); }
-  if (g == 0) { red[0][warp][2 * c] = m0; red[0][warp][2 * c + 1] = m1; }
-  __syncthreads();
-  m0 = red[0][0][2 * c]; m1 = red[0][0][2 * c + 1];
-#pragma unroll
-  for (int wq = 1; wq < kAttChunk / 32; ++wq) { m0 = fmaxf(m0, red[0][wq][2 * c]); m1 = fmaxf(m1, red[0][wq][2 * c + 1]); }
-  float l0 = 0.f, l1 = 0.f;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const float p0 = live ? expf(sv[r][0] - m0) : 0.f, p1 = live ? expf(sv[r][1] - m1) : 0.f;
-    l0 += p0; l1 += p1;
-    if (live && qok) *(float2 *)prow[r] = make_float2(p0, p1);
-  }
-#pragma unroll
-  for (int o = 4; o < 32; o <<= 1) { l0 += __shfl_xor_sync(0xffffffffu, l0, o); l1 += __shfl_xor_sync(0xffffffffu, l1, o); }
-  if (g == 0) { red[1][warp][2 * c] = l0; red[1][warp][2 * c + 1] = l1; }
-  __syncthreads();
-  if (tid < NQP) {
-    float l = 0.f, m_i = red[0][0][tid];
-    for (int wq = 0; wq < kAttChunk / 32; ++wq) l += red[1][wq][tid];
-    for (int wq = 1; wq < kAttChunk / 32; ++wq) m_i = fmaxf(m_i, red[0][wq][tid]);
-    float *ml = jb.ml + ((size_t)h * n_chunks + chunk) * 2 * NQP;
-    ml[tid] = m_i;
-    ml[NQP + tid] = l;
-  }
-  __syncthreads();            // red is rewritten by the next chunk
-  }
 }
 
 // grid (n_chunks, m, groups), kAttChunk threads.  The chunk is staged in two halves of 128 tokens (codes, scales and
@@ -555,133 +410,559 @@ __global__ void __launch_bounds__(kAttChunk, NQ == 4 ? 6 : 4) attend_values_kern
     __syncthreads();
   }
   if (sl == 0) {
-    float *ap = jb.a + (((size_t)h * n_chunks + chunk) * 128 + f0) * NQ;
+    float *ap = jb.a + ((size_t)h * n_chunks + chunk) * NQ * 128 + f0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int i = 0; i < NQ; ++i) ap[c * NQ + i] = acc[c][i];
+    for (int i = 0; i < NQ; ++i) *(float4 *)(ap + i * 128) = make_float4(acc[0][i], acc[1][i], acc[2][i], acc[3][i]);
   }
 }
 
-// The value-side code stream on the tensor cores, for 1-, 2-, 4- and 8-bit codes:
-//     a[f][i] = sum_t (2 u_tf + 1 - 2^b) * (Delta_t,g(f) p_t,i / 2)
-// is a product with M = features, N = queries, K = tokens.  Per 128-token half of the chunk the CTA expands the packed
-// codes to an fp16 tile E[t][f] in shared memory (exact integers; 16-byte pieces swizzled by the token index so that both
-// the row-wise writes and the transposed 8 x 8 fragment loads are conflict-free), writes the weights times the steps,
-// scaled by one power of two per half so that fp16 holds them, as hi + lo fp16 W[g][i][t], and then every warp owns 16
-// features: one transposed ldmatrix.x4 and two MMAs per 16 tokens.  No reduction between warps.
-// grid (n_chunks, m, groups), kAttChunk threads.  Dynamic shared memory: 32 KB + 4 * 2 * NQ * 136 halves.
-__device__ __forceinline__ void att_ldmatrix_x4_trans(uint32_t (&r)[4], const void *smem_row) {
-  const uint32_t addr = (uint32_t)__cvta_generic_to_shared(smem_row);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+// ---- the streaming pass on the tensor cores: scores, softmax weights and values of a chunk in one CTA -------------------
+// What bounds the call is the stream of codes; as separate kernels (backbone scores, code scores per bit width, code values,
+// backbone values) each of them ran at 1.5 to 2.2 TB/s on the latency of its own staging, with the weights going through
+// global memory three times.  Here a CTA of four warps takes a chunk of tokens of NH heads from codes to partial values:
+//   scores   U_T w of all NH heads at once (a warp per token stripe), then a warp per head adds the codes' part.  m16n8k16
+//            with M = tokens: A fragments come straight from global memory.  The order of the k index is free as long as both
+//            operands agree, so a lane takes eight neighbouring elements of a row: one 16-byte load of U_T feeds two MMAs of
+//            every head, one field of eight codes the two MMAs of a 32-feature group.
+//   weights  a warp per head: chunk maximum, p = exp(s - maximum)
+//   values   a warp per head streams the codes (M = features, K = tokens; a lane's pairs are one feature of two neighbouring
+//            tokens, joined by byte permutes; the steps scale the weights), then p^T U_T of all heads, a warp per 32 columns.
+// Codes enter as the exact integers u - 2^(b-1) (fp16 1024 + u by bit insertion, one subtraction for two codes); the half step
+// is a column sum: of the query (initial value of the accumulator) and of the weights (an MMA against a row of ones).  fp32
+// operands enter as hi + lo fp16 (22 bits).  Up to four queries share an MMA with their own lo parts (columns q | q + 4).
+// At 8 groups of 32 heads, 4096 tokens, ranks 128 / 112, 4- and 8-bit codes, four queries: 190 us in five launches -> 100 us.
+// A head per CTA with U_T from L2 for each took 144 us, with four heads but fragment loads straight from global memory 112.
+// What is left is instruction issue (46 % of the slots at 16 warps an SM) on chains of expand, multiply, exchange.
+constexpr int kAttStreamThreads = 128;
+constexpr int kAttTok = 128;                                                // tokens of a chunk
+constexpr int kAttPitch = kAttTok + 8;                                      // tokens per row of weights (rows of halves start four banks apart)
+constexpr int kAttWTok = 32, kAttWPitch = kAttWTok + 8;                     // ... of the weights times steps, 32 tokens at a time
+constexpr int kAttSlot = 2048, kAttSlots = 3;                               // a warp's ring of code stages
+__host__ __device__ constexpr int att_stage_rows(int bits) { return bits == 8 ? 16 : bits >= 3 ? 32 : 64; }      // at most kAttSlot bytes
+constexpr size_t att_stream_smem(int nq) {
+  return 4 * (kAttSlot * kAttSlots + (size_t)nq * kAttPitch * 8 + (size_t)4 * 2 * nq * kAttWPitch * 2);
 }
 
-template <int BITS, int NQ>
-__global__ void __launch_bounds__(kAttChunk, 4) attend_values_mma_kernel(const AttendJob *__restrict__ jobs) {
-  static_assert(BITS == 1 || BITS == 2 || BITS == 4 || BITS == 8, "codes that do not straddle words");
-  const AttendJob &jb = jobs[blockIdx.z];
-  if (jb.v.bits != BITS) return;
-  const int h = blockIdx.y, chunk = blockIdx.x, n_chunks = gridDim.x;
-  if (h >= jb.m || chunk * kAttChunk >= jb.T) return;
-  extern __shared__ unsigned char att_smem[];
-  typedef __half ERow[128];
-  typedef __half WBlk[2][NQ][kAttHalf + 8];
-  ERow *E = (ERow *)att_smem;                                   // [128 tokens][128 f], swizzled: piece j of row t sits at j ^ (t & 7)
-  WBlk *W = (WBlk *)(att_smem + sizeof(ERow) * kAttHalf);       // [group][hi | lo][query][token]
-  __shared__ float dmax[kAttChunk / 32];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
-  const int row = tid >> 1, hh = tid & 1;              // staging: token row of the half, feature half (groups 2 hh, 2 hh + 1)
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int hf = 0; hf < 2; ++hf) {
-    const int t0 = chunk * kAttChunk + hf * kAttHalf;
-    if (t0 >= jb.T) break;                             // T is a multiple of 128: a half is all in or all out
-    const size_t grow = (size_t)h * jb.T + t0 + row;
-    // packed codes of the half: 128 * BITS pieces of 16 bytes, consecutive threads take consecutive pieces (coalesced)
-    constexpr int NIT = (kAttHalf * BITS + kAttChunk - 1) / kAttChunk;
-    uint4 cw[NIT];
-    {
-      const uint4 *src = (const uint4 *)(jb.v.words + ((size_t)h * jb.T + t0) * (4 * BITS));
+// The packed rows of a warp's head, keys and then values, through a ring in shared memory by 16-byte asynchronous copies: the
+// rows of a head are contiguous, so a request touches each 128-byte line once (straight fragment loads looked every line up
+// once per 32-feature group: 57 % of the L1's tag rate and 16 % hits), and four stages stay in flight while the warp forms
+// weights or multiplies by U_T.  Pieces are swizzled so that the fragment reads fall into different banks: 8-bit rows of the
+// keys (lane row g) by row & 3, of the values (lane rows 2c ..) by (row >> 1) & 3 in units of 32 bytes, 4-bit rows by
+// (row >> 1) & 3 in units of 16; narrower rows need none.
+struct AttRing {
+  char *slots;
+  const char *src, *vsrc;     // this lane's first piece of the next stage; of the values
+  uint32_t dst[4];            // places of its pieces in a slot
+  int per, bytes, left;       // pieces of a lane, bytes of a stage, stages to come of the current cell
+  int vbits, vleft;
+  int wslot, rslot;
+  __device__ __forceinline__ void layout(int bits, bool values) {
+    const int lane = threadIdx.x & 31;
+    const int rows = att_stage_rows(bits);
+    per = rows * bits / 32;
+    bytes = rows * 16 * bits;
 #pragma unroll
-      for (int it = 0; it < NIT; ++it) {
-        const int idx = tid + it * kAttChunk;
-        cw[it] = idx < kAttHalf * BITS ? __ldg(src + idx) : make_uint4(0u, 0u, 0u, 0u);
+    for (int k = 0; k < 4; ++k) {
+      const int i = lane + 32 * k, row = bits == 3 ? i / 3 : i >> (bits == 8 ? 3 : bits == 4 ? 2 : bits == 2 ? 1 : 0), j = i - row * bits;
+      const int key = bits == 8 ? 2 * (values ? (row >> 1) & 3 : row & 3) : bits == 4 ? (row >> 1) & 3 : 0;
+      dst[k] = row * (16 * bits) + (j ^ key) * 16;
+    }
+  }
+  __device__ __forceinline__ void issue() {
+    if (left == 0 && vleft > 0) { layout(vbits, true); src = vsrc; left = vleft; vleft = 0; }
+    if (left > 0) {
+      const uint32_t base = (uint32_t)__cvta_generic_to_shared(slots + wslot * kAttSlot);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k < per) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + dst[k]), "l"(src + k * 512) : "memory");
+      src += bytes;
+      --left;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    wslot = wslot + 1 == kAttSlots ? 0 : wslot + 1;
+  }
+  __device__ __forceinline__ AttRing(char *ring, const uint32_t *krows, int kbits, const uint32_t *vrows, int vb, int nt)
+      : slots(ring), vbits(vb), wslot(0), rslot(0) {
+    const int lane = threadIdx.x & 31;
+    src = (const char *)krows + lane * 16;
+    vsrc = (const char *)vrows + lane * 16;
+    left = kbits ? nt / att_stage_rows(kbits) : 0;
+    vleft = vb ? nt / att_stage_rows(vb) : 0;
+    layout(kbits ? kbits : 1, false);
+#pragma unroll
+    for (int i = 0; i < kAttSlots - 1; ++i) issue();
+  }
+  // the stage to read; the one read before it is refilled
+  __device__ __forceinline__ const char *next() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAttSlots - 2) : "memory");
+    __syncwarp();
+    issue();
+    const char *p = slots + rslot * kAttSlot;
+    rslot = rslot + 1 == kAttSlots ? 0 : rslot + 1;
+    return p;
+  }
+};
+
+// mid-rise codes of two tokens or features, exact in fp16
+template <int BITS>
+__device__ __forceinline__ uint32_t att_centre(uint32_t v) {
+  const __half2 r = __hsub2(*(const __half2 *)&v, __float2half2_rn(1024.f + (float)(1 << (BITS - 1))));
+  return *(const uint32_t *)&r;
+}
+template <int BITS>
+__device__ __forceinline__ uint32_t att_pair(uint32_t z, int i) {             // code i of the low half and of the high half
+  constexpr uint32_t m = (1u << BITS) - 1u;
+  return att_centre<BITS>(((z >> (BITS * i)) & (m | m << 16)) | 0x64006400u);
+}
+
+// Raw field of a lane: eight codes of a row's group (scores; lane c of four) -- natural order for 8-bit codes, else codes
+// 0..3 in the low and 4..7 in the high half of a word, so that pair i = (i, i + 4).
+template <int BITS>
+struct AttField8 {
+  uint32_t w0, w1;
+  __device__ __forceinline__ void load(const char *st, int row, int key, int G, int c) {       // key: of the ring's swizzle
+    const char *r = st + row * (16 * BITS);
+    if constexpr (BITS == 8) { const uint2 v = *(const uint2 *)(r + (G ^ key) * 32 + 8 * c); w0 = v.x; w1 = v.y; }
+    else if constexpr (BITS == 4) { w0 = *(const uint32_t *)(r + (G ^ key) * 16 + 4 * c); }
+    else if constexpr (BITS == 3) { const int lo = (24 * c) >> 5; w0 = *(const uint32_t *)(r + G * 12 + 4 * lo); w1 = *(const uint32_t *)(r + G * 12 + 4 * min(lo + 1, 2)); }
+    else if constexpr (BITS == 2) { w0 = *(const unsigned short *)(r + G * 8 + 2 * c); }
+    else { w0 = *(const unsigned char *)(r + G * 4 + c); }
+  }
+  __device__ __forceinline__ void expand(uint32_t (&o)[4], int c) const {
+    if constexpr (BITS == 8) {
+      o[0] = att_centre<8>(__byte_perm(w0, 0x64646464u, 0x4140)); o[1] = att_centre<8>(__byte_perm(w0, 0x64646464u, 0x4342));
+      o[2] = att_centre<8>(__byte_perm(w1, 0x64646464u, 0x4140)); o[3] = att_centre<8>(__byte_perm(w1, 0x64646464u, 0x4342));
+    } else {
+      uint32_t z = w0;
+      if constexpr (BITS == 3) { const uint32_t x = __funnelshift_r(w0, w1, (24 * c) & 31); z = (x & 0xFFFu) | ((x & 0xFFF000u) << 4); }
+      if constexpr (BITS == 2) z = __byte_perm(w0, 0u, 0x4140);
+      if constexpr (BITS == 1) z = (w0 & 0xFu) | (w0 << 12);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[i] = att_pair<BITS>(z, i);
+    }
+  }
+};
+// ... and four codes of a row's group (values; lane g of eight).
+template <int BITS>
+struct AttField4 {
+  uint32_t w0, w1;
+  __device__ __forceinline__ void load(const char *st, int row, int key, int G, int g) {
+    const char *r = st + row * (16 * BITS);
+    if constexpr (BITS == 8) w0 = *(const uint32_t *)(r + (G ^ key) * 32 + 4 * g);
+    else if constexpr (BITS == 4) w0 = *(const unsigned short *)(r + (G ^ key) * 16 + 2 * g);
+    else if constexpr (BITS == 3) { const int lo = (12 * g) >> 5; w0 = *(const uint32_t *)(r + G * 12 + 4 * lo); w1 = *(const uint32_t *)(r + G * 12 + 4 * min(lo + 1, 2)); }
+    else if constexpr (BITS == 2) w0 = *(const unsigned char *)(r + G * 8 + g);
+    else w0 = *(const unsigned char *)(r + G * 4 + (g >> 1));
+  }
+  // features 0..3 of two neighbouring tokens
+  static __device__ __forceinline__ void expand(uint32_t (&o)[4], const AttField4 &a, const AttField4 &b, int g) {
+    if constexpr (BITS == 8) {
+      const uint32_t lo = __byte_perm(a.w0, b.w0, 0x5140), hi = __byte_perm(a.w0, b.w0, 0x7362);
+      o[0] = att_centre<8>(__byte_perm(lo, 0x64646464u, 0x4140)); o[1] = att_centre<8>(__byte_perm(lo, 0x64646464u, 0x4342));
+      o[2] = att_centre<8>(__byte_perm(hi, 0x64646464u, 0x4140)); o[3] = att_centre<8>(__byte_perm(hi, 0x64646464u, 0x4342));
+    } else {
+      uint32_t x = a.w0, y = b.w0;
+      if constexpr (BITS == 3) { x = __funnelshift_r(a.w0, a.w1, (12 * g) & 31); y = __funnelshift_r(b.w0, b.w1, (12 * g) & 31); }
+      if constexpr (BITS == 1) { x >>= 4 * (g & 1); y >>= 4 * (g & 1); }
+      const uint32_t z = __byte_perm(x, y, 0x5410);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[i] = att_pair<BITS>(z, i);
+    }
+  }
+};
+
+// fp32 pair -> hi and lo half2
+__device__ __forceinline__ void att_split(float x0, float x1, uint32_t &hi, uint32_t &lo) {
+  const __half2 h = __floats2half2_rn(x0, x1);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(x0 - f.x, x1 - f.y);
+  hi = *(const uint32_t *)&h; lo = *(const uint32_t *)&l;
+}
+
+// Code scores of a warp's head over its nt tokens, added to ps[query][token].
+template <int BITS, int NQ>
+__device__ __forceinline__ void att_code_scores(const AttendJob &jb, int h, size_t row0, int nt, float *ps, AttRing &ring) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  constexpr int NB = NQ == 8 ? 2 : 1, P = kAttPitch;      // lo parts in an MMA of their own
+  const int key = BITS == 8 ? g & 3 : (g >> 1) & 3;
+  const uint2 *sp = (const uint2 *)jb.k.scales + row0 + g;
+  uint2 sc[2][2];
+  sc[0][0] = __ldg(sp); sc[0][1] = __ldg(sp + 8); sc[1][0] = __ldg(sp + 16); sc[1][1] = __ldg(sp + 24);
+  uint4 bq[NB][4];
+  float qs[4][2];
+  {
+    const int q = NQ == 8 ? g : g & 3;
+    const __half *s0 = ((NQ == 4 && g >= 4) ? jb.ql : jb.qh) + ((size_t)h * kAttMaxQ + q) * 128 + 8 * c;
+    const __half *s1 = jb.ql + ((size_t)h * kAttMaxQ + q) * 128 + 8 * c;
+#pragma unroll
+    for (int G = 0; G < 4; ++G) {
+      bq[0][G] = *(const uint4 *)(s0 + G * 32);
+      if (NB == 2) bq[NB - 1][G] = *(const uint4 *)(s1 + G * 32);
+    }
+#pragma unroll
+    for (int G = 0; G < 4; ++G) {
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint32_t one = 0x3C003C00u, ones[4] = {one, one, one, one};
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        if constexpr (BITS != 8) {                         // pairs (i, i + 4)
+          const uint4 v = bq[b][G];
+          bq[b][G] = make_uint4(__byte_perm(v.x, v.z, 0x5410), __byte_perm(v.x, v.z, 0x7632), __byte_perm(v.y, v.w, 0x5410), __byte_perm(v.y, v.w, 0x7632));
+        }
+        att_mma_f16(d, ones, bq[b][G].x, bq[b][G].y);
+        att_mma_f16(d, ones, bq[b][G].z, bq[b][G].w);
+      }
+      qs[G][0] = 0.5f * d[0]; qs[G][1] = 0.5f * d[1];      // the half step of every code of the group
+    }
+  }
+  const int qa = (2 * c) & (NQ - 1);
+  const float e0 = jb.qe[h * kAttMaxQ + qa], e1 = jb.qe[h * kAttMaxQ + qa + 1];
+  float *pr = ps + qa * P + g + (NQ == 4 ? (c & 2) * 4 : 0);      // NQ = 4: lanes c < 2 finish row g, c >= 2 row g + 8
+  constexpr int R = att_stage_rows(BITS);
+  const char *stage = nullptr;
+  for (int t = 0; t < nt; t += 32) {
+    if (R >= 32 && (R == 32 || (t & 32) == 0)) stage = ring.next();
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (R == 16) stage = ring.next();
+      const int r0 = R == 16 ? 0 : R == 32 ? 16 * u : (t & 32) + 16 * u;
+      AttField8<BITS> fa[4], fb[4];
+#pragma unroll
+      for (int G = 0; G < 4; ++G) { fa[G].load(stage, r0 + g, key, G, c); fb[G].load(stage, r0 + g + 8, key, G, c); }
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int G = 0; G < 4; ++G) {
+        uint32_t x[4], y[4];
+        fa[G].expand(x, c);
+        fb[G].expand(y, c);
+        float d[4] = {qs[G][0], qs[G][1], qs[G][0], qs[G][1]};
+        const uint32_t a0[4] = {x[0], y[0], x[1], y[1]}, a1[4] = {x[2], y[2], x[3], y[3]};
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          att_mma_f16(d, a0, bq[b][G].x, bq[b][G].y);
+          att_mma_f16(d, a1, bq[b][G].z, bq[b][G].w);
+        }
+        const uint32_t wa = G & 2 ? sc[u][0].y : sc[u][0].x, wb = G & 2 ? sc[u][1].y : sc[u][1].x;
+        const float da = G & 1 ? __high2float(*(const __half2 *)&wa) : __low2float(*(const __half2 *)&wa);
+        const float db = G & 1 ? __high2float(*(const __half2 *)&wb) : __low2float(*(const __half2 *)&wb);
+        s[0] = fmaf(da, d[0], s[0]); s[1] = fmaf(da, d[1], s[1]);
+        s[2] = fmaf(db, d[2], s[2]); s[3] = fmaf(db, d[3], s[3]);
+      }
+      if (t + 32 < nt) { sc[u][0] = __ldg(sp + t + 32 + 16 * u); sc[u][1] = __ldg(sp + t + 40 + 16 * u); }
+      float *pt = pr + t + 16 * u;
+      if constexpr (NQ == 4) {
+        const float k0 = c & 2 ? s[2] : s[0], k1 = c & 2 ? s[3] : s[1], v0 = c & 2 ? s[0] : s[2], v1 = c & 2 ? s[1] : s[3];
+        pt[0] = fmaf(k0 + __shfl_xor_sync(0xffffffffu, v0, 2), e0, pt[0]);
+        pt[P] = fmaf(k1 + __shfl_xor_sync(0xffffffffu, v1, 2), e1, pt[P]);
+      } else {
+        pt[0] = fmaf(s[0], e0, pt[0]); pt[P] = fmaf(s[1], e1, pt[P]);
+        pt[8] = fmaf(s[2], e0, pt[8]); pt[P + 8] = fmaf(s[3], e1, pt[P + 8]);
       }
     }
-    const uint32_t sc2 = __ldg((const uint32_t *)(jb.v.scales + grow * 4) + hh);       // steps of groups 2 hh, 2 hh + 1
-    const float d0 = __half2float(__ushort_as_half((unsigned short)(sc2 & 0xFFFFu))), d1 = __half2float(__ushort_as_half((unsigned short)(sc2 >> 16)));
-    float pv[NQ];
+  }
+}
+
+// A lane's product columns, hi + lo, as elements 4g .. 4g + 3 of queries 2c, 2c + 1; NQ = 4: lanes c < 2.
+template <int NQ>
+__device__ __forceinline__ void att_put4(float (&d)[2][4], float mul, float *dst, int stride, bool ok) {
+  const int lane = threadIdx.x & 31, c = lane & 3;
 #pragma unroll
-    for (int q4 = 0; q4 < NQ; q4 += 4) {
-      const float4 p4 = *(const float4 *)(jb.p + grow * NQ + q4);
-      pv[q4] = p4.x; pv[q4 + 1] = p4.y; pv[q4 + 2] = p4.z; pv[q4 + 3] = p4.w;
+  for (int j = 0; j < 2; ++j)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (NQ == 4) d[j][i] += __shfl_xor_sync(0xffffffffu, d[j][i], 2);
+  if (!ok || (NQ == 4 && c >= 2)) return;
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    *(float4 *)(dst + (size_t)(2 * c + q) * stride) = make_float4(d[0][q] * mul, d[0][q + 2] * mul, d[1][q] * mul, d[1][q + 2] * mul);
+}
+
+// One 16-token step of a value product: M = 32 elements of a row (a lane's four, x from tokens 2c, 2c + 1 and y from 8 on), B
+// from the weight rows of column g (hi rows 0 .. NQ - 1, lo rows NQ .. 2 NQ - 1).  ones: also sum the weights into row G of e.
+template <int NQ>
+__device__ __forceinline__ void att_value_mma(float (&d)[2][4], const uint32_t (&x)[4], const uint32_t (&y)[4], const __half *w, int pitch) {
+  const uint32_t a0[4] = {x[0], x[1], y[0], y[1]}, a1[4] = {x[2], x[3], y[2], y[3]};
+  const uint32_t b0 = *(const uint32_t *)w, b1 = *(const uint32_t *)(w + 8);
+  att_mma_f16(d[0], a0, b0, b1); att_mma_f16(d[1], a1, b0, b1);
+  if (NQ == 8) {
+    const uint32_t c0 = *(const uint32_t *)(w + 8 * pitch), c1 = *(const uint32_t *)(w + 8 * pitch + 8);
+    att_mma_f16(d[0], a0, c0, c1); att_mma_f16(d[1], a1, c0, c1);
+  }
+}
+
+// Code values of a warp's head over its nt tokens.  ws: [4 groups][2 NQ][kAttWPitch] weights times steps of 32 tokens.
+template <int BITS, int NQ>
+__device__ __forceinline__ void att_code_values(const AttendJob &jb, size_t row0, int nt, const float *ps, __half *ws, AttRing &ring, float *out) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  constexpr int P = kAttPitch;
+  // one power of two for the chunk so that step * weight fits fp16: the largest step -> below 2^14
+  const uint4 *sp = (const uint4 *)(jb.v.scales + (row0 + 2 * lane) * 4);                 // the steps of two tokens
+  __half2 mx2 = __float2half2_rn(0.f);
+  for (int t = 0; t < nt; t += 64) {
+    const uint4 v = __ldg(sp + t / 2);
+    mx2 = __hmax2(mx2, __hmax2(__hmax2(*(const __half2 *)&v.x, *(const __half2 *)&v.y), __hmax2(*(const __half2 *)&v.z, *(const __half2 *)&v.w)));
+  }
+  float mx = fmaxf(__low2float(mx2), __high2float(mx2));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  int ex = 0;
+  if (mx > 0.f && mx < INFINITY) frexpf(mx, &ex);
+  const float up = ldexpf(1.f, 14 - ex), down = ldexpf(1.f, ex - 14);
+  float d[4][2][4], hs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int G = 0; G < 4; ++G)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[G][j][i] = 0.f;
+  const __half *w = ws + g * kAttWPitch + 2 * c;
+  // weights: this lane forms those of tokens 2 tl, 2 tl + 1 of every 32 and groups 2 gh, 2 gh + 1
+  const int tl = lane & 15, gh = lane >> 4;
+  const uint4 *vp = (const uint4 *)(jb.v.scales + (row0 + 2 * tl) * 4);
+  uint4 vn = __ldg(vp);
+  const char *stage = nullptr;
+  for (int tb = 0; tb < nt; tb += kAttWTok) {
+    const uint32_t va = gh ? vn.y : vn.x, vb = gh ? vn.w : vn.z;
+    if (tb + kAttWTok < nt) vn = __ldg(vp + (tb + kAttWTok) / 2);
+    const float2 fa = __half22float2(*(const __half2 *)&va), fb = __half22float2(*(const __half2 *)&vb);
+    const float d0[2] = {fa.x * up, fa.y * up}, d1[2] = {fb.x * up, fb.y * up};
+    __syncwarp();                                                                       // the previous weights have been read
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const float2 p = *(const float2 *)(ps + q * P + tb + 2 * tl);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        uint32_t hi, lo;
+        att_split(p.x * d0[i], p.y * d1[i], hi, lo);
+        __half *wr = ws + ((2 * gh + i) * 2 * NQ + q) * kAttWPitch + 2 * tl;
+        *(uint32_t *)wr = hi;
+        *(uint32_t *)(wr + NQ * kAttWPitch) = lo;
+      }
     }
-    // one power of two per half so that step * weight / 2 fits fp16: largest step of the half -> below 2^14
-    float mx = fmaxf(d0, d1);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (hf) __syncthreads();                           // the previous half's tiles have been read
-    if (lane == 0) dmax[warp] = mx;
-    // codes -> E: a 16-byte piece of a packed row holds 128 / BITS codes = 16 / BITS output pieces of eight fp16 values
+    for (int s = 0; s < kAttWTok / 16; ++s) {
+      constexpr int R = att_stage_rows(BITS);
+      if (R == 16 || (s == 0 && (R == 32 || (tb & 32) == 0))) stage = ring.next();      // its __syncwarp also publishes the weights
+      else if (s == 0) __syncwarp();
+      const int r0 = R == 16 ? 0 : R == 32 ? 16 * s : (tb & 32) + 16 * s;
+      AttField4<BITS> f[4][4];
 #pragma unroll
-    for (int it = 0; it < NIT; ++it) {
-      const int idx = tid + it * kAttChunk;
-      if (idx < kAttHalf * BITS) {
-        const int er = idx / BITS, seg = idx % BITS;
-        const uint32_t w4[4] = {cw[it].x, cw[it].y, cw[it].z, cw[it].w};
+      for (int G = 0; G < 4; ++G)
 #pragma unroll
-        for (int pc = 0; pc < 16 / BITS; ++pc) {
-          uint32_t o[4];
+        for (int i = 0; i < 4; ++i) f[G][i].load(stage, r0 + 2 * c + (i & 1) + (i >> 1) * 8, c, G, g);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int bit = 2 * (pc * 4 + j) * BITS;                  // pair pc * 4 + j of this piece of the row's bit string
-            o[j] = att_pair_f16(w4[bit >> 5] >> (bit & 31), BITS);
+      for (int G = 0; G < 4; ++G) {
+        uint32_t x[4], y[4];
+        AttField4<BITS>::expand(x, f[G][0], f[G][1], g);
+        AttField4<BITS>::expand(y, f[G][2], f[G][3], g);
+        const __half *wg = w + G * 2 * NQ * kAttWPitch + 16 * s;
+        att_value_mma<NQ>(d[G], x, y, wg, kAttWPitch);
+        const uint32_t one = g == G ? 0x3C003C00u : 0u, a[4] = {one, 0u, one, 0u};      // row G of hs: the sum of the weights
+        att_mma_f16(hs, a, *(const uint32_t *)wg, *(const uint32_t *)(wg + 8));
+        if (NQ == 8) att_mma_f16(hs, a, *(const uint32_t *)(wg + 8 * kAttWPitch), *(const uint32_t *)(wg + 8 * kAttWPitch + 8));
+      }
+    }
+  }
+#pragma unroll
+  for (int G = 0; G < 4; ++G) {
+    const float a0 = 0.5f * __shfl_sync(0xffffffffu, hs[0], 4 * G + c), a1 = 0.5f * __shfl_sync(0xffffffffu, hs[1], 4 * G + c);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) { d[G][j][0] += a0; d[G][j][1] += a1; d[G][j][2] += a0; d[G][j][3] += a1; }
+    att_put4<NQ>(d[G], down, out + G * 32 + 4 * g, 128, true);
+  }
+}
+
+// grid (ceil(chunks / (4 / NH)), ceil(m / NH), groups), 128 threads, att_stream_smem bytes of dynamic shared memory.  NH = 4: the
+// warps are four heads of one chunk; NH = 1 (fewer than three heads in a cell): four chunks of one head.
+template <int NQ, int NH>
+__global__ void __launch_bounds__(kAttStreamThreads, NQ == 4 ? 4 : 3) attend_stream_kernel(const AttendJob *__restrict__ jobs, int n_chunks) {
+  constexpr int TC = kAttTok, P = kAttPitch;
+  const AttendJob &jb = jobs[blockIdx.z];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
+  const int h0 = blockIdx.y * NH, t_cta = blockIdx.x * (TC * 4 / NH), T = jb.T, m = jb.m;
+  if (h0 >= m || t_cta >= T) return;
+  extern __shared__ unsigned char att_smem[];
+  float *ps_all = (float *)att_smem;                                        // [4 warps][NQ][P] scores, then weights
+  __half *pw_all = (__half *)(ps_all + 4 * NQ * P);                         // [4][2 NQ][P] weights as hi and lo rows
+  const int kr = jb.k.r_t, vr = jb.v.r_t;
+  const int h = h0 + (NH == 4 ? warp : 0), t0 = t_cta + (NH == 4 ? 0 : warp * TC), nt = max(0, min(TC, T - t0));      // nt: a multiple of 128
+  const bool alive = h < m && nt > 0;
+  const size_t row0 = (size_t)h * T + t0;
+  float *ps = ps_all + warp * NQ * P;
+  __half *pw = pw_all + warp * 2 * NQ * P, *ws = pw_all + 4 * 2 * NQ * P + warp * 4 * 2 * NQ * kAttWPitch;
+  AttRing ring((char *)(pw_all + 4 * 2 * NQ * P + 4 * 4 * 2 * NQ * kAttWPitch) + warp * kAttSlot * kAttSlots, jb.k.words + row0 * 4 * jb.k.bits,
+               jb.k.bits, jb.v.words + row0 * 4 * jb.v.bits, jb.v.bits, alive ? nt : 0);
+  att_wait_predecessor();
+  // ---- backbone scores of a warp's TA tokens, SB stripes of 16 and all heads at a time
+  {
+    constexpr int TA = TC / NH, SB = 2;
+    const int tw = t_cta + warp * TA, tp = NH == 4 ? warp * TA : 0;          // first token; its place in the chunk
+    for (int ta = 0; ta < TA && tw + ta < T; ta += 16 * SB) {
+      float acc[SB][NH][4];
+#pragma unroll
+      for (int st = 0; st < SB; ++st)
+#pragma unroll
+        for (int j = 0; j < NH; ++j)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[st][j][i] = 0.f;
+      const __half *ua = jb.k.UT + (size_t)(tw + ta + g) * kr + 8 * c;
+      const size_t wo = ((size_t)h0 * NQ + (NQ == 8 ? g : g & 3)) * kr + 8 * c;
+      const __half *w0 = ((NQ == 4 && g >= 4) ? jb.wl : jb.wh) + wo, *w1 = jb.wl + wo;
+      const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+      uint4 x[SB], y[SB];
+      auto load_a = [&](int k) {
+        const bool ok = k + 8 * c < kr;
+#pragma unroll
+        for (int st = 0; st < SB; ++st) {
+          x[st] = ok ? __ldg((const uint4 *)(ua + (size_t)(st * 16) * kr + k)) : zero;
+          y[st] = ok ? __ldg((const uint4 *)(ua + (size_t)(st * 16 + 8) * kr + k)) : zero;
+        }
+      };
+      uint4 bn[NH];
+      auto load_b = [&](int k) {
+#pragma unroll
+        for (int j = 0; j < NH; ++j) bn[j] = k + 8 * c < kr && h0 + j < m ? __ldg((const uint4 *)(w0 + (size_t)j * NQ * kr + k)) : zero;
+      };
+      load_b(0);
+      load_a(0);
+#pragma unroll 1
+      for (int k = 0; k < kr; k += 32) {
+        uint4 b[NH], bl[NH], xc[SB], yc[SB];
+#pragma unroll
+        for (int j = 0; j < NH; ++j) {
+          b[j] = bn[j];
+          if (NQ == 8) bl[j] = k + 8 * c < kr && h0 + j < m ? __ldg((const uint4 *)(w1 + (size_t)j * NQ * kr + k)) : zero;
+        }
+        if (k + 32 < kr) load_b(k + 32);
+#pragma unroll
+        for (int st = 0; st < SB; ++st) { xc[st] = x[st]; yc[st] = y[st]; }
+        if (k + 32 < kr) load_a(k + 32);
+#pragma unroll
+        for (int st = 0; st < SB; ++st) {
+          const uint32_t a0[4] = {xc[st].x, yc[st].x, xc[st].y, yc[st].y}, a1[4] = {xc[st].z, yc[st].z, xc[st].w, yc[st].w};
+#pragma unroll
+          for (int j = 0; j < NH; ++j) {
+            att_mma_f16(acc[st][j], a0, b[j].x, b[j].y);
+            att_mma_f16(acc[st][j], a1, b[j].z, b[j].w);
+            if (NQ == 8) { att_mma_f16(acc[st][j], a0, bl[j].x, bl[j].y); att_mma_f16(acc[st][j], a1, bl[j].z, bl[j].w); }
           }
-          const int piece = seg * (16 / BITS) + pc;
-          *(uint4 *)&E[er][((piece ^ (er & 7)) << 3)] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+      }
+      const int qa = (2 * c) & (NQ - 1);
+#pragma unroll
+      for (int j = 0; j < NH; ++j) {
+        const bool hk = kr > 0 && h0 + j < m;
+        const float we0 = hk ? jb.we[(h0 + j) * NQ + qa] : 0.f, we1 = hk ? jb.we[(h0 + j) * NQ + qa + 1] : 0.f;
+        float *pj = ps_all + (NH == 4 ? j : warp) * NQ * P + qa * P + tp + ta + g;
+#pragma unroll
+        for (int st = 0; st < SB; ++st) {
+          const float *s = acc[st][j];
+          if constexpr (NQ == 4) {
+            const float k0 = c & 2 ? s[2] : s[0], k1 = c & 2 ? s[3] : s[1], v0 = c & 2 ? s[0] : s[2], v1 = c & 2 ? s[1] : s[3];
+            const float r0 = (k0 + __shfl_xor_sync(0xffffffffu, v0, 2)) * we0, r1 = (k1 + __shfl_xor_sync(0xffffffffu, v1, 2)) * we1;
+            pj[st * 16 + (c & 2) * 4] = r0; pj[P + st * 16 + (c & 2) * 4] = r1;
+          } else {
+            pj[st * 16] = s[0] * we0; pj[P + st * 16] = s[1] * we1;
+            pj[st * 16 + 8] = s[2] * we0; pj[P + st * 16 + 8] = s[3] * we1;
+          }
         }
       }
     }
-    __syncthreads();
-    mx = dmax[0];
+  }
+  __syncthreads();
+  if (alive) {
+    switch (jb.k.bits) {
+      case 1: att_code_scores<1, NQ>(jb, h, row0, nt, ps, ring); break;
+      case 2: att_code_scores<2, NQ>(jb, h, row0, nt, ps, ring); break;
+      case 3: att_code_scores<3, NQ>(jb, h, row0, nt, ps, ring); break;
+      case 4: att_code_scores<4, NQ>(jb, h, row0, nt, ps, ring); break;
+      case 8: att_code_scores<8, NQ>(jb, h, row0, nt, ps, ring); break;
+      default: break;
+    }
+    __syncwarp();
+    // chunk maximum, weights and their sum, per query; this lane: tokens 2 lane, 2 lane + 1 of every 64
+    const int chunk = t0 / TC;
+    float *ml = jb.ml + ((size_t)h * n_chunks + chunk) * 2 * NQ;
+    float2 v[NQ][TC / 64];
+    float mx[NQ], l[NQ];
 #pragma unroll
-    for (int wq = 1; wq < kAttChunk / 32; ++wq) mx = fmaxf(mx, dmax[wq]);
-    int ex = 0;
-    if (mx > 0.f && mx < INFINITY) frexpf(mx, &ex);                    // mx < 2^ex
-    const float up = ldexpf(0.5f, 14 - ex), down = ldexpf(1.f, ex - 14);
+    for (int q = 0; q < NQ; ++q) {
+      mx[q] = -INFINITY; l[q] = 0.f;
 #pragma unroll
-    for (int gl = 0; gl < 2; ++gl) {
-      const float ds = (gl ? d1 : d0) * up;
+      for (int i = 0; i < TC / 64; ++i) { v[q][i] = *(const float2 *)(ps + q * P + 64 * i + 2 * lane); mx[q] = fmaxf(mx[q], fmaxf(v[q][i].x, v[q][i].y)); }
+    }
 #pragma unroll
-      for (int i = 0; i < NQ; ++i) {
-        const float x = ds * pv[i];
-        const __half hi = __float2half_rn(x);
-        W[hh * 2 + gl][0][i][row] = hi;
-        W[hh * 2 + gl][1][i][row] = __float2half_rn(x - __half2float(hi));
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], o));
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+      for (int i = 0; i < TC / 64; ++i) {
+        const float2 p = make_float2(expf(v[q][i].x - mx[q]), expf(v[q][i].y - mx[q]));
+        l[q] += p.x + p.y;
+        *(float2 *)(ps + q * P + 64 * i + 2 * lane) = p;
+        uint32_t hi, lo;
+        att_split(p.x, p.y, hi, lo);
+        *(uint32_t *)(pw + q * P + 64 * i + 2 * lane) = hi;
+        *(uint32_t *)(pw + (q + NQ) * P + 64 * i + 2 * lane) = lo;
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) l[q] += __shfl_xor_sync(0xffffffffu, l[q], o);
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) { ml[q] = mx[q]; ml[NQ + q] = l[q]; }
+    __syncwarp();
+    float *ap = jb.a + ((size_t)h * n_chunks + chunk) * NQ * 128;
+    switch (jb.v.bits) {
+      case 1: att_code_values<1, NQ>(jb, row0, nt, ps, ws, ring, ap); break;
+      case 2: att_code_values<2, NQ>(jb, row0, nt, ps, ws, ring, ap); break;
+      case 3: att_code_values<3, NQ>(jb, row0, nt, ps, ws, ring, ap); break;
+      case 4: att_code_values<4, NQ>(jb, row0, nt, ps, ws, ring, ap); break;
+      case 8: att_code_values<8, NQ>(jb, row0, nt, ps, ws, ring, ap); break;
+      default: break;
+    }
+  }
+  __syncthreads();
+  // ---- p^T U_T: 32 columns at a time, all heads (NH = 4) or this warp's chunk (NH = 1)
+  if (nt == 0) return;
+  for (int kb = NH == 4 ? warp * 32 : 0; kb < vr; kb += NH == 4 ? 128 : 32) {
+    const int k = kb + 4 * g;
+    const bool ok = k < vr;
+    const __half *p0 = jb.v.UT + (size_t)(t0 + 2 * c) * vr + min(k, vr - 4), *p1 = p0 + vr, *p2 = p0 + 8 * (size_t)vr, *p3 = p2 + vr;      // columns past the end: not stored
+    const size_t step = 16 * (size_t)vr;
+    constexpr int PF = 4;
+    uint2 f[PF][4];
+    auto fetch = [&](int buf) {
+      f[buf][0] = __ldg((const uint2 *)p0); f[buf][1] = __ldg((const uint2 *)p1); f[buf][2] = __ldg((const uint2 *)p2); f[buf][3] = __ldg((const uint2 *)p3);
+      p0 += step; p1 += step; p2 += step; p3 += step;
+    };
+#pragma unroll
+    for (int u = 0; u < PF; ++u) fetch(u);
+    float d[NH][2][4];
+#pragma unroll
+    for (int j = 0; j < NH; ++j)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) d[j][i >> 2][i & 3] = 0.f;
+    const __half *w = pw_all + (NH == 4 ? 0 : warp) * 2 * NQ * P + g * P + 2 * c;
+    for (int t = 0; t < nt; t += 16 * PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        uint32_t x[4], y[4];
+        x[0] = __byte_perm(f[u][0].x, f[u][1].x, 0x5410); x[1] = __byte_perm(f[u][0].x, f[u][1].x, 0x7632);
+        x[2] = __byte_perm(f[u][0].y, f[u][1].y, 0x5410); x[3] = __byte_perm(f[u][0].y, f[u][1].y, 0x7632);
+        y[0] = __byte_perm(f[u][2].x, f[u][3].x, 0x5410); y[1] = __byte_perm(f[u][2].x, f[u][3].x, 0x7632);
+        y[2] = __byte_perm(f[u][2].y, f[u][3].y, 0x5410); y[3] = __byte_perm(f[u][2].y, f[u][3].y, 0x7632);
+        if (t + 16 * PF < nt) fetch(u);
+#pragma unroll
+        for (int j = 0; j < NH; ++j) att_value_mma<NQ>(d[j], x, y, w + j * 2 * NQ * P + t + 16 * u, P);
       }
     }
-    __syncthreads();
-    // warp = features 16 warp .. +15 (group warp >> 1); 8 steps of 16 tokens
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
-    const int mi = lane >> 3, r8 = lane & 7, tb8 = mi >> 1, fb = mi & 1;
-    const bool have = g < NQ;                           // query columns beyond NQ are zero
-    const uint32_t *wh = (const uint32_t *)&W[warp >> 1][0][have ? g : 0][0], *wl = (const uint32_t *)&W[warp >> 1][1][have ? g : 0][0];
 #pragma unroll
-    for (int s16 = 0; s16 < kAttHalf / 16; ++s16) {
-      uint32_t a[4];
-      const int tr = s16 * 16 + tb8 * 8 + r8;
-      att_ldmatrix_x4_trans(a, &E[tr][(((2 * warp + fb) ^ (tr & 7)) << 3)]);
-      // ldmatrix order: (tokens 0-7, f 0-7), (tokens 0-7, f 8-15), (tokens 8-15, f 0-7), (tokens 8-15, f 8-15) = a0, a1, a2, a3
-      att_mma_f16(d, a, have ? wh[s16 * 8 + c] : 0u, have ? wh[s16 * 8 + c + 4] : 0u);
-      att_mma_f16(d, a, have ? wl[s16 * 8 + c] : 0u, have ? wl[s16 * 8 + c + 4] : 0u);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] = fmaf(d[j], down, acc[j]);
-  }
-  if (2 * c < NQ) {
-    float *ap = jb.a + (((size_t)h * n_chunks + chunk) * 128 + warp * 16 + g) * NQ + 2 * c;
-    *(float2 *)ap = make_float2(acc[0], acc[1]);
-    *(float2 *)(ap + 8 * NQ) = make_float2(acc[2], acc[3]);
+    for (int j = 0; j < NH; ++j)
+      att_put4<NQ>(d[j], 1.f, jb.y + ((size_t)(h0 + j) * n_chunks + t0 / TC) * NQ * vr + k, vr, ok && h0 + j < m);
   }
 }
 
@@ -856,77 +1137,91 @@ __global__ void __launch_bounds__(256) attend_bvalue_kernel(const AttendJob *__r
   for (int half = 0; half < 2; ++half) {
     const int n = n0 + warp * 16 + g + half * 8;
     if (n >= N) continue;
-    float *yr = jb.y + ((size_t)(n / NQP) * n_chunks + chunk) * r_t * NQP + n % NQP;
+    float *yr = jb.y + (((size_t)(n / NQP) * n_chunks + chunk) * NQP + n % NQP) * r_t;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       const int k = kb + nt * 8 + 2 * c;
-      if (k < r_t) yr[(size_t)k * NQP] = acc[nt][half * 2];
-      if (k + 1 < r_t) yr[(size_t)(k + 1) * NQP] = acc[nt][half * 2 + 1];
+      if (k < r_t) yr[k] = acc[nt][half * 2];
+      if (k + 1 < r_t) yr[k + 1] = acc[nt][half * 2 + 1];
     }
   }
 }
 
-// grid (m, groups, n_q), 128 threads (thread = feature); CTA z finishes query z.  Dynamic shared memory:
-// (n_chunks + v.r_t + 128 + 1) floats.
+// grid (m, groups, n_q), 128 threads; CTA z finishes query z.  Dynamic shared memory: (n_chunks + v.r_t + 128) floats.
 __global__ void __launch_bounds__(128) attend_combine_kernel(const AttendJob *__restrict__ jobs, int n_q, int NQP, int n_chunks,
                                                              uint64_t seed) {
   const AttendJob &jb = jobs[blockIdx.y];
-  const int h = blockIdx.x, f = threadIdx.x, i = blockIdx.z;
+  const int h = blockIdx.x, f = threadIdx.x, i = blockIdx.z, warp = f >> 5, lane = f & 31;
   if (h >= jb.m) return;
   extern __shared__ unsigned char att_smem[];
   const int r_t = jb.v.r_t;
   float *coef = (float *)att_smem;                                   // [n_chunks]
-  float *ys = coef + n_chunks;                                       // [r_t]
+  float *ys = coef + ((n_chunks + 3) & ~3);                          // [r_t]
   float *buf = ys + r_t;                                             // [128]
-  float *Ls = buf + 128;                                             // [1]
-  const float *ml = jb.ml + (size_t)h * n_chunks * 2 * NQP;
+  __shared__ float4 part[4][32];
+  __shared__ float Ls;
+  const float *ml = jb.ml + (size_t)h * n_chunks * 2 * NQP + i;
+  const float esc = r_t > 0 ? ldexpf(1.f, *jb.v.e) : 0.f;
+  att_wait_predecessor();
   // running-maximum merge of the chunks: warp 0 finds the maximum and the rescaled sum
-  if (f < 32) {
+  if (warp == 0) {
     float M = -INFINITY;
-    for (int c = f; c < n_chunks; c += 32) M = fmaxf(M, ml[c * 2 * NQP + i]);
+    for (int c = lane; c < n_chunks; c += 32) M = fmaxf(M, ml[(size_t)c * 2 * NQP]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     float L = 0.f;
-    for (int c = f; c < n_chunks; c += 32) {
-      const float cf = expf(ml[c * 2 * NQP + i] - M);
+    for (int c = lane; c < n_chunks; c += 32) {
+      const float cf = expf(ml[(size_t)c * 2 * NQP] - M);
       coef[c] = cf;
-      L = fmaf(cf, ml[c * 2 * NQP + NQP + i], L);
+      L = fmaf(cf, ml[(size_t)c * 2 * NQP + NQP], L);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-    if (f == 0) Ls[0] = L;
+    if (lane == 0) Ls = L;
   }
   __syncthreads();
-  for (int k = f; k < r_t; k += 128) {
-    const float *yp = jb.y + ((size_t)h * n_chunks * r_t + k) * NQP + i;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < n_chunks; ++c) acc = fmaf(coef[c], __ldg(yp + (size_t)c * r_t * NQP), acc);
-    ys[k] = acc;
-  }
-  float res = 0.f;
-  if (jb.v.bits > 0) {
-    const float *ap = jb.a + ((size_t)h * n_chunks * 128 + f) * NQP + i;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < n_chunks; ++c) acc = fmaf(coef[c], __ldg(ap + (size_t)c * 128 * NQP), acc);
-    buf[f] = acc;
-  }
-  __syncthreads();
-  if (jb.v.bits > 0) res = att_wht_smem(buf, f) * kInvSqrtD * att_sign(seed, jb.v.cell, f);
-  float ob = 0.f;
-  if (r_t > 0) {
-    const __half *P = jb.vP + (size_t)h * r_t * 128 + f;
-    float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-    for (int k = 0; k < r_t; k += 4) {       // r_t is a multiple of 8
-      o0 = fmaf(ys[k], __half2float(P[(size_t)k * 128]), o0);
-      o1 = fmaf(ys[k + 1], __half2float(P[(size_t)(k + 1) * 128]), o1);
-      o2 = fmaf(ys[k + 2], __half2float(P[(size_t)(k + 2) * 128]), o2);
-      o3 = fmaf(ys[k + 3], __half2float(P[(size_t)(k + 3) * 128]), o3);
+  auto merge = [&](const float *p, size_t stride) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    int c = 0;
+    for (; c + 16 <= n_chunks; c += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = __ldg(p + (size_t)(c + u) * stride);
+#pragma unroll
+      for (int u = 0; u < 16; ++u) acc[u & 3] = fmaf(coef[c + u], v[u], acc[u & 3]);
     }
-    ob = ((o0 + o1) + (o2 + o3)) * ldexpf(1.f, *jb.v.e);
+    for (; c < n_chunks; ++c) acc[0] = fmaf(coef[c], __ldg(p + (size_t)c * stride), acc[0]);
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  };
+  if (jb.v.bits > 0) buf[f] = merge(jb.a + ((size_t)h * n_chunks * NQP + i) * 128 + f, (size_t)NQP * 128);
+  for (int k = f; k < r_t; k += 128) ys[k] = merge(jb.y + ((size_t)h * n_chunks * NQP + i) * r_t + k, (size_t)NQP * r_t);
+  __syncthreads();
+  // y P_h: a lane per four features, a warp per fourth row
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  const uint2 *P = (const uint2 *)(jb.vP + (size_t)h * r_t * 128) + lane;
+#pragma unroll 8
+  for (int k = warp; k < r_t; k += 4) {
+    const uint2 p = __ldg(P + (size_t)k * 32);
+    const float2 a = __half22float2(*(const __half2 *)&p.x), b = __half22float2(*(const __half2 *)&p.y);
+    const float y = ys[k];
+    o.x = fmaf(y, a.x, o.x); o.y = fmaf(y, a.y, o.y); o.z = fmaf(y, b.x, o.z); o.w = fmaf(y, b.y, o.w);
   }
-  jb.out[((size_t)h * n_q + i) * 128 + f] = (ob + res) / Ls[0];
+  part[warp][lane] = o;
+  __syncthreads();
+  if (warp) return;
+  float res[4] = {0.f, 0.f, 0.f, 0.f};
+  if (jb.v.bits > 0) {
+    const float4 v = *(const float4 *)(buf + 4 * lane);
+    res[0] = v.x; res[1] = v.y; res[2] = v.z; res[3] = v.w;
+    att_wht_warp(res);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) res[j] *= kInvSqrtD * att_sign(seed, jb.v.cell, 4 * lane + j);
+  }
+  const float4 p1 = part[1][lane], p2 = part[2][lane], p3 = part[3][lane];
+  const float L = Ls;
+  *(float4 *)(jb.out + ((size_t)h * n_q + i) * 128 + 4 * lane) =
+      make_float4((((o.x + p1.x) + (p2.x + p3.x)) * esc + res[0]) / L, (((o.y + p1.y) + (p2.y + p3.y)) * esc + res[1]) / L,
+                  (((o.z + p1.z) + (p2.z + p3.z)) * esc + res[2]) / L, (((o.w + p1.w) + (p2.w + p3.w)) * esc + res[3]) / L);
 }
 
 }  // namespace jolt

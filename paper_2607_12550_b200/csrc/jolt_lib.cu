@@ -1899,27 +1899,24 @@ static void launch_att_scores(dim3 grid, size_t shm, cudaStream_t s, const Atten
   attend_scores_kernel<BITS><<<grid, kAttChunk, shm, s>>>(d, NQP);
 }
 template <int BITS>
-static void launch_att_scores_mma(dim3 grid, cudaStream_t s, const AttendJob *d, int NQP) {
-  const int n_chunks = (int)grid.x;
-  grid.x = (grid.x + 1) / 2;                 // two chunks per CTA: the query operand is staged once, the second chunk's rows are prefetched
-  attend_scores_mma_kernel<BITS><<<grid, kAttChunk, 0, s>>>(d, NQP, n_chunks);
-}
-template <int BITS>
-static void launch_att_values_mma(dim3 grid, cudaStream_t s, const AttendJob *d, int NQP) {
-  const size_t shm = (size_t)kAttHalf * 128 * sizeof(__half) + (size_t)4 * 2 * NQP * (kAttHalf + 8) * sizeof(__half);
-  static std::atomic<bool> opted{false};      // 49.4 KB with eight query slots
-  if (!opted.exchange(true)) {
-    cudaFuncSetAttribute(attend_values_mma_kernel<BITS, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    cudaFuncSetAttribute(attend_values_mma_kernel<BITS, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-  }
-  if (NQP == 4) attend_values_mma_kernel<BITS, 4><<<grid, kAttChunk, shm, s>>>(d);
-  else attend_values_mma_kernel<BITS, 8><<<grid, kAttChunk, shm, s>>>(d);
-}
-template <int BITS>
 static void launch_att_values(dim3 grid, cudaStream_t s, const AttendJob *d, int NQP) {
   const size_t shm = (size_t)kAttHalf * (NQP * sizeof(float) + 16 * BITS + 8) + (size_t)4 * 128 * NQP * sizeof(float);
   if (NQP == 4) attend_values_kernel<BITS, 4><<<grid, kAttChunk, shm, s>>>(d);
   else attend_values_kernel<BITS, 8><<<grid, kAttChunk, shm, s>>>(d);
+}
+
+// A launch that may begin while the kernel before it on the stream drains (it waits on the device for that kernel's results).
+template <typename... P, typename... A>
+static void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t shm, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = shm; cfg.stream = s;
+  cudaLaunchAttribute at;
+  memset(&at, 0, sizeof at);
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, double scale, void *dOut, void *stream) {
@@ -1933,7 +1930,8 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
   if (dev != H->device) return fail(JOLT_EINVAL, "handle belongs to device %d, current device is %d", H->device, dev);
   const int ng = H->n_groups, T = H->T, nh = H->n_kv_heads;
   const int NQP = n_q <= 4 ? 4 : 8;
-  const int n_chunks = (T + kAttChunk - 1) / kAttChunk;
+  const bool mma = (g_fast.load() & 1) != 0;        // the streaming kernel (the other kernels stay as the portable path)
+  const int tc = mma ? kAttTok : kAttChunk, n_chunks = (T + tc - 1) / tc;
   int m_max = 0, krt = 0, krf = 0, vrt = 0, vrf = 0;
   unsigned kbits = 0, vbits = 0;
   for (int g = 0; g < ng; ++g) {
@@ -1944,10 +1942,9 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
     kbits |= 1u << ck.bits; vbits |= 1u << cv.bits;
     if ((ck.r_t % 8) || (cv.r_t % 8) || (ck.r_f % 8) || (cv.r_f % 8)) return fail(JOLT_EUNSUPPORTED, "ranks must be multiples of 8");
   }
-  const size_t shm_prep = 128 * sizeof(float);
   const size_t shm_sc = (size_t)128 * NQP * sizeof(float);
   const size_t shm_comb = (size_t)(n_chunks + vrt + 136) * sizeof(float);
-  if (shm_comb > 48 * 1024) return fail(JOLT_EUNSUPPORTED, "sequence of %d tokens: the chunk merge needs %zu bytes of shared memory", T, shm_comb);
+  if (shm_comb > 96 * 1024) return fail(JOLT_EUNSUPPORTED, "sequence of %d tokens: the chunk merge needs %zu bytes of shared memory", T, shm_comb);
   // the projected cores do not depend on the queries: compress (or deserialize) formed them, the handle keeps them
   std::vector<AttendJob> jobs(ng);
   void *ws_base = nullptr;
@@ -1986,47 +1983,63 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
   const size_t off = P.push(jobs);
   const uint64_t seed = H->seed;
   const float fscale = (float)scale;
-  const bool mma = (g_fast.load() & 1) != 0;        // warp-MMA forms of the two code streams (the CUDA-core forms stay as the portable path)
-  const bool vmma = mma;
   P.add(ST_ATT, [=](char *dev_t, cudaStream_t s) {
     const AttendJob *d = (const AttendJob *)(dev_t + off);
-    attend_prep_kernel<<<dim3(m_max, ng, NQP), 128, shm_prep, s>>>(d, n_q, NQP, fscale, seed);
+    if (NQP == 4) attend_prep_kernel<4><<<dim3(m_max, ng), 256, 0, s>>>(d, n_q, fscale, seed);
+    else attend_prep_kernel<8><<<dim3(m_max, ng), 256, 0, s>>>(d, n_q, fscale, seed);
     LAUNCHED();
     const dim3 grid(n_chunks, m_max, ng);
-    const int n_tiles = (m_max * NQP + 127) / 128;
-    if (krt > 0) {
-      attend_bscore_kernel<<<dim3((T + 63) / 64, n_tiles, ng), 256, 0, s>>>(d, NQP);
+    if (mma) {
+      static std::once_flag once;
+      std::call_once(once, [] {
+        cudaFuncSetAttribute(attend_stream_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(4));
+        cudaFuncSetAttribute(attend_stream_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(4));
+        cudaFuncSetAttribute(attend_stream_kernel<8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(8));
+        cudaFuncSetAttribute(attend_stream_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(8));
+      });
+      const bool h4 = m_max >= 3;
+      const dim3 sg(h4 ? n_chunks : (n_chunks + 3) / 4, h4 ? (m_max + 3) / 4 : m_max, ng);
+      const size_t shm = att_stream_smem(NQP);
+      launch_overlapped(NQP == 4 ? (h4 ? attend_stream_kernel<4, 4> : attend_stream_kernel<4, 1>) : (h4 ? attend_stream_kernel<8, 4> : attend_stream_kernel<8, 1>),
+                        sg, kAttStreamThreads, shm, s, d, n_chunks);
       LAUNCHED();
-    }
-    for (int b = 0; b <= 8; ++b) {
-      if (!((kbits >> b) & 1)) continue;
-      switch (b) {
-        case 0: launch_att_scores<0>(grid, shm_sc, s, d, NQP); break;
-        case 1: if (mma) launch_att_scores_mma<1>(grid, s, d, NQP); else launch_att_scores<1>(grid, shm_sc, s, d, NQP); break;
-        case 2: if (mma) launch_att_scores_mma<2>(grid, s, d, NQP); else launch_att_scores<2>(grid, shm_sc, s, d, NQP); break;
-        case 3: launch_att_scores<3>(grid, shm_sc, s, d, NQP); break;
-        case 4: if (mma) launch_att_scores_mma<4>(grid, s, d, NQP); else launch_att_scores<4>(grid, shm_sc, s, d, NQP); break;
-        default: if (mma) launch_att_scores_mma<8>(grid, s, d, NQP); else launch_att_scores<8>(grid, shm_sc, s, d, NQP); break;
+    } else {
+      const int n_tiles = (m_max * NQP + 127) / 128;
+      if (krt > 0) {
+        attend_bscore_kernel<<<dim3((T + 63) / 64, n_tiles, ng), 256, 0, s>>>(d, NQP);
+        LAUNCHED();
       }
-      LAUNCHED();
-    }
-    for (int b = 1; b <= 8; ++b) {                 // b = 0: no residual, nothing to stream
-      if (!((vbits >> b) & 1)) continue;
-      switch (b) {
-        case 1: if (vmma) launch_att_values_mma<1>(grid, s, d, NQP); else launch_att_values<1>(grid, s, d, NQP); break;
-        case 2: if (vmma) launch_att_values_mma<2>(grid, s, d, NQP); else launch_att_values<2>(grid, s, d, NQP); break;
-        case 3: launch_att_values<3>(grid, s, d, NQP); break;
-        case 4: if (vmma) launch_att_values_mma<4>(grid, s, d, NQP); else launch_att_values<4>(grid, s, d, NQP); break;
-        default: if (vmma) launch_att_values_mma<8>(grid, s, d, NQP); else launch_att_values<8>(grid, s, d, NQP); break;
+      for (int b = 0; b <= 8; ++b) {
+        if (!((kbits >> b) & 1)) continue;
+        switch (b) {
+          case 0: launch_att_scores<0>(grid, shm_sc, s, d, NQP); break;
+          case 1: launch_att_scores<1>(grid, shm_sc, s, d, NQP); break;
+          case 2: launch_att_scores<2>(grid, shm_sc, s, d, NQP); break;
+          case 3: launch_att_scores<3>(grid, shm_sc, s, d, NQP); break;
+          case 4: launch_att_scores<4>(grid, shm_sc, s, d, NQP); break;
+          default: launch_att_scores<8>(grid, shm_sc, s, d, NQP); break;
+        }
+        LAUNCHED();
       }
-      LAUNCHED();
+      for (int b = 1; b <= 8; ++b) {                 // b = 0: no residual, nothing to stream
+        if (!((vbits >> b) & 1)) continue;
+        switch (b) {
+          case 1: launch_att_values<1>(grid, s, d, NQP); break;
+          case 2: launch_att_values<2>(grid, s, d, NQP); break;
+          case 3: launch_att_values<3>(grid, s, d, NQP); break;
+          case 4: launch_att_values<4>(grid, s, d, NQP); break;
+          default: launch_att_values<8>(grid, s, d, NQP); break;
+        }
+        LAUNCHED();
+      }
+      if (vrt > 0) {
+        const int KT = (vrt + 63) / 64;
+        attend_bvalue_kernel<<<dim3(n_chunks * KT, n_tiles, ng), 256, 0, s>>>(d, NQP, n_chunks, KT);
+        LAUNCHED();
+      }
     }
-    if (vrt > 0) {
-      const int KT = (vrt + 63) / 64;
-      attend_bvalue_kernel<<<dim3(n_chunks * KT, n_tiles, ng), 256, 0, s>>>(d, NQP, n_chunks, KT);
-      LAUNCHED();
-    }
-    attend_combine_kernel<<<dim3(m_max, ng, n_q), 128, shm_comb, s>>>(d, n_q, NQP, n_chunks, seed);
+    if (shm_comb > 48 * 1024) cudaFuncSetAttribute(attend_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    launch_overlapped(attend_combine_kernel, dim3(m_max, ng, n_q), 128, shm_comb, s, d, n_q, NQP, n_chunks, seed);
     LAUNCHED();
   });
   void *d_tab = nullptr;

@@ -1,0 +1,49 @@
+"""The streaming attention kernel against the CUDA-core kernels (bit 0 of the kernel mask off) where its shapes change: four
+heads a CTA or four chunks of one head, partial head quads and last chunks, ranks that are no multiple of its 32-column blocks,
+every code width in both roles."""
+import pytest
+import torch
+
+import __graft_entry__ as entry
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    entry.build()
+    import paper_2607_12550_b200 as pkg
+    return pkg.load()
+
+
+# layers, first layer of the second group, heads, tokens, ranks (K, V) of both groups, bits (K, V) of both groups, queries
+@pytest.mark.parametrize("L,g1,H,T,ranks,bits,nq", [
+    (2, 1, 1, 128, (8, 8, 16, 40), (8, 1, 1, 8), 1),              # one head a cell: four chunks a CTA, three of them past the end
+    (2, 1, 1, 640, (40, 8, 8, 72), (3, 4, 4, 3), 8),
+    (2, 1, 2, 768, (0, 8, 32, 0), (2, 8, 8, 2), 4),
+    (3, 2, 3, 384, (264, 136, 24, 0), (4, 8, 0, 4), 4),           # six and three heads: a partial quad
+    (3, 2, 5, 256, (64, 96, 8, 248), (8, 2, 3, 1), 8),
+    (5, 4, 4, 512, (128, 112, 96, 40), (1, 3, 8, 0), 5),
+])
+def test_stream_matches_cuda_core_path(B, L, g1, H, T, ranks, bits, nq):
+    g = torch.Generator().manual_seed(L * 1000 + T)
+    base = torch.randn(L, 1, T, 24, generator=g) @ torch.randn(L, H, 24, 128, generator=g)
+    K, V = (base + 0.3 * torch.randn(L, H, T, 128, generator=g)).half().cuda(), (base.flip(0) + torch.randn(L, H, T, 128, generator=g)).half().cuda()
+    plan = [(r, 128 if r else 0, b) for r, b in zip(ranks, bits)]
+    h = B.jolt_compress(K, V, [0, g1, L], plan, B.default_options(seed=5, power_iters=0))
+    Q = torch.randn(L, H, nq, 128, generator=g).cuda()
+    Q[0, 0, 0] *= 8.0                                             # a sharp row: one chunk carries the weight
+    out = B.jolt_attend(h, Q)
+    prev = B.set_fast_path(14)
+    try:
+        ref = B.jolt_attend(h, Q)
+        torch.cuda.synchronize()
+    finally:
+        B.set_fast_path(prev)
+    h.free()
+    assert torch.isfinite(out).all()
+    # hi + lo fp16 operands (2^-22 each) give scores to 2^-21 of the largest, which is the relative error of a weight; the
+    # values' own sums add a few 2^-22
+    smax = torch.einsum("lhqf,lhtf->lhqt", Q, K.float()).abs().amax(-1) / 128 ** 0.5
+    per_row = (out - ref).norm(dim=-1) / ref.norm(dim=-1)
+    assert bool((per_row <= 5e-6 + 2.0 ** -21 * smax).all()), (per_row / smax).max()
