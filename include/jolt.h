@@ -321,7 +321,8 @@ int jolt_test_set_wait_limit(int64_t cycles, int32_t skip_first_load);
 int jolt_test_set_decode_tail(int32_t percent, int32_t chunk_tiles);
 
 /* Wall-clock-free per-stage device timing of the last compress / decompress on this thread
- * (milliseconds, CUDA events): out[0..n) in stage order, names via jolt_stage_name. */
+ * (milliseconds, CUDA events; the start and end that the kernel itself took where a decode on the default stream is one
+ * kernel): out[0..n) in stage order, names via jolt_stage_name. */
 int jolt_last_stage_ms(float *out, int32_t cap, int32_t *n);
 const char *jolt_stage_name(int32_t i);
 

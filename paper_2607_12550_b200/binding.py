@@ -7,7 +7,6 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-from dataclasses import dataclass
 from typing import Sequence
 
 import numpy as np
@@ -112,26 +111,20 @@ def _check(status: int, allow=()):
     return status
 
 
-@dataclass
-class _Keep:
-    layout: Layout
-    gs: object
-
-
 def make_layout(K: torch.Tensor, group_start: Sequence[int], V: torch.Tensor | None = None) -> Layout:
     """Layout of a [n_layers, n_kv_heads, T, 128] tensor (any strides with unit feature stride).
 
     The C ABI describes K and V by ONE layout: when V is given it must match K in shape, strides, dtype and device."""
-    assert K.dim() == 4 and K.stride(3) == 1
-    if V is not None and (V.shape != K.shape or V.stride() != K.stride() or V.dtype != K.dtype or V.device != K.device):
+    shape, stride, dtype = K.shape, K.stride(), K.dtype
+    n_layers, n_heads, T, d = shape
+    s_layer, s_head, s_token, s_feature = stride
+    assert s_feature == 1
+    if V is not None and (V.shape != shape or V.stride() != stride or V.dtype != dtype or V.device != K.device):
         raise ValueError("K and V must share shape, strides, dtype and device (one jolt_layout describes both)")
-    gs = (C.c_int32 * len(group_start))(*group_start)
-    lay = Layout(K.shape[0], K.shape[1], K.shape[2], K.shape[3],
-                 F16 if K.dtype == torch.float16 else F32,
-                 MEM_DEVICE if K.is_cuda else MEM_HOST,
-                 K.stride(0), K.stride(1), K.stride(2), len(group_start) - 1, gs)
-    lay._gs = gs  # keep alive
-    return lay
+    n = len(group_start)
+    # (the structure keeps the array it points to alive)
+    return Layout(n_layers, n_heads, T, d, F16 if dtype is torch.float16 else F32, MEM_DEVICE if K.is_cuda else MEM_HOST,
+                  s_layer, s_head, s_token, n - 1, (C.c_int32 * n)(*group_start))
 
 
 def default_options(**kw) -> Options:

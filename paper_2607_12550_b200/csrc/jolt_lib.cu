@@ -58,32 +58,64 @@ static const char *kStageNames[] = {"stage_in", "sketch_gen", "gram", "eig_feat"
                                     "small_svd", "factors", "store", "backbone", "residual_quant", "decode_backbone",
                                     "decode_rows", "rope", "attend", "stage_out"};
 constexpr int kNumStages = sizeof(kStageNames) / sizeof(kStageNames[0]);
+constexpr int kStampedStage = 14;                // decode_rows
 struct StageTimer {
   cudaEvent_t ev[kNumStages + 1];
   bool have = false;
   int order[kNumStages + 1];
   int n = 0;
   float ms[kNumStages];
+  int stamp_dev = -1;          // >= 0: the last call was a single kernel that stamped its own start and end there
+  unsigned long long *stamps = nullptr;
   void init() {
     if (have) return;
     for (auto &e : ev) cudaEventCreate(&e);
     have = true;
   }
-  void begin(cudaStream_t s) { init(); n = 0; for (auto &m : ms) m = 0.f; cudaEventRecord(ev[0], s); }
+  void begin(cudaStream_t s) { init(); n = 0; stamp_dev = -1; for (auto &m : ms) m = 0.f; cudaEventRecord(ev[0], s); }
   void mark(int stage, cudaStream_t s) { if (n < kNumStages) { order[n] = stage; ++n; cudaEventRecord(ev[n], s); } }
+  void begin_stamped(int dev, unsigned long long *p) { n = 0; for (auto &m : ms) m = 0.f; stamp_dev = dev; stamps = p; }
   void finish() {
     for (auto &m : ms) m = 0.f;
+    if (stamp_dev >= 0) { finish_stamped(); return; }
     for (int i = 0; i < n; ++i) { float t = 0; if (cudaEventElapsedTime(&t, ev[i], ev[i + 1]) == cudaSuccess) ms[order[i]] += t; }
   }
+  void finish_stamped();
 };
 thread_local StageTimer g_timer;
 enum { ST_IN = 0, ST_SKGEN, ST_GRAM, ST_EIGF, ST_SKETCH, ST_ORTH, ST_POWER, ST_PROJ, ST_SVD, ST_FACT, ST_STORE, ST_BACK,
        ST_RQ, ST_DBACK, ST_DROWS, ST_ROPE, ST_ATT, ST_OUT };
+static_assert(ST_DROWS == kStampedStage, "stage order");
 
 // ------------------------------------------------------------------ workspace cache (per device)
 struct Workspace { void *base = nullptr; size_t cap = 0; };
 static std::mutex g_ws_mu;
 static Workspace g_ws[64];
+
+// Start and end (globaltimer) of the last single-kernel call of a thread: 64 slots of a device, dealt out to threads in turn (with
+// more threads than slots a time may be another thread's).  A pair of timing events around a short decode cost 5 us of GPU time.
+constexpr int kStampSlots = 64;
+static unsigned long long *g_stamps[64];          // under g_ws_mu
+static unsigned long long *stamp_slot(int dev) {
+  static std::atomic<unsigned> next{0};
+  static thread_local unsigned slot = next.fetch_add(1) % kStampSlots;
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  if (!g_stamps[dev]) {
+    if (cudaMalloc(&g_stamps[dev], kStampSlots * 16) != cudaSuccess || cudaMemset(g_stamps[dev], 0, kStampSlots * 16) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+  }
+  return g_stamps[dev] + 2 * slot;
+}
+void StageTimer::finish_stamped() {
+  unsigned long long t[2] = {0, 0};
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  const unsigned long long *base = g_stamps[stamp_dev];
+  if (!base || !stamps || stamps < base || stamps >= base + 2 * kStampSlots) return;       // given back since
+  if (cudaMemcpy(t, stamps, sizeof t, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); return; }
+  if (t[1] > t[0]) ms[kStampedStage] = (float)(t[1] - t[0]) * 1e-6f;
+}
 
 static int ws_reserve(int dev, size_t bytes, void **out) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
@@ -280,6 +312,7 @@ struct jolt_handle {
   int64_t stored_bytes = 0;
   bool subspace = false;     // token factors came from the converged block iteration (exact mode, large T)
   int *d_status = nullptr;   // 4 words per cell, written by the decode kernels of the last call on this handle (jolt_check_status): epoch << 8 | bits
+  mutable std::atomic<bool> unreleased{false};  // a call on the default stream since the last that left the arena's event behind
   mutable cudaStream_t last_stream = nullptr;   // stream of the last call that read the handle's buffers (jolt_free orders after it)
   // The tail of the same device allocation (not part of the stored bytes or of a serialised image): the status words, the
   // projected cores P_h = fp16(G_h U_F^T) of the cells that need them (CellStore::P16), the descriptors
@@ -1662,7 +1695,8 @@ static void of_this_epoch(const jolt_handle *H, std::vector<int> &words) {      
 
 // The cells on the tensor-core kernels: the persistent kernel for r_t <= 128, the per-item kernel for the others and for key
 // cells whose rotation happens in its epilogue (`rope`: their table).
-static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Kout, char *Vout, const float2 *rope, int dev, cudaStream_t st) {
+static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Kout, char *Vout, const float2 *rope, unsigned long long *stamps, int dev,
+                            cudaStream_t st) {
   static std::atomic<int> n_sm[64];
   if (!n_sm[dev].load()) {
     int v = 0;
@@ -1691,7 +1725,7 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   if ((g_fast.load() & 128) && d.end[pc] > 0 && d.tiles[pc] < (1ll << 30)) {
     const int total = (int)d.tiles[pc], pct = g_dec_tail_pct.load(), grid = std::min(n_sm[dev].load(), total);
     a.cells = (const tc::BBCell *)H->d_dec; a.n_cells = d.end[pc]; a.total = total;
-    a.nt = H->T / 128; a.seed = H->seed; a.epoch = H->status_epoch;
+    a.nt = H->T / 128; a.seed = H->seed; a.epoch = H->status_epoch; a.stamps = stamps;
     // The tail that is dealt out in chunks is empty unless a test asks for one: measured on the benchmark mix, a 5 % tail in
     // 8-tile chunks made the launch slower (0.199 against 0.192 ms), because every chunk reloads its head's projected
     // core into the single P buffer and restarts the unpack -> rotation pipeline.
@@ -1706,6 +1740,12 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   if (d.end[1] < d.end[2]) launch_decode_items(H, d.end[1], d.end[2] - d.end[1], a.out, rope, dbg, st);
   CU(cudaGetLastError());
   return JOLT_OK;
+}
+
+// arena_acquire for a call that reads a handle: also after the calls on the default stream that left no event behind
+static int handle_acquire(const jolt_handle *H, int dev, cudaStream_t st) {
+  if (st && H->unreleased.exchange(false)) arena_release(dev, nullptr);
+  return arena_acquire(dev, st);
 }
 
 static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kout, void *Vout, const jolt_rope *rope,
@@ -1734,6 +1774,26 @@ static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kou
   const size_t esz = L->dtype == JOLT_F16 ? 2 : 4;
   const size_t span = layout_span_elems(L) * esz;
   const bool fast = (g_fast.load() & 1) != 0;
+  // A device destination of a cache whose cells all take the persistent kernel needs nothing but its launch: no shared memory of
+  // the library, and what the kernel writes into the status words carries the epoch of the call.  The other kernels write
+  // plain bits: words cleared.
+  int epoch = 0;
+  if (fast && H->dec.end[2] == nc && H->dec.end[1] == nc && !rope && (g_fast.load() & 128)) epoch = H->epoch.fetch_add(1) + 1;
+  if (epoch >= 1 << 22) { H->epoch = 1; epoch = 0; }                               // the epochs start again
+  if (epoch && L->mem_space != JOLT_MEM_HOST) {
+    // Calls on the default stream that follow one another there are in order as it is; the event that orders the users of the
+    // shared memory is left out until another stream comes, and the kernel takes its own times.
+    const bool in_order = !st && !H->last_stream && g_dec_tail_pct.load() == 0;
+    if (!in_order && (rc = handle_acquire(H, dev, st))) return rc;
+    H->last_stream = st;
+    H->status_epoch = epoch;
+    unsigned long long *stamps = in_order ? stamp_slot(dev) : nullptr;
+    if (stamps) g_timer.begin_stamped(dev, stamps); else g_timer.begin(st);
+    if ((rc = launch_decode_tc(H, L, (char *)Kout, (char *)Vout, nullptr, stamps, dev, st))) return rc;
+    if (!stamps) g_timer.mark(ST_DROWS, st);
+    if (in_order) H->unreleased = true; else arena_release(dev, st);
+    return JOLT_OK;
+  }
   std::vector<CellWork> ws(nc);
   std::vector<char> use_tc(nc, 0);
   int n_tc = 0;
@@ -1830,14 +1890,9 @@ static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kou
   lap("program");
   void *d_tab = nullptr;
   if (!P.host.empty() && (rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
-  if ((rc = arena_acquire(dev, st))) return rc;
+  if ((rc = handle_acquire(H, dev, st))) return rc;
   H->last_stream = st;
   g_timer.begin(st);
-  // A device destination of a cache whose cells all take the persistent kernel needs nothing but its launch: what that
-  // kernel writes into the status words carries the epoch of the call.  The other kernels write plain bits: words cleared.
-  int epoch = 0;
-  if (n_tc == nc && H->dec.end[1] == H->dec.end[2] && !rope && (g_fast.load() & 128)) epoch = H->epoch.fetch_add(1) + 1;
-  if (epoch >= 1 << 22) { H->epoch = 1; epoch = 0; }                               // the epochs start again
   if (epoch == 0) CU(cudaMemsetAsync(d_status, 0, sizeof(int) * 4 * nc, st));
   H->status_epoch = epoch;
   lap("acquire+memset");
@@ -1848,7 +1903,7 @@ static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kou
     if ((rc = run_program(head, (char *)d_tab, st))) return rc;
   }
   if (n_tc) {
-    if ((rc = launch_decode_tc(H, L, Kd, Vd, n_rope_fused ? rope_tab : nullptr, dev, st))) return rc;
+    if ((rc = launch_decode_tc(H, L, Kd, Vd, n_rope_fused ? rope_tab : nullptr, nullptr, dev, st))) return rc;
     g_timer.mark(ST_DROWS, st);
   }
   if ((rc = run_program(P, (char *)d_tab, st))) return rc;
@@ -2044,7 +2099,7 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
   });
   void *d_tab = nullptr;
   if ((rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
-  if ((rc = arena_acquire(dev, st))) return rc;
+  if ((rc = handle_acquire(H, dev, st))) return rc;
   H->last_stream = st;
   g_timer.begin(st);
   if ((rc = run_program(P, (char *)d_tab, st))) return rc;
@@ -2496,6 +2551,7 @@ extern "C" int jolt_release_workspace(void) {
   cudaDeviceSynchronize();
   if (g_ws[dev].base) { cudaFree(g_ws[dev].base); g_ws[dev] = Workspace(); }
   if (g_tab[dev].base) { cudaFree(g_tab[dev].base); g_tab[dev] = Workspace(); }
+  if (g_stamps[dev]) { cudaFree(g_stamps[dev]); g_stamps[dev] = nullptr; }
   return JOLT_OK;
 }
 #ifdef JOLT_DEBUG
@@ -2529,7 +2585,7 @@ extern "C" int jolt_set_fast_path(int enabled) { return g_fast.exchange(enabled 
 extern "C" int jolt_last_stage_ms(float *out, int32_t cap, int32_t *n) {
   if (!out || !n) return fail(JOLT_EINVAL, "null argument");
   *n = std::min<int>(cap, kNumStages);
-  if (g_timer.have) g_timer.finish();
+  if (g_timer.have || g_timer.stamp_dev >= 0) g_timer.finish();
   for (int i = 0; i < *n; ++i) out[i] = g_timer.ms[i];
   return JOLT_OK;
 }

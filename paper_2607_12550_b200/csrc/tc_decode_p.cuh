@@ -44,11 +44,18 @@ struct DecPArgs {
   int pool;            // tiles [0, pool) are dealt out in equal shares; from here on in chunks ...
   int chunk;           // ... of this many tiles
   int *counter;        // chunks handed out so far (zero at launch when pool < total; not read otherwise)
+  unsigned long long *stamps;      // optional: start of the first CTA, end of the last (globaltimer, ns)
   int epoch;           // a failed wait writes (epoch << 8 | 8) into the status word of the first cell
 #ifdef JOLT_DEBUG
   long long *dbg;
 #endif
 };
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
 
 // linear tile p of the launch -> (cell, head, tile in head); cells[].tile_base is the first linear tile of a cell
 struct DecPos { int ci, h, tile; };
@@ -251,6 +258,8 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   const int run0_first = (int)((long long)pool * blockIdx.x / gridDim.x), run0_end = (int)((long long)pool * (blockIdx.x + 1) / gridDim.x);
   JOLT_DBG(long long *cta_dbg = a.dbg ? a.dbg + 128 + blockIdx.x * 4 : nullptr;)
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; unsigned sm; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)); cta_dbg[0] = g; cta_dbg[2] = sm; })
+
+  if (a.stamps && blockIdx.x == 0 && threadIdx.x == 0) a.stamps[0] = global_ns();
 
   // shared memory: P block (32 KB) | output staging (2 x 16 KB) | rotation operand H | U_T ring | operand tiles | barriers
   const uint32_t raw = smem_u32(smem_raw);
@@ -531,6 +540,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   tc_fence_before();
   __syncthreads();
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); cta_dbg[1] = g; cta_dbg[3] = 0; })
+  if (a.stamps && threadIdx.x == 0) atomicMax(a.stamps + 1, global_ns());
   if (*abort_flag) {
     if (threadIdx.x == 0) atomicMax(cells[0].status, a.epoch << 8 | 8);
     const long long t0 = clock64();

@@ -88,3 +88,31 @@ def test_memory_of_freed_handles_is_used_again_in_order(B):
     torch.cuda.synchronize()
     assert torch.equal(got[0][0], want[1][0])
     h.free()
+
+
+def test_default_stream_decodes_then_another_stream(B):
+    """Decodes that follow one another on the default stream leave no event behind; a call on another stream and the free after
+    it still come after all of them."""
+    g = torch.Generator().manual_seed(3)
+    K, V = (torch.randn(2, 4, 1024, 128, generator=g).half().cuda() for _ in range(2))
+    plan = [(32, 128, 4), (16, 64, 2)]
+    opts = B.default_options(seed=1, power_iters=0)
+    side = torch.cuda.Stream()
+    h = B.jolt_compress(K, V, [0, 2], plan, opts)
+    ref = [torch.empty_like(K), torch.empty_like(V)]
+    B.jolt_decompress(h, *ref, [0, 2])
+    torch.cuda.synchronize()
+    for _ in range(4):
+        outs = [[torch.zeros_like(K), torch.zeros_like(V)] for _ in range(4)]
+        torch.cuda.synchronize()
+        for o in outs[:3]:
+            B.jolt_decompress(h, *o, [0, 2])
+        B.jolt_decompress(h, *outs[3], [0, 2], stream=side)
+        h.free()
+        h2 = B.jolt_compress(-K, V.flip(0), [0, 2], plan, opts, stream=side)        # takes over the freed memory
+        h2.free()
+        h = B.jolt_compress(K, V, [0, 2], plan, opts)
+        torch.cuda.synchronize()
+        for o in outs:
+            assert torch.equal(o[0], ref[0]) and torch.equal(o[1], ref[1])
+    h.free()
