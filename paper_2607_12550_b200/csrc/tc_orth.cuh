@@ -204,9 +204,11 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
 // upper triangle X, the diagonal of X in `invd`).  Per panel: (1) warp 0 factors the 8 x 8 diagonal block in
 // registers, (2) one thread per row solves its 8 panel entries against the block (rows above the panel are rows of X,
 // rows below are rows of L, the same recurrence), (3) the trailing update W[i][j] -= sum_c P[i][c] P[j][c] for the
-// rows of X (i < panel end) and of the Schur complement (i >= j): first the next panel's eight columns, then -- while
-// warp 0 already factors the next diagonal block (look-ahead) -- the rest, four columns per warp pass.  Three barriers
-// per panel.
+// rows of X (i < panel end) and of the Schur complement (i >= j), four columns per warp pass, while warp 0 updates and
+// factors the next diagonal block by itself (look-ahead).  Two barriers per panel.  98 -> 80 us a launch at n up to 138, 66 -> 47 at
+// n up to 106: square roots left the pivots' chain (1880 cycles a block), the separate update of the next eight columns and its
+// barrier are gone, 16 loads in flight.  The update is bound by shared memory: it reads and writes the trailing matrix once per
+// eight columns (2400 of its 2850 cycles at n = 138).
 // A pivot not above `dead_rel` of its original diagonal entry belongs to a direction that is dependent to working
 // accuracy: its column of L and its row / column of L^-1 are zero, status bit 1.
 // Input: fp32 row-chunk partials of the Gram kernel (summed here in fp64) or an fp64 matrix.  Output: L^-1 as fp16
@@ -237,82 +239,87 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
   double *ipiv = (double *)(blkd + 8);      // [8]
   double *diag0 = ipiv + 8;                 // [n] original diagonal
   double *invd = diag0 + n;                 // [n] diagonal of X = 1 / L_ii (0 for a dead pivot)
-  __shared__ float s_red[32];
-  __shared__ int s_exp, s_dead;
+  __shared__ int s_red[32], s_dead;
   const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
   if (tid == 0) s_dead = 0;
   // a warp per column j, lanes over the rows i >= j: both the fp64 input (its upper triangle, (row j, column i): the
-  // matrix is symmetric) and the Gram partials are then read along contiguous addresses
+  // matrix is symmetric) and the Gram partials are then read along contiguous addresses.  Entry (i, j) of the partials is
+  // read as (row j, column i), which is stored for every such pair (row j < 128 holds all columns; j >= 128 implies i >= 128);
+  // 64 rows of eight chunks in flight per warp (one SM reads it all: 13 us with 32, the largest part after the pivots).
   for (int j = warp; j < n; j += nw) {
-    for (int i = lane; i < n; i += 32) {
-      double v = 0.0;
-      if (i >= j) {
-        if (t.A64) v = t.A64[(size_t)j * n + i];
-        else {
-          // entry (i, j), i >= j, is read as (row j, column i) of the partials, which is stored for every such pair
-          // (row j < 128 holds all columns; j >= 128 implies i >= 128)
-          const float *p = t.part + (size_t)j * kp + i;
-          const size_t cs = (size_t)kp * kp;
-          int ch = 0;
-          for (; ch + 8 <= t.n_chunks; ch += 8) {
-            float a[8];
+    const size_t cs = (size_t)kp * kp;
+    for (int i0 = j + lane; i0 < n + lane; i0 += 64) {
+      const int q0 = min(i0, n - 1), q1 = min(i0 + 32, n - 1);
+      double v0 = 0.0, v1 = 0.0;
+      if (t.A64) { v0 = t.A64[(size_t)j * n + q0]; v1 = t.A64[(size_t)j * n + q1]; }
+      else {
+        const float *p = t.part + (size_t)j * kp;
+        int ch = 0;
+        for (; ch + 8 <= t.n_chunks; ch += 8) {
+          float x[8], y[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) a[q] = __ldg(p + (size_t)(ch + q) * cs);
-            v += (((double)a[0] + (double)a[1]) + ((double)a[2] + (double)a[3])) + (((double)a[4] + (double)a[5]) + ((double)a[6] + (double)a[7]));
-          }
-          for (; ch < t.n_chunks; ++ch) v += (double)__ldg(p + (size_t)ch * cs);
+          for (int q = 0; q < 8; ++q) { x[q] = __ldg(p + (size_t)(ch + q) * cs + q0); y[q] = __ldg(p + (size_t)(ch + q) * cs + q1); }
+          v0 += (((double)x[0] + (double)x[1]) + ((double)x[2] + (double)x[3])) + (((double)x[4] + (double)x[5]) + ((double)x[6] + (double)x[7]));
+          v1 += (((double)y[0] + (double)y[1]) + ((double)y[2] + (double)y[3])) + (((double)y[4] + (double)y[5]) + ((double)y[6] + (double)y[7]));
         }
+        for (; ch < t.n_chunks; ++ch) { v0 += (double)__ldg(p + (size_t)ch * cs + q0); v1 += (double)__ldg(p + (size_t)ch * cs + q1); }
       }
-      W[(size_t)j * n + i] = v;
+      if (i0 < n) W[(size_t)j * n + i0] = v0;
+      if (i0 + 32 < n) W[(size_t)j * n + i0 + 32] = v1;
     }
+    for (int i = lane; i < j; i += 32) W[(size_t)j * n + i] = 0.0;
   }
   __syncthreads();
   for (int i = tid; i < n; i += nt) diag0[i] = W[(size_t)i * n + i];
   __syncthreads();
-  // (1) the 8 x 8 diagonal block at j0: every lane of warp 0 factors it in registers (broadcast loads, no shuffles on
-  // the dependent chain), then publishes the block and the reciprocal pivots
+  // (1) the 8 x 8 diagonal block at j0 (in blkd): every lane of warp 0 factors it in registers as L D L^T -- a reciprocal, a
+  // product and an FMA per pivot on the dependent chain, 86 cycles where the square root took 170 -- lane c finds the
+  // reciprocal square root of pivot c, then the block and those are published
   auto factor_block = [&](int j0) {
     const int w = min(8, n - j0);
-    double Lb[8][8], piv[8];
-    int dead = 0;
+    double Lb[8][8], mine = 0.0;
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
-      for (int cc = 0; cc <= r; ++cc) Lb[r][cc] = (r < w && cc < w) ? W[(size_t)(j0 + cc) * n + j0 + r] : (r == cc ? 1.0 : 0.0);
+      for (int cc = 0; cc <= r; ++cc) Lb[r][cc] = blkd[r][cc];
+    __syncwarp();
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
-      piv[cc] = 0.0;
-      if (cc < w) {
-        const double d = Lb[cc][cc], dg = diag0[j0 + cc];
-        const bool bad = !(d > t.dead_rel * dg) || !(dg > 0);
-        const double rs = bad ? 0.0 : rsqrt_pos(d);
-        Lb[cc][cc] = bad ? 0.0 : d * rs;
-        dead |= bad ? 1 : 0;
-        piv[cc] = rs;
+      const double d = Lb[cc][cc], dg = cc < w ? diag0[j0 + cc] : 0.0;
+      const bool bad = !(d > t.dead_rel * dg) || !(dg > 0);
+      const double inv = bad ? 0.0 : 1.0 / d;
+      if (lane == cc) mine = bad ? 0.0 : d;
+      double tr[8];
 #pragma unroll
-        for (int r = cc + 1; r < 8; ++r) Lb[r][cc] *= rs;
+      for (int r = cc + 1; r < 8; ++r) tr[r] = Lb[r][cc] * inv;
 #pragma unroll
-        for (int c2 = cc + 1; c2 < 8; ++c2)
+      for (int c2 = cc + 1; c2 < 8; ++c2)
 #pragma unroll
-          for (int r = c2; r < 8; ++r) Lb[r][c2] = fma(-Lb[r][cc], Lb[c2][cc], Lb[r][c2]);
-      }
+        for (int r = c2; r < 8; ++r) Lb[r][c2] = fma(-Lb[r][cc], tr[c2], Lb[r][c2]);
     }
+    const double rs = mine > 0.0 ? rsqrt_pos(mine) : 0.0;
+    if (lane < w && mine == 0.0) s_dead = 1;
+    if (lane < 8) ipiv[lane] = rs;
+    __syncwarp();
+    double piv[8];
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) piv[cc] = ipiv[cc];
     if (lane < 8) {
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr)
         if (rr == lane) {
 #pragma unroll
-          for (int cc = 0; cc < 8; ++cc) blkd[rr][cc] = cc <= rr ? Lb[rr][cc] : 0.0;
+          for (int cc = 0; cc < 8; ++cc) blkd[rr][cc] = cc <= rr ? Lb[rr][cc] * piv[cc] : 0.0;
         }
     }
-    if (lane == 0) {
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) ipiv[cc] = piv[cc];
-      if (dead) s_dead = 1;
-    }
   };
+  if (warp == 0) {
+    for (int e = lane; e < 64; e += 32) { const int r = e & 7, c = e >> 3; blkd[r][c] = r < n && c <= r ? W[(size_t)c * n + r] : 0.0; }
+    __syncwarp();
+  }
   if (warp == 0) factor_block(0);
   __syncthreads();
+  int mxh = 0;                                 // largest |X| so far: the high word of its fp64
   for (int j0 = 0; j0 < n; j0 += 8) {
     const int w = min(8, n - j0);
     // (2) the panel entries of every row: x_c = (p_c - sum_{l<c} x_l L[c][l]) / L[c][c]
@@ -339,44 +346,48 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
           else if (cc > r) W[(size_t)(j0 + cc) * n + i] = x[cc];              // row of X
           else W[(size_t)(j0 + cc) * n + i] = blkd[r][cc];                    // row of L (diagonal included)
           if (inside && cc == r) invd[i] = x[cc];
+          if (i < j0 + w && (!inside || cc >= r)) mxh = max(mxh, __double2hiint(x[cc]) & 0x7FFFFFFF);
         }
       }
     }
     __syncthreads();
     const int m0 = j0 + w;
     if (m0 >= n) break;
-    // (3a) trailing update of the NEXT panel's columns only (one thread per row), so that warp 0 can factor the next
-    // diagonal block while the other warps finish the update (look-ahead)
+    // (1') warp 0 brings the next diagonal block up to date and factors it || (3) the other warps update the trailing columns,
+    // four per warp pass; rows i < m0 belong to X, rows i >= column to the Schur complement.  The next diagonal block's own
+    // entries in W are left as they are: warp 0 reads them meanwhile and nobody needs them afterwards.
     const int wn = min(8, n - m0);
-    for (int i = tid; i < n; i += nt) {
-      double pi[8];
+    if (warp == 0) {
+      double bv[2];
 #pragma unroll
-      for (int cc = 0; cc < 8; ++cc) pi[cc] = pan[cc * n + i];
+      for (int u = 0; u < 2; ++u) {
+        const int e = lane + 32 * u, r = e & 7, c = e >> 3;
+        bv[u] = 0.0;
+        if (r < wn && c <= r) {
+          double a0 = W[(size_t)(m0 + c) * n + m0 + r], a1 = 0.0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int j = m0 + q;
-        if (q < wn && (i < m0 || i >= j)) {
-          double a0 = 0, a1 = 0;
-#pragma unroll
-          for (int cc = 0; cc < 8; cc += 2) { a0 = fma(pi[cc], pan[cc * n + j], a0); a1 = fma(pi[cc + 1], pan[(cc + 1) * n + j], a1); }
-          W[(size_t)j * n + i] -= a0 + a1;
+          for (int cc = 0; cc < 8; cc += 2) {
+            a0 = fma(-pan[cc * n + m0 + r], pan[cc * n + m0 + c], a0);
+            a1 = fma(-pan[(cc + 1) * n + m0 + r], pan[(cc + 1) * n + m0 + c], a1);
+          }
+          bv[u] = a0 + a1;
         }
       }
-    }
-    __syncthreads();
-    // (1') next diagonal block on warp 0 || (3b) the other columns on the other warps, four columns per warp pass;
-    // rows i < m0 belong to X, rows i >= column to the Schur complement
-    if (warp == 0) factor_block(m0);
-    else {
-      for (int j = m0 + wn + 4 * (warp - 1); j < n; j += 4 * (nw - 1)) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) { const int e = lane + 32 * u; blkd[e & 7][e >> 3] = bv[u]; }
+      __syncwarp();
+      factor_block(m0);
+    } else if (warp & 3) {                                     // (warp 0 has the fp64 pipe of its quarter of the SM to itself)
+      for (int j = m0 + 4 * (warp - 1 - (warp >> 2)); j < n; j += 4 * (nw - nw / 4)) {
         double pj[4][8];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
           for (int cc = 0; cc < 8; ++cc) pj[q][cc] = (j + q < n) ? pan[cc * n + j + q] : 0.0;
-        const int nv = m0 + (n - j);
+        const int jr = j < m0 + 8 ? m0 + wn : j;               // first Schur row
+        const int nv = m0 + (n - jr);
         for (int v = lane; v < nv; v += 32) {
-          const int i = v < m0 ? v : j + (v - m0);
+          const int i = v < m0 ? v : jr + (v - m0);
           double acc[4] = {0, 0, 0, 0};
 #pragma unroll
           for (int cc = 0; cc < 8; ++cc) {
@@ -406,38 +417,33 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
   }
   if (!t.Lhi) return;
   // ---- L^-1: (L^-1)_ic = X[c][i] for c < i, diagonal invd.  Scaled so that the largest entry lies in [2^9, 2^10).
-  float mx = 0.f;
-  for (int i = warp; i < n; i += nw) {           // column i of W, rows cidx < i hold row i of L^-1
-    for (int cidx = lane; cidx < i; cidx += 32) mx = fmaxf(mx, fabsf((float)W[(size_t)i * n + cidx]));
-    if (lane == 0) mx = fmaxf(mx, (float)invd[i]);
-  }
-  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) s_red[warp] = mx;
+  mxh = __reduce_max_sync(0xffffffffu, mxh);
+  if (lane == 0) s_red[warp] = mxh;
   __syncthreads();
-  if (tid == 0) {
-    for (int i = 0; i < nw; ++i) mx = fmaxf(mx, s_red[i]);
-    int e = 0;
-    if (mx > 0.f && isfinite(mx)) e = 9 - ilogbf(mx);
-    s_exp = e;
-    *t.l_exp = e;
-  }
-  __syncthreads();
-  const double sc = ldexp(1.0, s_exp);
-  for (int i = warp; i < kp; i += nw) {          // row i (output column of Q), a pair of columns cidx (contraction index) per lane
-    for (int c2 = 2 * lane; c2 < kp; c2 += 64) {
-      float f[2];
+  mxh = __reduce_max_sync(0xffffffffu, lane < nw ? s_red[lane] : 0);
+  const int xe = (mxh >> 20) - 1023, le = mxh > 0 && xe < 1024 ? 9 - xe : 0;
+  if (tid == 0) *t.l_exp = le;
+  const double sc = ldexp(1.0, le);
+  for (int i = warp; i < kp; i += nw) {          // row i (output column of Q), a pair of columns (contraction index) per lane
+    float f[3][2];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int cidx = c2 + u;
+        const int cidx = 2 * lane + 64 * q + u;
         double v = 0.0;
         if (i < n && cidx < i) v = W[(size_t)i * n + cidx];
         else if (i < n && cidx == i) v = invd[i];
-        f[u] = (float)(v * sc);
+        f[q][u] = (float)(v * sc);
       }
-      const __half2 h = __floats2half2_rn(f[0], f[1]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int c2 = 2 * lane + 64 * q;
+      if (c2 >= kp) continue;
+      const __half2 h = __floats2half2_rn(f[q][0], f[q][1]);
       const float2 hf = __half22float2(h);
       *(__half2 *)(t.Lhi + (size_t)i * kp + c2) = h;
-      *(__half2 *)(t.Llo + (size_t)i * kp + c2) = __floats2half2_rn(f[0] - hf.x, f[1] - hf.y);
+      *(__half2 *)(t.Llo + (size_t)i * kp + c2) = __floats2half2_rn(f[q][0] - hf.x, f[q][1] - hf.y);
     }
   }
 }
