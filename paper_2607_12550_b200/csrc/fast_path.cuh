@@ -68,20 +68,16 @@ inline void bb_split(int total_heads, int n_tiles, int &tiles_per_item, int &ite
   items_per_head = (n_tiles + tiles_per_item - 1) / tiles_per_item;
 }
 
-template <bool RESIDUAL>
 inline void add_backbone_tc(Program &P, int stage, const std::vector<tc::BBCell> &cells, uint64_t seed) {
   if (cells.empty()) return;
-  static bool attr_done[2] = {false, false};
-  if (!attr_done[RESIDUAL]) {
-    cudaFuncSetAttribute(tc::backbone_kernel<RESIDUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::BB_SMEM_BYTES);
-    attr_done[RESIDUAL] = true;
-  }
+  static std::once_flag once;
+  std::call_once(once, [] { cudaFuncSetAttribute(tc::backbone_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::BB_SMEM_BYTES); });
   int gx = 0;
   for (auto &c : cells) gx = std::max(gx, c.m * c.items_per_head);
   const size_t off = P.push(cells);
   const int n = (int)cells.size();
   P.add(stage, [=](char *dev_t, cudaStream_t s) {
-    launch_heavy(tc::backbone_kernel<RESIDUAL>, dim3(gx, n), dim3(tc::BB_THREADS), (size_t)tc::BB_SMEM_BYTES, s, (const tc::BBCell *)(dev_t + off), seed);
+    launch_heavy(tc::backbone_kernel, dim3(gx, n), dim3(tc::BB_THREADS), (size_t)tc::BB_SMEM_BYTES, s, (const tc::BBCell *)(dev_t + off), seed);
     LAUNCHED();
   });
 }

@@ -1598,7 +1598,7 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
       rows += (long long)c.m * c.T;
       rj.push_back(j);
     }
-    add_backbone_tc<true>(PP, ST_RQ, bbc, o->seed);
+    add_backbone_tc(PP, ST_RQ, bbc, o->seed);
     add_backbone(PP, ST_BACK, br_port);
     if (!rj.empty()) {
       const size_t off = PP.push(rj);

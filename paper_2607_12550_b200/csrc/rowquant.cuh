@@ -30,39 +30,94 @@ __device__ __forceinline__ void apply_signs(float (&v)[128], const uint32_t (&sw
     v[f] = __uint_as_float(__float_as_uint(v[f]) ^ (((sw[f >> 5] >> (f & 31)) & 1u) << 31));
 }
 
-// Rotate, quantise and pack one residual row.  words: 4*BITS uint32, scales: 4 halves.
+// ---- pairs of floats in one register pair: one instruction for two additions, products or FMAs, each rounded as the single one
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) { f32x2 d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b)); return d; }
+__device__ __forceinline__ void f2_unpack(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) { f32x2 d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) { f32x2 d; asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) { f32x2 d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) { f32x2 d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
+__device__ __forceinline__ f32x2 f2_add_rz(f32x2 a, f32x2 b) { f32x2 d; asm("add.rz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+
+// Rotate, quantise and pack one residual row whose signs are applied: v[k] = entries 2k, 2k + 1.  words: 4*BITS uint32,
+// scales: 4 halves.  The pass is bound by its straight-line code (fetch and issue; a thread holds a row, so every entry is
+// code of its own): pairs halve the transform, the scaling and the rounding; the clamp of two codes is one 16-bit-pair
+// instruction; codes i and i + 16 / BITS share a pair, so a word is a chain of shift-adds.  1370 instead of 2650
+// instructions a row.
+template <int BITS>
+__device__ __forceinline__ void quantize_pack_pairs(f32x2 (&v)[64], uint32_t *__restrict__ words, __half *__restrict__ scales, int *bad_scale) {
+#pragma unroll
+  for (int k = 0; k < 64; ++k) { float a, b; f2_unpack(v[k], a, b); v[k] = f2_pack(a + b, a - b); }
+#pragma unroll
+  for (int len = 1; len < 64; len <<= 1)
+#pragma unroll
+    for (int k = 0; k < 64; ++k)
+      if ((k & len) == 0) { const f32x2 a = v[k], b = v[k | len]; v[k] = f2_add(a, b); v[k | len] = f2_sub(a, b); }
+  constexpr float L = (float)(1 << (BITS - 1));
+  constexpr int levels = (1 << BITS) - 1;
+  const f32x2 isd = f2_pack(kInvSqrtD, kInvSqrtD), magic = f2_pack(8388608.0f + L, 8388608.0f + L);
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    f32x2 *q = v + 16 * g;
+    float a = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) { float x, y; q[k] = f2_mul(q[k], isd); f2_unpack(q[k], x, y); a = fmaxf(a, fmaxf(fabsf(x), fabsf(y))); }
+    const __half dh = __float2half_rn(a * (1.0f / L));
+    const float delta = __half2float(dh);
+    if (isinf(delta) || isnan(delta)) *bad_scale = 1;
+    const float inv = (delta == 0.f) ? 0.f : 1.0f / delta;
+    scales[g] = dh;
+    const f32x2 inv2 = f2_pack(inv, inv);
+    // clamp(floor(x), -L, L-1) + L without a rounding or conversion instruction: a round-toward-zero addition of 2^23 + L leaves
+    // floor(x + L) in the low mantissa bits of a positive float (-1 or -2 in its low 16 bits when x < -L: |x| exceeds L
+    // by the rounding of the step at most), clamped to [0, 2L - 1] as 16-bit integers
+    uint32_t code[32];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const f32x2 t = f2_add_rz(f2_mul(q[k], inv2), magic);
+      code[2 * k] = (uint32_t)t; code[2 * k + 1] = (uint32_t)(t >> 32);
+    }
+    const uint32_t zero_word = delta == 0.f ? 1u : 0u;                                  // no step: every code is L
+    if constexpr (BITS == 3) {
+      uint64_t accw = 0;
+      int nb = 0, wi = 0;
+#pragma unroll
+      for (int j = 0; j < 32; j += 2) {
+        const uint32_t c2 = __vimin_s16x2_relu(__byte_perm(code[j], code[j + 1], 0x5410), (uint32_t)(levels | levels << 16));
+        const uint32_t c6 = zero_word ? 4u | 4u << 3 : (c2 & 7u) | (c2 >> 13);
+        accw |= (uint64_t)c6 << nb;
+        nb += 6;
+        if (nb >= 32) { words[g * 3 + wi] = (uint32_t)accw; accw >>= 32; nb -= 32; ++wi; }
+      }
+    } else {
+      constexpr int H = 16 / BITS;                                                      // codes of half a word
+      uint32_t lw = 0;
+#pragma unroll
+      for (int i = 0; i < 32 / BITS; ++i) lw |= (1u << (BITS - 1)) << (i * BITS);
+#pragma unroll
+      for (int w = 0; w < BITS; ++w) {
+        uint32_t acc = 0;
+#pragma unroll
+        for (int i = H - 1; i >= 0; --i) {
+          const int j = w * 2 * H + i;
+          acc = (acc << BITS) + __vimin_s16x2_relu(__byte_perm(code[j], code[j + H], 0x5410), (uint32_t)(levels | levels << 16));
+        }
+        words[g * BITS + w] = zero_word ? lw : acc;
+      }
+    }
+  }
+}
+
 template <int BITS>
 __device__ __forceinline__ void quantize_pack_row(float (&r)[128], const uint32_t (&sw)[4],
                                                   uint32_t *__restrict__ words, __half *__restrict__ scales,
                                                   int *bad_scale) {
   apply_signs(r, sw);
-  wht128(r);
-  constexpr float half_levels = (float)(1 << (BITS - 1));
+  f32x2 v[64];
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    float a = 0.f;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) { r[g * 32 + j] *= kInvSqrtD; a = fmaxf(a, fabsf(r[g * 32 + j])); }
-    const __half dh = __float2half_rn(a * (1.0f / half_levels));
-    const float delta = __half2float(dh);
-    if (isinf(delta) || isnan(delta)) *bad_scale = 1;
-    const float inv = (delta == 0.f) ? 0.f : 1.0f / delta;
-    scales[g] = dh;
-    uint64_t accw = 0;
-    int nb = 0, wi = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      // clamp(floor(v), -L, L-1) + L without a rounding or conversion instruction (both run on the quarter-rate
-      // pipe and bound this pass): clamp v to [-L, L - 1/2] first (same result: floor is monotone), then one
-      // round-toward-zero add of 2^23 + L leaves floor(v + L) in the low mantissa bits of a positive float
-      const float v = fminf(fmaxf(__fmul_rn(r[g * 32 + j], inv), -half_levels), half_levels - 0.5f);
-      const uint32_t code = __float_as_uint(__fadd_rz(v, 8388608.0f + half_levels)) & 0x1FFu;
-      const uint32_t u = (delta == 0.f) ? (uint32_t)half_levels : code;
-      accw |= (uint64_t)u << nb;
-      nb += BITS;
-      if (nb >= 32) { words[g * BITS + wi] = (uint32_t)accw; accw >>= 32; nb -= 32; ++wi; }
-    }
-  }
+  for (int k = 0; k < 64; ++k) v[k] = f2_pack(r[2 * k], r[2 * k + 1]);
+  quantize_pack_pairs<BITS>(v, words, scales, bad_scale);
 }
 
 // Unpack, dequantise and rotate back one row: r = s . H(delta * (u - 2^(b-1) + 1/2)) / sqrt(d).

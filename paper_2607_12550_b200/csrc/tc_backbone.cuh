@@ -1,14 +1,14 @@
-// Fused backbone pass on tcgen05 tensor cores, in two modes that share everything but the epilogue:
-//
-//   DECODE  : X^  = 2^e U_T P_h + s . H(dequant(codes)) / sqrt(d)       -> fp16 / fp32 rows
-//   RESIDUAL: r   = x - 2^e U_T P_h ; rotate ; quantise ; pack            -> codes + scales
+// Fused residual pass on tcgen05 tensor cores:   r = x - 2^e U_T P_h ; rotate ; quantise ; pack   -> codes + scales
 //
 // One CTA owns a (cell, head, run of 128-token tiles).  The projected core P_h = fp16(G_h U_F^T) was formed once
 // when the cell was compressed and is kept with the handle: the CTA fetches its head's [r_t][128] block by TMA as
 // two 64-feature panels (an MN-major B operand) and streams U_T tiles through a TMA ring into  D = U_T[tile] P_h
 // with two TMEM accumulators, so the epilogue of one tile overlaps the MMA of the next.  Residual and decode read
-// the SAME stored P, so the backbone the residual is taken against is bit for bit the one the decoder adds back.  Two epilogue warpgroups alternate tiles; each thread owns one
-// 128-feature row in registers (TMEM lane = token).
+// the SAME stored P, so the backbone the residual is taken against is bit for bit the one the decoder adds back.  Two
+// epilogue warpgroups alternate tiles; each thread owns one 128-feature row in registers (TMEM lane = token), as 64 pairs.
+// The epilogue's code is the bound (quantize_pack_pairs): the signs of the rotation go onto the fp16 words of x and onto
+// the factor of the backbone, both read from shared memory, so applying them costs an instruction per pair.
+// 13 million rows (40 layers, 40 heads, 4096 tokens): 2.13 -> 1.44 ms; 2.1 million: 394 -> 262 us.
 #pragma once
 #include "rowquant.cuh"
 #include "tc_common.cuh"
@@ -21,13 +21,14 @@ constexpr int BB_P_BYTES = 65536;            // P: two panels of [r_t rows][128 
 constexpr int BB_BIG_BYTES = 131072;         // ring (+ X tiles)
 constexpr int BB_STAGE_BYTES = 16384;        // one [128 tokens][64 fp16] box of U_T
 constexpr int BB_XTILE_BYTES = 32768;        // two [128 tokens][64 fp16] boxes of X
-constexpr int BB_SMEM_BYTES = BB_P_BYTES + BB_BIG_BYTES + 1024 /*align*/ + 512 /*barriers*/;
+constexpr int BB_SIGN_BYTES = 768;           // sign masks of x (64 words), signed factors of the backbone (128 floats)
+constexpr int BB_SMEM_BYTES = BB_P_BYTES + BB_BIG_BYTES + 1024 /*align*/ + 512 /*barriers*/ + BB_SIGN_BYTES;
 constexpr int BB_TMEM_COLS = 256;
 
 struct alignas(64) BBCell {
   CUtensorMap tmUT;     // fp16 [T][r_t]           dims {r_t, T},       box {64, 128}
   CUtensorMap tmP;      // fp16 [m*r_t][128]       dims {128, m*r_t},   box {64, r_t}
-  CUtensorMap tmX;      // fp16 [L][n_h][T][128]   dims {128, T, n_h, L}, box {64, 128, 1, 1}   (RESIDUAL)
+  CUtensorMap tmX;      // fp16 [L][n_h][T][128]   dims {128, T, n_h, L}, box {64, 128, 1, 1}   (residual)
   int tma_out;          // DECODE: filled in from the launch's destination (DecOut)
   long long *dbg;       // optional: cycle stamps of CTA 0 (profiling aid), 8 per tile per warpgroup
   uint32_t *words;      // [m][T][4*bits]
@@ -45,31 +46,11 @@ struct alignas(64) BBCell {
 };
 
 template <int BITS>
-__device__ __forceinline__ void bb_decode_row(const BBCell &c, uint64_t seed, long long row, float (&r)[128]) {
-  if constexpr (BITS > 0) {
-    uint32_t words[4 * BITS];
-    const uint4 *wp = (const uint4 *)(c.words + row * (4 * BITS));
-#pragma unroll
-    for (int i = 0; i < BITS; ++i) { const uint4 v = __ldg(wp + i); words[4 * i] = v.x; words[4 * i + 1] = v.y; words[4 * i + 2] = v.z; words[4 * i + 3] = v.w; }
-    __half sc[4];
-    *(uint2 *)sc = __ldg((const uint2 *)(c.scales + row * 4));
-    uint32_t sw[4];
-    cell_sign_words(seed, c.cell, sw);
-    unpack_dequant_row<BITS>(words, sc, sw, r);
-  } else {
-#pragma unroll
-    for (int f = 0; f < 128; ++f) r[f] = 0.f;
-  }
-}
-
-template <int BITS>
-__device__ __forceinline__ void bb_quant_row(const BBCell &c, uint64_t seed, long long row, float (&r)[128]) {
-  uint32_t sw[4];
-  cell_sign_words(seed, c.cell, sw);
+__device__ __forceinline__ void bb_quant_row(const BBCell &c, long long row, f32x2 (&v)[64]) {
   uint32_t words[4 * BITS];
   __half sc[4];
   int bad = 0;
-  quantize_pack_row<BITS>(r, sw, words, sc, &bad);
+  quantize_pack_pairs<BITS>(v, words, sc, &bad);
   if (bad) *c.status = 4;
   uint4 *wo = (uint4 *)(c.words + row * (4 * BITS));
 #pragma unroll
@@ -77,7 +58,6 @@ __device__ __forceinline__ void bb_quant_row(const BBCell &c, uint64_t seed, lon
   *(uint2 *)(c.scales + row * 4) = *(const uint2 *)sc;
 }
 
-template <bool RESIDUAL>
 __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *__restrict__ cells, uint64_t seed) {
   extern __shared__ unsigned char smem_raw[];
   const BBCell &c = cells[blockIdx.y];
@@ -99,9 +79,9 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
   volatile int *abort_flag = (volatile int *)(sm + BB_P_BYTES + BB_BIG_BYTES + 256);
   uint32_t *tmem_slot = (uint32_t *)(sm + BB_P_BYTES + BB_BIG_BYTES + 264);
 
-  constexpr int NS = RESIDUAL ? 4 : 8;                 // ring stages
+  constexpr int NS = 4;                                // ring stages
   const uint32_t sRing = sBig;
-  const uint32_t sX = sBig + 4 * BB_STAGE_BYTES;       // RESIDUAL: two X tiles behind a 4-stage ring
+  const uint32_t sX = sBig + 4 * BB_STAGE_BYTES;       // two X tiles behind the ring
   // barrier slots (8 bytes each)
   const uint32_t bSetup = sBar + 0;
   auto bFull = [=](int s) { return sBar + 24 + 8 * s; };
@@ -124,6 +104,17 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
     fence_barrier_init();
   }
   if (warp == 8) { tmem_alloc(smem_u32(tmem_slot), BB_TMEM_COLS); tmem_relinquish(); }
+  uint32_t *xmask = (uint32_t *)(sm + BB_P_BYTES + BB_BIG_BYTES + 512);
+  float *bfac = (float *)(xmask + 64);
+  if (threadIdx.x < 128) {
+    const int f = threadIdx.x;
+    uint32_t sw[4];
+    cell_sign_words(seed, c.cell, sw);
+    const uint32_t wv = f < 64 ? (f < 32 ? sw[0] : sw[1]) : (f < 96 ? sw[2] : sw[3]);
+    const uint32_t neg = (wv >> (f & 31)) & 1u, next = __shfl_down_sync(0xffffffffu, neg, 1);
+    bfac[f] = neg ? ldexpf(1.0f, *c.e) : -ldexpf(1.0f, *c.e);
+    if (!(f & 1)) xmask[f >> 1] = neg << 15 | next << 31;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -134,7 +125,7 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
     if (warp == 8 && lane == 0) {
       // ---------------- TMA producer
       tma_prefetch_desc(&c.tmUT); tma_prefetch_desc(&c.tmP);
-      if (RESIDUAL) tma_prefetch_desc(&c.tmX);
+      tma_prefetch_desc(&c.tmX);
       mbar_expect_tx(bSetup, 2u * panel);
       tma_load_2d(sP, &c.tmP, bSetup, 0, h * c.r_t);
       tma_load_2d(sP + panel, &c.tmP, bSetup, 64, h * c.r_t);
@@ -143,13 +134,11 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
       const int l = h / c.n_heads, hd = h - l * c.n_heads;
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int tt = tile0 + i, b = i & 1, nb = i >> 1;
-        if (RESIDUAL) {
-          ok = mbar_wait(bXempty(b), (nb & 1) ^ 1, abort_flag);
-          if (!ok) break;
-          mbar_expect_tx(bXfull(b), BB_XTILE_BYTES);
-          tma_load_4d(sX + b * BB_XTILE_BYTES, &c.tmX, bXfull(b), 0, tt * 128, hd, l);
-          tma_load_4d(sX + b * BB_XTILE_BYTES + 16384, &c.tmX, bXfull(b), 64, tt * 128, hd, l);
-        }
+        ok = mbar_wait(bXempty(b), (nb & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        mbar_expect_tx(bXfull(b), BB_XTILE_BYTES);
+        tma_load_4d(sX + b * BB_XTILE_BYTES, &c.tmX, bXfull(b), 0, tt * 128, hd, l);
+        tma_load_4d(sX + b * BB_XTILE_BYTES + 16384, &c.tmX, bXfull(b), 64, tt * 128, hd, l);
         for (int kb = 0; kb < nkt; ++kb, ++cnt) {
           const int s = cnt % NS, n = cnt / NS;
           ok = mbar_wait(bEmpty(s), (n & 1) ^ 1, abort_flag);
@@ -195,35 +184,22 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
     const int row_in_tile = q * 32 + lane;
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
     bool ok = true;
-    const float scale = ldexpf(1.0f, *c.e);
-    const int l = h / c.n_heads, hd = h - l * c.n_heads;
     for (int i = wg; ok && i < n_tiles; i += 2) {
       const int tt = tile0 + i, nb = i >> 1;
-      const int token = tt * 128 + row_in_tile;
-      const long long row = (long long)h * c.T + token;
-      float r[128];
-      if constexpr (RESIDUAL) {
-        ok = __all_sync(0xffffffffu, mbar_wait(bXfull(wg), nb & 1, abort_flag));
-        if (!ok) break;
-        const unsigned char *xb = sm + BB_P_BYTES + 4 * BB_STAGE_BYTES + wg * BB_XTILE_BYTES;
+      const long long row = (long long)h * c.T + tt * 128 + row_in_tile;
+      f32x2 r[64];
+      ok = __all_sync(0xffffffffu, mbar_wait(bXfull(wg), nb & 1, abort_flag));
+      if (!ok) break;
+      const unsigned char *xb = sm + BB_P_BYTES + 4 * BB_STAGE_BYTES + wg * BB_XTILE_BYTES;
 #pragma unroll
-        for (int ck = 0; ck < 16; ++ck) {
-          const uint4 v = *(const uint4 *)(xb + (ck >> 3) * 16384 + row_in_tile * 128 + (((ck & 7) ^ (row_in_tile & 7)) << 4));
-          const __half2 *hp = (const __half2 *)&v;
+      for (int ck = 0; ck < 16; ++ck) {
+        const uint4 v = *(const uint4 *)(xb + (ck >> 3) * 16384 + row_in_tile * 128 + (((ck & 7) ^ (row_in_tile & 7)) << 4));
+        const uint4 mk = *(const uint4 *)(xmask + 4 * ck);
+        const uint32_t w[4] = {v.x ^ mk.x, v.y ^ mk.y, v.z ^ mk.z, v.w ^ mk.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); r[ck * 8 + 2 * j] = f.x; r[ck * 8 + 2 * j + 1] = f.y; }
-        }
-        mbar_arrive(bXempty(wg));
-      } else {
-        switch (c.bits) {
-          case 0: bb_decode_row<0>(c, seed, row, r); break;
-          case 1: bb_decode_row<1>(c, seed, row, r); break;
-          case 2: bb_decode_row<2>(c, seed, row, r); break;
-          case 3: bb_decode_row<3>(c, seed, row, r); break;
-          case 4: bb_decode_row<4>(c, seed, row, r); break;
-          default: bb_decode_row<8>(c, seed, row, r); break;
-        }
+        for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(*(const __half2 *)&w[j]); r[ck * 4 + j] = f2_pack(f.x, f.y); }
       }
+      mbar_arrive(bXempty(wg));
       ok = __all_sync(0xffffffffu, mbar_wait(bTfull(wg), nb & 1, abort_flag));
       if (!ok) break;
       tc_fence_after();
@@ -233,39 +209,22 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
         tmem_ld32(t_lane + wg * 128 + ch * 32, v);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if constexpr (RESIDUAL) r[ch * 32 + j] -= scale * v[j];
-          else r[ch * 32 + j] += scale * v[j];
+        for (int j = 0; j < 32; j += 4) {
+          const float4 f = *(const float4 *)(bfac + ch * 32 + j);
+          const int k = ch * 16 + j / 2;
+          r[k] = f2_fma(f2_pack(f.x, f.y), f2_pack(v[j], v[j + 1]), r[k]);
+          r[k + 1] = f2_fma(f2_pack(f.z, f.w), f2_pack(v[j + 2], v[j + 3]), r[k + 1]);
         }
       }
       tc_fence_before();
       mbar_arrive(bTempty(wg));
-      if constexpr (RESIDUAL) {
-        switch (c.bits) {
-          case 1: bb_quant_row<1>(c, seed, row, r); break;
-          case 2: bb_quant_row<2>(c, seed, row, r); break;
-          case 3: bb_quant_row<3>(c, seed, row, r); break;
-          case 4: bb_quant_row<4>(c, seed, row, r); break;
-          case 8: bb_quant_row<8>(c, seed, row, r); break;
-          default: break;
-        }
-      } else {
-        const long long off = (long long)l * c.osl + (long long)hd * c.osh + (long long)token * c.ost;
-        if (c.out_dtype == DT_F16) {
-          uint4 *p = (uint4 *)((__half *)c.out + off);
-#pragma unroll
-          for (int k8 = 0; k8 < 16; ++k8) {
-            uint4 v;
-            __half2 *hp = (__half2 *)&v;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) hp[j] = __floats2half2_rn(r[k8 * 8 + 2 * j], r[k8 * 8 + 2 * j + 1]);
-            p[k8] = v;
-          }
-        } else {
-          float4 *p = (float4 *)((float *)c.out + off);
-#pragma unroll
-          for (int k4 = 0; k4 < 32; ++k4) p[k4] = make_float4(r[4 * k4], r[4 * k4 + 1], r[4 * k4 + 2], r[4 * k4 + 3]);
-        }
+      switch (c.bits) {
+        case 1: bb_quant_row<1>(c, row, r); break;
+        case 2: bb_quant_row<2>(c, row, r); break;
+        case 3: bb_quant_row<3>(c, row, r); break;
+        case 4: bb_quant_row<4>(c, row, r); break;
+        case 8: bb_quant_row<8>(c, row, r); break;
+        default: break;
       }
     }
   }
