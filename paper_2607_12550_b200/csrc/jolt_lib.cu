@@ -1269,60 +1269,76 @@ static size_t carve_handle_blob(jolt_handle &H) {
   return b.off + 256;
 }
 
-// Runs the programs of the cell groups concurrently, one side stream per group, forked from and joined back into the
-// caller's stream; the groups' steps are enqueued round-robin, so every side stream has work from the start.
-static int run_group_programs(int dev, cudaStream_t st, std::vector<Program> &PG, int n_groups, void *d_tab,
-                              const std::vector<size_t> &tab_off) {
-  {
-    GroupStreams *gs = group_streams(dev);
-    if (!gs) return fail(JOLT_ECUDA, "cannot create side streams");
-    cudaError_t ce = cudaEventRecord(gs->fork, st);
-    for (int g = 0; g < n_groups && ce == cudaSuccess; ++g) {
-      ce = cudaStreamWaitEvent(gs->s[g], gs->fork, 0);
-      if (ce == cudaSuccess && !PG[g].host.empty())
-        ce = cudaMemcpyAsync((char *)d_tab + tab_off[g], PG[g].host.data(), PG[g].host.size(), cudaMemcpyHostToDevice, gs->s[g]);
+// The programs of the cell groups, run concurrently: one side stream per group, forked from and joined back into the caller's
+// stream.  A program's first steps are enqueued as soon as it is built, so that the device works while the host builds the
+// others (16 cells: the first kernel came 170 us into the call when all were built first); the rest goes round-robin.  A
+// program's tables are one copy of its own on its stream.
+constexpr int kEarlySteps = 5;
+struct GroupRun {
+  int dev;
+  cudaStream_t st;
+  GroupStreams *gs = nullptr;
+  char *tab = nullptr;
+  size_t cap = 0, at = 0;                    // of the table memory: reserved, used
+  std::vector<Program> &PG;
+  std::vector<size_t> off;                   // where each program's tables are
+  std::vector<size_t> done;                  // steps enqueued
+  cudaError_t ce = cudaSuccess;
+  GroupRun(int d, cudaStream_t s, std::vector<Program> &p) : dev(d), st(s), PG(p) {}
+  int start(size_t table_bytes) {
+    cap = table_bytes;
+    void *p = nullptr;
+    if (int rc = tab_reserve(dev, cap, &p)) return rc;
+    tab = (char *)p;
+    gs = group_streams(dev);
+    return gs ? JOLT_OK : fail(JOLT_ECUDA, "cannot create side streams");
+  }
+  void fork() { ce = cudaEventRecord(gs->fork, st); }
+  // `bytes` of table memory; where the estimate was too low the tables move to a larger allocation
+  size_t take(size_t bytes) {
+    const size_t o = (at + 255) & ~(size_t)255;
+    if (o + bytes > cap && ce == cudaSuccess) {
+      ce = cudaDeviceSynchronize();
+      void *p = nullptr;
+      cap = 2 * (o + bytes);
+      if (tab_reserve(dev, cap, &p)) ce = cudaErrorMemoryAllocation;
+      tab = (char *)p;
+      for (size_t g = 0; g < off.size() && ce == cudaSuccess; ++g)
+        if (!PG[g].host.empty()) ce = cudaMemcpyAsync(tab + off[g], PG[g].host.data(), PG[g].host.size(), cudaMemcpyHostToDevice, gs->s[g]);
     }
-    // enqueue the groups' steps round-robin, so every side stream has work from the start
-    size_t max_steps = 0;
-    for (int g = 0; g < n_groups; ++g) max_steps = std::max(max_steps, PG[g].steps.size());
-#ifdef JOLT_DEBUG
-    const bool tl = getenv("JOLT_DEBUG_TIMELINE") != nullptr;      // per-group stage boundaries, printed after the call
-    struct TL { int g, stage; cudaEvent_t ev; };
-    std::vector<TL> tls;
-    cudaEvent_t tl0 = nullptr;
-    if (tl) { cudaEventCreate(&tl0); cudaEventRecord(tl0, st); }
-#endif
-    for (size_t si = 0; si < max_steps && ce == cudaSuccess; ++si)
-      for (int g = 0; g < n_groups; ++g)
-        if (si < PG[g].steps.size()) {
-          PG[g].steps[si].run((char *)d_tab + tab_off[g], gs->s[g]);
-#ifdef JOLT_DEBUG
-          if (tl && (si + 1 == PG[g].steps.size() || PG[g].steps[si + 1].stage != PG[g].steps[si].stage)) {
-            TL t{g, PG[g].steps[si].stage, nullptr}; cudaEventCreate(&t.ev); cudaEventRecord(t.ev, gs->s[g]); tls.push_back(t);
-          }
-#endif
-        }
-#ifdef JOLT_DEBUG
-    if (tl) {
-      cudaDeviceSynchronize();
-      for (int g = 0; g < n_groups; ++g) {
-        fprintf(stderr, "[jolt] group %d:", g);
-        for (auto &t : tls) if (t.g == g) { float ms = 0; cudaEventElapsedTime(&ms, tl0, t.ev); fprintf(stderr, " %s@%.2f", kStageNames[t.stage], ms); }
-        fprintf(stderr, "\n");
-      }
-      for (auto &t : tls) cudaEventDestroy(t.ev);
-      cudaEventDestroy(tl0);
+    at = o + bytes;
+    return o;
+  }
+  void add(int g) {                          // program g (they come in order) is built
+    const size_t o = take(PG[g].host.size());
+    if (ce == cudaSuccess) ce = cudaStreamWaitEvent(gs->s[g], gs->fork, 0);
+    if (ce == cudaSuccess && !PG[g].host.empty())
+      ce = cudaMemcpyAsync(tab + o, PG[g].host.data(), PG[g].host.size(), cudaMemcpyHostToDevice, gs->s[g]);
+    off.push_back(o);
+    done.push_back(0);
+    for (; ce == cudaSuccess && done[g] < std::min<size_t>(kEarlySteps, PG[g].steps.size()); ++done[g]) PG[g].steps[done[g]].run(tab + o, gs->s[g]);
+  }
+  int finish() {
+    for (bool any = true; any && ce == cudaSuccess;) {
+      any = false;
+      for (size_t g = 0; g < off.size(); ++g)
+        if (done[g] < PG[g].steps.size()) { PG[g].steps[done[g]++].run(tab + off[g], gs->s[g]); any = true; }
     }
-#endif
     if (ce == cudaSuccess) ce = cudaGetLastError();
-    for (int g = 0; g < n_groups && ce == cudaSuccess; ++g) {
+    for (size_t g = 0; g < off.size() && ce == cudaSuccess; ++g) {
       ce = cudaEventRecord(gs->join[g], gs->s[g]);
       if (ce == cudaSuccess) ce = cudaStreamWaitEvent(st, gs->join[g], 0);
     }
     if (ce != cudaSuccess) { cudaDeviceSynchronize(); return fail(JOLT_ECUDA, "side streams: %s", cudaGetErrorString(ce)); }
+    return JOLT_OK;
   }
-  return JOLT_OK;
-}
+  // what the argument tables of a call may take: a bound that holds for every list of tasks built here
+  static size_t estimate(const std::vector<CellDesc> &cells) {
+    size_t b = 1 << 16;
+    for (auto &c : cells) b += 16384 + (size_t)c.m * 3072;
+    return b;
+  }
+};
 
 // Device memory of freed handles, kept for the next ones.  The stream-ordered pool alone does not serve a program that
 // compresses caches one after another: blocks of neighbouring sizes whose release is still in flight do not fit, and it
@@ -1537,17 +1553,16 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
   }
 
   lap("workspace");
-  // ---- program
+  // ---- programs
   Program P;
   std::vector<int> cell_group;
   const int n_groups = assign_groups(ws, cell_group);
   std::vector<Program> PG(std::max(n_groups, 1));
-  for (int g = 0; g < n_groups; ++g) {
+  auto build_group = [&](int g) {
     std::vector<CellWork> sub = ws;
     for (int i = 0; i < nc; ++i) if (cell_group[i] != g) sub[i].active = false;
     build_factor_program(PG[g], sub, mode, false, power_iters, o->seed, fast, subspace);
-  }
-  lap("factor program");
+  };
   // fp16 storage of the factors and the residual / rotate / quantise / pack pass (tensor-core kernel where the cell
   // fits it, portable kernels otherwise).  With several cell groups each group's program ends with the tail of its
   // own cells, so only the last group's tail is left when the others have finished.
@@ -1632,28 +1647,21 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
       });
     }
   };
+  GroupRun run(dev, st, PG);
+  void *d_tab = nullptr;
   if (n_groups > 1) {
-    std::vector<int> rest;
-    for (int g = 0; g < n_groups; ++g) {
-      std::vector<int> idx;
-      for (int i = 0; i < nc; ++i) if (cell_group[i] == g) idx.push_back(i);
-      build_tail(PG[g], idx);
-    }
-    for (int i = 0; i < nc; ++i) if (cell_group[i] < 0) rest.push_back(i);
-    build_tail(P, rest);
+    if ((rc = run.start(GroupRun::estimate(cells)))) { free_blob(); return rc; }
   } else {
+    if (n_groups == 1) build_group(0);
     std::vector<int> all(nc);
     for (int i = 0; i < nc; ++i) all[i] = i;
     build_tail(P, all);
+    if ((rc = tab_reserve(dev, PG[0].host.size() + P.host.size() + 512, &d_tab))) { free_blob(); return rc; }
   }
-  void *d_tab = nullptr;
-  std::vector<size_t> tab_off(PG.size() + 1, 0);
-  for (size_t g = 0; g < PG.size(); ++g) tab_off[g + 1] = tab_off[g] + ((PG[g].host.size() + 255) & ~(size_t)255);
-  if ((rc = tab_reserve(dev, tab_off.back() + P.host.size() + 256, &d_tab))) { free_blob(); return rc; }
-  lap("residual program");
+  lap("programs");
 
   // ---- run
-  if ((rc = arena_acquire(dev, st)) || (rc = upload_decode_table(*H, st))) { free_blob(); return rc; }
+  if ((rc = arena_acquire(dev, st))) { free_blob(); return rc; }
   g_timer.begin(st);
   std::vector<ClearRange> cl = {{(uint32_t *)d_status, 4 * nc}, {(uint32_t *)H->d_status, 4 * nc}};
   for (int i = 0; i < nc; ++i) {
@@ -1679,11 +1687,25 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
   if (ce != cudaSuccess) { free_blob(); return fail(JOLT_ECUDA, "staging copy: %s", cudaGetErrorString(ce)); }
   if (n_groups <= 1) {
     if (n_groups == 1 && (rc = run_program(PG[0], (char *)d_tab, st))) { free_blob(); return rc; }
+    if ((rc = run_program(P, (char *)d_tab + ((PG[0].host.size() + 255) & ~(size_t)255), st))) { free_blob(); return rc; }
   } else {
-    if ((rc = run_group_programs(dev, st, PG, n_groups, d_tab, tab_off))) { free_blob(); return rc; }
+    run.fork();
+    for (int g = 0; g < n_groups; ++g) {
+      std::vector<int> idx;
+      for (int i = 0; i < nc; ++i) if (cell_group[i] == g) idx.push_back(i);
+      build_group(g);
+      build_tail(PG[g], idx);
+      run.add(g);
+    }
+    std::vector<int> rest;
+    for (int i = 0; i < nc; ++i) if (cell_group[i] < 0) rest.push_back(i);
+    build_tail(P, rest);
+    const size_t o_rest = run.take(P.host.size());
+    if ((rc = run.finish())) { free_blob(); return rc; }
     g_timer.mark(ST_FACT, st);
+    if ((rc = run_program(P, run.tab + o_rest, st))) { free_blob(); return rc; }
   }
-  if ((rc = run_program(P, (char *)d_tab + tab_off.back(), st))) { free_blob(); return rc; }
+  if ((rc = upload_decode_table(*H, st))) { free_blob(); return rc; }
   arena_release(dev, st);
   lap("launches");
   std::vector<int> hstat(4 * nc);
@@ -2457,16 +2479,13 @@ extern "C" int jolt_probe(const jolt_layout *L, const void *K, const void *V, do
   // program of their own on one more stream instead of lengthening every group's chain
   const bool split = mode == FM_RANDOMIZED && n_groups > 1 && n_groups < kMaxGroups;
   std::vector<Program> PG(std::max(n_groups, 1) + (split ? 1 : 0));
-  for (int g = 0; g < n_groups; ++g) {
+  auto build_group = [&](int g) {
     std::vector<CellWork> sub = ws;
+    if (split && g + 1 == n_groups) { build_factor_program(PG[g], sub, mode, true, power_iters, o->seed, fast, false, 1); return; }
     for (int i = 0; i < nc; ++i) if (cell_group[i] != g) sub[i].active = false;
     build_factor_program(PG[g], sub, mode, true, power_iters, o->seed, fast, false, split ? 2 : 3);
-  }
-  if (split) {
-    std::vector<CellWork> sub = ws;
-    build_factor_program(PG[n_groups], sub, mode, true, power_iters, o->seed, fast, false, 1);
-    ++n_groups;
-  }
+  };
+  if (split) ++n_groups;
   Program P;
   {
     std::vector<PackJob> pj;
@@ -2479,10 +2498,14 @@ extern "C" int jolt_probe(const jolt_layout *L, const void *K, const void *V, do
     const int n = (int)pj.size();
     P.add(ST_SVD, [=](char *dev_t, cudaStream_t s) { pack_spectra_kernel<<<n, 128, 0, s>>>((const PackJob *)(dev_t + poff)); LAUNCHED(); });
   }
+  GroupRun run(dev, st, PG);
   void *d_tab = nullptr;
-  std::vector<size_t> tab_off(PG.size() + 1, 0);
-  for (size_t g = 0; g < PG.size(); ++g) tab_off[g + 1] = tab_off[g] + ((PG[g].host.size() + 255) & ~(size_t)255);
-  if ((rc = tab_reserve(dev, tab_off.back() + P.host.size() + 256, &d_tab))) return rc;
+  if (n_groups > 1) {
+    if ((rc = run.start(GroupRun::estimate(cells)))) return rc;
+  } else {
+    if (n_groups == 1) build_group(0);
+    if ((rc = tab_reserve(dev, PG[0].host.size() + P.host.size() + 512, &d_tab))) return rc;
+  }
   if ((rc = arena_acquire(dev, st))) return rc;
   g_timer.begin(st);
   CU(cudaMemsetAsync(d_status, 0, sizeof(int) * 4 * nc, st));
@@ -2492,8 +2515,14 @@ extern "C" int jolt_probe(const jolt_layout *L, const void *K, const void *V, do
   }
   if (n_groups <= 1) {
     if (n_groups == 1 && (rc = run_program(PG[0], (char *)d_tab, st))) return rc;
-  } else if ((rc = run_group_programs(dev, st, PG, n_groups, d_tab, tab_off))) return rc;
-  if ((rc = run_program(P, (char *)d_tab + tab_off.back(), st))) return rc;
+    if ((rc = run_program(P, (char *)d_tab + ((PG[0].host.size() + 255) & ~(size_t)255), st))) return rc;
+  } else {
+    run.fork();
+    for (int g = 0; g < n_groups; ++g) { build_group(g); run.add(g); }
+    const size_t o_pack = run.take(P.host.size());
+    if ((rc = run.finish())) return rc;
+    if ((rc = run_program(P, run.tab + o_pack, st))) return rc;
+  }
   arena_release(dev, st);
   std::vector<int> hstat(4 * nc);
   std::vector<float> pack(pack_floats);
