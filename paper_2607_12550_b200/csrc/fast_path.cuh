@@ -92,7 +92,8 @@ inline void fill_bb_common(tc::BBCell &b, const CellStore &cs, int *status) {
 }
 
 
-// Per-item decode kernel: cells of r_t > 128, keys rotated at decode, and every cell when the persistent kernel is off.
+// Per-item decode kernel: cells of r_t > 128, keys rotated into a destination that bulk stores cannot write, and every cell when
+// the persistent kernel is off.
 inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, cudaStream_t s) {
   using LY = tc::DecLayout;
   static std::once_flag once;
@@ -112,12 +113,12 @@ inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc
   LAUNCHED();
 }
 
-template <bool TMA_ONLY, unsigned BITMASK>
+template <bool TMA_ONLY, unsigned BITMASK, bool ROPE = false>
 inline void launch_decode_p(const tc::DecPArgs &a, int grid, cudaStream_t s) {
   using LY = tc::DecLayout;
   static std::once_flag once;
-  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
-  tc::decode_persistent_kernel<TMA_ONLY, BITMASK><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
 }
 
 // The persistent kernel is instantiated per output mode and per set of bit widths: with at most two tile loops compiled
@@ -136,7 +137,7 @@ inline void launch_decode_widths(const tc::DecPArgs &a, unsigned bitmask, int gr
 
 // Descriptors of the cells that take the tensor-core decode, in the order [values, r_t <= 128][keys, r_t <= 128][r_t > 128]
 // and in each class the costliest first (most residual bits, then largest r_t: the last wave of per-item CTAs is then the
-// cheapest).  The persistent kernel takes the first two classes in one launch, or only the first when keys are rotated.
+// cheapest).  The persistent kernel takes the first two classes in one launch, or each in its own when keys are rotated.
 inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
   table.clear();
   H.dec = jolt_handle::DecTable();

@@ -1764,22 +1764,42 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
 #ifdef JOLT_DEBUG
   dbg = a.dbg = g_dbg_stamps;
 #endif
-  // the persistent kernel walks the first two classes, or the values alone
+  // The persistent kernel walks the first two classes, or the values and then the keys that it rotates.  The tail that is dealt
+  // out in chunks is empty unless a test asks for one: measured on the benchmark mix, a 5 % tail in 8-tile chunks made the
+  // launch slower (0.199 against 0.192 ms), because every chunk reloads its head's projected core into the single P buffer
+  // and restarts the unpack -> rotation pipeline.
   const int pc = rope ? 0 : 1;
   int done = 0;
-  if ((g_fast.load() & 128) && d.end[pc] > 0 && d.tiles[pc] < (1ll << 30)) {
-    const int total = (int)d.tiles[pc], pct = g_dec_tail_pct.load(), grid = std::min(n_sm[dev].load(), total);
-    a.cells = (const tc::BBCell *)H->d_dec; a.n_cells = d.end[pc]; a.total = total;
+  auto persistent = [&](int c0, int c1, long long t0, long long t1) {      // cells [c0, c1), tiles [t0, t1)
+    const int pct = g_dec_tail_pct.load();
+    a.cells = (const tc::BBCell *)H->d_dec + c0; a.n_cells = c1 - c0;
+    a.first = (int)t0; a.total = (int)t1;
     a.nt = H->T / 128; a.seed = H->seed; a.epoch = H->status_epoch; a.stamps = stamps;
-    // The tail that is dealt out in chunks is empty unless a test asks for one: measured on the benchmark mix, a 5 % tail in
-    // 8-tile chunks made the launch slower (0.199 against 0.192 ms), because every chunk reloads its head's projected
-    // core into the single P buffer and restarts the unpack -> rotation pipeline.
-    a.pool = (int)((long long)total * (100 - pct) / 100); a.chunk = std::max(1, g_dec_tail_chunk.load());
+    a.pool = (int)(t0 + (t1 - t0) * (100 - pct) / 100); a.chunk = std::max(1, g_dec_tail_chunk.load());
     a.counter = H->d_counter;
-    if (a.pool < a.total) CU(cudaMemsetAsync(H->d_counter, 0, sizeof(int), st));
-    launch_decode_widths(a, d.bitmask[pc], grid, st);
+    done = c1;
+    return a.pool < a.total ? cudaMemsetAsync(H->d_counter, 0, sizeof(int), st) : cudaSuccess;
+  };
+  const bool use_p = (g_fast.load() & 128) && d.tiles[1] < (1ll << 30);
+  if (use_p && d.end[pc] > 0) {
+    CU(persistent(0, d.end[pc], 0, d.tiles[pc]));
+    launch_decode_widths(a, d.bitmask[pc], (int)std::min<long long>(n_sm[dev].load(), d.tiles[pc]), st);
     LAUNCHED();
-    done = d.end[pc];
+  }
+  if (use_p && rope && d.end[1] > d.end[0] && a.out.tma_out) {
+    const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)L->seq_len, (uint64_t)L->n_kv_heads, (uint64_t)L->n_layers};
+    const uint64_t str[3] = {(uint64_t)L->stride_token * 2, (uint64_t)L->stride_head * 2, (uint64_t)L->stride_layer * 2};
+    const uint32_t box[4] = {32, 32, 1, 1};
+    const CUtensorMap keep = a.out.tm[0];
+    if (make_tmap_f16(&a.out.tm[0], Kout, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_64B)) {
+      CU(persistent(d.end[0], d.end[1], d.tiles[0], d.tiles[1]));
+      a.rope = rope;
+      const int grid = (int)std::min<long long>(n_sm[dev].load(), d.tiles[1] - d.tiles[0]);
+      if ((d.bitmask[1] & ~0x110u) == 0) launch_decode_p<true, 0x110u, true>(a, grid, st);
+      else launch_decode_p<true, 0x11Fu, true>(a, grid, st);
+      LAUNCHED();
+    }
+    a.out.tm[0] = keep;
   }
   if (done < d.end[1] && done < d.end[2]) launch_decode_items(H, done, d.end[1] - done, a.out, rope, dbg, st);
   if (d.end[1] < d.end[2]) launch_decode_items(H, d.end[1], d.end[2] - d.end[1], a.out, rope, dbg, st);

@@ -25,7 +25,12 @@
 //          rotation MMAs of the old cell are complete by then: each warpgroup has read its last accumulator), copy
 //          the new descriptor, rebuild the rotation operand and re-enter the tile loop compiled for the new bit
 //          width.  A CTA's share touches two cells at most once in a while; cells are never interleaved.
-// Cells of r_t > 128 (their P block needs the whole P region) and keys rotated at decode take the per-item kernel.  A
+// Keys that are rotated at decode (ROPE, fp16 through bulk stores only) are a launch of their own: an accumulator is then read as
+// features {0..31, 64..95} and {32..63, 96..127}, so that both features of a pair are at hand, and each half leaves as two
+// boxes of 32 features.  The first half's (cos, sin) are requested before the wait for the tile, the second half's behind
+// the unpacking of the next tile.  256 heads of 4096 tokens (8 cells,
+// 4 and 8 bits): 185 us per-item, 156 here, 86 without rotation; the difference is the 64 KB of table per tile from L2.
+// Cells of r_t > 128 (their P block needs the whole P region) take the per-item kernel.  A
 // layout with 64 KB for P and a ring of two U_T stages was tried for r_t > 128: the ring of two cannot cover the loads
 // (0.345 ms against 0.29 ms per-item for the eleven such cells of a 8192-token cache).
 #pragma once
@@ -39,11 +44,12 @@ struct DecPArgs {
   const BBCell *cells;
   int n_cells;
   int nt;              // 128-token tiles per head (all cells of a handle share T)
-  int total;           // tiles of the launch
+  int first, total;    // the launch's tiles [first, total) of that order
   uint64_t seed;
-  int pool;            // tiles [0, pool) are dealt out in equal shares; from here on in chunks ...
+  int pool;            // tiles [first, pool) are dealt out in equal shares; from here on in chunks ...
   int chunk;           // ... of this many tiles
   int *counter;        // chunks handed out so far (zero at launch when pool < total; not read otherwise)
+  const float2 *rope;  // ROPE: (cos, sin) of feature pair j at token t in rope[j * T + t]
   unsigned long long *stamps;      // optional: start of the first CTA, end of the last (globaltimer, ns)
   int epoch;           // a failed wait writes (epoch << 8 | 8) into the status word of the first cell
 #ifdef JOLT_DEBUG
@@ -84,6 +90,7 @@ struct DecPCtx {
   uint32_t t_acc;
   unsigned char *rbuf, *stg;              // the warpgroup's operand tile; the warp's 32 staging rows (128 bytes each)
   const DecOut *out;                      // kernel argument: the destination
+  const float2 *rope;
   volatile int *abort_flag;
   int rit;
   int nt, base;                           // tiles per head; first linear tile of the cell
@@ -102,7 +109,7 @@ __device__ __forceinline__ void tma_prefetch_l2_2d(const void *tmap, int c0, int
 // scale, round to fp16, stage the warp's 32 rows and hand them to one bulk tensor store per half.  `pending` says
 // whether a bulk store of this warp may still be reading its staging rows.
 // returns bit 0: no wait ran out, bit 1: a bulk store of this warp is still pending
-template <int BITS, bool TMA_ONLY>
+template <int BITS, bool TMA_ONLY, bool ROPE>
 __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x, int p0, int p_end, bool pending) {
   DecCodes<BITS> cur;
   bool ok = true;
@@ -133,6 +140,12 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
     const int j = p + x.joff, n = j >> 1, acc = n & 1, ph = n >> 1;
     JOLT_DBG(long long *dbg = (c.dbg && blockIdx.x == gridDim.x / 2 && x.rit == 0 && j >= 40 && j < 56) ? c.dbg + (size_t)(j - 40) * 8 : nullptr;)
     JOLT_DBG(if (dbg) dbg[0] = clock64();)
+    float2 tb[ROPE ? 32 : 1];
+    const float2 *tp = ROPE ? x.rope + tt * 128 + x.rit : nullptr;
+    if constexpr (ROPE) {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) tb[k] = __ldg(tp + (size_t)k * c.T);
+    }
     ok = __all_sync(0xffffffffu, mbar_wait(x.bTfull + 16 * acc, ph & 1, x.abort_flag));
     if (!ok) break;
     tc_fence_after();
@@ -142,10 +155,18 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       float va[2][32];
-      tmem_ld32(t_acc + half * 64, va[0]);
-      tmem_ld32(t_acc + half * 64 + 32, va[1]);
+      tmem_ld32(t_acc + half * (ROPE ? 32 : 64), va[0]);
+      tmem_ld32(t_acc + (ROPE ? 64 + half * 32 : half * 64 + 32), va[1]);
       tmem_wait_ld();
       if (half == 1) { tc_fence_before(); mbar_arrive(x.bTempty() + 16 * acc); }
+      if constexpr (ROPE) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          const float a = va[0][k], b = va[1][k];
+          va[0][k] = __fmaf_rn(a, tb[k].x, -__fmul_rn(b, tb[k].y));
+          va[1][k] = __fmaf_rn(b, tb[k].x, __fmul_rn(a, tb[k].y));
+        }
+      }
       if (!f16) {
         float4 *pf = (float4 *)((float *)c.out + (long long)l * c.osl + (long long)hd * c.osh + (long long)(tt * 128 + x.rit) * c.ost) + half * 16;
 #pragma unroll
@@ -168,12 +189,20 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
         pending = false;
       }
 #pragma unroll
-      for (int k8 = 0; k8 < 8; ++k8) *(uint4 *)(rowp + ((k8 ^ (lane & 7)) << 4)) = o[k8];
+      for (int k8 = 0; k8 < 8; ++k8) {
+        if (ROPE) *(uint4 *)(x.stg + (k8 >> 2) * 2048 + lane * 64 + (((k8 & 3) ^ ((lane >> 1) & 3)) << 4)) = o[k8];
+        else *(uint4 *)(rowp + ((k8 ^ (lane & 7)) << 4)) = o[k8];
+      }
       if (tma_out) {
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) {
-          tma_store_4d(&x.out->tm[c.cell & 1], smem_u32(x.stg), half * 64, tt * 128 + wrow0, hd, c.layer0 + l);
+          if (ROPE) {
+            tma_store_4d(&x.out->tm[0], smem_u32(x.stg), half * 32, tt * 128 + wrow0, hd, c.layer0 + l);
+            tma_store_4d(&x.out->tm[0], smem_u32(x.stg) + 2048, 64 + half * 32, tt * 128 + wrow0, hd, c.layer0 + l);
+          } else {
+            tma_store_4d(&x.out->tm[c.cell & 1], smem_u32(x.stg), half * 64, tt * 128 + wrow0, hd, c.layer0 + l);
+          }
           tma_store_commit();
         }
         pending = true;
@@ -203,6 +232,10 @@ __device__ __forceinline__ int dec_tile_loop_p(const BBCell &c, const DecPCtx &x
           if constexpr (BITS > 0) {
             if (p + 4 < p_end) { dec_load_codes<BITS>(c, (long long)hl * c.T + tl * 128 + x.rit, cur); advance(hl, tl); }
           }
+        }
+        if constexpr (ROPE) {        // (across the unpack they would spill)
+#pragma unroll
+          for (int k = 0; k < 32; ++k) tb[k] = __ldg(tp + (size_t)(32 + k) * c.T);
         }
         JOLT_DBG(if (dbg) dbg[3] = clock64();)
       }
@@ -247,7 +280,8 @@ struct DecRunQ {
 // the fp32 and read-back paths)
 // BITMASK: bit b set = the tile loop for b-bit cells is compiled in (a launch takes the smallest instantiated superset
 // of its cells' bit widths: fewer tile loops, a smaller instruction footprint)
-template <bool TMA_ONLY, unsigned BITMASK>
+// ROPE: the cells are keys, rotated by a.rope (with TMA_ONLY; the destination's map has boxes of 32 features)
+template <bool TMA_ONLY, unsigned BITMASK, bool ROPE>
 __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kernel(const __grid_constant__ DecPArgs a) {
   using LY = DecLayout;
   constexpr int NWG = DEC_NWG, NS = LY::NS;
@@ -255,7 +289,8 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   const BBCell *cells = a.cells;
   const int nt = a.nt, total = a.total;
   const int pool = a.pool;
-  const int run0_first = (int)((long long)pool * blockIdx.x / gridDim.x), run0_end = (int)((long long)pool * (blockIdx.x + 1) / gridDim.x);
+  const int run0_first = a.first + (int)((long long)(pool - a.first) * blockIdx.x / gridDim.x);
+  const int run0_end = a.first + (int)((long long)(pool - a.first) * (blockIdx.x + 1) / gridDim.x);
   JOLT_DBG(long long *cta_dbg = a.dbg ? a.dbg + 128 + blockIdx.x * 4 : nullptr;)
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; unsigned sm; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)); cta_dbg[0] = g; cta_dbg[2] = sm; })
 
@@ -512,7 +547,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
         const int cell_end = min(end, cell_last);
         if (ok) {
           DecPCtx x;
-          x.out = &a.out;
+          x.out = &a.out; x.rope = a.rope;
           x.ex = *c.e;
           x.bTfull = bTfull(wg);
           x.t_acc = t_lane + wg * 128; x.rbuf = smR + wg * 32768;
@@ -521,12 +556,12 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           const int p0 = p + (((j & 1) == wg) ? 0 : 1);      // this warpgroup's first tile of the piece
           int rcode = pending ? 2 : 0;      // a bit width that is not compiled in: reported as a failed launch
           const int bits = c.bits;
-          if ((BITMASK & 1u) && bits == 0) rcode = dec_tile_loop_p<0, TMA_ONLY>(c, x, p0, cell_end, pending);
-          if ((BITMASK & 2u) && bits == 1) rcode = dec_tile_loop_p<1, TMA_ONLY>(c, x, p0, cell_end, pending);
-          if ((BITMASK & 4u) && bits == 2) rcode = dec_tile_loop_p<2, TMA_ONLY>(c, x, p0, cell_end, pending);
-          if ((BITMASK & 8u) && bits == 3) rcode = dec_tile_loop_p<3, TMA_ONLY>(c, x, p0, cell_end, pending);
-          if ((BITMASK & 16u) && bits == 4) rcode = dec_tile_loop_p<4, TMA_ONLY>(c, x, p0, cell_end, pending);
-          if ((BITMASK & 256u) && bits == 8) rcode = dec_tile_loop_p<8, TMA_ONLY>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 1u) && bits == 0) rcode = dec_tile_loop_p<0, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 2u) && bits == 1) rcode = dec_tile_loop_p<1, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 4u) && bits == 2) rcode = dec_tile_loop_p<2, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 8u) && bits == 3) rcode = dec_tile_loop_p<3, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 16u) && bits == 4) rcode = dec_tile_loop_p<4, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
+          if ((BITMASK & 256u) && bits == 8) rcode = dec_tile_loop_p<8, TMA_ONLY, ROPE>(c, x, p0, cell_end, pending);
           ok = (rcode & 1) != 0; pending = (rcode & 2) != 0;
         }
         j += cell_end - p;

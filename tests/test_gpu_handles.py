@@ -116,3 +116,28 @@ def test_default_stream_decodes_then_another_stream(B):
         for o in outs:
             assert torch.equal(o[0], ref[0]) and torch.equal(o[1], ref[1])
     h.free()
+
+
+@pytest.mark.parametrize("bits", [(0, 1), (2, 3), (4, 8)])
+@pytest.mark.parametrize("T,tail", [(128, 0), (640, 0), (384, 60)])
+def test_rotated_keys_of_the_persistent_kernel(B, bits, T, tail):
+    """Every key width, one and several tiles a head, tiles dealt out in chunks: against the per-item kernel (bit 7 off)."""
+    K, V = _cache(4, 3, T, 9)
+    gs = [0, 2, 4]
+    plans = [(32, 128, bits[0]), (48, 128, 4), (128, 96, bits[1]), (16, 128, 2)]
+    h = B.jolt_compress(K, V, gs, plans, B.default_options(seed=2, power_iters=0))
+    outs = []
+    for mask in (255, 255 - 128):
+        Ko, Vo = torch.empty_like(K), torch.empty_like(V)
+        prev = B.set_fast_path(mask)
+        B.set_test_decode_tail(tail, 2)
+        try:
+            B.jolt_decompress_rope(h, Ko, Vo, gs, base=10000.0, pos0=100)
+            torch.cuda.synchronize()
+        finally:
+            B.set_fast_path(prev)
+            B.set_test_decode_tail(0)
+        outs.append((Ko, Vo))
+    h.free()
+    # the same operands, accumulators and rounding in both kernels
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
