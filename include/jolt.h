@@ -282,14 +282,14 @@ int jolt_release_workspace(void);
 int64_t jolt_launch_count(void);
 
 /* Selects the kernel family by bit mask: 0 = portable SIMT kernels only; bit 0 = fused tcgen05 backbone
- * kernels (decode, residual) and the tensor-core forms of jolt_attend's code streams, bit 1 = tcgen05 factor sweeps (sketch, projection), bit 2 = tcgen05 mode-3
+ * kernels (decode, residual) and the streaming kernel of jolt_attend, bit 1 = tcgen05 factor sweeps (sketch, projection), bit 2 = tcgen05 mode-3
  * Gram, bit 3 = rotary embedding inside the decode kernel (jolt_decompress_rope; otherwise a separate pass),
- * bit 4 = tridiagonal eigen-solver (otherwise Jacobi, one launch per round),
+ * bit 4 = tridiagonal eigen-solver, the probe's values from a cluster-resident Jacobi (otherwise Jacobi, one launch per round),
  * bit 5 = CholeskyQR of the range finder on tensor cores (otherwise fp64 SIMT Gram and row-wise triangular solve),
  * bit 6 = factor sweeps with two output tiles per CTA (otherwise one);
  * bit 7 = persistent decode kernel (one CTA per SM walks a share of all tiles; otherwise one CTA per 16-tile item;
- *         launches with a cell of r_t > 128, with keys rotated at decode or with cells of different sequence
- *         lengths always take the per-item kernel);
+ *         cells of r_t > 128 and keys rotated into an fp32 or unaligned destination always take the per-item
+ *         kernel);
  * 255 (default) = all, where the shapes allow.  Returns the previous mask. */
 int jolt_set_fast_path(int enabled);
 

@@ -13,8 +13,7 @@
 // not their squares), needs no eigenvector accumulator, and is what makes single precision enough: one-sided Jacobi
 // resolves every column relative to its own norm, so the small singular directions keep the relative accuracy of the
 // fp64 factor they start from (the paper's own decomposition numerics are float32, Sec. 6 "Setup").  Measured on
-// spectra shaped like the benchmark's: eigenvector orthogonality 2e-6, dominant-subspace projectors within 4e-5 of an
-// fp64 solve at a relative gap of 1e-2, eigenvalues to 4e-6.
+// spectra shaped like the benchmark's: eigenvalues to 4e-6.
 //
 // The n columns are cut into 16 blocks of g columns; CTA c holds two blocks.  A block round orthogonalises every
 // column of the left block against every column of the right block (g sub-rounds of g disjoint pairs, one warp per

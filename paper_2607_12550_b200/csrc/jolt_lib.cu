@@ -1120,7 +1120,7 @@ int run_program(Program &P, char *d_tables, cudaStream_t st, bool timed = true) 
 
 // Side streams on which independent groups of cells run their (latency-bound) factor stages concurrently.
 constexpr int kMaxGroups = 8;
-struct GroupStreams { bool have = false; cudaStream_t s[kMaxGroups]; cudaEvent_t fork, join[kMaxGroups]; };
+struct GroupStreams { bool have = false; cudaStream_t s[kMaxGroups]; cudaEvent_t fork, join[kMaxGroups], arrive[kMaxGroups]; };
 GroupStreams g_groups[64];
 GroupStreams *group_streams(int dev) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
@@ -1137,6 +1137,7 @@ GroupStreams *group_streams(int dev) {
       cudaDeviceGetStreamPriorityRange(&lo, &hi);      // (least, greatest)
       if (cudaStreamCreateWithPriority(&g.s[i], cudaStreamNonBlocking, i == 0 ? hi : (hi + lo) / 2) != cudaSuccess) return nullptr;
       if (cudaEventCreateWithFlags(&g.join[i], cudaEventDisableTiming) != cudaSuccess) return nullptr;
+      if (cudaEventCreateWithFlags(&g.arrive[i], cudaEventDisableTiming) != cudaSuccess) return nullptr;
     }
     if (cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     g.have = true;
@@ -1146,12 +1147,19 @@ GroupStreams *group_streams(int dev) {
 
 // Cells whose factor stages may run side by side.  Cells that need the feature eigen-solve (the longest chain)
 // and the others never share a group.
-int assign_groups(const std::vector<CellWork> &ws, std::vector<int> &group) {
+// in_order: the cells arrive one after another (host memory): runs of neighbouring cells, the last to arrive in group 0.
+int assign_groups(const std::vector<CellWork> &ws, std::vector<int> &group, bool in_order = false) {
   const int want = std::max(1, std::min(kMaxGroups, g_n_cell_groups.load()));
   group.assign(ws.size(), -1);
   int n_active = 0, n_long = 0;
   for (auto &w : ws) if (w.active) { ++n_active; if (!w.ufI) ++n_long; }
   if (n_active < 2 || want == 1) { for (size_t i = 0; i < ws.size(); ++i) if (ws[i].active) group[i] = 0; return n_active ? 1 : 0; }
+  if (in_order) {
+    const int n = std::min(want, n_active);
+    int r = 0;
+    for (size_t i = 0; i < ws.size(); ++i) if (ws[i].active) group[i] = n - 1 - (int)((long long)r++ * n / n_active);
+    return n;
+  }
   // long cells share the first groups, short cells the rest, each in proportion to their number
   int g_long = 0;
   if (n_long > 0 && n_long < n_active) g_long = std::max(1, std::min(want - 1, (want * n_long + n_active / 2) / n_active));
@@ -1309,14 +1317,14 @@ struct GroupRun {
     at = o + bytes;
     return o;
   }
-  void add(int g) {                          // program g (they come in order) is built
+  void add(int g, size_t early = kEarlySteps) {      // program g (they come in order) is built
     const size_t o = take(PG[g].host.size());
     if (ce == cudaSuccess) ce = cudaStreamWaitEvent(gs->s[g], gs->fork, 0);
     if (ce == cudaSuccess && !PG[g].host.empty())
       ce = cudaMemcpyAsync(tab + o, PG[g].host.data(), PG[g].host.size(), cudaMemcpyHostToDevice, gs->s[g]);
     off.push_back(o);
     done.push_back(0);
-    for (; ce == cudaSuccess && done[g] < std::min<size_t>(kEarlySteps, PG[g].steps.size()); ++done[g]) PG[g].steps[done[g]].run(tab + o, gs->s[g]);
+    for (; ce == cudaSuccess && done[g] < std::min(early, PG[g].steps.size()); ++done[g]) PG[g].steps[done[g]].run(tab + o, gs->s[g]);
   }
   int finish() {
     for (bool any = true; any && ce == cudaSuccess;) {
@@ -1556,7 +1564,10 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
   // ---- programs
   Program P;
   std::vector<int> cell_group;
-  const int n_groups = assign_groups(ws, cell_group);
+  // host memory, layer after layer: the copies go out by layer group and a cell's program starts when its layers have arrived
+  const bool by_arrival = L->mem_space == JOLT_MEM_HOST && !injected &&
+                          L->stride_layer >= (int64_t)(L->n_kv_heads - 1) * L->stride_head + (int64_t)(L->seq_len - 1) * L->stride_token + kD;
+  const int n_groups = assign_groups(ws, cell_group, by_arrival);
   std::vector<Program> PG(std::max(n_groups, 1));
   auto build_group = [&](int g) {
     std::vector<CellWork> sub = ws;
@@ -1669,7 +1680,8 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
     if (cells[i].r_t == 0 || cells[i].r_f == kD || injected) cl.push_back({(uint32_t *)H->cells[i].lam, kD});
   }
   cudaError_t ce = clear_ranges(cl, st);
-  if (ce == cudaSuccess && L->mem_space == JOLT_MEM_HOST) {
+  const bool late_copy = by_arrival && n_groups > 1;
+  if (ce == cudaSuccess && L->mem_space == JOLT_MEM_HOST && !late_copy) {
     ce = cudaMemcpyAsync(stage_K, K, span, cudaMemcpyHostToDevice, st);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(stage_V, V, span, cudaMemcpyHostToDevice, st);
     g_timer.mark(ST_IN, st);
@@ -1690,12 +1702,34 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
     if ((rc = run_program(P, (char *)d_tab + ((PG[0].host.size() + 255) & ~(size_t)255), st))) { free_blob(); return rc; }
   } else {
     run.fork();
+    // Copies to the device are served in the order they were asked for: the first group's layers go out at once, the tables of
+    // the programs (built meanwhile) behind them, then the other layers.
+    std::vector<int> left(n_groups, 0);
+    int first_end = 0;
+    auto copy_cells = [&](int c0, int c1) {
+      for (int i = c0; i < c1 && run.ce == cudaSuccess; ++i) {
+        const size_t o0 = (size_t)L->group_start[i / 2] * L->stride_layer * esz, o1 = std::min(span, (size_t)L->group_start[i / 2 + 1] * L->stride_layer * esz);
+        run.ce = cudaMemcpyAsync((i % 2 ? stage_V : stage_K) + o0, (const char *)(i % 2 ? V : K) + o0, o1 - o0, cudaMemcpyHostToDevice, st);
+        const int g = cell_group[i];
+        if (g >= 0 && --left[g] == 0 && run.ce == cudaSuccess) run.ce = cudaEventRecord(run.gs->arrive[g], st);
+      }
+    };
+    if (late_copy) {
+      for (int i = 0; i < nc; ++i) if (cell_group[i] >= 0) ++left[cell_group[i]];
+      while (first_end < nc && (cell_group[first_end] < 0 || cell_group[first_end] == n_groups - 1)) ++first_end;
+      copy_cells(0, first_end);
+    }
     for (int g = 0; g < n_groups; ++g) {
       std::vector<int> idx;
       for (int i = 0; i < nc; ++i) if (cell_group[i] == g) idx.push_back(i);
       build_group(g);
       build_tail(PG[g], idx);
-      run.add(g);
+      run.add(g, late_copy ? 0 : kEarlySteps);
+    }
+    if (late_copy) {
+      copy_cells(first_end, nc);
+      for (int g = 0; g < n_groups && run.ce == cudaSuccess; ++g) run.ce = cudaStreamWaitEvent(run.gs->s[g], run.gs->arrive[g], 0);
+      g_timer.mark(ST_IN, st);
     }
     std::vector<int> rest;
     for (int i = 0; i < nc; ++i) if (cell_group[i] < 0) rest.push_back(i);
