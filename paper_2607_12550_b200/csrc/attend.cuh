@@ -58,6 +58,16 @@ struct AttendJob {                  // one per layer group
   float *a;                         // [m][n_chunks][NQP][128]
 };
 
+// The descriptors of a short call travel as a kernel argument (up to 15 layer groups): the copy ahead of it cost more than its
+// kernels' ramps (35 -> 31 us at 384 tokens).  A call of more than one wave of CTAs has them in the table arena: the streaming
+// kernel that reads them from its argument spills 48 bytes (128.5 against 126.3 us at 4096 tokens).
+constexpr int kAttArgJobs = 15;
+struct AttendArgs {
+  const AttendJob *table;           // null: j
+  AttendJob j[kAttArgJobs];
+};
+__device__ __forceinline__ const AttendJob &att_job(const AttendArgs &a, int i) { return a.table ? a.table[i] : a.j[i]; }
+
 // 128-point Walsh-Hadamard transform by one warp: lane l holds elements 4 l .. 4 l + 3.
 __device__ __forceinline__ void att_wht_warp(float (&v)[4]) {
   const int lane = threadIdx.x & 31;
@@ -103,8 +113,8 @@ __device__ __forceinline__ float att_sign(uint64_t seed, int cell, int f) {
 // four rows in flight.  Bound by the latency of its few loads: with a CTA per query, block-wide transforms and five shuffles
 // per value and row it took 19.6 us at 8 groups of 32 heads, rank 128; now 8.8.
 template <int NQ>
-__global__ void __launch_bounds__(256) attend_prep_kernel(const AttendJob *__restrict__ jobs, int n_q, float scale, uint64_t seed) {
-  const AttendJob &jb = jobs[blockIdx.y];
+__global__ void __launch_bounds__(256) attend_prep_kernel(const __grid_constant__ AttendArgs args, int n_q, float scale, uint64_t seed) {
+  const AttendJob &jb = att_job(args, blockIdx.y);
   const int h = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (h >= jb.m) return;
   att_let_successor_start();
@@ -774,10 +784,10 @@ __device__ __forceinline__ void att_code_values(const AttendJob &jb, size_t row0
 
 // grid (ceil(chunks / (4 / NH)), ceil(m / NH), groups), 128 threads, att_stream_smem bytes of dynamic shared memory.  NH = 4: the
 // warps are four heads of one chunk; NH = 1 (fewer than three heads in a cell): four chunks of one head.
-template <int NQ, int NH>
-__global__ void __launch_bounds__(kAttStreamThreads, NQ == 4 ? 4 : 3) attend_stream_kernel(const AttendJob *__restrict__ jobs, int n_chunks) {
+template <int NQ, int NH, bool BYARG>
+__global__ void __launch_bounds__(kAttStreamThreads, NQ == 4 ? 4 : 3) attend_stream_kernel(const __grid_constant__ AttendArgs args, int n_chunks) {
   constexpr int TC = kAttTok, P = kAttPitch;
-  const AttendJob &jb = jobs[blockIdx.z];
+  const AttendJob &jb = BYARG ? args.j[blockIdx.z] : args.table[blockIdx.z];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, c = lane & 3;
   const int h0 = blockIdx.y * NH, t_cta = blockIdx.x * (TC * 4 / NH), T = jb.T, m = jb.m;
   if (h0 >= m || t_cta >= T) return;
@@ -1148,9 +1158,9 @@ __global__ void __launch_bounds__(256) attend_bvalue_kernel(const AttendJob *__r
 }
 
 // grid (m, groups, n_q), 128 threads; CTA z finishes query z.  Dynamic shared memory: (n_chunks + v.r_t + 128) floats.
-__global__ void __launch_bounds__(128) attend_combine_kernel(const AttendJob *__restrict__ jobs, int n_q, int NQP, int n_chunks,
+__global__ void __launch_bounds__(128) attend_combine_kernel(const __grid_constant__ AttendArgs args, int n_q, int NQP, int n_chunks,
                                                              uint64_t seed) {
-  const AttendJob &jb = jobs[blockIdx.y];
+  const AttendJob &jb = att_job(args, blockIdx.y);
   const int h = blockIdx.x, f = threadIdx.x, i = blockIdx.z, warp = f >> 5, lane = f & 31;
   if (h >= jb.m) return;
   extern __shared__ unsigned char att_smem[];

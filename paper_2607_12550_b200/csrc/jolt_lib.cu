@@ -2061,7 +2061,7 @@ static void launch_att_values(dim3 grid, cudaStream_t s, const AttendJob *d, int
 
 // A launch that may begin while the kernel before it on the stream drains (it waits on the device for that kernel's results).
 template <typename... P, typename... A>
-static void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t shm, cudaStream_t s, A... args) {
+static void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t shm, cudaStream_t s, const A &...args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = shm; cfg.stream = s;
@@ -2134,28 +2134,33 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
     if (pass == 0 && (rc = ws_reserve(dev, b.off + 256, &ws_base))) return rc;
   }
   Program P;
-  const size_t off = P.push(jobs);
+  const bool h4 = m_max >= 3;                       // a CTA of the streaming kernel: four heads, or four chunks of one
+  const dim3 sg(h4 ? n_chunks : (n_chunks + 3) / 4, h4 ? (m_max + 3) / 4 : m_max, ng);
+  const bool by_arg = mma && ng <= kAttArgJobs && (long long)sg.x * sg.y * sg.z <= 592;
+  const size_t off = by_arg ? 0 : P.push(jobs);
   const uint64_t seed = H->seed;
   const float fscale = (float)scale;
-  P.add(ST_ATT, [=](char *dev_t, cudaStream_t s) {
-    const AttendJob *d = (const AttendJob *)(dev_t + off);
-    if (NQP == 4) attend_prep_kernel<4><<<dim3(m_max, ng), 256, 0, s>>>(d, n_q, fscale, seed);
-    else attend_prep_kernel<8><<<dim3(m_max, ng), 256, 0, s>>>(d, n_q, fscale, seed);
+  P.add(ST_ATT, [&, off](char *dev_t, cudaStream_t s) {              // run before this function returns
+    const AttendJob *d = by_arg ? nullptr : (const AttendJob *)(dev_t + off);
+    AttendArgs args;
+    memset(&args, 0, sizeof args);
+    args.table = d;
+    if (by_arg) std::copy(jobs.begin(), jobs.end(), args.j);
+    if (NQP == 4) attend_prep_kernel<4><<<dim3(m_max, ng), 256, 0, s>>>(args, n_q, fscale, seed);
+    else attend_prep_kernel<8><<<dim3(m_max, ng), 256, 0, s>>>(args, n_q, fscale, seed);
     LAUNCHED();
     const dim3 grid(n_chunks, m_max, ng);
     if (mma) {
       static std::once_flag once;
       std::call_once(once, [] {
-        cudaFuncSetAttribute(attend_stream_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(4));
-        cudaFuncSetAttribute(attend_stream_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(4));
-        cudaFuncSetAttribute(attend_stream_kernel<8, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(8));
-        cudaFuncSetAttribute(attend_stream_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(8));
+        auto allow = [](auto k, int nq) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(nq)); };
+        allow(attend_stream_kernel<4, 4, true>, 4); allow(attend_stream_kernel<4, 1, true>, 4); allow(attend_stream_kernel<8, 4, true>, 8); allow(attend_stream_kernel<8, 1, true>, 8);
+        allow(attend_stream_kernel<4, 4, false>, 4); allow(attend_stream_kernel<4, 1, false>, 4); allow(attend_stream_kernel<8, 4, false>, 8); allow(attend_stream_kernel<8, 1, false>, 8);
       });
-      const bool h4 = m_max >= 3;
-      const dim3 sg(h4 ? n_chunks : (n_chunks + 3) / 4, h4 ? (m_max + 3) / 4 : m_max, ng);
       const size_t shm = att_stream_smem(NQP);
-      launch_overlapped(NQP == 4 ? (h4 ? attend_stream_kernel<4, 4> : attend_stream_kernel<4, 1>) : (h4 ? attend_stream_kernel<8, 4> : attend_stream_kernel<8, 1>),
-                        sg, kAttStreamThreads, shm, s, d, n_chunks);
+      auto k = by_arg ? (NQP == 4 ? (h4 ? attend_stream_kernel<4, 4, true> : attend_stream_kernel<4, 1, true>) : (h4 ? attend_stream_kernel<8, 4, true> : attend_stream_kernel<8, 1, true>))
+                      : (NQP == 4 ? (h4 ? attend_stream_kernel<4, 4, false> : attend_stream_kernel<4, 1, false>) : (h4 ? attend_stream_kernel<8, 4, false> : attend_stream_kernel<8, 1, false>));
+      launch_overlapped(k, sg, kAttStreamThreads, shm, s, args, n_chunks);
       LAUNCHED();
     } else {
       const int n_tiles = (m_max * NQP + 127) / 128;
@@ -2193,11 +2198,11 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
       }
     }
     if (shm_comb > 48 * 1024) cudaFuncSetAttribute(attend_combine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-    launch_overlapped(attend_combine_kernel, dim3(m_max, ng, n_q), 128, shm_comb, s, d, n_q, NQP, n_chunks, seed);
+    launch_overlapped(attend_combine_kernel, dim3(m_max, ng, n_q), 128, shm_comb, s, args, n_q, NQP, n_chunks, seed);
     LAUNCHED();
   });
   void *d_tab = nullptr;
-  if ((rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
+  if (!by_arg && (rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
   if ((rc = handle_acquire(H, dev, st))) return rc;
   H->last_stream = st;
   g_timer.begin(st);

@@ -24,6 +24,8 @@ def B():
     (3, 2, 3, 384, (264, 136, 24, 0), (4, 8, 0, 4), 4),           # six and three heads: a partial quad
     (3, 2, 5, 256, (64, 96, 8, 248), (8, 2, 3, 1), 8),
     (5, 4, 4, 512, (128, 112, 96, 40), (1, 3, 8, 0), 5),
+    (4, 2, 10, 9600, (16, 32, 24, 8), (4, 8, 2, 3), 4),           # more than one wave of CTAs: descriptors in the table arena
+    (4, 2, 1, 40960, (16, 8, 8, 24), (8, 4, 3, 1), 6),
 ])
 def test_stream_matches_cuda_core_path(B, L, g1, H, T, ranks, bits, nq):
     g = torch.Generator().manual_seed(L * 1000 + T)
@@ -47,3 +49,22 @@ def test_stream_matches_cuda_core_path(B, L, g1, H, T, ranks, bits, nq):
     smax = torch.einsum("lhqf,lhtf->lhqt", Q, K.float()).abs().amax(-1) / 128 ** 0.5
     per_row = (out - ref).norm(dim=-1) / ref.norm(dim=-1)
     assert bool((per_row <= 5e-6 + 2.0 ** -21 * smax).all()), (per_row / smax).max()
+
+
+@pytest.mark.parametrize("groups", [15, 16])                       # descriptors as a kernel argument / in the table arena
+def test_many_layer_groups(B, groups):
+    g = torch.Generator().manual_seed(groups)
+    K, V = (torch.randn(groups, 2, 256, 128, generator=g).half().cuda() for _ in range(2))
+    gs = list(range(groups + 1))
+    h = B.jolt_compress(K, V, gs, [(16, 128, 8), (24, 128, 4)] * groups, B.default_options(seed=1, power_iters=0))
+    Q = torch.randn(groups, 2, 4, 128, generator=g).cuda()
+    out = B.jolt_attend(h, Q)
+    prev = B.set_fast_path(14)                                     # (always the table)
+    try:
+        ref = B.jolt_attend(h, Q)
+        torch.cuda.synchronize()
+    finally:
+        B.set_fast_path(prev)
+    h.free()
+    # scores of size one: 2^-21 of a weight, and the values' own sums
+    assert float(((out - ref).norm(dim=-1) / ref.norm(dim=-1)).max()) <= 1e-5
