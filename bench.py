@@ -438,7 +438,7 @@ def main():
                     "frac": ach / pk["tensor"], "traffic": traffic, "algorithmic_flops": fd, "kernel_ms": t_dec,
                     "peak_source": pk["source"] + " (MEASURED_PEAKS.json bf16_tflops, burst)"}
 
-    # compress: its largest GPU-filling kernel is the fused residual pass (tc::backbone_kernel<true>: X in, codes and
+    # compress: its largest GPU-filling kernel is the fused residual pass (tc::backbone_kernel: X in, codes and
     # scales out), HBM-bound; the factor sweeps (tc::tc_gemm2_kernel) read X once each and are bound by the tensor
     # pipe once the dense operand is split in hi + lo (two MMAs per K step)
     fr, br_ = tot["residual_quant"]
@@ -447,7 +447,7 @@ def main():
     if t_res:
         tr = dram_traffic("tc::backbone_kernel<1>", cfg.name)
         ach = br_ / (t_res * 1e-3) / 1e9
-        roof_c = {"kernel": "tc::backbone_kernel<1>", "bound": "hbm", "achieved": ach, "peak": pk["hbm"], "unit": "GB/s",
+        roof_c = {"kernel": "tc::backbone_kernel", "bound": "hbm", "achieved": ach, "peak": pk["hbm"], "unit": "GB/s",
                   "frac": ach / pk["hbm"], "traffic": (tr["read"] + tr["write"]) * (2 * ng) / tr["cells"] if tr else None,
                   "algorithmic_bytes": br_, "kernel_ms": t_res,
                   "peak_source": pk["source"] + " (MEASURED_PEAKS.json hbm_gbs)"}
