@@ -137,6 +137,7 @@ static int ws_reserve(int dev, size_t bytes, void **out) {
 // The workspace and the argument-table arena are shared by every call on a device.  A call makes its stream wait for
 // the last launch of the previous call that used them (whatever stream that ran on) and leaves an event behind.
 static cudaEvent_t g_arena_ev[64] = {};
+static cudaEvent_t g_default_ev[64] = {};       // calls on the default stream that left no event in g_arena_ev (handle_acquire)
 static int arena_acquire(int dev, cudaStream_t st) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
   if (!g_arena_ev[dev]) {
@@ -1841,9 +1842,18 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   return JOLT_OK;
 }
 
-// arena_acquire for a call that reads a handle: also after the calls on the default stream that left no event behind
+// arena_acquire for a call that reads a handle: also after the calls on the default stream that left no event behind.  They get
+// an event of their own, recorded and waited for in one step: the arena's event holds the last user of the shared memory,
+// which may be on a stream that the default stream has not waited for.
 static int handle_acquire(const jolt_handle *H, int dev, cudaStream_t st) {
-  if (st && H->unreleased.exchange(false)) arena_release(dev, nullptr);
+  if (st && H->unreleased.exchange(false)) {
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    cudaEvent_t &ev = g_default_ev[dev];
+    cudaError_t e = ev ? cudaSuccess : cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, nullptr);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
+    if (e != cudaSuccess) { cudaGetLastError(); H->unreleased = true; return fail(JOLT_ECUDA, "event: %s", cudaGetErrorString(e)); }
+  }
   return arena_acquire(dev, st);
 }
 

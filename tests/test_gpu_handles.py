@@ -1,4 +1,6 @@
 """Decode of caches whose cells fall into different kernel classes, and the memory of freed handles used again."""
+import time
+
 import pytest
 import torch
 
@@ -116,6 +118,50 @@ def test_default_stream_decodes_then_another_stream(B):
         for o in outs:
             assert torch.equal(o[0], ref[0]) and torch.equal(o[1], ref[1])
     h.free()
+
+
+def _held(stream, seconds=0.2):
+    """The stream is busy for about that long (a bounded spin of SM clocks, up to 2 GHz)."""
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(int(seconds * 1.9e9))
+
+
+def _after(stream):
+    ev = torch.cuda.Event()
+    ev.record(stream)
+    return ev
+
+
+def test_call_on_a_third_stream_waits_for_the_second(B):
+    """h1 was decoded on the default stream, h2 is used on stream C (held back): a call that reads h1 on stream A uses the same
+    shared memory as C's and comes after it, and both give what they give alone."""
+    K, V = _cache(2, 4, 1024, 11)
+    gs, plan = [0, 2], [(32, 128, 4), (16, 64, 2)]
+    opts = B.default_options(seed=1, power_iters=0)
+    h1, h2 = B.jolt_compress(K, V, gs, plan, opts), B.jolt_compress(V, K, gs, plan, opts)
+    Q1, Q2 = (torch.randn(2, 4, 4, 128, generator=torch.Generator().manual_seed(i)).cuda() for i in (1, 2))
+    o = torch.empty_like(K), torch.empty_like(V)
+    want1, want2 = B.jolt_attend(h1, Q1), B.jolt_attend(h2, Q2)
+    B.jolt_decompress_rope(h1, *o, gs, base=10000.0, pos0=3)
+    torch.cuda.synchronize()
+    want_rope = [t.clone() for t in o]
+    C, A = torch.cuda.Stream(), torch.cuda.Stream()
+    for call in ("attend", "rope"):
+        B.jolt_decompress(h1, *o, gs)
+        torch.cuda.synchronize()
+        _held(C)
+        got2 = B.jolt_attend(h2, Q2, stream=C)
+        if call == "attend":
+            got1 = B.jolt_attend(h1, Q1, stream=A)
+        else:
+            B.jolt_decompress_rope(h1, *o, gs, base=10000.0, pos0=3, stream=A)
+        done = _after(A)
+        time.sleep(0.03)
+        assert not done.query()
+        torch.cuda.synchronize()
+        assert torch.equal(got2, want2)
+        assert torch.equal(got1, want1) if call == "attend" else torch.equal(o[0], want_rope[0]) and torch.equal(o[1], want_rope[1])
+    h1.free(); h2.free()
 
 
 @pytest.mark.parametrize("bits", [(0, 1), (2, 3), (4, 8)])
