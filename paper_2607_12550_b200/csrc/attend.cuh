@@ -99,7 +99,8 @@ __device__ __forceinline__ float att_warp_sums(float (&v)[N]) {
   return v[0];
 }
 
-// A kernel launched while its predecessor still runs waits here before it reads what that one wrote.
+// A kernel launched while its predecessor still runs waits here before it reads what that one wrote: by plain loads (the read-only
+// path, __ldg, is for memory that nobody writes while the kernel is resident, and may be moved across the wait).
 __device__ __forceinline__ void att_wait_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void att_let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -831,7 +832,7 @@ __global__ void __launch_bounds__(kAttStreamThreads, NQ == 4 ? 4 : 3) attend_str
       uint4 bn[NH];
       auto load_b = [&](int k) {
 #pragma unroll
-        for (int j = 0; j < NH; ++j) bn[j] = k + 8 * c < kr && h0 + j < m ? __ldg((const uint4 *)(w0 + (size_t)j * NQ * kr + k)) : zero;
+        for (int j = 0; j < NH; ++j) bn[j] = k + 8 * c < kr && h0 + j < m ? *(const uint4 *)(w0 + (size_t)j * NQ * kr + k) : zero;
       };
       load_b(0);
       load_a(0);
@@ -841,7 +842,7 @@ __global__ void __launch_bounds__(kAttStreamThreads, NQ == 4 ? 4 : 3) attend_str
 #pragma unroll
         for (int j = 0; j < NH; ++j) {
           b[j] = bn[j];
-          if (NQ == 8) bl[j] = k + 8 * c < kr && h0 + j < m ? __ldg((const uint4 *)(w1 + (size_t)j * NQ * kr + k)) : zero;
+          if (NQ == 8) bl[j] = k + 8 * c < kr && h0 + j < m ? *(const uint4 *)(w1 + (size_t)j * NQ * kr + k) : zero;
         }
         if (k + 32 < kr) load_b(k + 32);
 #pragma unroll
@@ -1196,11 +1197,11 @@ __global__ void __launch_bounds__(128) attend_combine_kernel(const __grid_consta
     for (; c + 16 <= n_chunks; c += 16) {
       float v[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = __ldg(p + (size_t)(c + u) * stride);
+      for (int u = 0; u < 16; ++u) v[u] = p[(size_t)(c + u) * stride];
 #pragma unroll
       for (int u = 0; u < 16; ++u) acc[u & 3] = fmaf(coef[c + u], v[u], acc[u & 3]);
     }
-    for (; c < n_chunks; ++c) acc[0] = fmaf(coef[c], __ldg(p + (size_t)c * stride), acc[0]);
+    for (; c < n_chunks; ++c) acc[0] = fmaf(coef[c], p[(size_t)c * stride], acc[0]);
     return (acc[0] + acc[1]) + (acc[2] + acc[3]);
   };
   if (jb.v.bits > 0) buf[f] = merge(jb.a + ((size_t)h * n_chunks * NQP + i) * 128 + f, (size_t)NQP * 128);

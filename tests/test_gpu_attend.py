@@ -68,3 +68,21 @@ def test_many_layer_groups(B, groups):
     h.free()
     # scores of size one: 2^-21 of a weight, and the values' own sums
     assert float(((out - ref).norm(dim=-1) / ref.norm(dim=-1)).max()) <= 1e-5
+
+
+# the second and third kernel of a call start while their predecessor runs: one head a CTA and four, descriptors by argument and table
+@pytest.mark.parametrize("L,H,T,nq", [(2, 1, 512, 4), (4, 8, 1024, 8), (2, 16, 16384, 4)])
+def test_calls_in_a_row_use_their_own_queries(B, L, H, T, nq):
+    g = torch.Generator().manual_seed(T)
+    K, V = (torch.randn(L, H, T, 128, generator=g).half().cuda() for _ in range(2))
+    h = B.jolt_compress(K, V, [0, L], [(32, 128, 4), (48, 128, 8)], B.default_options(seed=3, power_iters=0))
+    Q = [torch.randn(L, H, nq, 128, generator=g).cuda() * 2.0 ** i for i in range(5)]
+    want = []
+    for q in Q:
+        want.append(B.jolt_attend(h, q))
+        torch.cuda.synchronize()
+    got = [B.jolt_attend(h, Q[i % 5]) for i in range(25)]
+    torch.cuda.synchronize()
+    h.free()
+    for i, o in enumerate(got):
+        assert torch.equal(o, want[i % 5]), i
