@@ -505,10 +505,13 @@ __global__ void __launch_bounds__(kTdValThreads) td_values_kernel(const TdTask *
   __shared__ double s_lo[4], s_hi[4];
   const int tid = threadIdx.x, lane = tid & 31, n8 = (n + 7) & ~7;
   double lo = 1e300, hi = -1e300;
+  bool finite = true;
   for (int i = tid; i < n; i += kTdValThreads) {
     const double r = (i > 0 ? fabs(t.e[i - 1]) : 0.0) + (i + 1 < n ? fabs(t.e[i]) : 0.0), d = t.d[i];
+    finite = finite && fabs(d) + r < 1e300;                         // (false for a NaN, which fmin and fmax pass over)
     lo = fmin(lo, d - r); hi = fmax(hi, d + r);
   }
+  if (!finite && blockIdx.x == 0 && t.status) atomicOr(t.status, 1);
   for (int o = 16; o; o >>= 1) { lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
   if (lane == 0) { s_lo[tid >> 5] = lo; s_hi[tid >> 5] = hi; }
   __syncthreads();

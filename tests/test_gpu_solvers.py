@@ -108,3 +108,28 @@ def test_probe_values_give_the_portable_plan(B, q_cap):
         # values agree to some 1e-6 of the largest: a near-tie moves one cell by one step of the grid, and nothing else moves
         assert sum(x != y for x, y in zip(p, q)) <= 1, (p, q)
         assert all(abs(x[0] - y[0]) <= 16 and x[1] == y[1] and x[2] == y[2] for x, y in zip(p, q)), (p, q)
+
+
+# one entry of the cache is no number: the spectra do not exist, and the call has to say so
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
+@pytest.mark.parametrize("mask", [255, 255 - 16, 0])
+def test_planning_a_cache_that_is_not_finite_fails(B, bad, dtype, mask):
+    T = 512
+    K, V = _cache(T, 4, 40, 0.05, 1).to(dtype), _cache(T, 4, 70, 0.3, 2).to(dtype)
+    raw = 2 * K.numel() * 2
+    prev = B.set_fast_path(mask)
+    try:
+        for opts in (B.default_options(seed=3, q_cap=64), B.default_options(seed=3, q_cap=300),
+                     B.default_options(seed=3, token_mode=B.TOKEN_EXACT)):
+            for X, at in ((K, (0, 0, 0, 0)), (V, (0, 3, T - 1, 77))):
+                keep = X[at].clone()
+                X[at] = bad
+                for call in (lambda: B.jolt_plan(K, V, [0, 1], raw / 2, opts), lambda: B.jolt_probe(K, V, [0, 1], 2.0, opts)):
+                    with pytest.raises(B.JoltError) as e:
+                        call()
+                    assert e.value.status == B.ENUMERIC
+                X[at] = keep
+            assert B.jolt_plan(K, V, [0, 1], raw / 2, opts)[1] <= raw / 2
+    finally:
+        B.set_fast_path(prev)
