@@ -13,10 +13,11 @@
  *
  * Concurrency.  Scratch memory and kernel argument tables are one cached arena per device.  Calls may be issued on
  * different streams: every call makes its stream wait (an event, no host synchronisation) for the last launch of the
- * previous call that used the arena, so the GPU work of two library calls on one device never overlaps.  Calls from
- * several host threads on one device must still be serialised by the caller (the event is recorded when a call
- * returns; a second thread that enters in between would build its tables in the same arena).  jolt_decompress_static
- * has a scratch array of its own and the rules stated there.
+ * previous call on the device, so the GPU work of two library calls on one device never overlaps.  (Decodes that follow one
+ * another on the default stream are in order as they are; the next call on another stream, whatever handle it is for, waits
+ * for them.)  Calls from several host threads on one device must still be serialised by the caller (the event is
+ * recorded when a call returns; a second thread that enters in between would build its tables in the same arena).
+ * jolt_decompress_static has a scratch array of its own and the rules stated there.
  */
 #ifndef JOLT_H
 #define JOLT_H

@@ -134,22 +134,49 @@ static int ws_reserve(int dev, size_t bytes, void **out) {
   return JOLT_OK;
 }
 
-// The workspace and the argument-table arena are shared by every call on a device.  A call makes its stream wait for
-// the last launch of the previous call that used them (whatever stream that ran on) and leaves an event behind.
-static cudaEvent_t g_arena_ev[64] = {};
-static cudaEvent_t g_default_ev[64] = {};       // calls on the default stream that left no event in g_arena_ev (handle_acquire)
+// The workspace and the argument-table arena are shared by every call on a device.  A call makes its stream wait for the last
+// launch of the previous call (whatever stream that ran on) and leaves an event behind.  A call on the default stream that
+// follows one there, and uses nothing of the shared memory, needs neither (in_default_order): it is only noted, and the next call
+// on another stream waits for the default stream by an event of its own -- the arena's may hold work that the default
+// stream has not waited for.
+struct Arena {
+  cudaEvent_t ev = nullptr, default_ev = nullptr;
+  bool on_default = true;        // ev, once recorded, was recorded on the default stream
+  bool noted = false;            // calls on the default stream since then that left no event
+};
+static Arena g_arena[64];        // under g_ws_mu
+static cudaError_t order_after(cudaEvent_t &ev, cudaStream_t first, cudaStream_t then) {
+  cudaError_t e = ev ? cudaSuccess : cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(ev, first);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(then, ev, 0);
+  return e;
+}
 static int arena_acquire(int dev, cudaStream_t st) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
-  if (!g_arena_ev[dev]) {
-    if (cudaEventCreateWithFlags(&g_arena_ev[dev], cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); g_arena_ev[dev] = nullptr; return fail(JOLT_ECUDA, "event"); }
-    return JOLT_OK;        // first use: nothing to wait for
-  }
-  if (cudaStreamWaitEvent(st, g_arena_ev[dev], 0) != cudaSuccess) { cudaGetLastError(); return fail(JOLT_ECUDA, "cudaStreamWaitEvent"); }
+  Arena &a = g_arena[dev];
+  cudaError_t e = cudaSuccess;
+  if (!a.ev) e = cudaEventCreateWithFlags(&a.ev, cudaEventDisableTiming);        // first use: nothing to wait for
+  else e = cudaStreamWaitEvent(st, a.ev, 0);
+  if (e == cudaSuccess && st && a.noted) e = order_after(a.default_ev, nullptr, st);
+  if (e != cudaSuccess) { cudaGetLastError(); return fail(JOLT_ECUDA, "order of the calls: %s", cudaGetErrorString(e)); }
   return JOLT_OK;
 }
 static void arena_release(int dev, cudaStream_t st) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
-  if (g_arena_ev[dev]) { if (cudaEventRecord(g_arena_ev[dev], st) != cudaSuccess) cudaGetLastError(); }
+  Arena &a = g_arena[dev];
+  if (!a.ev) return;
+  if (cudaEventRecord(a.ev, st) != cudaSuccess) { cudaGetLastError(); return; }
+  a.on_default = st == nullptr;
+  a.noted = false;
+}
+// The previous call was on the default stream as well: a call there is behind it without an event.
+static bool in_default_order(int dev) {
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  return g_arena[dev].on_default;
+}
+static void note_default(int dev) {
+  std::lock_guard<std::mutex> lk(g_ws_mu);
+  g_arena[dev].noted = true;
 }
 
 struct Bump {
@@ -332,7 +359,6 @@ struct jolt_handle {
   int64_t stored_bytes = 0;
   bool subspace = false;     // token factors came from the converged block iteration (exact mode, large T)
   int *d_status = nullptr;   // 4 words per cell, written by the decode kernels of the last call on this handle (jolt_check_status): epoch << 8 | bits
-  mutable std::atomic<bool> unreleased{false};  // a call on the default stream since the last that left the arena's event behind
   mutable cudaStream_t last_stream = nullptr;   // stream of the last call that read the handle's buffers (jolt_free orders after it)
   // The tail of the same device allocation (not part of the stored bytes or of a serialised image): the status words, the
   // projected cores P_h = fp16(G_h U_F^T) of the cells that need them (CellStore::P16), the descriptors
@@ -1842,21 +1868,6 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   return JOLT_OK;
 }
 
-// arena_acquire for a call that reads a handle: also after the calls on the default stream that left no event behind.  They get
-// an event of their own, recorded and waited for in one step: the arena's event holds the last user of the shared memory,
-// which may be on a stream that the default stream has not waited for.
-static int handle_acquire(const jolt_handle *H, int dev, cudaStream_t st) {
-  if (st && H->unreleased.exchange(false)) {
-    std::lock_guard<std::mutex> lk(g_ws_mu);
-    cudaEvent_t &ev = g_default_ev[dev];
-    cudaError_t e = ev ? cudaSuccess : cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(ev, nullptr);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
-    if (e != cudaSuccess) { cudaGetLastError(); H->unreleased = true; return fail(JOLT_ECUDA, "event: %s", cudaGetErrorString(e)); }
-  }
-  return arena_acquire(dev, st);
-}
-
 static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kout, void *Vout, const jolt_rope *rope,
                            void *stream) {
   if (!H || !Kout || !Vout) return fail(JOLT_EINVAL, "null argument");
@@ -1890,17 +1901,17 @@ static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kou
   if (fast && H->dec.end[2] == nc && H->dec.end[1] == nc && !rope && (g_fast.load() & 128)) epoch = H->epoch.fetch_add(1) + 1;
   if (epoch >= 1 << 22) { H->epoch = 1; epoch = 0; }                               // the epochs start again
   if (epoch && L->mem_space != JOLT_MEM_HOST) {
-    // Calls on the default stream that follow one another there are in order as it is; the event that orders the users of the
-    // shared memory is left out until another stream comes, and the kernel takes its own times.
-    const bool in_order = !st && !H->last_stream && g_dec_tail_pct.load() == 0;
-    if (!in_order && (rc = handle_acquire(H, dev, st))) return rc;
+    // Calls on the default stream that follow one another there are in order as it is; the event is left out until another
+    // stream comes, and the kernel takes its own times.
+    const bool in_order = !st && in_default_order(dev) && g_dec_tail_pct.load() == 0;
+    if (!in_order && (rc = arena_acquire(dev, st))) return rc;
     H->last_stream = st;
     H->status_epoch = epoch;
     unsigned long long *stamps = in_order ? stamp_slot(dev) : nullptr;
     if (stamps) g_timer.begin_stamped(dev, stamps); else g_timer.begin(st);
     if ((rc = launch_decode_tc(H, L, (char *)Kout, (char *)Vout, nullptr, stamps, dev, st))) return rc;
     if (!stamps) g_timer.mark(ST_DROWS, st);
-    if (in_order) H->unreleased = true; else arena_release(dev, st);
+    if (in_order) note_default(dev); else arena_release(dev, st);
     return JOLT_OK;
   }
   std::vector<CellWork> ws(nc);
@@ -1999,7 +2010,7 @@ static int decompress_impl(const jolt_handle *H, const jolt_layout *L, void *Kou
   lap("program");
   void *d_tab = nullptr;
   if (!P.host.empty() && (rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
-  if ((rc = handle_acquire(H, dev, st))) return rc;
+  if ((rc = arena_acquire(dev, st))) return rc;
   H->last_stream = st;
   g_timer.begin(st);
   if (epoch == 0) CU(cudaMemsetAsync(d_status, 0, sizeof(int) * 4 * nc, st));
@@ -2213,7 +2224,7 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
   });
   void *d_tab = nullptr;
   if (!by_arg && (rc = tab_reserve(dev, P.host.size() + 256, &d_tab))) return rc;
-  if ((rc = handle_acquire(H, dev, st))) return rc;
+  if ((rc = arena_acquire(dev, st))) return rc;
   H->last_stream = st;
   g_timer.begin(st);
   if ((rc = run_program(P, (char *)d_tab, st))) return rc;

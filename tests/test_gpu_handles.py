@@ -164,6 +164,38 @@ def test_call_on_a_third_stream_waits_for_the_second(B):
     h1.free(); h2.free()
 
 
+def test_calls_on_other_handles_come_after_default_stream_decodes_and_before_them(B):
+    """Short decodes on the default stream leave no event behind, but a call on another stream comes after them whatever handle
+    it reads or makes, and they come after the calls on other streams before them."""
+    K, V = _cache(2, 4, 1024, 12)
+    gs, plan = [0, 2], [(32, 128, 4), (16, 64, 2)]
+    opts = B.default_options(seed=1, power_iters=0)
+    h1, h2 = B.jolt_compress(K, V, gs, plan, opts), B.jolt_compress(V, K, gs, plan, opts)
+    Q = torch.randn(2, 4, 4, 128, generator=torch.Generator().manual_seed(1)).cuda()
+    o = torch.empty_like(K), torch.empty_like(V)
+    B.jolt_attend(h2, Q)
+    B.jolt_decompress(h2, *o, gs)
+    torch.cuda.synchronize()
+    C, default = torch.cuda.Stream(), torch.cuda.default_stream()
+    for first, then in ((default, C), (C, default)):
+        for call in ("attend", "decode"):
+            torch.cuda.synchronize()
+            B.jolt_decompress(h1, *o, gs)
+            torch.cuda.synchronize()
+            _held(first)
+            B.jolt_decompress(h1, *o, gs, stream=None if first == default else C)
+            st = None if then == default else C
+            if call == "attend":
+                B.jolt_attend(h2, Q, stream=st)
+            else:
+                B.jolt_decompress(h2, *o, gs, stream=st)
+            done = _after(then)
+            time.sleep(0.03)
+            assert not done.query(), (call, then)
+    torch.cuda.synchronize()
+    h1.free(); h2.free()
+
+
 @pytest.mark.parametrize("bits", [(0, 1), (2, 3), (4, 8)])
 @pytest.mark.parametrize("T,tail", [(128, 0), (640, 0), (384, 60)])
 def test_rotated_keys_of_the_persistent_kernel(B, bits, T, tail):
