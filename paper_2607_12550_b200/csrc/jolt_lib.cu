@@ -118,17 +118,87 @@ void StageTimer::finish_stamped() {
   if (t[1] > t[0]) ms[kStampedStage] = (float)(t[1] - t[0]) * 1e-6f;
 }
 
+// Device memory of freed handles, kept for the next ones.  The stream-ordered pool alone does not serve a program that
+// compresses caches one after another: blocks of neighbouring sizes whose release is still in flight do not fit, and it
+// maps new memory instead (2 - 12 ms a call measured).  At most kMemCacheBlocks blocks per device stay here, each with an
+// event behind the last call that used it; a block is only handed out for a size of at least 7/8 of its own; the rest
+// goes back to the pool.  Blocks and pool go back to the driver with jolt_release_workspace, or when an allocation fails.
+struct MemBlock { void *p = nullptr; size_t bytes = 0; cudaEvent_t ev = nullptr; };
+constexpr int kMemCacheBlocks = 3;
+static std::mutex g_mem_mu;
+static std::vector<MemBlock> g_mem_cache[64];
+
+static bool mem_cache_take(int dev, size_t bytes, cudaStream_t st, MemBlock &out) {
+  std::lock_guard<std::mutex> lk(g_mem_mu);
+  auto &v = g_mem_cache[dev];
+  int best = -1;
+  for (int i = 0; i < (int)v.size(); ++i)
+    if (v[i].bytes >= bytes && bytes >= v[i].bytes / 8 * 7 && (best < 0 || v[i].bytes < v[best].bytes)) best = i;
+  if (best < 0) return false;
+  if (cudaStreamWaitEvent(st, v[best].ev, 0) != cudaSuccess) { cudaGetLastError(); return false; }
+  out = v[best];
+  v.erase(v.begin() + best);
+  return true;
+}
+
+static void mem_block_release(const MemBlock &b) {                     // back to the stream-ordered pool
+  cudaEventSynchronize(b.ev);
+  cudaEventDestroy(b.ev);
+  if (cudaFreeAsync(b.p, 0) != cudaSuccess) cudaGetLastError();
+}
+
+// `last`: the stream of the last call that used the block (if it no longer exists, the device is waited for)
+static void mem_cache_put(int dev, MemBlock b, cudaStream_t last) {
+  if (!b.ev && cudaEventCreateWithFlags(&b.ev, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    cudaDeviceSynchronize();
+    if (cudaFreeAsync(b.p, 0) != cudaSuccess) cudaGetLastError();
+    return;
+  }
+  if (cudaEventRecord(b.ev, last) != cudaSuccess) { cudaGetLastError(); cudaDeviceSynchronize(); cudaEventRecord(b.ev, 0); }
+  MemBlock old;
+  {
+    std::lock_guard<std::mutex> lk(g_mem_mu);
+    auto &v = g_mem_cache[dev];
+    v.push_back(b);
+    if ((int)v.size() > kMemCacheBlocks) { old = v.front(); v.erase(v.begin()); }
+  }
+  if (old.p) mem_block_release(old);
+}
+
+// all of it, and what the stream-ordered pool holds on to, to the driver
+static void give_back_kept_memory(int dev) {
+  std::vector<MemBlock> v;
+  { std::lock_guard<std::mutex> lk(g_mem_mu); v.swap(g_mem_cache[dev]); }
+  for (auto &b : v) mem_block_release(b);
+  cudaDeviceSynchronize();                 // what was freed in stream order is free
+  cudaMemPool_t pool;
+  if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+}
+
+// cudaMalloc that gives the kept memory back before it gives up
+static cudaError_t device_malloc(int dev, void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();
+  give_back_kept_memory(dev);
+  if ((e = cudaMalloc(p, bytes)) != cudaSuccess) { cudaGetLastError(); *p = nullptr; }
+  return e;
+}
+
 static int ws_reserve(int dev, size_t bytes, void **out) {
   std::lock_guard<std::mutex> lk(g_ws_mu);
   Workspace &w = g_ws[dev];
   if (w.cap < bytes) {
     if (w.base) { cudaDeviceSynchronize(); cudaFree(w.base); w.base = nullptr; w.cap = 0; }
     const size_t want = bytes + (bytes >> 3);
-    if (cudaMalloc(&w.base, want) != cudaSuccess) {
+    if (cudaMalloc(&w.base, want) == cudaSuccess) w.cap = want;
+    else {
       cudaGetLastError();
-      if (cudaMalloc(&w.base, bytes) != cudaSuccess) { cudaGetLastError(); w.base = nullptr; return fail(JOLT_ENOMEM, "workspace of %zu bytes", bytes); }
+      if (device_malloc(dev, &w.base, bytes) != cudaSuccess) return fail(JOLT_ENOMEM, "workspace of %zu bytes", bytes);
       w.cap = bytes;
-    } else w.cap = want;
+    }
   }
   *out = w.base;
   return JOLT_OK;
@@ -1213,7 +1283,7 @@ static int tab_reserve(int dev, size_t bytes, void **out) {
   if (w.cap < bytes) {
     if (w.base) { cudaDeviceSynchronize(); cudaFree(w.base); w.base = nullptr; w.cap = 0; }
     const size_t want = std::max<size_t>(bytes * 2, 1 << 20);
-    if (cudaMalloc(&w.base, want) != cudaSuccess) { cudaGetLastError(); return fail(JOLT_ENOMEM, "task tables of %zu bytes", want); }
+    if (device_malloc(dev, &w.base, want) != cudaSuccess) return fail(JOLT_ENOMEM, "task tables of %zu bytes", want);
     w.cap = want;
   }
   *out = w.base;
@@ -1375,60 +1445,6 @@ struct GroupRun {
   }
 };
 
-// Device memory of freed handles, kept for the next ones.  The stream-ordered pool alone does not serve a program that
-// compresses caches one after another: blocks of neighbouring sizes whose release is still in flight do not fit, and it
-// maps new memory instead (2 - 12 ms a call measured).  At most kMemCacheBlocks blocks per device stay here, each with an
-// event behind the last call that used it; a block is only handed out for a size of at least 7/8 of its own; the rest
-// goes back to the pool, all of it with jolt_release_workspace.
-struct MemBlock { void *p = nullptr; size_t bytes = 0; cudaEvent_t ev = nullptr; };
-constexpr int kMemCacheBlocks = 3;
-static std::mutex g_mem_mu;
-static std::vector<MemBlock> g_mem_cache[64];
-
-static bool mem_cache_take(int dev, size_t bytes, cudaStream_t st, MemBlock &out) {
-  std::lock_guard<std::mutex> lk(g_mem_mu);
-  auto &v = g_mem_cache[dev];
-  int best = -1;
-  for (int i = 0; i < (int)v.size(); ++i)
-    if (v[i].bytes >= bytes && bytes >= v[i].bytes / 8 * 7 && (best < 0 || v[i].bytes < v[best].bytes)) best = i;
-  if (best < 0) return false;
-  if (cudaStreamWaitEvent(st, v[best].ev, 0) != cudaSuccess) { cudaGetLastError(); return false; }
-  out = v[best];
-  v.erase(v.begin() + best);
-  return true;
-}
-
-static void mem_block_release(const MemBlock &b) {                     // back to the stream-ordered pool
-  cudaEventSynchronize(b.ev);
-  cudaEventDestroy(b.ev);
-  if (cudaFreeAsync(b.p, 0) != cudaSuccess) cudaGetLastError();
-}
-
-// `last`: the stream of the last call that used the block (if it no longer exists, the device is waited for)
-static void mem_cache_put(int dev, MemBlock b, cudaStream_t last) {
-  if (!b.ev && cudaEventCreateWithFlags(&b.ev, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    cudaDeviceSynchronize();
-    if (cudaFreeAsync(b.p, 0) != cudaSuccess) cudaGetLastError();
-    return;
-  }
-  if (cudaEventRecord(b.ev, last) != cudaSuccess) { cudaGetLastError(); cudaDeviceSynchronize(); cudaEventRecord(b.ev, 0); }
-  MemBlock old;
-  {
-    std::lock_guard<std::mutex> lk(g_mem_mu);
-    auto &v = g_mem_cache[dev];
-    v.push_back(b);
-    if ((int)v.size() > kMemCacheBlocks) { old = v.front(); v.erase(v.begin()); }
-  }
-  if (old.p) mem_block_release(old);
-}
-
-static void mem_cache_clear(int dev) {
-  std::vector<MemBlock> v;
-  { std::lock_guard<std::mutex> lk(g_mem_mu); v.swap(g_mem_cache[dev]); }
-  for (auto &b : v) mem_block_release(b);
-}
-
 // Allocates the handle's device memory: the stored arrays (payload) and, behind them, the parts that are not stored.  A cell
 // whose feature factor is exactly the identity (`identity_uf[c]`: r_f = d, factors not injected) needs no projected
 // core of its own: P = G there.  One stream-ordered allocation: cudaMalloc and cudaFree of the separate parts took up to
@@ -1463,7 +1479,7 @@ static int alloc_handle_memory(jolt_handle &H, size_t payload, const std::vector
         cudaError_t e = cudaMallocAsync(&H.blob, want, st);
         if (e != cudaSuccess) {           // out of memory: what is kept for later handles may be enough
           cudaGetLastError();
-          mem_cache_clear(H.device);
+          give_back_kept_memory(H.device);
           e = cudaMallocAsync(&H.blob, want, st);
         }
         if (e != cudaSuccess) { cudaGetLastError(); H.blob = nullptr; return fail(JOLT_ENOMEM, "compressed cache of %zu bytes", want); }
@@ -2678,9 +2694,8 @@ extern "C" int jolt_signs_host(uint64_t seed, int32_t cell, float out[128]) {
 extern "C" int jolt_release_workspace(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return JOLT_OK; }
-  mem_cache_clear(dev);
+  give_back_kept_memory(dev);
   std::lock_guard<std::mutex> lk(g_ws_mu);
-  cudaDeviceSynchronize();
   if (g_ws[dev].base) { cudaFree(g_ws[dev].base); g_ws[dev] = Workspace(); }
   if (g_tab[dev].base) { cudaFree(g_tab[dev].base); g_tab[dev] = Workspace(); }
   if (g_stamps[dev]) { cudaFree(g_stamps[dev]); g_stamps[dev] = nullptr; }

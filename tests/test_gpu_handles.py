@@ -196,6 +196,35 @@ def test_calls_on_other_handles_come_after_default_stream_decodes_and_before_the
     h1.free(); h2.free()
 
 
+def _free_bytes():
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_kept_memory_is_given_back(B):
+    """Blocks of freed handles are kept for the next ones, but not against the workspace: a call whose workspace only fits
+    without them succeeds, and jolt_release_workspace returns everything to the driver."""
+    K = torch.randn(4, 8, 32768, 128, device="cuda", dtype=torch.float16)
+    V, gs, opts = K.flip(0).contiguous(), [0, 4], B.default_options(seed=1)
+    Ko, Vo = torch.empty(K.shape, dtype=K.dtype), torch.empty(V.shape, dtype=V.dtype)       # host: the call stages 2 x 268 MB
+    small = B.jolt_compress(K[:, :, :128], V[:, :, :128], gs, [(0, 0, 8)] * 2, opts)        # what the library allocates once
+    B.jolt_decompress(small, K[:, :, :128], V[:, :, :128], gs)
+    small.free()
+    B.release_workspace()
+    base = _free_bytes()
+    hs = [B.jolt_compress(K, V, gs, [(0, 0, 8)] * 2, opts) for _ in range(3)]               # 285 MB each
+    hs.pop().free()
+    hs.pop().free()
+    filler = torch.empty(_free_bytes() - (200 << 20), dtype=torch.uint8, device="cuda")
+    B.jolt_decompress(hs[0], Ko, Vo, gs)
+    del filler
+    assert float((Ko.cuda().float() - K.float()).norm() / K.float().norm()) <= 1e-2
+    hs[0].free()
+    B.release_workspace()
+    assert _free_bytes() >= base - (8 << 20)
+
+
 @pytest.mark.parametrize("bits", [(0, 1), (2, 3), (4, 8)])
 @pytest.mark.parametrize("T,tail", [(128, 0), (640, 0), (384, 60)])
 def test_rotated_keys_of_the_persistent_kernel(B, bits, T, tail):
