@@ -116,9 +116,9 @@ def make_layout(K: torch.Tensor, group_start: Sequence[int], V: torch.Tensor | N
 
     The C ABI describes K and V by ONE layout: when V is given it must match K in shape, strides, dtype and device."""
     shape, stride, dtype = K.shape, K.stride(), K.dtype
+    assert len(shape) == 4 and stride[3] == 1
     n_layers, n_heads, T, d = shape
-    s_layer, s_head, s_token, s_feature = stride
-    assert s_feature == 1
+    s_layer, s_head, s_token, _ = stride
     if V is not None and (V.shape != shape or V.stride() != stride or V.dtype != dtype or V.device != K.device):
         raise ValueError("K and V must share shape, strides, dtype and device (one jolt_layout describes both)")
     n = len(group_start)

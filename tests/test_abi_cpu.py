@@ -41,6 +41,13 @@ def _cpu_cache(L=2, nh=2, T=128, dtype=torch.float16):
     return K, K.clone()
 
 
+def test_layout_takes_four_dimensions_of_unit_feature_stride(B):
+    K, _ = _cpu_cache()
+    for bad in (K[0], K[None], K.transpose(2, 3)):
+        with pytest.raises(AssertionError):
+            B.make_layout(bad, [0, 2])
+
+
 def test_argument_validation_needs_no_gpu(B):
     K, V = _cpu_cache()
     opts = B.default_options()
