@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <mutex>
 #include <cooperative_groups.h>
+#include "device_once.h"
 #include "small_solvers.cuh"
 
 namespace jolt {
@@ -335,8 +336,8 @@ __global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(kCholThre
 }
 
 inline void chol_cluster_launch(const CholTask *d_tasks, int count, int max_n, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] { cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024)); });
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024)); });
   gram_sum_kernel<<<dim3((max_n + kGramRedRows - 1) / kGramRedRows, count), 32 * kGramRedRows, 0, s>>>(d_tasks);
   chol_cluster_kernel<<<dim3(kCholCluster, count), kCholThreads, chol_smem_bytes_cl(max_n), s>>>(d_tasks);
 }

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include <cooperative_groups.h>
+#include "device_once.h"
 #include "small_solvers.cuh"
 
 namespace jolt {
@@ -894,8 +895,8 @@ __global__ void __launch_bounds__(kTdBackThreads) td_back_kernel(const TdTask *_
 
 // ---------------------------------------------------------------------------------------------- host
 inline void td_opt_in() {
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static DeviceOnce once;
+  once([] {
     const int lim = (int)(kSmemOptIn - 1024);
     cudaFuncSetAttribute(td_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(td_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);

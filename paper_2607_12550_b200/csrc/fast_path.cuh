@@ -70,8 +70,8 @@ inline void bb_split(int total_heads, int n_tiles, int &tiles_per_item, int &ite
 
 inline void add_backbone_tc(Program &P, int stage, const std::vector<tc::BBCell> &cells, uint64_t seed) {
   if (cells.empty()) return;
-  static std::once_flag once;
-  std::call_once(once, [] { cudaFuncSetAttribute(tc::backbone_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::BB_SMEM_BYTES); });
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(tc::backbone_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::BB_SMEM_BYTES); });
   int gx = 0;
   for (auto &c : cells) gx = std::max(gx, c.m * c.items_per_head);
   const size_t off = P.push(cells);
@@ -96,8 +96,8 @@ inline void fill_bb_common(tc::BBCell &b, const CellStore &cs, int *status) {
 // the persistent kernel is off.
 inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, cudaStream_t s) {
   using LY = tc::DecLayout;
-  static std::once_flag once;
-  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
   tc::DecIArgs a;
   memset(&a, 0, sizeof a);
   a.out = out; a.cells = (const tc::BBCell *)H->d_dec + first; a.rope = rope; a.seed = H->seed;
@@ -116,8 +116,8 @@ inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc
 template <bool TMA_ONLY, unsigned BITMASK, bool ROPE = false>
 inline void launch_decode_p(const tc::DecPArgs &a, int grid, cudaStream_t s) {
   using LY = tc::DecLayout;
-  static std::once_flag once;
-  std::call_once(once, [] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
   tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
 }
 
@@ -210,11 +210,8 @@ inline void launch_tc_gemm(Program &P, int stage, std::vector<tc::GemmCell> &cel
   }
   int n_stages = std::min(8, (int)((tc::GM_SMEM_LIMIT - 1536) / max_stage));
   const size_t smem = (size_t)n_stages * max_stage + 1024 + 512;
-  static size_t attr[3] = {0, 0, 0};
-  if (attr[MODE] < smem) {
-    cudaFuncSetAttribute(tc::tc_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::GM_SMEM_LIMIT);
-    attr[MODE] = tc::GM_SMEM_LIMIT;
-  }
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(tc::tc_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::GM_SMEM_LIMIT); });
   const size_t off = P.push(cells);
   const int n = (int)cells.size();
   P.add(stage, [=](char *dev_t, cudaStream_t s) {
@@ -235,11 +232,8 @@ inline void launch_tc_gemm2(Program &P, int stage, std::vector<tc::Gemm2Cell> &c
   }
   const int n_stages = std::min(8, (int)((tc::GM_SMEM_LIMIT - 1536) / max_stage));
   const size_t smem = (size_t)n_stages * max_stage + 1024 + 512;
-  static bool attr[3] = {false, false, false};
-  if (!attr[MODE]) {
-    cudaFuncSetAttribute(tc::tc_gemm2_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::GM_SMEM_LIMIT);
-    attr[MODE] = true;
-  }
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(tc::tc_gemm2_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::GM_SMEM_LIMIT); });
   const size_t off = P.push(cells);
   const int n = (int)cells.size();
   P.add(stage, [=](char *dev_t, cudaStream_t s) {
@@ -497,8 +491,8 @@ constexpr double kOrthRedoRel = 5e-7;      // about eight times the error of a s
 inline void add_orth_wide(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side, int passes,
                           bool want_fp32) {
   if (idx.empty()) return;
-  static std::once_flag once;
-  std::call_once(once, [] {
+  static DeviceOnce once;
+  once([] {
     cudaFuncSetAttribute(tc::orthw_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OW_GRAM_SMEM);
     cudaFuncSetAttribute(tc::orthw_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OW_APPLY_SMEM);
   });
@@ -573,13 +567,12 @@ inline void add_orth_wide(Program &P, int stage, std::vector<CellWork> &ws, cons
 inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side, int passes,
                         bool want_fp32) {
   if (idx.empty()) return;
-  static bool attr_done = false;
-  if (!attr_done) {
+  static DeviceOnce once;
+  once([] {
     cudaFuncSetAttribute(tc::orth_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OR_SMEM_LIMIT);
     cudaFuncSetAttribute(tc::orth_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::OR_SMEM_LIMIT);
     cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN));
-    attr_done = true;
-  }
+  });
   add_orth_split(P, stage, ws, idx, token_side);
   std::vector<tc::OrthCell> oc, oc_last;      // the fp32 rows of Q are only written by the last pass, and only if someone reads them
   std::vector<tc::CholInvTask> ci;

@@ -16,6 +16,7 @@
 #include <cuda.h>
 #include "allocator.h"
 #include "common.cuh"
+#include "device_once.h"
 #include "rowquant.cuh"
 #include "simt_gemm.cuh"
 #include "small_solvers.cuh"
@@ -597,8 +598,8 @@ void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sw
     int cmn = 0;
     for (auto &c : cfs) cmn = std::max(cmn, c.k);
     const size_t cshm = tc::cholinv_smem_bytes(cmn);
-    static std::once_flag once;
-    std::call_once(once, [] { cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN)); });
+    static DeviceOnce once;
+    once([] { cudaFuncSetAttribute(tc::cholinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::cholinv_smem_bytes(tc::kCholInvMaxN)); });
     P.add(stage, [=](char *dev, cudaStream_t s) { tc::cholinv_kernel<<<n, tc::kCholInvThreads, cshm, s>>>((const tc::CholInvTask *)(dev + off)); LAUNCHED(); });
   }
   if (!cf.empty()) {
@@ -607,13 +608,13 @@ void add_eig(Program &P, int stage, const std::vector<EigTask> &tasks, int bj_sw
     int cmn = 0;
     for (auto &c : cf) cmn = std::max(cmn, c.n);
     const size_t cshm = std::max(chol_factor_smem_bytes(kCholFactorSmemN), chol_factor_smem_bytes(cmn));
-    static std::once_flag once;
-    std::call_once(once, [] { cudaFuncSetAttribute(chol_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 2048)); });
+    static DeviceOnce once;
+    once([] { cudaFuncSetAttribute(chol_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 2048)); });
     P.add(stage, [=](char *dev, cudaStream_t s) { chol_factor_kernel<<<n, kCholFactorThreads, cshm, s>>>((const CholFactorTask *)(dev + off)); LAUNCHED(); });
   }
   if (!cj.empty()) {
-    static std::once_flag once;
-    std::call_once(once, [] { cj_opt_in_smem(); });
+    static DeviceOnce once;
+    once([] { cj_opt_in_smem(); });
     int mn = 0;
     for (auto &c : cj) mn = std::max(mn, c.n);
     const int nr = cj_rows_per_lane(mn), nt = (int)cj.size();
@@ -863,14 +864,13 @@ void add_orth(Program &P, int stage, std::vector<CellWork> &ws, bool token_side,
       max_k[cls] = std::max(max_k[cls], k);
     }
     add_tall_gram(P, stage, tg);
-    static bool attr_done = false;
-    if (!attr_done) {
+    static DeviceOnce once;
+    once([] {
       cudaFuncSetAttribute(cholesky_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chol_smem_bytes(kCholSmemMaxN));
       cudaFuncSetAttribute(trsm_rows_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024));
       cudaFuncSetAttribute(trsm_rows_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024));
       cudaFuncSetAttribute(trsm_rows_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemOptIn - 1024));
-      attr_done = true;
-    }
+    });
     for (int cls = 0; cls < 2; ++cls) {
       if (chs[cls].empty()) continue;
       const size_t o1 = P.push(chs[cls]), o2 = P.push(tj[cls]);
@@ -1502,8 +1502,8 @@ static int upload_decode_table(jolt_handle &H, cudaStream_t st) {
 }
 
 static void launch_project_cores(const ProjJob *d_jobs, int n, int max_rows, int max_rf, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) { cudaFuncSetAttribute(project_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 2); attr = true; }
+  static DeviceOnce once;
+  once([] { cudaFuncSetAttribute(project_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 2); });
   project_core_kernel<<<dim3((max_rows + 31) / 32, n), 128, (size_t)128 * max_rf * sizeof(__half), s>>>(d_jobs);
   LAUNCHED();
 }
@@ -2188,8 +2188,8 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
     LAUNCHED();
     const dim3 grid(n_chunks, m_max, ng);
     if (mma) {
-      static std::once_flag once;
-      std::call_once(once, [] {
+      static DeviceOnce once;
+      once([] {
         auto allow = [](auto k, int nq) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_stream_smem(nq)); };
         allow(attend_stream_kernel<4, 4, true>, 4); allow(attend_stream_kernel<4, 1, true>, 4); allow(attend_stream_kernel<8, 4, true>, 8); allow(attend_stream_kernel<8, 1, true>, 8);
         allow(attend_stream_kernel<4, 4, false>, 4); allow(attend_stream_kernel<4, 1, false>, 4); allow(attend_stream_kernel<8, 4, false>, 8); allow(attend_stream_kernel<8, 1, false>, 8);

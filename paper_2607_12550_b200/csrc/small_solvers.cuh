@@ -3,6 +3,7 @@
 // CholeskyQR2: tall Gram (fp64), Cholesky with dead-pivot deflation (fp64), row-wise triangular solve (fp32).
 #pragma once
 #include "common.cuh"
+#include "device_once.h"
 
 namespace jolt {
 
