@@ -309,7 +309,7 @@ inline void add_tok_tc(Program &P, int stage, std::vector<CellWork> &ws, const s
       if (src[i] == 2) { in = w.ufI ? w.Z : w.W; se = ilog2_floor((long long)c.N) / 2; }
       tc::SplitJob j;
       j.in = in; j.hi = w.Bhi; j.lo = w.Blo; j.batch = c.m; j.rows = kD; j.cols = c.k; j.ld_in = c.k;
-      j.kp = w.kp; j.scale_exp = se; j.absmax = nullptr;
+      j.kp = w.kp; j.scale_exp = se; j.absmax = nullptr; j.top = 0;
       sp.push_back(j);
     }
     std::vector<std::pair<int, int>> ch;
@@ -368,7 +368,7 @@ inline void add_feat_tc(Program &P, int stage, std::vector<CellWork> &ws) {
     const int se = ilog2_floor(c.T) / 2;
     if (w.split_ready != 1) {      // else the triangular solve of orth(S) has written the operand already
       tc::SplitJob j;
-      j.in = w.S; j.hi = w.Bhi; j.lo = w.Blo; j.batch = 1; j.rows = c.T; j.cols = c.k; j.ld_in = c.k; j.kp = w.kp; j.scale_exp = se; j.absmax = nullptr;
+      j.in = w.S; j.hi = w.Bhi; j.lo = w.Blo; j.batch = 1; j.rows = c.T; j.cols = c.k; j.ld_in = c.k; j.kp = w.kp; j.scale_exp = se; j.absmax = nullptr; j.top = 0;
       sp.push_back(j);
     }
     w.split_ready = 0;
@@ -461,7 +461,11 @@ inline bool orth_tc_ok(const CellWork &w) {
 inline bool orth_is_wide(const CellWork &w) { return w.c.k > tc::OR_MAX_K || w.kp > tc::OR_MAX_KP; }
 
 // The sweep left the raw basis as fp32 rows: measure its magnitude (unless the sweep's epilogue did), split it into the
-// operand layout.
+// operand layout.  After a power iteration the columns are graded like the spectrum: with the largest entry below 1 the lo part of
+// an entry 1e-4 of it is a subnormal of three or four bits, and the weak directions of the span were lost with them.
+// Wide sketches, which reach furthest down the spectrum, use all of fp16's range (kOrthWideTop).  Distance of the span from an
+// fp64 one, key caches: 7.1e-4 -> 1.04e-4 at k = 160, 1.3e-2 -> 5.0e-4 at k = 522 (fp64 Gram and CUDA-core solve: 1.05e-4, 5.0e-4).
+constexpr int kOrthWideTop = 15;
 inline void add_orth_split(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side) {
   std::vector<tc::AbsMaxJob> am;
   std::vector<tc::SplitJob> sp;
@@ -475,7 +479,7 @@ inline void add_orth_split(Program &P, int stage, std::vector<CellWork> &ws, con
     w.absmax_ready = false;
     tc::SplitJob j;
     j.in = src; j.hi = w.Bhi; j.lo = w.Blo; j.batch = panels; j.rows = rpp; j.cols = c.k; j.ld_in = c.k; j.kp = w.kp; j.scale_exp = 0;
-    j.absmax = slot;
+    j.absmax = slot; j.top = orth_is_wide(w) ? kOrthWideTop : 0;
     sp.push_back(j);
   }
   const size_t o_am = P.push(am), o_sp = P.push(sp);

@@ -88,6 +88,60 @@ def test_wide_choleskyqr_matches_cuda_core_path(B, r_t):
         assert np.linalg.norm(UT[c][:, :n] @ UT[c][:, :n].T - UT2[c][:, :n] @ UT2[c][:, :n].T) <= 1e-3
 
 
+def _graded_cache(T, m, seed):
+    """A key cache (decaying terms, four outlier channels) and a value cache, as the synthetic caches are made."""
+    g = torch.Generator().manual_seed(seed)
+    out = []
+    for alpha, sigma in ((1.0, 0.05), (0.6, 0.1)):
+        n = 256
+        q, _ = torch.linalg.qr(torch.randn(128, 128, generator=g, dtype=torch.float64))
+        q = (q * 128 ** 0.5)[:, torch.arange(n) % 128]
+        w = torch.arange(1, n + 1, dtype=torch.float64) ** -alpha
+        p = torch.randn(T, n, generator=g, dtype=torch.float64)
+        a = (1.0 + 0.1 * torch.randn(m, n, generator=g, dtype=torch.float64)) * w
+        x = (p * a[:, None, :]) @ q.t() + sigma * torch.randn(m, T, 128, generator=g, dtype=torch.float64)
+        if not out:
+            x[:, :, [5, 37, 70, 101]] *= 10.0
+        out.append(x.half().view(1, m, T, 128).cuda())
+    return out
+
+
+def _range_fp64(B, X, cell, seed, k, q):
+    """Basis of the range finder with the library's own sketch, in fp64, in the order of the singular values."""
+    _, m, T, _ = X.shape
+    A = X[0].permute(1, 0, 2).reshape(T, m * 128).double()
+    om = torch.from_numpy(B.sketch_host(seed, cell, 0, m * 128, k).astype(np.float64)).cuda().reshape(m * 128, k)
+    Q = torch.linalg.qr(A @ om)[0]
+    for _ in range(q):
+        Q = torch.linalg.qr(A @ torch.linalg.qr(A.T @ Q)[0])[0]
+    M = Q.T @ A
+    return Q @ torch.linalg.eigh(M @ M.T)[1].flip(1)
+
+
+def _distance(P, R):
+    return max(float((P.T @ P).norm() ** 2 + (R.T @ R).norm() ** 2 - 2 * (P.T @ R).norm() ** 2), 0.0) ** 0.5
+
+
+# the whole sketch is kept (no oversampling), so the span of the factor is the span of the basis: it has to be as close to the
+# fp64 one as with the fp64 Gram and the CUDA-core solve (bit 5 off); what both have is the error of the sweeps
+@pytest.mark.parametrize("T,m,k,q", [(2048, 8, 160, 1), (1024, 8, 272, 2), (2048, 8, 400, 1)])
+def test_wide_basis_is_as_good_as_the_fp64_one(B, T, m, k, q):
+    KV = _graded_cache(T, m, 7)
+    got = []
+    for mask in (255 - 32, 255):
+        prev = B.set_fast_path(mask)
+        try:
+            h = B.jolt_compress(*KV, [0, 1], [(k, 128, 4)] * 2, B.default_options(seed=7, power_iters=q, oversample=0))
+            got.append([torch.from_numpy(h.component(c, 8).reshape(T, k).astype(np.float64)).cuda() for c in (0, 1)])
+            h.free()
+        finally:
+            B.set_fast_path(prev)
+    for c in (0, 1):
+        R = _range_fp64(B, KV[c], c, 7, k, q)
+        for n in (64, k):
+            assert _distance(got[1][c][:, :n], R[:, :n]) <= 1.2 * _distance(got[0][c][:, :n], R[:, :n]), (c, n)
+
+
 # sketch width = cap + 10: portable up to 32, Cholesky in shared memory to 152, in global memory to 288, tridiagonal beyond
 @pytest.mark.parametrize("q_cap", [16, 32, 142, 144, 278, 279, 320])
 def test_probe_values_give_the_portable_plan(B, q_cap):
