@@ -532,6 +532,8 @@ inline void add_orth_wide(Program &P, int stage, std::vector<CellWork> &ws, cons
     o.n_chunks = (steps + tc::OW_GRAM_STEPS - 1) / tc::OW_GRAM_STEPS;
     o.out_exp = ilog2_floor((long long)rpp * panels) / 2;
     o.status = w.status;
+    o.hi = w.Bhi; o.lo = w.Blo; o.unit = w.Gs;      // (the fp64 Gram of the first pass is used up by then)
+    if (want_fp32) w.unit = w.Gs;
     oc.push_back(o);
     o.out32 = want_fp32 ? (token_side ? w.S : w.Z) : nullptr;
     oc_last.push_back(o);
@@ -566,6 +568,10 @@ inline void add_orth_wide(Program &P, int stage, std::vector<CellWork> &ws, cons
       tc::orthw_apply_kernel<<<dim3(max_tiles, n), tc::OW_THREADS, tc::OW_APPLY_SMEM, s>>>((const tc::OrthWCell *)(dev_t + o_app)); LAUNCHED();
     });
   }
+  if (want_fp32)
+    P.add(stage, [=](char *dev_t, cudaStream_t s) {
+      tc::orthw_norms_kernel<<<dim3((max_k + 7) / 8, n), 256, 0, s>>>((const tc::OrthWCell *)(dev_t + o_oc)); LAUNCHED();
+    });
 }
 
 inline void add_orth_tc(Program &P, int stage, std::vector<CellWork> &ws, const std::vector<int> &idx, bool token_side, int passes,

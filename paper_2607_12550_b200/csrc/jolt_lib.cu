@@ -392,6 +392,18 @@ __global__ void __launch_bounds__(128) project_core_kernel(const ProjJob *__rest
   }
 }
 
+// Q D in place of Q (D: the factors that make its columns unit vectors): B B^T -> D B B^T D, and D goes into the rows of the small
+// SVD's vectors, which both the token factor (Q U) and the core (U^T B) are made from.
+struct UnitJob { const double *d; double *BBt; float *U; int k, r; };
+__global__ void unit_gram_kernel(const UnitJob *__restrict__ jobs) {
+  const UnitJob j = jobs[blockIdx.y];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < j.k * j.k; e += gridDim.x * blockDim.x) j.BBt[e] *= j.d[e / j.k] * j.d[e % j.k];
+}
+__global__ void unit_rows_kernel(const UnitJob *__restrict__ jobs) {
+  const UnitJob j = jobs[blockIdx.y];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < j.k * j.r; e += gridDim.x * blockDim.x) j.U[e] = (float)((double)j.U[e] * j.d[e / j.r]);
+}
+
 __global__ void round_to_half_inplace_kernel(float *const *ptrs, const long long *counts) {
   const int ci = blockIdx.y;
   float *p = ptrs[ci];
@@ -703,6 +715,7 @@ struct CellWork {      // device scratch of one cell
   // CholeskyQR on tensor cores: Gram partials, L^-1 as fp16 hi + lo, its exponent, slots for measured magnitudes
   float *orthPart = nullptr; __half *orthLhi = nullptr, *orthLlo = nullptr; int *orthExp = nullptr;
   double *cholW = nullptr;                     // cluster Cholesky of wide sketches: work matrix and panels
+  const double *unit = nullptr;                // wide sketches: factors that make the columns of the final basis unit vectors
   unsigned *orthMax = nullptr; int orthMaxUsed = 0; bool absmax_ready = false;
   int split_ready = 0;       // 1 / 2: Bhi, Blo already hold the split of S / Z (written by the last triangular solve)
 };
@@ -1119,8 +1132,14 @@ void build_factor_program(Program &P, std::vector<CellWork> &ws, int mode, bool 
         }
       }
     }
+    std::vector<UnitJob> uj;
+    for (int i : act) if (ws[i].unit) uj.push_back({ws[i].unit, ws[i].BBt, probe ? nullptr : ws[i].Ut, ws[i].c.k, ws[i].c.r_t});
+    const size_t o_uj = P.push(uj);
+    const int n_uj = (int)uj.size();
     add_tall_gram(P, ST_SVD, tgb);
+    if (n_uj) P.add(ST_SVD, [=](char *dev, cudaStream_t s) { unit_gram_kernel<<<dim3(32, n_uj), 256, 0, s>>>((const UnitJob *)(dev + o_uj)); LAUNCHED(); });
     add_eig(P, ST_SVD, eg, 9);          // k x k, 6-7 sweeps observed
+    if (n_uj && !probe) P.add(ST_SVD, [=](char *dev, cudaStream_t s) { unit_rows_kernel<<<dim3(32, n_uj), 256, 0, s>>>((const UnitJob *)(dev + o_uj)); LAUNCHED(); });
     add_gemm(P, ST_FACT, g2, false);
     add_gemm(P, ST_FACT, g3, false);
     if (check_subspace && !probe) {

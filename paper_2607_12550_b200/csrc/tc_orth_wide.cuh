@@ -35,7 +35,38 @@ struct alignas(64) OrthWCell {
   float *out32;
   int ld, k, kp, rpp, panels, n_chunks, out_exp;
   int *status;
+  const __half *hi, *lo;      // the basis
+  double *unit;               // [k] orthw_norms_kernel
 };
+
+// unit[c] = 1 / |column c| of the finished basis (1 for a dead one).  The tensor core's accumulation truncates, which shows where
+// every term has one sign: on the diagonal of the Gram, and in Q = R L^-T through the one large term of each entry.  The columns
+// come out up to 2e-7 long; what is made of them takes the factor along (UnitJob).  A warp per column, eight rows a lane and
+// step; bound by reading the basis once (4 bytes an entry).
+__global__ void __launch_bounds__(256) orthw_norms_kernel(const OrthWCell *__restrict__ cells) {
+  const OrthWCell &c = cells[blockIdx.y];
+  const int col = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (col >= c.k) return;
+  const int per = c.rpp / 8, total = c.panels * per;           // pieces of eight rows: of a panel, of the column
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 2
+  for (int e = lane; e < total; e += 32) {
+    const int panel = e / per;
+    const size_t o = ((size_t)panel * c.kp + col) * c.rpp + (size_t)(e - panel * per) * 8;
+    const uint4 h = __ldg((const uint4 *)(c.hi + o)), l = __ldg((const uint4 *)(c.lo + o));
+    const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 a = __half22float2(*(const __half2 *)&hw[q]), b = __half22float2(*(const __half2 *)&lw[q]);
+      const double x = (double)a.x + (double)b.x, y = (double)a.y + (double)b.y;
+      s0 = fma(x, x, s0); s1 = fma(y, y, s1);
+    }
+  }
+  s0 += s1;
+  for (int o = 16; o; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+  const double n2 = ldexp(s0, -2 * c.out_exp);
+  if (lane == 0) c.unit[col] = n2 > 0.25 ? rsqrt(n2) : 1.0;
+}
 
 __global__ void __launch_bounds__(OW_THREADS, 1) orthw_gram_kernel(const OrthWCell *__restrict__ cells) {
   extern __shared__ unsigned char smem_raw[];

@@ -138,6 +138,9 @@ def test_wide_basis_is_as_good_as_the_fp64_one(B, T, m, k, q):
             B.set_fast_path(prev)
     for c in (0, 1):
         R = _range_fp64(B, KV[c], c, 7, k, q)
+        # columns of unit length: the rounding of the fp32 factor and of the product with the small SVD's vectors, 2^-23 each
+        assert float((got[1][c].T @ got[1][c] - torch.eye(k, dtype=torch.float64, device="cuda")).abs().max()) <= 2.0 ** -22
+        assert abs(float(got[1][c].norm() ** 2) / k - 1.0) <= 2.0 ** -24
         for n in (64, k):
             assert _distance(got[1][c][:, :n], R[:, :n]) <= 1.2 * _distance(got[0][c][:, :n], R[:, :n]), (c, n)
 
