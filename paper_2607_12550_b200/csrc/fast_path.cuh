@@ -156,7 +156,7 @@ inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
     for (auto &b : v) {
       b.tile_base = (int)std::min<long long>(total, 1 << 30);
       total += (long long)b.m * (b.T / 128);
-      for (int q = cls; q < 2; ++q) H.dec.bitmask[q] |= 1u << b.bits;
+      if (cls < 2) H.dec.bitmask[cls] |= 1u << b.bits;
       H.dec.m.push_back(b.m);
     }
     table.insert(table.end(), v.begin(), v.end());

@@ -449,7 +449,7 @@ struct jolt_handle {
   void *d_dec = nullptr;
   int *d_counter = nullptr;
   // decode descriptors by class (values r_t <= 128, keys r_t <= 128, r_t > 128): cells and tiles up to the end of each class,
-  // bit widths of the first class and of the first two, heads of each cell
+  // bit widths of the first two, heads of each cell
   struct DecTable { int end[3] = {0, 0, 0}; long long tiles[3] = {0, 0, 0}; unsigned bitmask[2] = {0, 0}; std::vector<int> m; } dec;
   // A decode that launches only the persistent kernel does not clear the status words: it marks what it writes with its epoch
   mutable std::atomic<int> epoch{0}, status_epoch{0};
@@ -1879,7 +1879,7 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   const bool use_p = (g_fast.load() & 128) && d.tiles[1] < (1ll << 30);
   if (use_p && d.end[pc] > 0) {
     CU(persistent(0, d.end[pc], 0, d.tiles[pc]));
-    launch_decode_widths(a, d.bitmask[pc], (int)std::min<long long>(n_sm[dev].load(), d.tiles[pc]), st);
+    launch_decode_widths(a, d.bitmask[0] | (rope ? 0u : d.bitmask[1]), (int)std::min<long long>(n_sm[dev].load(), d.tiles[pc]), st);
     LAUNCHED();
   }
   if (use_p && rope && d.end[1] > d.end[0] && a.out.tma_out) {
