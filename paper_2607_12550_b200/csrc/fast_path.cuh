@@ -92,9 +92,23 @@ inline void fill_bb_common(tc::BBCell &b, const CellStore &cs, int *status) {
 }
 
 
-// Per-item decode kernel: cells of r_t > 128, keys rotated into a destination that bulk stores cannot write, and every cell when
-// the persistent kernel is off.
-inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, cudaStream_t s) {
+// A launch that may begin while the kernel before it on the stream drains (on the device it waits for that kernel).
+template <typename... P, typename... A>
+inline void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t shm, cudaStream_t s, const A &...args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = shm; cfg.stream = s;
+  cudaLaunchAttribute at;
+  memset(&at, 0, sizeof at);
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+// Per-item decode kernel over descriptors [first, first + n).  overlap: behind a launch of the persistent kernel, which writes other
+// cells: this one's CTAs take the SMs that come free.
+inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, bool overlap, cudaStream_t s) {
   using LY = tc::DecLayout;
   static DeviceOnce once;
   once([] { cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
@@ -109,16 +123,19 @@ inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc
   int heads = 0, m_max = 0;
   for (int i = first; i < first + n; ++i) { heads += H->dec.m[i]; m_max = std::max(m_max, H->dec.m[i]); }
   bb_split(heads, H->T / 128, a.tiles_per_item, a.items_per_head);
-  tc::decode_kernel<<<dim3(m_max * a.items_per_head, n), LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+  const dim3 grid(m_max * a.items_per_head, n);
+  if (overlap) launch_overlapped(tc::decode_kernel, grid, LY::THREADS, LY::SMEM_BYTES, s, a);
+  else tc::decode_kernel<<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
   LAUNCHED();
 }
 
 template <bool TMA_ONLY, unsigned BITMASK, bool ROPE = false>
-inline void launch_decode_p(const tc::DecPArgs &a, int grid, cudaStream_t s) {
+inline void launch_decode_p(const tc::DecPArgs &a, int grid, cudaStream_t s, bool overlap = false) {
   using LY = tc::DecLayout;
   static DeviceOnce once;
   once([] { cudaFuncSetAttribute(tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
-  tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+  if (overlap) launch_overlapped(tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE>, dim3(grid), LY::THREADS, LY::SMEM_BYTES, s, a);
+  else tc::decode_persistent_kernel<TMA_ONLY, BITMASK, ROPE><<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
 }
 
 // The persistent kernel is instantiated per output mode and per set of bit widths: with at most two tile loops compiled
@@ -135,12 +152,13 @@ inline void launch_decode_widths(const tc::DecPArgs &a, unsigned bitmask, int gr
   else launch_decode_p<true, 0x11Fu>(a, grid, s);
 }
 
-// Descriptors of the cells that take the tensor-core decode, in the order [values, r_t <= 128][keys, r_t <= 128][r_t > 128]
-// and in each class the costliest first (most residual bits, then largest r_t: the last wave of per-item CTAs is then the
-// cheapest).  The persistent kernel takes the first two classes in one launch, or each in its own when keys are rotated.
+// Descriptors of the cells that take the tensor-core decode, in the order [values, r_t <= 128][keys, r_t <= 128][r_t > 128] and in each
+// class the costliest first (most residual bits, then largest r_t: the last wave of per-item CTAs is then the cheapest), for the
+// persistent kernel; then all of them once more, the costliest first, for one launch of the per-item kernel.
 inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
   table.clear();
   H.dec = jolt_handle::DecTable();
+  auto costlier = [](const tc::BBCell &x, const tc::BBCell &y) { return x.bits != y.bits ? x.bits > y.bits : x.r_t > y.r_t; };
   long long total = 0;
   for (int cls = 0; cls < 3; ++cls) {
     std::vector<tc::BBCell> v;
@@ -152,7 +170,7 @@ inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
       b.layer0 = H.group_start[i / 2];
       v.push_back(b);
     }
-    std::stable_sort(v.begin(), v.end(), [](const tc::BBCell &x, const tc::BBCell &y) { return x.bits != y.bits ? x.bits > y.bits : x.r_t > y.r_t; });
+    std::stable_sort(v.begin(), v.end(), costlier);
     for (auto &b : v) {
       b.tile_base = (int)std::min<long long>(total, 1 << 30);
       total += (long long)b.m * (b.T / 128);
@@ -163,6 +181,10 @@ inline void make_decode_table(jolt_handle &H, std::vector<tc::BBCell> &table) {
     H.dec.end[cls] = (int)table.size();
     H.dec.tiles[cls] = total;
   }
+  std::vector<tc::BBCell> all = table;
+  std::stable_sort(all.begin(), all.end(), costlier);
+  for (auto &b : all) H.dec.m.push_back(b.m);
+  table.insert(table.end(), all.begin(), all.end());
 }
 
 // ------------------------------------------------------------------ tensor-core sweeps of the factor stage

@@ -448,8 +448,8 @@ struct jolt_handle {
   // of the persistent decode kernel and its chunk counter
   void *d_dec = nullptr;
   int *d_counter = nullptr;
-  // decode descriptors by class (values r_t <= 128, keys r_t <= 128, r_t > 128): cells and tiles up to the end of each class,
-  // bit widths of the first two, heads of each cell
+  // decode descriptors by class (values r_t <= 128, keys r_t <= 128, r_t > 128), and once more all of them, the costliest first: cells
+  // and tiles up to the end of each class, bit widths of the first two, heads of each descriptor
   struct DecTable { int end[3] = {0, 0, 0}; long long tiles[3] = {0, 0, 0}; unsigned bitmask[2] = {0, 0}; std::vector<int> m; } dec;
   // A decode that launches only the persistent kernel does not clear the status words: it marks what it writes with its epoch
   mutable std::atomic<int> epoch{0}, status_epoch{0};
@@ -1477,7 +1477,7 @@ static int alloc_handle_memory(jolt_handle &H, size_t payload, const std::vector
     b.take<char>(payload);
     H.d_status = b.take<int>(4 * nc);
     H.d_counter = b.take<int>(4);
-    H.d_dec = b.take<tc::BBCell>(nc);
+    H.d_dec = b.take<tc::BBCell>(2 * nc);
     for (size_t c = 0; c < nc; ++c) {
       CellStore &cs = H.cells[c];
       if (cs.c.r_t == 0) { cs.P16 = nullptr; continue; }
@@ -1834,8 +1834,22 @@ static void of_this_epoch(const jolt_handle *H, std::vector<int> &words) {      
   for (auto &w : words) w = (w >> 8) == epoch ? w & 0xff : 0;
 }
 
-// The cells on the tensor-core kernels: the persistent kernel for r_t <= 128, the per-item kernel for the others and for key
-// cells whose rotation happens in its epilogue (`rope`: their table).
+// map of a decode's destination: boxes of 32 tokens by `features`
+static bool decode_map(CUtensorMap *tm, void *base, const jolt_layout *L, uint32_t features, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
+  const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)L->seq_len, (uint64_t)L->n_kv_heads, (uint64_t)L->n_layers};
+  const uint64_t str[3] = {(uint64_t)L->stride_token * 2, (uint64_t)L->stride_head * 2, (uint64_t)L->stride_layer * 2};
+  const uint32_t box[4] = {features, 32, 1, 1};
+  return make_tmap_f16(tm, base, 4, dims, str, box, swizzle);
+}
+
+// The cells on the tensor-core kernels.  The persistent kernel takes cells of r_t <= 128: all of a plain decode in one launch, or
+// the values and then the keys that it rotates.  Everything else is one launch of the per-item kernel over all cells, the
+// costliest first: any mixture balances there, where a launch per class pays a start and a tail of its own (caches of r_t 208 and
+// 64 in equal parts, 256 / 2048 / 16384 tiles: 27 / 65 / 245 us in one launch, 28 / 68 / 260 in two, 26 / 66 / 253 in two that
+// overlap).  Two overlapping launches are ahead where three quarters of the tiles are the persistent kernel's and there are more
+// than two a CTA (one cell of 16 above 128: 199 against 224 us at 16384 tiles, 29 against 41 at 512), and for rotated keys above
+// that size where no cell is above 128 (16384 tiles: 234 against 272 us; 48 tiles: 27 against 24; with one cell above, 275 against 279
+// and 119 against 114 at 4096).  `rope`: the rotation's table, or null.
 static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Kout, char *Vout, const float2 *rope, unsigned long long *stamps, int dev,
                             cudaStream_t st) {
   static std::atomic<int> n_sm[64];
@@ -1850,22 +1864,14 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
   a.out.base[0] = Kout; a.out.base[1] = Vout;
   a.out.osl = L->stride_layer; a.out.osh = L->stride_head; a.out.ost = L->stride_token;
   a.out.out_dtype = L->dtype == JOLT_F16 ? DT_F16 : DT_F32;
-  if (L->dtype == JOLT_F16) {
-    const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)L->seq_len, (uint64_t)L->n_kv_heads, (uint64_t)L->n_layers};
-    const uint64_t str[3] = {(uint64_t)L->stride_token * 2, (uint64_t)L->stride_head * 2, (uint64_t)L->stride_layer * 2};
-    const uint32_t box[4] = {64, 32, 1, 1};
-    a.out.tma_out = make_tmap_f16(&a.out.tm[0], Kout, 4, dims, str, box) && make_tmap_f16(&a.out.tm[1], Vout, 4, dims, str, box);
-  }
+  if (L->dtype == JOLT_F16) a.out.tma_out = decode_map(&a.out.tm[0], Kout, L, 64) && decode_map(&a.out.tm[1], Vout, L, 64);
   long long *dbg = nullptr;
 #ifdef JOLT_DEBUG
   dbg = a.dbg = g_dbg_stamps;
 #endif
-  // The persistent kernel walks the first two classes, or the values and then the keys that it rotates.  The tail that is dealt
-  // out in chunks is empty unless a test asks for one: measured on the benchmark mix, a 5 % tail in 8-tile chunks made the
-  // launch slower (0.199 against 0.192 ms), because every chunk reloads its head's projected core into the single P buffer
-  // and restarts the unpack -> rotation pipeline.
-  const int pc = rope ? 0 : 1;
-  int done = 0;
+  // The tail of the persistent kernel that is dealt out in chunks is empty unless a test asks for one: measured on the benchmark mix,
+  // a 5 % tail in 8-tile chunks made the launch slower (0.199 against 0.192 ms), because every chunk reloads its head's projected
+  // core into the single P buffer and restarts the unpack -> rotation pipeline.
   auto persistent = [&](int c0, int c1, long long t0, long long t1) {      // cells [c0, c1), tiles [t0, t1)
     const int pct = g_dec_tail_pct.load();
     a.cells = (const tc::BBCell *)H->d_dec + c0; a.n_cells = c1 - c0;
@@ -1873,32 +1879,33 @@ static int launch_decode_tc(const jolt_handle *H, const jolt_layout *L, char *Ko
     a.nt = H->T / 128; a.seed = H->seed; a.epoch = H->status_epoch; a.stamps = stamps;
     a.pool = (int)(t0 + (t1 - t0) * (100 - pct) / 100); a.chunk = std::max(1, g_dec_tail_chunk.load());
     a.counter = H->d_counter;
-    done = c1;
+    a.more = c1 < d.end[2];
     return a.pool < a.total ? cudaMemsetAsync(H->d_counter, 0, sizeof(int), st) : cudaSuccess;
   };
-  const bool use_p = (g_fast.load() & 128) && d.tiles[1] < (1ll << 30);
-  if (use_p && d.end[pc] > 0) {
-    CU(persistent(0, d.end[pc], 0, d.tiles[pc]));
-    launch_decode_widths(a, d.bitmask[0] | (rope ? 0u : d.bitmask[1]), (int)std::min<long long>(n_sm[dev].load(), d.tiles[pc]), st);
+  const int sms = n_sm[dev].load();
+  const bool use_p = (g_fast.load() & 128) && d.tiles[1] < (1ll << 30) && d.end[1] > 0, some_high = d.end[2] > d.end[1], large = d.tiles[2] > 2 * sms;
+  CUtensorMap keys;
+  if (use_p && !rope && (!some_high || (large && 4 * d.tiles[1] >= 3 * d.tiles[2]))) {
+    CU(persistent(0, d.end[1], 0, d.tiles[1]));
+    launch_decode_widths(a, d.bitmask[0] | d.bitmask[1], (int)std::min<long long>(sms, d.tiles[1]), st);
     LAUNCHED();
-  }
-  if (use_p && rope && d.end[1] > d.end[0] && a.out.tma_out) {
-    const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)L->seq_len, (uint64_t)L->n_kv_heads, (uint64_t)L->n_layers};
-    const uint64_t str[3] = {(uint64_t)L->stride_token * 2, (uint64_t)L->stride_head * 2, (uint64_t)L->stride_layer * 2};
-    const uint32_t box[4] = {32, 32, 1, 1};
-    const CUtensorMap keep = a.out.tm[0];
-    if (make_tmap_f16(&a.out.tm[0], Kout, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_64B)) {
-      CU(persistent(d.end[0], d.end[1], d.tiles[0], d.tiles[1]));
-      a.rope = rope;
-      const int grid = (int)std::min<long long>(n_sm[dev].load(), d.tiles[1] - d.tiles[0]);
-      if ((d.bitmask[1] & ~0x110u) == 0) launch_decode_p<true, 0x110u, true>(a, grid, st);
-      else launch_decode_p<true, 0x11Fu, true>(a, grid, st);
+    if (some_high) launch_decode_items(H, d.end[1], d.end[2] - d.end[1], a.out, nullptr, dbg, true, st);
+  } else if (use_p && rope && !some_high && large && d.end[1] > d.end[0] && a.out.tma_out && decode_map(&keys, Kout, L, 32, CU_TENSOR_MAP_SWIZZLE_64B)) {
+    if (d.end[0] > 0) {
+      CU(persistent(0, d.end[0], 0, d.tiles[0]));
+      launch_decode_widths(a, d.bitmask[0], (int)std::min<long long>(sms, d.tiles[0]), st);
       LAUNCHED();
     }
-    a.out.tm[0] = keep;
+    CU(persistent(d.end[0], d.end[1], d.tiles[0], d.tiles[1]));
+    a.out.tm[0] = keys;
+    a.rope = rope;
+    const int grid = (int)std::min<long long>(sms, d.tiles[1] - d.tiles[0]);
+    if ((d.bitmask[1] & ~0x110u) == 0) launch_decode_p<true, 0x110u, true>(a, grid, st, d.end[0] > 0);
+    else launch_decode_p<true, 0x11Fu, true>(a, grid, st, d.end[0] > 0);
+    LAUNCHED();
+  } else if (d.end[2] > 0) {
+    launch_decode_items(H, d.end[2], d.end[2], a.out, rope, dbg, false, st);
   }
-  if (done < d.end[1] && done < d.end[2]) launch_decode_items(H, done, d.end[1] - done, a.out, rope, dbg, st);
-  if (d.end[1] < d.end[2]) launch_decode_items(H, d.end[1], d.end[2] - d.end[1], a.out, rope, dbg, st);
   CU(cudaGetLastError());
   return JOLT_OK;
 }
@@ -2113,20 +2120,6 @@ static void launch_att_values(dim3 grid, cudaStream_t s, const AttendJob *d, int
   const size_t shm = (size_t)kAttHalf * (NQP * sizeof(float) + 16 * BITS + 8) + (size_t)4 * 128 * NQP * sizeof(float);
   if (NQP == 4) attend_values_kernel<BITS, 4><<<grid, kAttChunk, shm, s>>>(d);
   else attend_values_kernel<BITS, 8><<<grid, kAttChunk, shm, s>>>(d);
-}
-
-// A launch that may begin while the kernel before it on the stream drains (it waits on the device for that kernel's results).
-template <typename... P, typename... A>
-static void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t shm, cudaStream_t s, const A &...args) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = shm; cfg.stream = s;
-  cudaLaunchAttribute at;
-  memset(&at, 0, sizeof at);
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at; cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, double scale, void *dOut, void *stream) {

@@ -59,6 +59,11 @@ __device__ __forceinline__ void dec_fill_out(BBCell &c, const DecOut &o) {      
   c.out_dtype = o.out_dtype; c.tma_out = o.tma_out;
 }
 
+// Two launches of one decode overlap: the second may start when every CTA of the first has, and one CTA of it ends after the
+// first launch has, so that what follows on the stream comes after both.
+__device__ __forceinline__ void dec_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dec_end_after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <int BITS>
 struct DecCodesRow { uint32_t words[BITS > 0 ? 4 * BITS : 1]; uint2 sc; };
 
@@ -865,6 +870,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
     __syncthreads();
   }
   if (warp == NWG * 4) { tc_fence_after(); tmem_dealloc(tmem_base, LY::TMEM_COLS); }
+  if (blockIdx.x == 0 && blockIdx.y + 1 == gridDim.y) dec_end_after_previous();
 }
 
 }  // namespace tc

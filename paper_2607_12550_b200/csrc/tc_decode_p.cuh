@@ -51,6 +51,7 @@ struct DecPArgs {
   int *counter;        // chunks handed out so far (zero at launch when pool < total; not read otherwise)
   const float2 *rope;  // ROPE: (cos, sin) of feature pair j at token t in rope[j * T + t]
   unsigned long long *stamps;      // optional: start of the first CTA, end of the last (globaltimer, ns)
+  int more;            // a second launch of the same decode follows
   int epoch;           // a failed wait writes (epoch << 8 | 8) into the status word of the first cell
 #ifdef JOLT_DEBUG
   long long *dbg;
@@ -294,6 +295,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   JOLT_DBG(long long *cta_dbg = a.dbg ? a.dbg + 128 + blockIdx.x * 4 : nullptr;)
   JOLT_DBG(if (cta_dbg && threadIdx.x == 0) { long long g; unsigned sm; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g)); asm volatile("mov.u32 %0, %%smid;" : "=r"(sm)); cta_dbg[0] = g; cta_dbg[2] = sm; })
 
+  if (a.more) dec_let_next_start();
   if (a.stamps && blockIdx.x == 0 && threadIdx.x == 0) a.stamps[0] = global_ns();
 
   // shared memory: P block (32 KB) | output staging (2 x 16 KB) | rotation operand H | U_T ring | operand tiles | barriers
@@ -583,6 +585,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
     __syncthreads();
   }
   if (warp == NWG * 4) { tc_fence_after(); tmem_dealloc(tmem_base, LY::TMEM_COLS); }
+  if (blockIdx.x + 1 == gridDim.x) dec_end_after_previous();
 }
 
 }  // namespace tc

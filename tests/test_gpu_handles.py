@@ -248,3 +248,54 @@ def test_rotated_keys_of_the_persistent_kernel(B, bits, T, tail):
     h.free()
     # the same operands, accumulators and rounding in both kernels
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+def _decode_both(B, h, like, gs, rope, tail=0):
+    outs = []
+    for mask in (255, 255 - 128):
+        o = torch.empty_like(like), torch.empty_like(like)
+        prev = B.set_fast_path(mask)
+        B.set_test_decode_tail(tail, 2)
+        try:
+            for _ in range(4):                          # on one stream, without a host wait: what follows a decode sees all of it
+                o[0].zero_(); o[1].zero_()
+                if rope:
+                    B.jolt_decompress_rope(h, *o, gs, base=10000.0, pos0=100)
+                else:
+                    B.jolt_decompress(h, *o, gs)
+                outs.append((o[0].clone(), o[1].clone()))
+            B.check_status(h)
+        finally:
+            B.set_fast_path(prev)
+            B.set_test_decode_tail(0)
+    return outs
+
+
+# more than two tiles a CTA (640): one cell, half and all but one of them above r_t = 128, keys or values; widths with an
+# instantiation of their own and without
+@pytest.mark.parametrize("high", [(1,), (0, 5), (0, 2, 4, 6), (1, 3, 5, 7), (0, 1, 2, 4, 5, 6, 7), ()])
+@pytest.mark.parametrize("bits", [(4, 8), (2, 3)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_overlapping_launches_decode_like_one(B, high, bits, rope):
+    K, V = _cache(4, 4, 2560, 31)
+    gs = [0, 1, 2, 3, 4]
+    plans = [(176 if c in high else 48 + 16 * (c % 3), 128, bits[c % 2]) for c in range(8)]
+    h = B.jolt_compress(K, V, gs, plans, B.default_options(seed=2, power_iters=0))
+    outs = _decode_both(B, h, K, gs, rope)
+    h.free()
+    for o in outs[1:]:
+        assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
+
+
+# as test_rotated_keys_of_the_persistent_kernel, with enough tiles for the persistent kernel to take the rotation
+@pytest.mark.parametrize("bits", [(0, 1), (2, 3), (4, 8)])
+@pytest.mark.parametrize("heads,T,tail", [(40, 128, 0), (8, 640, 0), (13, 384, 60)])
+def test_rotated_keys_of_many_tiles(B, bits, heads, T, tail):
+    K, V = _cache(4, heads, T, 9)
+    gs = [0, 2, 4]
+    plans = [(32, 128, bits[0]), (48, 128, 4), (128, 96, bits[1]), (16, 128, 2)]
+    h = B.jolt_compress(K, V, gs, plans, B.default_options(seed=2, power_iters=0))
+    outs = _decode_both(B, h, K, gs, True, tail)
+    h.free()
+    for o in outs[1:]:
+        assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
