@@ -2175,7 +2175,7 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
       j.qh = b.take<__half>((size_t)j.m * kAttMaxQ * kD);
       j.ql = b.take<__half>((size_t)j.m * kAttMaxQ * kD);
       j.qe = b.take<float>((size_t)j.m * kAttMaxQ);
-      j.p = b.take<float>((size_t)j.m * T * NQP);
+      j.p = mma ? nullptr : b.take<float>((size_t)j.m * T * NQP);       // (the streaming kernel keeps the weights to itself)
       j.ml = b.take<float>((size_t)j.m * n_chunks * 2 * NQP);
       j.y = b.take<float>((size_t)j.m * n_chunks * std::max(j.v.r_t, 1) * NQP);
       j.a = b.take<float>((size_t)j.m * n_chunks * kD * NQP);

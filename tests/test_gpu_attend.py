@@ -86,3 +86,25 @@ def test_calls_in_a_row_use_their_own_queries(B, L, H, T, nq):
     h.free()
     for i, o in enumerate(got):
         assert torch.equal(o, want[i % 5]), i
+
+
+def test_scratch_of_a_call(B):
+    """What a call takes from the device: per head and 128-token chunk the partial values (ranks and features) of four queries, and
+    nothing per token."""
+    L, H, T, nq, r = 2, 4, 65536, 4, 64
+    K, V = (torch.randn(L, H, T, 128, device="cuda").half() for _ in range(2))
+    h = B.jolt_compress(K, V, [0, L], [(r, 128, 4), (r, 128, 4)], B.default_options(seed=3, power_iters=0))
+    Q = torch.randn(L, H, nq, 128, device="cuda")
+    B.jolt_attend(h, Q)
+    del K, V
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    B.release_workspace()
+    out = torch.empty_like(Q)
+    before = torch.cuda.mem_get_info()[0]
+    B._check(B.lib.jolt_attend(h.ptr, Q.data_ptr(), nq, 0.1, out.data_ptr(), None))
+    torch.cuda.synchronize()
+    taken = before - torch.cuda.mem_get_info()[0]
+    h.free()
+    partial = L * H * (T // 128) * 4 * (r + 128 + 2) * 4
+    assert taken <= partial * 9 // 8 + (6 << 20), (taken, partial)           # an eighth of headroom, tables, pages of 2 MB
