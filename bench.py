@@ -445,7 +445,7 @@ def main():
     t_res = lock.get("residual_quant")
     roof_c = None
     if t_res:
-        tr = dram_traffic("tc::backbone_kernel<1>", cfg.name)
+        tr = dram_traffic("tc::backbone_kernel", cfg.name)
         ach = br_ / (t_res * 1e-3) / 1e9
         roof_c = {"kernel": "tc::backbone_kernel", "bound": "hbm", "achieved": ach, "peak": pk["hbm"], "unit": "GB/s",
                   "frac": ach / pk["hbm"], "traffic": (tr["read"] + tr["write"]) * (2 * ng) / tr["cells"] if tr else None,
@@ -463,7 +463,7 @@ def main():
 
     line = {"metric": METRIC, "value": job_throughput(world, cache_bytes, ms), "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": W, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "f16 operands, f32 accumulate (f64 Cholesky, f32 Jacobi)", "data": "synthetic",
+            "vs_baseline": None, "dtype": "f16 operands, f32 accumulate (f64 Cholesky and eigen-solves)", "data": "synthetic",
             "config": {"workload": f"{cfg.name}: {ng * cfg.layers_per_group} layers / {cfg.layers_per_group} per group, "
                                    f"{cfg.n_kv_heads} KV heads, T={cfg.seq_len}, d=128, fp16, budget {ratio}x, "
                                    + (f"randomized q={q}" if args.token_mode == "randomized" else "exact (converged block iteration)"),

@@ -162,7 +162,7 @@ int jolt_decompress(const jolt_handle *h, const jolt_layout *out_layout, void *d
  *     K_out[.., t, j]      = K^[.., t, j] cos - K^[.., t, j + 64] sin
  *     K_out[.., t, j + 64] = K^[.., t, j + 64] cos + K^[.., t, j] sin
  * where K^ is the decoded key before it is rounded to the destination type.  V is written as by
- * jolt_decompress.  Angles are evaluated in fp64, the rotation in fp32.  Key cells decoded by the tensor-core
+ * jolt_decompress.  Angles are evaluated in fp64, the rotation in fp32.  Key cells decoded by a tensor-core
  * kernel with r_t <= 128 are rotated inside that kernel and rounded once; the other key cells are rotated by a
  * separate in-place pass over the decoded tensor, so an fp16 destination is rounded after decoding and again
  * after the rotation (jolt_set_fast_path bit 3 off sends every cell that way).  rope: host pointer; 1 < base < 1e12, 0 <= pos0 <= 2^40 (JOLT_EINVAL otherwise).  All other
@@ -184,11 +184,10 @@ int jolt_decompress_rope(const jolt_handle *h, const jolt_layout *out_layout, vo
  *   dQ, dOut: device, fp32, contiguous [n_layers][n_kv_heads][n_q][128], 16-byte aligned; n_q = queries per KV head,
  *   1..8 (the grouped-query group size).  Keys are used as stored: a cache whose keys were compressed before a rotary
  *   embedding needs jolt_decompress_rope instead (the rotation differs per token and does not commute with the
- *   contraction).  Scratch comes from the library's per-device workspace (grown on first use).  The first call on a
- *   handle also forms the projected cores P_h = fp16(G_h U_F^T) of all cells (m * r_t * 128 fp16 values per cell,
- *   about 5 % of the compressed size on the benchmark workload) in a device buffer that stays with the handle
- *   until jolt_free; later calls, on any stream, reuse them (a first call that fails leaves nothing behind; the next
- *   call forms them again).  Errors: JOLT_EINVAL
+ *   contraction).  Scratch comes from the library's per-device workspace (grown on first use).  The projected cores
+ *   P_h = fp16(G_h U_F^T) that the call reads were formed by jolt_compress / jolt_deserialize and stay with the handle
+ *   (m * r_t * 128 fp16 values per cell with r_f < 128, about 5 % of the compressed size on the benchmark workload).
+ *   Errors: JOLT_EINVAL
  *   (null / misaligned pointers, n_q out of range, wrong device), JOLT_EUNSUPPORTED (ranks that are not multiples
  *   of 8; sequences beyond about 3 million tokens), JOLT_ENOMEM, JOLT_ECUDA.  Asynchronous on `stream`.  Arithmetic:
  *   fp32; the contractions that run on the tensor cores take their fp32 operand as hi + lo fp16 (about 22 bits) and
@@ -289,8 +288,8 @@ int64_t jolt_launch_count(void);
  * bit 5 = CholeskyQR of the range finder on tensor cores (otherwise fp64 SIMT Gram and row-wise triangular solve),
  * bit 6 = factor sweeps with two output tiles per CTA (otherwise one);
  * bit 7 = persistent decode kernel (one CTA per SM walks a share of all tiles; otherwise one CTA per 16-tile item;
- *         cells of r_t > 128 and keys rotated into an fp32 or unaligned destination always take the per-item
- *         kernel);
+ *         cells of r_t > 128, caches of which they are more than a quarter, and keys rotated into an fp32 or unaligned
+ *         destination or in caches of few tiles always take the per-item kernel);
  * 255 (default) = all, where the shapes allow.  Returns the previous mask. */
 int jolt_set_fast_path(int enabled);
 

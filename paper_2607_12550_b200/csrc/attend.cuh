@@ -15,7 +15,7 @@
 // operand entering as hi + lo fp16; the rest is CUDA-core fp32):
 //   (P_h = fp16(G_h U_F^T), the projected core the decoder also reads, is kept with the handle since compress)
 //   attend_prep_kernel     per (group, head, query): rotated scaled query (fp32, and scaled hi + lo fp16), w = P_h q
-//   attend_stream_kernel   per (group, head, 256-token chunk): scores, chunk maximum, p = exp(s - max), chunk sum,
+//   attend_stream_kernel   per (group, four heads, 128-token chunk): scores, chunk maximum, p = exp(s - max), chunk sum,
 //                          sum_t p_t r^'_t and p^T U_T
 //   attend_combine_kernel  per (group, head, query): merges the chunks (running-maximum rescaling), applies P_h of the
 //                          value cell and the inverse rotation, divides by the softmax denominator
@@ -30,7 +30,7 @@
 
 namespace jolt {
 
-constexpr int kAttChunk = 256;      // tokens per chunk = threads per CTA of the two streaming kernels
+constexpr int kAttChunk = 256;      // portable kernels: tokens per chunk = threads per CTA (the streaming kernel: kAttTok)
 constexpr int kAttMaxQ = 8;         // queries per KV head (padded to 4 or 8 inside)
 
 struct AttendCell {

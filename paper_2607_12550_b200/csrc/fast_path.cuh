@@ -16,8 +16,6 @@ inline bool tc_shape_ok(const CellDesc &c) {
   return c.r_t > 0 && c.r_t % 16 == 0 && c.r_t <= 256 && c.r_f % 8 == 0 && c.r_f >= 8 && c.T % 128 == 0;
 }
 
-inline void fast_carve(Bump &, std::vector<CellWork> &, bool) {}
-
 // Tensor maps of the stored factors (constant for the life of a handle).
 inline bool encode_store_maps(CellStore &cs) {
   const CellDesc &c = cs.c;

@@ -404,13 +404,6 @@ __global__ void unit_rows_kernel(const UnitJob *__restrict__ jobs) {
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < j.k * j.r; e += gridDim.x * blockDim.x) j.U[e] = (float)((double)j.U[e] * j.d[e / j.r]);
 }
 
-__global__ void round_to_half_inplace_kernel(float *const *ptrs, const long long *counts) {
-  const int ci = blockIdx.y;
-  float *p = ptrs[ci];
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < counts[ci]; i += (long long)gridDim.x * blockDim.x)
-    p[i] = __half2float(__float2half_rn(p[i]));
-}
-
 }  // namespace jolt
 
 // ------------------------------------------------------------------ handle
@@ -1350,11 +1343,6 @@ int check_plan(const std::vector<CellDesc> &cells, const jolt_cell_plan *plan) {
   return JOLT_OK;
 }
 
-struct StatusReader {
-  int *d = nullptr;
-  std::vector<int> h;
-};
-
 int status_to_code(const std::vector<int> &st) {
   for (size_t i = 0; i < st.size(); i += 4) {
     if (st[i] & 1) return fail(JOLT_ENUMERIC, "cell %zu: eigen-solver did not converge", i / 4);
@@ -1749,7 +1737,6 @@ static int compress_impl(const jolt_layout *L, const void *K, const void *V, con
     g_timer.mark(ST_IN, st);
   }
   if (ce == cudaSuccess && injected) {
-    std::vector<float *> ptrs; std::vector<long long> cnts;
     for (int i = 0; i < nc && ce == cudaSuccess; ++i) {
       const CellDesc &c = cells[i];
       if (c.r_t == 0) continue;
@@ -2135,13 +2122,13 @@ extern "C" int jolt_attend(const jolt_handle *H, const void *dQ, int32_t n_q, do
   const int NQP = n_q <= 4 ? 4 : 8;
   const bool mma = (g_fast.load() & 1) != 0;        // the streaming kernel (the other kernels stay as the portable path)
   const int tc = mma ? kAttTok : kAttChunk, n_chunks = (T + tc - 1) / tc;
-  int m_max = 0, krt = 0, krf = 0, vrt = 0, vrf = 0;
+  int m_max = 0, krt = 0, vrt = 0;
   unsigned kbits = 0, vbits = 0;
   for (int g = 0; g < ng; ++g) {
     const CellDesc &ck = H->cells[2 * g].c, &cv = H->cells[2 * g + 1].c;
     m_max = std::max(m_max, ck.m);
-    krt = std::max(krt, ck.r_t); krf = std::max(krf, ck.r_t > 0 ? ck.r_f : 0);
-    vrt = std::max(vrt, cv.r_t); vrf = std::max(vrf, cv.r_t > 0 ? cv.r_f : 0);
+    krt = std::max(krt, ck.r_t);
+    vrt = std::max(vrt, cv.r_t);
     kbits |= 1u << ck.bits; vbits |= 1u << cv.bits;
     if ((ck.r_t % 8) || (cv.r_t % 8) || (ck.r_f % 8) || (cv.r_f % 8)) return fail(JOLT_EUNSUPPORTED, "ranks must be multiples of 8");
   }

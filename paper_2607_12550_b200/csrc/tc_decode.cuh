@@ -67,16 +67,6 @@ __device__ __forceinline__ void dec_end_after_previous() { asm volatile("griddep
 template <int BITS>
 struct DecCodesRow { uint32_t words[BITS > 0 ? 4 * BITS : 1]; uint2 sc; };
 
-template <int BITS>
-__device__ __forceinline__ void dec_load_codes_row(const BBCell &c, long long row, DecCodesRow<BITS> &d) {
-  if constexpr (BITS > 0) {
-    const uint4 *wp = (const uint4 *)(c.words + row * (4 * BITS));
-#pragma unroll
-    for (int i = 0; i < BITS; ++i) { const uint4 v = __ldg(wp + i); d.words[4 * i] = v.x; d.words[4 * i + 1] = v.y; d.words[4 * i + 2] = v.z; d.words[4 * i + 3] = v.w; }
-    d.sc = __ldg((const uint2 *)(c.scales + row * 4));
-  }
-}
-
 // Code j of a 32-code group as the bit pattern of the float 2^23 + code (the code dropped into the low mantissa
 // byte of 0x4B000000 by one byte permute): adding -(2^23 + 2^(BITS-1)) gives code - 2^(BITS-1) exactly, without an
 // integer conversion, and one FMA with dq and dq/2 the dequantised value (code - 2^(BITS-1) + 1/2) dq, rounded once.  W = the group's BITS words, code j at bits [j*BITS, j*BITS + BITS).
