@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
   auto bXfull = [=](int b) { return sBar + 184 + 8 * b; };
   auto bXempty = [=](int b) { return sBar + 200 + 8 * b; };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   const int wg = warp >> 2;
   const int nkt = (c.r_t + 63) / 64;
   const uint32_t panel = (uint32_t)c.r_t * 128u;       // bytes of one 64-feature panel of P (r_t is a multiple of 16)
@@ -147,9 +147,9 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
           tma_load_2d(sRing + s * BB_STAGE_BYTES, &c.tmUT, bFull(s), kb * 64, tt * 128);
         }
       }
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == 9) {
       // ---------------- MMA issuer
-      bool ok = mbar_wait(bSetup, 0, abort_flag);      // the head's projected core has landed
+      bool ok = mbar_wait_warp(bSetup, 0, abort_flag);      // the head's projected core has landed
       if (ok) {
         tc_fence_after();
         const uint32_t idesc = umma_idesc_f16(128, 128, 0, 1);   // A = U_T tile, K-major; B = P panels, MN-major
@@ -157,12 +157,12 @@ __global__ void __launch_bounds__(BB_THREADS, 1) backbone_kernel(const BBCell *_
         int cnt = 0;
         for (int i = 0; ok && i < n_tiles; ++i) {
           const int b = i & 1, nb = i >> 1;
-          ok = mbar_wait(bTempty(b), (nb & 1) ^ 1, abort_flag);
+          ok = mbar_wait_warp(bTempty(b), (nb & 1) ^ 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
           for (int kb = 0; kb < nkt; ++kb, ++cnt) {
             const int s = cnt % NS, n = cnt / NS;
-            ok = mbar_wait(bFull(s), n & 1, abort_flag);
+            ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
             for (int k4 = 0; k4 < 4 && kb * 4 + k4 < ksteps; ++k4) {

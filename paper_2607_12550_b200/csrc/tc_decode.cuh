@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
   auto bRready = [=](int b) { return sBar + 184 + 8 * b; };
   auto bBB = [=](int b) { return sBar + 216 + 8 * b; };           // backbone of the accumulator's tile complete
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   const int wg = warp >> 2;
   JOLT_DBG(long long *kdbg = (a.dbg && blockIdx.x == 0 && blockIdx.y == gridDim.y / 2 && threadIdx.x == 0) ? a.dbg + 16 * 8 : nullptr;)
   JOLT_DBG(if (kdbg) { kdbg[0] = clock64(); long long gt; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(gt)); kdbg[6] = gt; })
@@ -733,14 +733,14 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
           tma_load_2d(sStage(s), &cg.tmUT, bFull(s), kb * 64, tt * 128);
         }
       }
-    } else if (warp == NWG * 4 + 1 && lane == 0) {
+    } else if (warp == NWG * 4 + 1) {
       // ---------------- backbone MMA issuer.  Issuing an MMA costs its thread tens of cycles of dependent
       // instructions, and a tile needs sixteen of them: the two halves of a tile's accumulation (backbone, rotation)
       // are issued by two threads on different schedulers, ordered per accumulator through bBB.  The backbone thread
       // runs ahead as far as free accumulators and landed U_T stages allow (two accumulators per warpgroup when
       // r_t <= 128), so backbones wait in TMEM instead of U_T tiles in shared memory, and a late U_T stage never
       // holds back a rotation whose operands are complete.
-      bool ok = mbar_wait(bSetup, 0, abort_flag);        // the head's projected core has landed
+      bool ok = mbar_wait_warp(bSetup, 0, abort_flag);        // the head's projected core has landed
       if (ok) {
         tc_fence_after();
         const uint32_t idescB = umma_idesc_f16(128, 128, 0, 1);     // A = U_T tile, K-major; B = P panels, MN-major
@@ -754,13 +754,13 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
           // accumulator / barrier index b of tile j and how often it was used before (nb)
           const int wgi = j % NWG, ni = j / NWG;
           const int b = acc4 ? wgi + 2 * (ni & 1) : wgi, nb = acc4 ? ni >> 1 : ni;
-          ok = mbar_wait(bTempty(b), (nb & 1) ^ 1, abort_flag);
+          ok = mbar_wait_warp(bTempty(b), (nb & 1) ^ 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint32_t tacc = tmem_base + b * 128;
           for (int kb = 0; kb < nkt; ++kb, ++cnt) {
             const int s = cnt % ns, n = cnt / ns;
-            ok = mbar_wait(bFull(s), n & 1, abort_flag);
+            ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
             const uint64_t da = s < 4 ? dS0 + (uint64_t)s * kStep16K : dS4 + (uint64_t)(s - 4) * kStep16K;
@@ -773,9 +773,9 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
           if (ok) umma_commit(bBB(b));
         }
       }
-    } else if (warp == NWG * 4 + 2 && lane == 0) {
+    } else if (warp == NWG * 4 + 2) {
       // ---------------- rotation MMA issuer: A = the warpgroup's dequantised residual tile, B = H
-      bool ok = mbar_wait(bHready, 0, abort_flag);    // the rotation operand is built
+      bool ok = mbar_wait_warp(bHready, 0, abort_flag);    // the rotation operand is built
       if (ok) {
         tc_fence_after();
         const uint32_t idesc = umma_idesc_f16(128, 128, 0, 0);      // both operands K-major
@@ -787,8 +787,8 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
         for (int j = 0; ok && j < n_tiles; ++j) {
           const int wgi = j % NWG, ni = j / NWG;
           const int b = acc4 ? wgi + 2 * (ni & 1) : wgi, nb = acc4 ? ni >> 1 : ni;
-          ok = mbar_wait(bBB(b), nb & 1, abort_flag);                 // the tile's backbone is in the accumulator
-          if (ok && has_res) ok = mbar_wait(bRready(b), nb & 1, abort_flag);
+          ok = mbar_wait_warp(bBB(b), nb & 1, abort_flag);                 // the tile's backbone is in the accumulator
+          if (ok && has_res) ok = mbar_wait_warp(bRready(b), nb & 1, abort_flag);
           if (!ok) break;
           if (has_res) {
             tc_fence_after();

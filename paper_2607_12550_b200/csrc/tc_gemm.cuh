@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm_kernel(const GemmCell *
   auto bEmpty = [=](int s) { return sBar + 64 + 8 * s; };
   const uint32_t bDone = sBar + 128;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int s = 0; s < 8; ++s) { mbar_init(bFull(s), 1); mbar_init(bEmpty(s), 1); }
@@ -106,14 +106,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm_kernel(const GemmCell *
         }
       }
     }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     const uint32_t idesc = MODE == GM_TOK ? umma_idesc_f16(128, kp, 0, 0)
                          : MODE == GM_FEAT ? umma_idesc_f16(128, kp, 1, 0)
                                            : umma_idesc_f16(128, 128, 1, 1);
     bool ok = true;
     for (int j = 0; ok && j < n_steps; ++j) {
       const int s = j % n_stages, n = j / n_stages;
-      ok = mbar_wait(bFull(s), n & 1, abort_flag);
+      ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t st = sStages + s * stage_bytes;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm2_kernel(const Gemm2Cell
   auto bEmpty = [=](int s) { return sBar + 64 + 8 * s; };
   const uint32_t bDone = sBar + 128;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int s = 0; s < 8; ++s) { mbar_init(bFull(s), 1); mbar_init(bEmpty(s), 1); }
@@ -256,12 +256,12 @@ __global__ void __launch_bounds__(GM_THREADS, 1) tc_gemm2_kernel(const Gemm2Cell
         if (c.has_lo) tma_load_2d(st + a_bytes + b_pitch, &c.tmBlo, bFull(s), tok, 0);
       }
     }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     const uint32_t idesc = MODE == GM_TOK ? umma_idesc_f16(128, kp, 0, 0) : umma_idesc_f16(128, kp, 1, 0);
     bool ok = true;
     for (int j = 0; ok && j < n_steps; ++j) {
       const int s = j % n_stages, n = j / n_stages;
-      ok = mbar_wait(bFull(s), n & 1, abort_flag);
+      ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t st = sStages + s * stage_bytes;

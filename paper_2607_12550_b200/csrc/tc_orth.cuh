@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
   auto bAfull = [=](int b) { return sBar + 128 + 8 * b; };
   auto bAempty = [=](int b) { return sBar + 144 + 8 * b; };
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int s = 0; s < 8; ++s) { mbar_init(bFull(s), 1); mbar_init(bEmpty(s), 1); }
@@ -105,14 +105,14 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
       tma_load_3d(st, &c.tmHi, bFull(s), r0, 0, panel);
       tma_load_3d(st + tile, &c.tmLo, bFull(s), r0, 0, panel);
     }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     const uint32_t id0 = umma_idesc_f16(128, kp, 0, 0);
     const uint32_t id1 = umma_idesc_f16(128, n1 > 0 ? n1 : 16, 0, 0);
     bool ok = true;
     for (int j = 0; ok && j < n_steps; ++j) {
       const int s = j % n_stages, n = j / n_stages, b = j & 1, nb = j >> 1;
-      ok = mbar_wait(bFull(s), n & 1, abort_flag);
-      if (ok) ok = mbar_wait(bAempty(b), (nb & 1) ^ 1, abort_flag);
+      ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
+      if (ok) ok = mbar_wait_warp(bAempty(b), (nb & 1) ^ 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t hi = base + s * stage_bytes, lo = hi + tile;
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_apply_kernel(const OrthCel
   uint32_t *tmem_slot = (uint32_t *)(sm + bar_off + 72);
   const uint32_t bLoad = sBar, bDone = sBar + 8;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     mbar_init(bLoad, 1); mbar_init(bDone, 1);
@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_apply_kernel(const OrthCel
       tma_load_2d(sBhi + kb * tile, &c.tmLhi, bLoad, kb * 64, 0);
       tma_load_2d(sBlo + kb * tile, &c.tmLlo, bLoad, kb * 64, 0);
     }
-  } else if (warp == 5 && lane == 0) {
-    if (mbar_wait(bLoad, 0, abort_flag)) {
+  } else if (warp == 5) {
+    if (mbar_wait_warp(bLoad, 0, abort_flag)) {
       tc_fence_after();
       const uint32_t idesc = umma_idesc_f16(128, kp, 1, 0);
       for (int ks = 0; ks < kp / 16; ++ks) {

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(OW_THREADS, 1) orthw_gram_kernel(const OrthWCe
   auto bEmpty = [=](int s) { return sBar + 64 + 8 * s; };
   auto bAfull = [=](int b) { return sBar + 128 + 8 * b; };
   auto bAempty = [=](int b) { return sBar + 144 + 8 * b; };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int s = 0; s < OW_STAGES; ++s) { mbar_init(bFull(s), 1); mbar_init(bEmpty(s), 1); }
@@ -118,12 +118,12 @@ __global__ void __launch_bounds__(OW_THREADS, 1) orthw_gram_kernel(const OrthWCe
         tma_load_3d(st + 49152, &c.tmLo, bFull(s), r0, rb * 128, panel);
       }
     }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     const uint32_t idesc = umma_idesc_f16(128, 128, 0, 0);
     for (int j = 0; j < n_steps; ++j) {
       const int s = j % OW_STAGES, n = j / OW_STAGES, b = j & 1, q = j >> 1;
-      if (!mbar_wait(bFull(s), n & 1, abort_flag)) break;
-      if (!mbar_wait(bAempty(b), (q & 1) ^ 1, abort_flag)) break;
+      if (!mbar_wait_warp(bFull(s), n & 1, abort_flag)) break;
+      if (!mbar_wait_warp(bAempty(b), (q & 1) ^ 1, abort_flag)) break;
       tc_fence_after();
       const uint32_t bt = base + s * OW_STAGE_BYTES, at = diag ? bt : bt + 32768;
       const uint32_t d0 = tmem_base + b * 256, d1 = d0 + 128;
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(OW_THREADS, 1) orthw_apply_kernel(const OrthWC
   auto bEmpty = [=](int s) { return sBar + 64 + 8 * s; };
   auto bAfull = [=](int b) { return sBar + 128 + 8 * b; };
   auto bAempty = [=](int b) { return sBar + 144 + 8 * b; };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int s = 0; s < OW_STAGES; ++s) { mbar_init(bFull(s), 1); mbar_init(bEmpty(s), 1); }
@@ -232,19 +232,19 @@ __global__ void __launch_bounds__(OW_THREADS, 1) orthw_apply_kernel(const OrthWC
         tma_load_2d(st + 32768, &c.tmLhi, bFull(s), j * 64, cbk * 128);
         tma_load_2d(st + 49152, &c.tmLlo, bFull(s), j * 64, cbk * 128);
       }
-  } else if (warp == 5 && lane == 0) {
+  } else if (warp == 5) {
     const uint32_t idesc = umma_idesc_f16(128, 128, 1, 0);
     bool ok = true;
     int cnt = 0;
     for (int i = 0; ok && i < nb; ++i) {
       const int cbk = nb - 1 - i, b = i & 1, q = i >> 1, ns = steps_of(cbk);
-      ok = mbar_wait(bAempty(b), (q & 1) ^ 1, abort_flag);
+      ok = mbar_wait_warp(bAempty(b), (q & 1) ^ 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t d0 = tmem_base + b * 256, d1 = d0 + 128;
       for (int j = 0; j < ns; ++j, ++cnt) {
         const int s = cnt % OW_STAGES, n = cnt / OW_STAGES;
-        ok = mbar_wait(bFull(s), n & 1, abort_flag);
+        ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint32_t st = base + s * OW_STAGE_BYTES;
