@@ -274,7 +274,7 @@ inline void launch_split(Program &P, int stage, const std::vector<tc::SplitJob> 
   const size_t off = P.push(jobs);
   const int n = (int)jobs.size();
   P.add(stage, [=](char *dev_t, cudaStream_t s) {
-    tc::split_transpose_kernel<<<dim3(148, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + off));
+    tc::split_transpose_kernel<<<dim3(296, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + off));
     LAUNCHED();
   });
 }
@@ -506,7 +506,7 @@ inline void add_orth_split(Program &P, int stage, std::vector<CellWork> &ws, con
   const int n = (int)idx.size(), n_am = (int)am.size();
   P.add(stage, [=](char *dev_t, cudaStream_t s) {
     if (n_am) { tc::absmax_kernel<<<dim3(32, n_am), 256, 0, s>>>((const tc::AbsMaxJob *)(dev_t + o_am)); LAUNCHED(); }
-    tc::split_transpose_kernel<<<dim3(148, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + o_sp)); LAUNCHED();
+    tc::split_transpose_kernel<<<dim3(296, 1, n), 256, 0, s>>>((const tc::SplitJob *)(dev_t + o_sp)); LAUNCHED();
   });
 }
 
