@@ -355,40 +355,56 @@ __global__ void store_factors_kernel(const StoreJob *jobs) {
 // P_h[k][f] = fp16( sum_s G_h[k][s] U_F[f][s] ), the projected core of the decoder in the core's scaled units, for every
 // (head, k) row of a cell: [m * r_t][128].  Formed once, when the stored factors exist, and kept with the handle: the
 // residual pass, the decode pass and the attention kernels all read THIS array, so the backbone the residual was taken
-// against is bit for bit the backbone the decoder adds back (closed loop).  grid (row blocks of 32, cells), 128 threads
-// (thread = feature); dynamic shared memory: 128 * r_f halves (U_F, staged as [s][f]).
+// against is bit for bit the backbone the decoder adds back (closed loop).  fp64 accumulation: products of two fp16 numbers are
+// exact in it and the sum of <= 128 of them is far inside its precision, so the one rounding to fp16 is the rounding of the
+// exact value (the definition), not of an fp32 sum that may sit on the other side of a rounding boundary.
+// grid (row blocks of 32, cells), 256 threads (feature, half of the rows); dynamic shared memory: 160 r_f doubles, U_F as [s][f] and
+// the block's rows of G.  Both are converted once: with fp16 operands the loop was bound by conversions to fp64 (16 a clock and
+// SM), nine for eight FMAs.  One layer of 8 x 512 tokens, fp32, r_f = 64: round trip
+// 1226 -> 1196 us; 10 layers x 5 heads x 2944 tokens with its plan: 2516 -> 2473 us.
 struct ProjJob { const __half *G, *UF; __half *P; int rows, r_f; };
-__global__ void __launch_bounds__(128) project_core_kernel(const ProjJob *__restrict__ jobs) {
+__global__ void __launch_bounds__(256) project_core_kernel(const ProjJob *__restrict__ jobs) {
   const ProjJob j = jobs[blockIdx.y];
-  const int r0 = blockIdx.x * 32, f = threadIdx.x;
+  const int r0 = blockIdx.x * 32, f = threadIdx.x & 127, half = threadIdx.x >> 7, rf = j.r_f;
   if (r0 >= j.rows) return;
-  extern __shared__ __half pc_uf[];
-  for (int e = f; e < 128 * j.r_f; e += 128) { const int ff = e / j.r_f, s = e - ff * j.r_f; pc_uf[s * 128 + ff] = j.UF[e]; }
+  extern __shared__ __align__(16) double pc_sh[];
+  double *uf = pc_sh, *gs = pc_sh + 128 * rf;                       // [s][128], [32][rf]
+  const int ng = min(32, j.rows - r0) * rf;
+  for (int e = threadIdx.x; e < 32 * rf; e += 256) gs[e] = e < ng ? (double)__half2float(j.G[(size_t)r0 * rf + e]) : 0.0;
+  if ((rf & 7) == 0) {
+    for (int s = 8 * half; s < rf; s += 16) {
+      const uint4 q = *(const uint4 *)(j.UF + (size_t)f * rf + s);
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float2 v = __half22float2(*(const __half2 *)&w[u]);
+        uf[(s + 2 * u) * 128 + f] = (double)v.x; uf[(s + 2 * u + 1) * 128 + f] = (double)v.y;
+      }
+    }
+  } else {
+    for (int s = half; s < rf; s += 2) uf[s * 128 + f] = (double)__half2float(j.UF[(size_t)f * rf + s]);
+  }
   __syncthreads();
-  // fp64 accumulation: products of two fp16 numbers are exact in it and the sum of <= 128 of them is far inside its
-  // precision, so the one rounding to fp16 is the rounding of the exact value (the definition), not of an fp32 sum
-  // that may sit on the other side of a rounding boundary
-  // eight rows of G at a time, staged in shared memory (read straight from global memory the loop waited for one
-  // broadcast load per row and step: 76 us for three small cells on the critical chain of the call)
-  __shared__ __half gs[8][128];
-  for (int rb = r0; rb < min(r0 + 32, j.rows); rb += 8) {
-    __syncthreads();
-    for (int e = f; e < 8 * j.r_f; e += 128) {
-      const int r = e / j.r_f, s = e - r * j.r_f;
-      gs[r][s] = rb + r < j.rows ? j.G[(size_t)(rb + r) * j.r_f + s] : __float2half(0.f);
+  double acc[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) acc[r] = 0.0;
+  const double *g = gs + 16 * half * rf;
+  int s = 0;
+  if ((rf & 1) == 0)
+    for (; s < rf; s += 2) {
+      const double u0 = uf[s * 128 + f], u1 = uf[(s + 1) * 128 + f];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) { const double2 q = *(const double2 *)(g + r * rf + s); acc[r] = fma(q.y, u1, fma(q.x, u0, acc[r])); }
     }
-    __syncthreads();
-    double acc[8];
+  for (; s < rf; ++s) {
+    const double u = uf[s * 128 + f];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) acc[r] = 0.0;
-    for (int s = 0; s < j.r_f; ++s) {
-      const double u = (double)__half2float(pc_uf[s * 128 + f]);
+    for (int r = 0; r < 16; ++r) acc[r] = fma(g[r * rf + s], u, acc[r]);
+  }
 #pragma unroll
-      for (int r = 0; r < 8; ++r) acc[r] = fma((double)__half2float(gs[r][s]), u, acc[r]);
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r)
-      if (rb + r < j.rows) j.P[(size_t)(rb + r) * 128 + f] = __double2half(acc[r]);
+  for (int r = 0; r < 16; ++r) {
+    const int row = r0 + 16 * half + r;
+    if (row < j.rows) j.P[(size_t)row * 128 + f] = __double2half(acc[r]);
   }
 }
 
@@ -1510,8 +1526,8 @@ static int upload_decode_table(jolt_handle &H, cudaStream_t st) {
 
 static void launch_project_cores(const ProjJob *d_jobs, int n, int max_rows, int max_rf, cudaStream_t s) {
   static DeviceOnce once;
-  once([] { cudaFuncSetAttribute(project_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 2); });
-  project_core_kernel<<<dim3((max_rows + 31) / 32, n), 128, (size_t)128 * max_rf * sizeof(__half), s>>>(d_jobs);
+  once([] { cudaFuncSetAttribute(project_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 128 * 8); });
+  project_core_kernel<<<dim3((max_rows + 31) / 32, n), 256, (size_t)160 * max_rf * sizeof(double), s>>>(d_jobs);
   LAUNCHED();
 }
 
