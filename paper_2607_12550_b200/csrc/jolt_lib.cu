@@ -826,7 +826,7 @@ void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs) {
       for (int bj = 0; bj <= bi; ++bj)
         fastj[cls + (bi == bj ? 0 : 3)].push_back({j.M, j.rows, j.k, chunk, j.part, bi * bw, std::min(bw, j.k - bi * bw), bj * bw, std::min(bw, j.k - bj * bw), j.only});
     fast_chunks[cls] = std::max(fast_chunks[cls], n);
-    rj.push_back({j.part, j.out, n, j.k * j.k, j.only});
+    rj.push_back({j.part, j.out, n, j.k, j.only});
   }
   for (int q = 0; q < 6; ++q) {
     if (fastj[q].empty()) continue;
