@@ -199,16 +199,23 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
 
 // ---------------------------------------------------------------------------------------------- Cholesky + inverse
 // G = L L^T in fp64, one CTA per matrix, right-looking by panels of 8 columns, with X = L^-T formed by the same
-// panel operations on the rows of an identity appended below G ([G; I] = [L; X] L^T).  X is upper triangular and the
-// Schur complement only needs its lower triangle, so both live in one n x n array (column-major: lower triangle L,
-// upper triangle X, the diagonal of X in `invd`).  Per panel: (1) warp 0 factors the 8 x 8 diagonal block in
-// registers, (2) one thread per row solves its 8 panel entries against the block (rows above the panel are rows of X,
-// rows below are rows of L, the same recurrence), (3) the trailing update W[i][j] -= sum_c P[i][c] P[j][c] for the
-// rows of X (i < panel end) and of the Schur complement (i >= j), four columns per warp pass, while warp 0 updates and
-// factors the next diagonal block by itself (look-ahead).  Two barriers per panel.  98 -> 80 us a launch at n up to 138, 66 -> 47 at
-// n up to 106: square roots left the pivots' chain (1880 cycles a block), the separate update of the next eight columns and its
-// barrier are gone, 16 loads in flight.  The update is bound by shared memory: it reads and writes the trailing matrix once per
-// eight columns (2400 of its 2850 cycles at n = 138).
+// panel operations on the rows of an identity appended below G ([G; I] = [L; X] L^T).
+//
+// 8 x 8 tiles in shared memory, row by row of the lower triangle, the updates on fp64 matrix instructions.  Tile
+// (I, J), I >= J, of the Schur complement is finished when panel J is, and exactly then the tile (J, I) of X comes to life, so
+// one place serves both, and the living tiles of panel p are all those of the rows I > p.
+// Tiles hold the negative of the matrix: the update is then a plain product added.  An accumulator's two registers of a lane are
+// entries 2 c and 2 c + 1 of row r (lane = 4 r + c), 16 bytes of the row-major tile; taken as the k indices {2 c} and {2 c + 1} of two
+// k = 4 instructions they are an operand as they stand, of either side: no tile is ever rearranged.
+// Warp 0 owns the chain: it factors the 8 x 8 diagonal block (L D L^T in registers, every lane the whole block) and forms
+// its inverse Y = L^-T while twelve others update.  The rest of its quarter of the SM stays idle: a product there takes the fp64
+// pipe for 16 cycles, and the chain's dependent operations queue behind them.  Panel p, two barriers:
+//   solve    tiles of column p times Y (Schur rows below: rows of L; rows above: final rows of X), published
+//   update   every living tile; the owner of the next diagonal block does that one first and hands it to warp 0
+// What bounds it: the chain, 8 x (reciprocal, product, FMA) and the inverse, against 16 cycles of shared memory a tile.  The loops
+// are short on purpose: nothing runs more than a few times, and with tiles in registers (unrolled bodies, 40 KB of code) the fetch of the
+// instructions took as long as all the rest.  Against a matrix in shared memory updated by FMAs (two passes over it every eight
+// columns): round trip of 32 layers x 8 heads x 4096 tokens (four factorisations in its chain) 2164 -> 2069 us.
 // A pivot not above `dead_rel` of its original diagonal entry belongs to a direction that is dependent to working
 // accuracy: its column of L and its row / column of L^-1 are zero, status bit 1.
 // Input: fp32 row-chunk partials of the Gram kernel (summed here in fp64) or an fp64 matrix.  Output: L^-1 as fp16
@@ -226,225 +233,225 @@ struct CholInvTask {
 };
 constexpr int kCholInvThreads = 512;
 constexpr int kCholInvMaxN = 152;
-inline size_t cholinv_smem_bytes(int k) { return ((size_t)k * k + 8 * (size_t)k + 72 + 8 + 2 * (size_t)k + 64) * sizeof(double); }
+constexpr int kCholInvRows = kCholInvMaxN / 8;      // block rows
+constexpr int kCholInvWorkers = 12;
+inline size_t cholinv_smem_bytes(int k) {
+  const size_t nt = (k + 7) / 8;
+  return ((nt * (nt + 1) / 2 + 2 * kCholInvRows + 1) * 64 + kCholInvMaxN) * sizeof(double);
+}
+
+// 1 / d for d > 0: single-precision seed (relative error e below 2^-22) and one third-order step, 1 / d = y / (1 - e) = y (1 + e + e^2 + ..)
+__device__ __forceinline__ double rcp_pos(double d) {
+  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+  const double y = (double)__fdividef(1.0f, (float)d), e = fma(-d, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 
 __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholInvTask *__restrict__ tasks) {
   const CholInvTask t = tasks[blockIdx.x];
-  const int n = t.k, kp = t.kp;
+  const int n = t.k, kp = t.kp, NT = (n + 7) >> 3, n_tiles = NT * (NT + 1) / 2;
   if (n <= 0) return;
-  extern __shared__ double ci_sh[];
-  double *W = ci_sh;                        // element (row i, column j) at W[j * n + i]
-  double *pan = W + (size_t)n * n;          // [8][n] the solved panel: X values for rows up to the panel, L values below
-  double (*blkd)[9] = (double (*)[9])(pan + 8 * (size_t)n);
-  double *ipiv = (double *)(blkd + 8);      // [8]
-  double *diag0 = ipiv + 8;                 // [n] original diagonal
-  double *invd = diag0 + n;                 // [n] diagonal of X = 1 / L_ii (0 for a dead pivot)
-  __shared__ int s_red[32], s_dead;
-  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+  extern __shared__ __align__(16) double ci_sh[];
+  double2 *tile = (double2 *)ci_sh;                      // [tile][lane]; finished tiles (J, I) of X stay here
+  double2 *pan = tile + n_tiles * 32;                    // [2][block row][lane] solved tiles of a panel, by parity
+  double2 *ybuf = pan + 2 * kCholInvRows * 32;           // -Y as the right operand: its transpose
+  double *diag0 = (double *)(ybuf + 32);                 // original diagonal
+  __shared__ int s_red[kCholInvThreads / 32], s_dead;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = lane >> 2, c = lane & 3;
+  constexpr int NW = kCholInvThreads / 32;
+  auto row_start = [](int I) { return I * (I + 1) / 2; };
   if (tid == 0) s_dead = 0;
-  // a warp per column j, lanes over the rows i >= j: both the fp64 input (its upper triangle, (row j, column i): the
-  // matrix is symmetric) and the Gram partials are then read along contiguous addresses.  Entry (i, j) of the partials is
-  // read as (row j, column i), which is stored for every such pair (row j < 128 holds all columns; j >= 128 implies i >= 128);
-  // 64 rows of eight chunks in flight per warp (one SM reads it all: 13 us with 32, the largest part after the pivots).
-  for (int j = warp; j < n; j += nw) {
-    const size_t cs = (size_t)kp * kp;
-    for (int i0 = j + lane; i0 < n + lane; i0 += 64) {
-      const int q0 = min(i0, n - 1), q1 = min(i0 + 32, n - 1);
-      double v0 = 0.0, v1 = 0.0;
-      if (t.A64) { v0 = t.A64[(size_t)j * n + q0]; v1 = t.A64[(size_t)j * n + q1]; }
-      else {
-        const float *p = t.part + (size_t)j * kp;
-        int ch = 0;
-        for (; ch + 8 <= t.n_chunks; ch += 8) {
-          float x[8], y[8];
+  {
+    int I = 0, J = warp;
+    for (int q = warp; q < n_tiles; q += NW, J += NW) {
+      while (J > I) { J -= I + 1; ++I; }
+      double v[2] = {0.0, 0.0};
+      int at[2];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) { x[q] = __ldg(p + (size_t)(ch + q) * cs + q0); y[q] = __ldg(p + (size_t)(ch + q) * cs + q1); }
-          v0 += (((double)x[0] + (double)x[1]) + ((double)x[2] + (double)x[3])) + (((double)x[4] + (double)x[5]) + ((double)x[6] + (double)x[7]));
-          v1 += (((double)y[0] + (double)y[1]) + ((double)y[2] + (double)y[3])) + (((double)y[4] + (double)y[5]) + ((double)y[6] + (double)y[7]));
-        }
-        for (; ch < t.n_chunks; ++ch) { v0 += (double)__ldg(p + (size_t)ch * cs + q0); v1 += (double)__ldg(p + (size_t)ch * cs + q1); }
+      for (int e = 0; e < 2; ++e) {                      // entry (row, column) with row <= column: stored for every such pair
+        const int i = 8 * I + r, j = 8 * J + 2 * c + e, lo = min(i, j), hi = max(i, j);
+        at[e] = hi < n ? lo * (t.A64 ? n : kp) + hi : -1;
       }
-      if (i0 < n) W[(size_t)j * n + i0] = v0;
-      if (i0 + 32 < n) W[(size_t)j * n + i0 + 32] = v1;
+      if (t.A64) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) if (at[e] >= 0) v[e] = t.A64[at[e]];
+      } else {
+        const float *p = t.part;
+        const int cs = kp * kp;
+#pragma unroll 1
+        for (int ch = 0; ch < t.n_chunks; ch += 8, p += 8 * cs) {
+          float x[2][8];
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[e][u] = at[e] >= 0 && ch + u < t.n_chunks ? __ldg(p + u * cs + at[e]) : 0.f;
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            v[e] += (((double)x[e][0] + (double)x[e][1]) + ((double)x[e][2] + (double)x[e][3])) + (((double)x[e][4] + (double)x[e][5]) + ((double)x[e][6] + (double)x[e][7]));
+        }
+      }
+      tile[q * 32 + lane] = make_double2(-v[0], -v[1]);
+      if (I == J) {
+        if (2 * c == r) diag0[8 * I + r] = v[0];
+        if (2 * c + 1 == r) diag0[8 * I + r] = v[1];
+      }
     }
-    for (int i = lane; i < j; i += 32) W[(size_t)j * n + i] = 0.0;
   }
   __syncthreads();
-  for (int i = tid; i < n; i += nt) diag0[i] = W[(size_t)i * n + i];
-  __syncthreads();
-  // (1) the 8 x 8 diagonal block at j0 (in blkd): every lane of warp 0 factors it in registers as L D L^T -- a reciprocal, a
-  // product and an FMA per pivot on the dependent chain, 86 cycles where the square root took 170 -- lane c finds the
-  // reciprocal square root of pivot c, then the block and those are published
-  auto factor_block = [&](int j0) {
-    const int w = min(8, n - j0);
-    double Lb[8][8], mine = 0.0;
+  int mxh = 0;                                           // largest |X| so far: the high word of its fp64
+  if (warp & 3) {
+    const int wi = 3 * (warp >> 2) + (warp & 3) - 1;
+#pragma unroll 1
+    for (int p = 0; p < NT; ++p) {
+      __syncthreads();                                   // A: Y is in
+      double2 *pp = pan + (p & 1) * kCholInvRows * 32;
+      const double2 y = ybuf[lane];
+#pragma unroll 1
+      for (int q = wi; q < NT - 1; q += kCholInvWorkers) {      // block row q above the panel (X), q + 1 below it (L)
+        const bool above = q < p;
+        const int b = above ? q : q + 1;
+        double2 *w = tile + (above ? row_start(p) + q : row_start(b) + p) * 32 + lane;
+        double d[2] = {0.0, 0.0};
+        dmma(d, w->x, y.x);
+        dmma(d, w->y, y.y);
+        pp[b * 32 + lane] = make_double2(d[0], d[1]);
+        if (above) {                                     // final
+          *w = make_double2(d[0], d[1]);
+          mxh = max(mxh, max(__double2hiint(d[0]) & 0x7FFFFFFF, __double2hiint(d[1]) & 0x7FFFFFFF));
+        } else {                                         // the place is X's from here on
+          *w = make_double2(0.0, 0.0);
+          if (t.L64) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-      for (int cc = 0; cc <= r; ++cc) Lb[r][cc] = blkd[r][cc];
-    __syncwarp();
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const double d = Lb[cc][cc], dg = cc < w ? diag0[j0 + cc] : 0.0;
-      const bool bad = !(d > t.dead_rel * dg) || !(dg > 0);
-      const double inv = bad ? 0.0 : 1.0 / d;
-      if (lane == cc) mine = bad ? 0.0 : d;
-      double tr[8];
-#pragma unroll
-      for (int r = cc + 1; r < 8; ++r) tr[r] = Lb[r][cc] * inv;
-#pragma unroll
-      for (int c2 = cc + 1; c2 < 8; ++c2)
-#pragma unroll
-        for (int r = c2; r < 8; ++r) Lb[r][c2] = fma(-Lb[r][cc], tr[c2], Lb[r][c2]);
-    }
-    const double rs = mine > 0.0 ? rsqrt_pos(mine) : 0.0;
-    if (lane < w && mine == 0.0) s_dead = 1;
-    if (lane < 8) ipiv[lane] = rs;
-    __syncwarp();
-    double piv[8];
-#pragma unroll
-    for (int cc = 0; cc < 8; ++cc) piv[cc] = ipiv[cc];
-    if (lane < 8) {
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr)
-        if (rr == lane) {
-#pragma unroll
-          for (int cc = 0; cc < 8; ++cc) blkd[rr][cc] = cc <= rr ? Lb[rr][cc] * piv[cc] : 0.0;
-        }
-    }
-  };
-  if (warp == 0) {
-    for (int e = lane; e < 64; e += 32) { const int r = e & 7, c = e >> 3; blkd[r][c] = r < n && c <= r ? W[(size_t)c * n + r] : 0.0; }
-    __syncwarp();
-  }
-  if (warp == 0) factor_block(0);
-  __syncthreads();
-  int mxh = 0;                                 // largest |X| so far: the high word of its fp64
-  for (int j0 = 0; j0 < n; j0 += 8) {
-    const int w = min(8, n - j0);
-    // (2) the panel entries of every row: x_c = (p_c - sum_{l<c} x_l L[c][l]) / L[c][c]
-    for (int i = tid; i < n; i += nt) {
-      const int r = i - j0;                   // row inside the panel when 0 <= r < w
-      const bool inside = r >= 0 && r < w;
-      double x[8];
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) x[cc] = inside ? (cc == r ? 1.0 : 0.0) : (cc < w ? W[(size_t)(j0 + cc) * n + i] : 0.0);
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        if (cc < w) {
-          double a = x[cc];
-#pragma unroll
-          for (int l = 0; l < cc; ++l) a = fma(-x[l], blkd[cc][l], a);
-          x[cc] = a * ipiv[cc];
+            for (int e = 0; e < 2; ++e)
+              if (8 * b + r < n && 8 * p + 2 * c + e < n) t.L64[(size_t)(8 * p + 2 * c + e) * n + 8 * b + r] = d[e];
+          }
         }
       }
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        if (cc < w) {
-          pan[cc * n + i] = x[cc];
-          if (!inside) W[(size_t)(j0 + cc) * n + i] = x[cc];
-          else if (cc > r) W[(size_t)(j0 + cc) * n + i] = x[cc];              // row of X
-          else W[(size_t)(j0 + cc) * n + i] = blkd[r][cc];                    // row of L (diagonal included)
-          if (inside && cc == r) invd[i] = x[cc];
-          if (i < j0 + w && (!inside || cc >= r)) mxh = max(mxh, __double2hiint(x[cc]) & 0x7FFFFFFF);
-        }
+      __syncthreads();                                   // B: the panel is published
+      if (p + 1 == NT) break;
+      auto update = [&](int q, int I, int J) {           // Schur complement (J > p): P_I P_J^T; X (J, I): X_J P_I^T
+        const double2 f = pp[(J > p ? I : J) * 32 + lane], g = pp[(J > p ? J : I) * 32 + lane], w = tile[q * 32 + lane];
+        double d[2] = {w.x, w.y};
+        dmma(d, f.x, g.x);
+        dmma(d, f.y, g.y);
+        tile[q * 32 + lane] = make_double2(d[0], d[1]);
+      };
+      const int q0 = row_start(p + 1), next = q0 + p + 1;
+      if (wi == 0) {                                     // the next diagonal block, to the warp that factors it
+        update(next, p + 1, p + 1);
+        asm volatile("bar.arrive 1, 64;" ::: "memory");
+      }
+      int I = p + 1, J = wi;
+#pragma unroll 2
+      for (int q = q0 + wi; q < n_tiles; q += kCholInvWorkers, J += kCholInvWorkers) {
+        while (J > I) { J -= I + 1; ++I; }
+        if (q != next) update(q, I, J);
       }
     }
-    __syncthreads();
-    const int m0 = j0 + w;
-    if (m0 >= n) break;
-    // (1') warp 0 brings the next diagonal block up to date and factors it || (3) the other warps update the trailing columns,
-    // four per warp pass; rows i < m0 belong to X, rows i >= column to the Schur complement.  The next diagonal block's own
-    // entries in W are left as they are: warp 0 reads them meanwhile and nobody needs them afterwards.
-    const int wn = min(8, n - m0);
-    if (warp == 0) {
-      double bv[2];
+  } else if (warp) {
+    for (int p = 0; p < NT; ++p) { __syncthreads(); __syncthreads(); }
+  } else {
+    // ---------------- the chain
+#pragma unroll 1
+    for (int p = 0; p < NT; ++p) {
+      if (p > 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+      const int w = min(8, n - 8 * p), row = lane & 7;
+      double *const blk = (double *)(tile + (row_start(p) + p) * 32);
+      double Lb[8][8], mine = 0.0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) Lb[i][j] = -blk[i * 8 + j];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {          // L D L^T: below the diagonal the unit lower factor stays behind
+        const double d = Lb[q][q], dg = q < w ? diag0[8 * p + q] : 0.0;
+        const bool bad = !(d > t.dead_rel * dg) || !(dg > 0);
+        const double inv = bad ? 0.0 : rcp_pos(d);
+        if (row == q) mine = bad ? 0.0 : d;
+        double u[8];
+#pragma unroll
+        for (int i = q + 1; i < 8; ++i) u[i] = Lb[i][q] * inv;
+#pragma unroll
+        for (int j = q + 1; j < 8; ++j)
+#pragma unroll
+          for (int i = j; i < 8; ++i) Lb[i][j] = fma(-Lb[i][q], u[j], Lb[i][j]);
+#pragma unroll
+        for (int i = q + 1; i < 8; ++i) Lb[i][q] = u[i];
+      }
+      const double rs = mine > 0.0 ? rsqrt_pos(mine) : 0.0;
+      if (lane < w && mine == 0.0) s_dead = 1;
+      // row `row` of Y: the unit row times the inverse of the unit factor, then the pivots; a lane stores two columns of it
+      double z[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        z[j] = j == row ? 1.0 : 0.0;
+#pragma unroll
+        for (int l = 0; l < j; ++l) z[j] = fma(-z[l], Lb[j][l], z[j]);
+      }
+      const int j0 = 2 * (lane >> 3);
+      const bool h1 = lane & 8, h2 = lane & 16;
+      double v[2];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int e = lane + 32 * u, r = e & 7, c = e >> 3;
-        bv[u] = 0.0;
-        if (r < wn && c <= r) {
-          double a0 = W[(size_t)(m0 + c) * n + m0 + r], a1 = 0.0;
-#pragma unroll
-          for (int cc = 0; cc < 8; cc += 2) {
-            a0 = fma(-pan[cc * n + m0 + r], pan[cc * n + m0 + c], a0);
-            a1 = fma(-pan[(cc + 1) * n + m0 + r], pan[(cc + 1) * n + m0 + c], a1);
-          }
-          bv[u] = a0 + a1;
-        }
+        const double a = h1 ? z[2 + u] : z[u], b = h1 ? z[6 + u] : z[4 + u];
+        v[u] = (h2 ? b : a) * __shfl_sync(0xffffffffu, rs, j0 + u);
+        ((double *)ybuf)[(j0 + u) * 8 + row] = -v[u];
+        mxh = max(mxh, __double2hiint(v[u]) & 0x7FFFFFFF);
       }
-#pragma unroll
-      for (int u = 0; u < 2; ++u) { const int e = lane + 32 * u; blkd[e & 7][e >> 3] = bv[u]; }
+      pan[((p & 1) * kCholInvRows + p) * 32 + row * 4 + (j0 >> 1)] = make_double2(v[0], v[1]);
       __syncwarp();
-      factor_block(m0);
-    } else if (warp & 3) {                                     // (warp 0 has the fp64 pipe of its quarter of the SM to itself)
-      for (int j = m0 + 4 * (warp - 1 - (warp >> 2)); j < n; j += 4 * (nw - nw / 4)) {
-        double pj[4][8];
+      ((double2 *)blk)[row * 4 + (j0 >> 1)] = make_double2(v[0], v[1]);
+      if (t.L64) {
+        const double sd = mine * rs;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int j = 0; j < 8; ++j) {
+          const double sj = __shfl_sync(0xffffffffu, sd, j);
 #pragma unroll
-          for (int cc = 0; cc < 8; ++cc) pj[q][cc] = (j + q < n) ? pan[cc * n + j + q] : 0.0;
-        const int jr = j < m0 + 8 ? m0 + wn : j;               // first Schur row
-        const int nv = m0 + (n - jr);
-        for (int v = lane; v < nv; v += 32) {
-          const int i = v < m0 ? v : jr + (v - m0);
-          double acc[4] = {0, 0, 0, 0};
-#pragma unroll
-          for (int cc = 0; cc < 8; ++cc) {
-            const double pv = pan[cc * n + i];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] = fma(pv, pj[q][cc], acc[q]);
-          }
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (j + q < n && (i < m0 || i >= j + q)) W[(size_t)(j + q) * n + i] -= acc[q];
+          for (int i = j; i < 8; ++i)
+            if (lane == i && i < w) t.L64[(size_t)(8 * p + j) * n + 8 * p + i] = j == i ? sj : Lb[i][j] * sj;
         }
       }
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && s_dead && t.status) atomicOr(t.status, 2);
-  if (t.L64) {
-    for (int j = warp; j < n; j += nw)
-      for (int i = lane; i < n; i += 32) t.L64[(size_t)j * n + i] = i >= j ? W[(size_t)j * n + i] : 0.0;
-    if (tid == 0) {      // max |L_ij|^2 <= max G_ii: exponent for the single-precision Jacobi iteration
-      double mxd = 0.0;
-      for (int i = 0; i < n; ++i) mxd = fmax(mxd, diag0[i]);
-      int e2 = 0;
-      if (mxd > 0.0 && mxd < 1e300) frexp(mxd, &e2);
-      t.L64[(size_t)n * n] = (double)((e2 + 1) / 2 + 1);
+      __syncthreads();                                   // A
+      __syncthreads();                                   // B
     }
   }
-  if (!t.Lhi) return;
-  // ---- L^-1: (L^-1)_ic = X[c][i] for c < i, diagonal invd.  Scaled so that the largest entry lies in [2^9, 2^10).
   mxh = __reduce_max_sync(0xffffffffu, mxh);
   if (lane == 0) s_red[warp] = mxh;
   __syncthreads();
-  mxh = __reduce_max_sync(0xffffffffu, lane < nw ? s_red[lane] : 0);
+  if (tid == 0 && s_dead && t.status) atomicOr(t.status, 2);
+  if (t.L64) {
+    for (int j = warp; j < n; j += NW)
+      for (int i = lane; i < j; i += 32) t.L64[(size_t)j * n + i] = 0.0;
+    if (warp == 0) {     // max |L_ij|^2 <= max G_ii: exponent for the single-precision Jacobi iteration
+      double mxd = 0.0;
+      for (int i = lane; i < n; i += 32) mxd = fmax(mxd, diag0[i]);
+      for (int o = 16; o; o >>= 1) mxd = fmax(mxd, __shfl_xor_sync(0xffffffffu, mxd, o));
+      int e2 = 0;
+      if (mxd > 0.0 && mxd < 1e300) frexp(mxd, &e2);
+      if (lane == 0) t.L64[(size_t)n * n] = (double)((e2 + 1) / 2 + 1);
+    }
+  }
+  if (!t.Lhi) return;
+  // ---- L^-1: (L^-1)_ic = X[c][i] for c <= i.  Scaled so that the largest entry lies in [2^9, 2^10).
+  mxh = __reduce_max_sync(0xffffffffu, lane < NW ? s_red[lane] : 0);
   const int xe = (mxh >> 20) - 1023, le = mxh > 0 && xe < 1024 ? 9 - xe : 0;
   if (tid == 0) *t.l_exp = le;
   const double sc = ldexp(1.0, le);
-  for (int i = warp; i < kp; i += nw) {          // row i (output column of Q), a pair of columns (contraction index) per lane
-    float f[3][2];
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int cidx = 2 * lane + 64 * q + u;
-        double v = 0.0;
-        if (i < n && cidx < i) v = W[(size_t)i * n + cidx];
-        else if (i < n && cidx == i) v = invd[i];
-        f[q][u] = (float)(v * sc);
-      }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int c2 = 2 * lane + 64 * q;
-      if (c2 >= kp) continue;
-      const __half2 h = __floats2half2_rn(f[q][0], f[q][1]);
-      const float2 hf = __half22float2(h);
-      *(__half2 *)(t.Lhi + (size_t)i * kp + c2) = h;
-      *(__half2 *)(t.Llo + (size_t)i * kp + c2) = __floats2half2_rn(f[q][0] - hf.x, f[q][1] - hf.y);
-    }
+  const int nb = kp >> 3;
+#pragma unroll 2
+  for (int q = warp; q < nb * nb; q += NW) {             // rows 8 I .., columns 8 J .. of L^-1: the transpose of X (J, I)
+    const int I = q / nb, J = q - I * nb;
+    double2 x = make_double2(0.0, 0.0);
+    if (J <= I && I < NT) x = tile[(row_start(I) + J) * 32 + lane];
+    const float f0 = (float)(x.x * sc), f1 = (float)(x.y * sc);
+    // lanes r and r ^ 1 trade: the even one keeps column 2 c of X, the odd one column 2 c + 1, each a pair of rows
+    const bool odd = r & 1;
+    const float o = __shfl_xor_sync(0xffffffffu, odd ? f0 : f1, 4);
+    const __half2 h = odd ? __floats2half2_rn(o, f1) : __floats2half2_rn(f0, o);
+    const float2 hf = __half22float2(h);
+    const size_t at = (size_t)(8 * I + 2 * c + (odd ? 1 : 0)) * kp + 8 * J + (r & ~1);
+    *(__half2 *)(t.Lhi + at) = h;
+    *(__half2 *)(t.Llo + at) = odd ? __floats2half2_rn(o - hf.x, f1 - hf.y) : __floats2half2_rn(f0 - hf.x, o - hf.y);
   }
 }
 
