@@ -203,19 +203,24 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
 //
 // 8 x 8 tiles in shared memory, row by row of the lower triangle, the updates on fp64 matrix instructions.  Tile
 // (I, J), I >= J, of the Schur complement is finished when panel J is, and exactly then the tile (J, I) of X comes to life, so
-// one place serves both, and the living tiles of panel p are all those of the rows I > p.
-// Tiles hold the negative of the matrix: the update is then a plain product added.  An accumulator's two registers of a lane are
-// entries 2 c and 2 c + 1 of row r (lane = 4 r + c), 16 bytes of the row-major tile; taken as the k indices {2 c} and {2 c + 1} of two
-// k = 4 instructions they are an operand as they stand, of either side: no tile is ever rearranged.
-// Warp 0 owns the chain: it factors the 8 x 8 diagonal block (L D L^T in registers, every lane the whole block) and forms
-// its inverse Y = L^-T while twelve others update.  The rest of its quarter of the SM stays idle: a product there takes the fp64
+// one place serves both, and the living tiles of panel p are all those of the rows I > p.  Tiles hold the negative of the matrix.
+// An accumulator's two registers of a lane are entries 2 c and 2 c + 1 of row r (lane = 4 r + c), 16 bytes of the row-major tile; the pairs
+// of rows 2 i and 2 i + 1 are stored exchanged by i (pair c in place c ^ i), so that a lane per row reads its eight entries without
+// bank conflicts too.  The solved panel is kept as pairs (c, c + 4): the operand of two k = 4 instructions, columns 0 .. 3 and 4 .. 7.
+// Warp 0 owns the chain: it brings the next 8 x 8 diagonal block up to date and factors it (L D L^T in registers, every lane the whole
+// block) while twelve others update.  The rest of its quarter of the SM stays idle: a product there takes the fp64
 // pipe for 16 cycles, and the chain's dependent operations queue behind them.  Panel p, two barriers:
-//   solve    tiles of column p times Y (Schur rows below: rows of L; rows above: final rows of X), published
-//   update   every living tile; the owner of the next diagonal block does that one first and hands it to warp 0
-// What bounds it: the chain, 8 x (reciprocal, product, FMA) and the inverse, against 16 cycles of shared memory a tile.  The loops
-// are short on purpose: nothing runs more than a few times, and with tiles in registers (unrolled bodies, 40 KB of code) the fetch of the
-// instructions took as long as all the rest.  Against a matrix in shared memory updated by FMAs (two passes over it every eight
-// columns): round trip of 32 layers x 8 heads x 4096 tokens (four factorisations in its chain) 2164 -> 2069 us.
+//   solve    a thread per row, substitution against the block: rows of L below it, final rows of X above it; published
+//   update   every living tile but the next diagonal block; its eight products are summed first and then subtracted
+// The order of the operations is that of a matrix in shared memory updated by FMAs, one rounding each (the matrix instruction is four
+// FMAs in the order of k, the reciprocal is correctly rounded), and so are the results, bit for bit.  Multiplying the panel by the explicit inverse
+// of the block instead is 5 us shorter at n = 138 but not as good: the residual of L L^T in units of 2^-53 of the diagonal, 1081 against 3.2
+// where neighbouring columns are close (n = 74), 7.6 against 4.1 on a graded matrix.
+// What bounds it: fp64 operations and their latency: the chain, 8 x (estimate, five FMAs, product, FMA) and the substitution, and
+// at n > 100 the products of the early panels.  The loops are short on purpose: nothing runs more than a few times, and with tiles in
+// registers (unrolled bodies, 40 KB of code) the fetch of the instructions took as long as all the rest.  One matrix of n = 138 / 74 / 26 alone:
+// 53 / 22 / 10 us, the same from 32 partial Grams 78 / 29 / 11 us; updates by FMAs (two passes over the matrix every eight
+// columns) 78 / 34 / 15 and 103 / 43 / 19 us.
 // A pivot not above `dead_rel` of its original diagonal entry belongs to a direction that is dependent to working
 // accuracy: its column of L and its row / column of L^-1 are zero, status bit 1.
 // Input: fp32 row-chunk partials of the Gram kernel (summed here in fp64) or an fp64 matrix.  Output: L^-1 as fp16
@@ -237,14 +242,19 @@ constexpr int kCholInvRows = kCholInvMaxN / 8;      // block rows
 constexpr int kCholInvWorkers = 12;
 inline size_t cholinv_smem_bytes(int k) {
   const size_t nt = (k + 7) / 8;
-  return ((nt * (nt + 1) / 2 + 2 * kCholInvRows + 1) * 64 + kCholInvMaxN) * sizeof(double);
+  return ((nt * (nt + 1) / 2 + kCholInvRows + 2) * 64 + 8 + kCholInvMaxN) * sizeof(double);
 }
 
-// 1 / d for d > 0: single-precision seed (relative error e below 2^-22) and one third-order step, 1 / d = y / (1 - e) = y (1 + e + e^2 + ..)
+// 1 / d, correctly rounded, for 2^-1000 < d < 2^1000: the hardware's estimate (relative error e of 2^-20 or less), one third-order step,
+// 1 / d = y / (1 - e) = y (1 + e + e^2 + ..), which is good to a unit in the last place, and one of Newton's, which rounds such a number
+// correctly (Markstein 1990; all ones in d's fraction excepted).
 __device__ __forceinline__ double rcp_pos(double d) {
-  if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
-  const double y = (double)__fdividef(1.0f, (float)d), e = fma(-d, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  double e = fma(-d, y, 1.0);
+  y = fma(y, fma(e, e, e), y);
+  e = fma(-d, y, 1.0);
+  return fma(y, e, y);
 }
 
 __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholInvTask *__restrict__ tasks) {
@@ -252,12 +262,14 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
   const int n = t.k, kp = t.kp, NT = (n + 7) >> 3, n_tiles = NT * (NT + 1) / 2;
   if (n <= 0) return;
   extern __shared__ __align__(16) double ci_sh[];
-  double2 *tile = (double2 *)ci_sh;                      // [tile][lane]; finished tiles (J, I) of X stay here
-  double2 *pan = tile + n_tiles * 32;                    // [2][block row][lane] solved tiles of a panel, by parity
-  double2 *ybuf = pan + 2 * kCholInvRows * 32;           // -Y as the right operand: its transpose
-  double *diag0 = (double *)(ybuf + 32);                 // original diagonal
+  double2 *tile = (double2 *)ci_sh;                      // [tile][row][pair of columns]; finished tiles (J, I) of X stay here
+  double2 *pan = tile + n_tiles * 32;                    // [row][pair c, c + 4] the solved panel
+  double *blk = (double *)(pan + kCholInvRows * 32);     // [8][8] the next diagonal block, and its factor
+  double *lb = blk + 64, *ipiv = lb + 64;                // ... 1 / L_qq (0 for a dead pivot)
+  double *diag0 = ipiv + 8;                              // original diagonal
   __shared__ int s_red[kCholInvThreads / 32], s_dead;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = lane >> 2, c = lane & 3;
+  const int at_lane = lane ^ (lane >> 3);                // pair c of row r of a tile
   constexpr int NW = kCholInvThreads / 32;
   auto row_start = [](int I) { return I * (I + 1) / 2; };
   if (tid == 0) s_dead = 0;
@@ -286,11 +298,14 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[e][u] = at[e] >= 0 && ch + u < t.n_chunks ? __ldg(p + u * cs + at[e]) : 0.f;
 #pragma unroll
-          for (int e = 0; e < 2; ++e)
-            v[e] += (((double)x[e][0] + (double)x[e][1]) + ((double)x[e][2] + (double)x[e][3])) + (((double)x[e][4] + (double)x[e][5]) + ((double)x[e][6] + (double)x[e][7]));
+          for (int e = 0; e < 2; ++e) {
+            const double x0 = x[e][0], x1 = x[e][1], x2 = x[e][2], x3 = x[e][3], x4 = x[e][4], x5 = x[e][5], x6 = x[e][6], x7 = x[e][7];
+            if (ch + 8 <= t.n_chunks) v[e] += ((x0 + x1) + (x2 + x3)) + ((x4 + x5) + (x6 + x7));
+            else v[e] = ((((((v[e] + x0) + x1) + x2) + x3) + x4) + x5) + x6;
+          }
         }
       }
-      tile[q * 32 + lane] = make_double2(-v[0], -v[1]);
+      tile[q * 32 + at_lane] = make_double2(-v[0], -v[1]);
       if (I == J) {
         if (2 * c == r) diag0[8 * I + r] = v[0];
         if (2 * c + 1 == r) diag0[8 * I + r] = v[1];
@@ -303,49 +318,60 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
     const int wi = 3 * (warp >> 2) + (warp & 3) - 1;
 #pragma unroll 1
     for (int p = 0; p < NT; ++p) {
-      __syncthreads();                                   // A: Y is in
-      double2 *pp = pan + (p & 1) * kCholInvRows * 32;
-      const double2 y = ybuf[lane];
-#pragma unroll 1
-      for (int q = wi; q < NT - 1; q += kCholInvWorkers) {      // block row q above the panel (X), q + 1 below it (L)
-        const bool above = q < p;
-        const int b = above ? q : q + 1;
-        double2 *w = tile + (above ? row_start(p) + q : row_start(b) + p) * 32 + lane;
-        double d[2] = {0.0, 0.0};
-        dmma(d, w->x, y.x);
-        dmma(d, w->y, y.y);
-        pp[b * 32 + lane] = make_double2(d[0], d[1]);
-        if (above) {                                     // final
-          *w = make_double2(d[0], d[1]);
-          mxh = max(mxh, max(__double2hiint(d[0]) & 0x7FFFFFFF, __double2hiint(d[1]) & 0x7FFFFFFF));
-        } else {                                         // the place is X's from here on
-          *w = make_double2(0.0, 0.0);
-          if (t.L64) {
+      __syncthreads();                                   // A: the block is factored
+      const int i = wi * 32 + lane, b = i >> 3, rr = i & 7, s2 = rr >> 1;
+      if (b < NT) {                                      // x_j = (p_j - sum_{l<j} x_l L_jl) / L_jj
+        const bool below = b > p;
+        double2 *w = tile + (below ? row_start(b) + p : row_start(p) + b) * 32 + rr * 4;
+        double x[8];
 #pragma unroll
-            for (int e = 0; e < 2; ++e)
-              if (8 * b + r < n && 8 * p + 2 * c + e < n) t.L64[(size_t)(8 * p + 2 * c + e) * n + 8 * b + r] = d[e];
+        for (int j = 0; j < 4; ++j) { const double2 q = w[j ^ s2]; x[2 * j] = -q.x; x[2 * j + 1] = -q.y; }
+        if (b == p) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[j] = j == rr ? 1.0 : 0.0;
+        }
+        double2 f[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = ((const double2 *)ipiv)[j];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+#pragma unroll
+          for (int l = 0; l < j; l += 2) {
+            const double2 q = ((const double2 *)lb)[4 * j + (l >> 1)];
+            x[j] = fma(-x[l], q.x, x[j]);
+            if (l + 1 < j) x[j] = fma(-x[l + 1], q.y, x[j]);
           }
+          x[j] *= j & 1 ? f[j >> 1].y : f[j >> 1].x;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          pan[i * 4 + (j ^ s2)] = make_double2(x[j], x[j + 4]);
+          w[j ^ s2] = below ? make_double2(0.0, 0.0) : make_double2(x[2 * j], x[2 * j + 1]);      // X's from here on / final
+        }
+        if (!below) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) mxh = max(mxh, __double2hiint(x[j]) & 0x7FFFFFFF);
+        }
+        if (t.L64 && b >= p && i < n) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (below || j <= rr) t.L64[(size_t)(8 * p + j) * n + i] = below ? x[j] : lb[8 * rr + j];
         }
       }
       __syncthreads();                                   // B: the panel is published
       if (p + 1 == NT) break;
-      auto update = [&](int q, int I, int J) {           // Schur complement (J > p): P_I P_J^T; X (J, I): X_J P_I^T
-        const double2 f = pp[(J > p ? I : J) * 32 + lane], g = pp[(J > p ? J : I) * 32 + lane], w = tile[q * 32 + lane];
-        double d[2] = {w.x, w.y};
-        dmma(d, f.x, g.x);
-        dmma(d, f.y, g.y);
-        tile[q * 32 + lane] = make_double2(d[0], d[1]);
-      };
-      const int q0 = row_start(p + 1), next = q0 + p + 1;
-      if (wi == 0) {                                     // the next diagonal block, to the warp that factors it
-        update(next, p + 1, p + 1);
-        asm volatile("bar.arrive 1, 64;" ::: "memory");
-      }
+      const int q0 = row_start(p + 1), next = q0 + p + 1;      // (the next diagonal block is warp 0's)
       int I = p + 1, J = wi;
 #pragma unroll 2
       for (int q = q0 + wi; q < n_tiles; q += kCholInvWorkers, J += kCholInvWorkers) {
         while (J > I) { J -= I + 1; ++I; }
-        if (q != next) update(q, I, J);
+        if (q == next) continue;
+        // Schur complement (J > p): P_I P_J^T; X (J, I): X_J P_I^T
+        const double2 f = pan[(J > p ? I : J) * 32 + at_lane], g = pan[(J > p ? J : I) * 32 + at_lane], w = tile[q * 32 + at_lane];
+        double d[2] = {0.0, 0.0};
+        dmma(d, f.x, g.x);
+        dmma(d, f.y, g.y);
+        tile[q * 32 + at_lane] = make_double2(w.x + d[0], w.y + d[1]);
       }
     }
   } else if (warp) {
@@ -354,20 +380,34 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
     // ---------------- the chain
 #pragma unroll 1
     for (int p = 0; p < NT; ++p) {
-      if (p > 0) asm volatile("bar.sync 1, 64;" ::: "memory");
-      const int w = min(8, n - 8 * p), row = lane & 7;
-      double *const blk = (double *)(tile + (row_start(p) + p) * 32);
+      const double2 w0 = tile[(row_start(p) + p) * 32 + at_lane];
+      double a0[2] = {w0.x, w0.y};
+      if (p > 0) {                                       // columns 0, 2, 4, 6 of the panel, and 1, 3, 5, 7
+        const double *q = (const double *)(pan + (8 * p + r) * 4) + (c >> 1);
+        const double ev = q[2 * ((2 * (c & 1)) ^ (r >> 1))], od = q[2 * ((2 * (c & 1) + 1) ^ (r >> 1))];
+        double a1[2] = {0.0, 0.0};
+        dmma(a0, ev, ev);
+        dmma(a1, od, od);
+        a0[0] += a1[0]; a0[1] += a1[1];
+      }
+      __syncwarp();
+      ((double2 *)blk)[lane] = make_double2(a0[0], a0[1]);
+      __syncwarp();
+      const int w = min(8, n - 8 * p);
       double Lb[8][8], mine = 0.0;
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j <= i; ++j) Lb[i][j] = -blk[i * 8 + j];
+      __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {          // L D L^T: below the diagonal the unit lower factor stays behind
+      for (int q = 0; q < 8; ++q) {          // L D L^T, the columns not yet divided by their pivots
         const double d = Lb[q][q], dg = q < w ? diag0[8 * p + q] : 0.0;
         const bool bad = !(d > t.dead_rel * dg) || !(dg > 0);
         const double inv = bad ? 0.0 : rcp_pos(d);
-        if (row == q) mine = bad ? 0.0 : d;
+        if (lane == q) mine = bad ? 0.0 : d;
+#pragma unroll
+        for (int i = q; i < 8; ++i) if (lane == 0) blk[8 * i + q] = Lb[i][q];
         double u[8];
 #pragma unroll
         for (int i = q + 1; i < 8; ++i) u[i] = Lb[i][q] * inv;
@@ -375,41 +415,14 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
         for (int j = q + 1; j < 8; ++j)
 #pragma unroll
           for (int i = j; i < 8; ++i) Lb[i][j] = fma(-Lb[i][q], u[j], Lb[i][j]);
-#pragma unroll
-        for (int i = q + 1; i < 8; ++i) Lb[i][q] = u[i];
       }
       const double rs = mine > 0.0 ? rsqrt_pos(mine) : 0.0;
       if (lane < w && mine == 0.0) s_dead = 1;
-      // row `row` of Y: the unit row times the inverse of the unit factor, then the pivots; a lane stores two columns of it
-      double z[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        z[j] = j == row ? 1.0 : 0.0;
-#pragma unroll
-        for (int l = 0; l < j; ++l) z[j] = fma(-z[l], Lb[j][l], z[j]);
-      }
-      const int j0 = 2 * (lane >> 3);
-      const bool h1 = lane & 8, h2 = lane & 16;
-      double v[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const double a = h1 ? z[2 + u] : z[u], b = h1 ? z[6 + u] : z[4 + u];
-        v[u] = (h2 ? b : a) * __shfl_sync(0xffffffffu, rs, j0 + u);
-        ((double *)ybuf)[(j0 + u) * 8 + row] = -v[u];
-        mxh = max(mxh, __double2hiint(v[u]) & 0x7FFFFFFF);
-      }
-      pan[((p & 1) * kCholInvRows + p) * 32 + row * 4 + (j0 >> 1)] = make_double2(v[0], v[1]);
+      if (lane < 8) ipiv[lane] = rs;
       __syncwarp();
-      ((double2 *)blk)[row * 4 + (j0 >> 1)] = make_double2(v[0], v[1]);
-      if (t.L64) {
-        const double sd = mine * rs;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const double sj = __shfl_sync(0xffffffffu, sd, j);
-#pragma unroll
-          for (int i = j; i < 8; ++i)
-            if (lane == i && i < w) t.L64[(size_t)(8 * p + j) * n + 8 * p + i] = j == i ? sj : Lb[i][j] * sj;
-        }
+      {
+        const double2 x = ((const double2 *)blk)[lane], f = ((const double2 *)ipiv)[c];
+        ((double2 *)lb)[lane] = make_double2(x.x * f.x, x.y * f.y);
       }
       __syncthreads();                                   // A
       __syncthreads();                                   // B
@@ -442,7 +455,7 @@ __global__ void __launch_bounds__(kCholInvThreads, 1) cholinv_kernel(const CholI
   for (int q = warp; q < nb * nb; q += NW) {             // rows 8 I .., columns 8 J .. of L^-1: the transpose of X (J, I)
     const int I = q / nb, J = q - I * nb;
     double2 x = make_double2(0.0, 0.0);
-    if (J <= I && I < NT) x = tile[(row_start(I) + J) * 32 + lane];
+    if (J <= I && I < NT) x = tile[(row_start(I) + J) * 32 + at_lane];
     const float f0 = (float)(x.x * sc), f1 = (float)(x.y * sc);
     // lanes r and r ^ 1 trade: the even one keeps column 2 c of X, the odd one column 2 c + 1, each a pair of rows
     const bool odd = r & 1;
