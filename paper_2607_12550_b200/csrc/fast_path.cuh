@@ -109,7 +109,10 @@ inline void launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size
 inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc::DecOut &out, const float2 *rope, long long *dbg, bool overlap, cudaStream_t s) {
   using LY = tc::DecLayout;
   static DeviceOnce once;
-  once([] { cudaFuncSetAttribute(tc::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES); });
+  once([] {
+    cudaFuncSetAttribute(tc::decode_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
+    cudaFuncSetAttribute(tc::decode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, LY::SMEM_BYTES);
+  });
   tc::DecIArgs a;
   memset(&a, 0, sizeof a);
   a.out = out; a.cells = (const tc::BBCell *)H->d_dec + first; a.rope = rope; a.seed = H->seed;
@@ -122,8 +125,9 @@ inline void launch_decode_items(const jolt_handle *H, int first, int n, const tc
   for (int i = first; i < first + n; ++i) { heads += H->dec.m[i]; m_max = std::max(m_max, H->dec.m[i]); }
   bb_split(heads, H->T / 128, a.tiles_per_item, a.items_per_head);
   const dim3 grid(m_max * a.items_per_head, n);
-  if (overlap) launch_overlapped(tc::decode_kernel, grid, LY::THREADS, LY::SMEM_BYTES, s, a);
-  else tc::decode_kernel<<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
+  const auto kernel = rope ? tc::decode_kernel<true> : tc::decode_kernel<false>;
+  if (overlap) launch_overlapped(kernel, grid, LY::THREADS, LY::SMEM_BYTES, s, a);
+  else kernel<<<grid, LY::THREADS, LY::SMEM_BYTES, s>>>(a);
   LAUNCHED();
 }
 

@@ -321,7 +321,10 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   auto bRready = [=](int b) { return sBar + 184 + 8 * b; };
   auto bBB = [=](int b) { return sBar + 216 + 8 * b; };           // backbone of the accumulator's tile complete
 
-  const int warp = warp_uniform(), lane = threadIdx.x & 31;
+  // The warp number as one value per warp (a shuffle) leaves the tile loops of 4 and 8 bits without spills, and adds some to the others:
+  // 32 layers x 8 heads x 4096 tokens at 2x 205.6 -> 203.1 us, keys rotated 276 -> 273; with it, 2 bits everywhere took 107 instead of
+  // 100 us (16 layers), one layer of 128 tokens 8.7 instead of 8.2.
+  const int warp = BITMASK == 272u ? warp_uniform() : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int wg = warp >> 2;
   BBCell *sc_cell = (BBCell *)(smBar + 512);      // the epilogue's copy of the current cell's descriptor
 
@@ -417,7 +420,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
         }
         ci = min(w.ci, a.n_cells - 1);
       }
-    } else if (warp == NWG * 4 + 1) {
+    } else if (warp == NWG * 4 + 1 && lane == 0) {
       // ---------------- backbone MMA issuer
       const uint32_t idescB = umma_idesc_f16(128, 128, 0, 1);     // A = U_T tile, K-major; B = P panels, MN-major
       const uint64_t dS0 = umma_desc_sw128(sRing, 16, 1024);
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
       bool ok = true;
       for (int k = 0; ok; ++k) {
         int first = run0_first, end = run0_end;
-        if (k >= 1) { ok = __all_sync(0xffffffffu, runq.get(k, first, end)); if (!ok || first >= total) break; }
+        if (k >= 1) { ok = runq.get(k, first, end); if (!ok || first >= total) break; }
         int left = end - first;
         if (left <= 0) continue;
         DecPos w = dec_locate(cells, a.n_cells, nt, first, ci);
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           const BBCell &cg = cells[w.ci];
           const int r_t = cg.r_t, nkt = (r_t + 63) / 64, ksteps = r_t / 16, m = cg.m;
           const uint32_t panel = (uint32_t)r_t * 128u;
-          ok = mbar_wait_warp(bSetup, seg & 1, abort_flag);      // the head's projected core has landed
+          ok = mbar_wait(bSetup, seg & 1, abort_flag);      // the head's projected core has landed
           if (!ok) break;
           tc_fence_after();
           const uint64_t dP0 = umma_desc_sw128(sP, panel, 1024);
@@ -442,32 +445,32 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           for (int i = 0; ok && i < len; ++i, ++j) {
             int b, nb;
             dec_acc_of(j, b, nb);
-            ok = mbar_wait_warp(bTempty(b), (nb & 1) ^ 1, abort_flag);
+            ok = mbar_wait(bTempty(b), (nb & 1) ^ 1, abort_flag);
             if (!ok) break;
             tc_fence_after();
             const uint32_t tacc = tmem_base + b * 128;
             for (int kb = 0; kb < nkt; ++kb, ++cnt) {
               const int s = cnt % NS, n = cnt / NS;
-              ok = mbar_wait_warp(bFull(s), n & 1, abort_flag);
+              ok = mbar_wait(bFull(s), n & 1, abort_flag);
               if (!ok) break;
               tc_fence_after();
               const uint64_t da = dS0 + (uint64_t)s * kStep16K;
               const uint64_t db = dP0 + (uint64_t)kb * (8192 >> 4);
 #pragma unroll
               for (int k4 = 0; k4 < 4; ++k4)
-                if (kb * 4 + k4 < ksteps) umma_f16(tacc, umma_desc_kslice(da, k4), db + (uint64_t)k4 * (2048 >> 4), idescB, (kb | k4) != 0);
-              umma_commit(bEmpty(s));
+                if (kb * 4 + k4 < ksteps) umma_f16_lane(tacc, umma_desc_kslice(da, k4), db + (uint64_t)k4 * (2048 >> 4), idescB, (kb | k4) != 0);
+              umma_commit_lane(bEmpty(s));
             }
-            if (ok) umma_commit(bBB(b));
+            if (ok) umma_commit_lane(bBB(b));
           }
-          if (ok) umma_commit(bPfree);
+          if (ok) umma_commit_lane(bPfree);
           left -= len; ++seg;
           w.tile = 0;
           if (++w.h >= m) { w.h = 0; ++w.ci; }
         }
         ci = min(w.ci, a.n_cells - 1);
       }
-    } else if (warp == NWG * 4 + 2) {
+    } else if (warp == NWG * 4 + 2 && lane == 0) {
       // ---------------- rotation MMA issuer: A = the warpgroup's dequantised residual tile, B = H of the current cell
       const uint32_t idesc = umma_idesc_f16(128, 128, 0, 0);
       const uint64_t dH0 = umma_desc_sw128(sH, 16, 1024), dR0 = umma_desc_sw128(sR, 16, 1024);
@@ -479,7 +482,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
       bool ok = true;
       for (int k = 0; ok; ++k) {
         int p = run0_first, end = run0_end;
-        if (k >= 1) { ok = __all_sync(0xffffffffu, runq.get(k, p, end)); if (!ok || p >= total) break; }
+        if (k >= 1) { ok = runq.get(k, p, end); if (!ok || p >= total) break; }
         if (p >= end) continue;
         ci = dec_locate(cells, a.n_cells, nt, p, ci).ci;
         while (ok && p < end) {
@@ -487,7 +490,7 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           const bool has_res = cg.bits > 0;
           const int cell_end = min(end, cg.tile_base + cg.m * nt);
           if (ci != cur_ci) {
-            ok = mbar_wait_warp(bHready, n_built & 1, abort_flag);      // the cell's rotation operand is built
+            ok = mbar_wait(bHready, n_built & 1, abort_flag);      // the cell's rotation operand is built
             if (!ok) break;
             tc_fence_after();
             cur_ci = ci; ++n_built;
@@ -495,8 +498,8 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
           for (; ok && p < cell_end; ++p, ++j) {
             int b, nb;
             dec_acc_of(j, b, nb);
-            ok = mbar_wait_warp(bBB(b), nb & 1, abort_flag);          // the tile's backbone is in the accumulator
-            if (ok) ok = mbar_wait_warp(bRready(b), nb & 1, abort_flag);      // ... and its residual operand is unpacked
+            ok = mbar_wait(bBB(b), nb & 1, abort_flag);          // the tile's backbone is in the accumulator
+            if (ok) ok = mbar_wait(bRready(b), nb & 1, abort_flag);      // ... and its residual operand is unpacked
             if (!ok) break;
             if (has_res) {
               tc_fence_after();
@@ -504,9 +507,9 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
               const uint64_t dR = dR0 + (uint64_t)(j & 1) * kStep32K;
 #pragma unroll
               for (int ks = 0; ks < 8; ++ks)
-                umma_f16(tacc, umma_desc_kslice(dR + (uint64_t)(ks >> 2) * kStep16K, ks & 3), dH[ks], idesc, 1);
+                umma_f16_lane(tacc, umma_desc_kslice(dR + (uint64_t)(ks >> 2) * kStep16K, ks & 3), dH[ks], idesc, 1);
             }
-            umma_commit(bTfull(b));
+            umma_commit_lane(bTfull(b));
           }
           if (p >= cg.tile_base + cg.m * nt) ++ci;
         }
