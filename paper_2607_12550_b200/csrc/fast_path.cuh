@@ -250,10 +250,10 @@ inline void launch_tc_gemm2(Program &P, int stage, std::vector<tc::Gemm2Cell> &c
   uint32_t max_stage = 0;
   int gx = 0;
   for (auto &c : cells) {
-    max_stage = std::max(max_stage, 32768u + (c.has_lo ? 2u : 1u) * (uint32_t)c.kp * 64u);
+    const uint32_t b_pitch = ((uint32_t)c.kp * 128u + 1023u) & ~1023u;
+    max_stage = std::max(max_stage, 32768u + (c.has_lo ? 2 * b_pitch : b_pitch));
     gx = std::max(gx, MODE == tc::GM_TOK ? (c.T / 128 + 1) / 2 : c.m / 2);
   }
-  gx = (gx + 1) & ~1;                  // pairs of CTAs
   const int n_stages = std::min(8, (int)((tc::GM_SMEM_LIMIT - 1536) / max_stage));
   const size_t smem = (size_t)n_stages * max_stage + 1024 + 512;
   static DeviceOnce once;
@@ -348,7 +348,7 @@ inline void add_tok_tc(Program &P, int stage, std::vector<CellWork> &ws, const s
         memset(&g, 0, sizeof g);
         const uint64_t dims[3] = {(uint64_t)kD, (uint64_t)kc, (uint64_t)c.m};
         const uint64_t str[2] = {(uint64_t)kD * 2, (uint64_t)w.kp * kD * 2};
-        const uint32_t box[3] = {64, (uint32_t)kc / 2, 1};
+        const uint32_t box[3] = {64, (uint32_t)kc, 1};
         bool okm = make_x_map4(&g.tmX, c, 256, 1) && make_tmap_f16(&g.tmBhi, w.Bhi + (size_t)c0 * kD, 3, dims, str, box) &&
                    make_tmap_f16(&g.tmBlo, w.Blo + (size_t)c0 * kD, 3, dims, str, box);
         (void)okm;
@@ -410,7 +410,7 @@ inline void add_feat_tc(Program &P, int stage, std::vector<CellWork> &ws) {
         memset(&g, 0, sizeof g);
         const uint64_t dims[2] = {(uint64_t)c.T, (uint64_t)kc};
         const uint64_t str[1] = {(uint64_t)c.T * 2};
-        const uint32_t box[2] = {64, (uint32_t)kc / 2};
+        const uint32_t box[2] = {64, (uint32_t)kc};
         bool okm = make_x_map4(&g.tmX, c, 64, 2) && make_tmap_f16(&g.tmBhi, w.Bhi + (size_t)c0 * c.T, 2, dims, str, box) &&
                    make_tmap_f16(&g.tmBlo, w.Blo + (size_t)c0 * c.T, 2, dims, str, box);
         (void)okm;
