@@ -845,8 +845,11 @@ void add_tall_gram(Program &P, int stage, const std::vector<TallGram> &jobs) {
   if (rj.empty()) return;
   const size_t off = P.push(rj);
   const int n = (int)rj.size();
+  int max_k = 0;
+  for (auto &r : rj) max_k = std::max(max_k, r.k);
+  const int gx = (max_k * max_k + kReduceThreads - 1) / kReduceThreads;
   P.add(stage, [=](char *dev, cudaStream_t s) {
-    reduce_partials_var_kernel<<<dim3(32, n), 256, 0, s>>>((const ReduceJob *)(dev + off));
+    reduce_partials_var_kernel<<<dim3(gx, n), kReduceThreads, 0, s>>>((const ReduceJob *)(dev + off));
     LAUNCHED();
   });
 }
