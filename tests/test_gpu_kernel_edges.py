@@ -118,3 +118,35 @@ def test_reciprocal_is_correctly_rounded(E):
     y, ref = out.view(2, -1).cpu().numpy()
     assert (y[:m] == ref[:m]).all()
     assert np.all(np.abs(y - ref) <= 2 * U * np.abs(ref))
+
+
+# staging and sums of the projected core: sixteen bytes (r_f a multiple of 8), pairs (even), single entries (odd); 21 rows end inside the second
+# half of a block of 32, 72 in a third block.  Saved and loaded handles form it again.
+@pytest.mark.parametrize("r_t", [7, 24])
+@pytest.mark.parametrize("r_f", [1, 2, 8, 10, 12, 126, 127])
+def test_projected_core(r_f, r_t):
+    import __graft_entry__ as entry
+    entry.build()
+    import paper_2607_12550_b200 as pkg
+    from tests.helpers import cell_from_handle, cell_view, decode_elementwise_bound
+    from oracle import jolt_oracle as O
+    B = pkg.load()
+    cfg = pkg.synth.CacheConfig("t", 1, 1, 3, 256, n_terms=40, seed=r_f)
+    K, V = pkg.synth.make_cache(cfg, device="cuda")
+    r_t = min(r_t, 3 * r_f)                  # (no more than the rows of the projected unfolding)
+    gs, plans = [0, 1], [(r_t, r_f, 0), (r_t, r_f, 4)]
+    h = B.jolt_compress(K, V, gs, plans, B.default_options(seed=4, power_iters=1))
+    h2 = B.jolt_deserialize(B.jolt_serialize(h))
+    got = []
+    for x in (h, h2):
+        Ko, Vo = torch.empty(K.shape, device="cuda"), torch.empty(K.shape, device="cuda")
+        B.jolt_decompress(x, Ko, Vo, gs)
+        got.append((Ko, Vo))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    out = [t.cpu().numpy() for t in got[0]]
+    for c, plan in enumerate(plans):
+        oc = cell_from_handle(h, c, 3, 256, plan, 4, "f32")
+        err = np.abs(cell_view(*out, gs, c) - O.decompress_cell(oc))
+        assert np.all(err <= decode_elementwise_bound(oc, "f32")), float(err.max())
+    h.free()
+    h2.free()
