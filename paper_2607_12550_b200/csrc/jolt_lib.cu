@@ -360,8 +360,7 @@ __global__ void store_factors_kernel(const StoreJob *jobs) {
 // exact value (the definition), not of an fp32 sum that may sit on the other side of a rounding boundary.
 // grid (row blocks of 32, cells), 256 threads (feature, half of the rows); dynamic shared memory: 160 r_f doubles, U_F as [s][f] and
 // the block's rows of G.  Both are converted once: with fp16 operands the loop was bound by conversions to fp64 (16 a clock and
-// SM), nine for eight FMAs.  One layer of 8 x 512 tokens, fp32, r_f = 64: round trip
-// 1226 -> 1196 us; 10 layers x 5 heads x 2944 tokens with its plan: 2516 -> 2473 us.
+// SM), nine for eight FMAs.  One cell of 8 heads, r_t = r_f = 64: 41.9 -> 11.1 us a launch; 20 heads x 2944 tokens with its plan: 77.6 -> 15.5.
 struct ProjJob { const __half *G, *UF; __half *P; int rows, r_f; };
 __global__ void __launch_bounds__(256) project_core_kernel(const ProjJob *__restrict__ jobs) {
   const ProjJob j = jobs[blockIdx.y];

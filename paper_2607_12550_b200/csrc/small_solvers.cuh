@@ -526,8 +526,8 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partials_var_kernel(con
 // Rows stream through shared memory 16 at a time (converted to fp64 once, on the way in).  The block is 8 x 8 tiles, accumulators
 // of fp64 matrix instructions, dealt out over a 4 x 2 grid of warps; a diagonal block (SAME) holds its lower tiles only.  Bound by the
 // fp64 rate (64 FMAs a clock and SM): the matrix instructions do not raise it, but their operands are one load for eight columns where a
-// 9 x 9 register tile took eighteen for 81 FMAs, and half the tiles need not be formed.  Round trip of 40 layers x 40 heads x 4096 tokens: 9.28 -> 9.03 ms,
-// 32 x 8 heads: 2301 -> 2264 us; one fp32 layer of 8 x 512: 1196 -> 1169 us.
+// 9 x 9 register tile took eighteen for 81 FMAs, and half the tiles need not be formed.  20480 rows, k = 138 (two matrices): 178.5 -> 91.3 us a launch;
+// 4096 rows, k up to 106: 19.5 -> 12.0; 512 rows, k = 74: 21.4 -> 11.5.
 struct TallGramJob { const float *M; int rows, k, chunk; double *part; int ca, wa, cb, wb; const int *only; };
 
 __device__ __forceinline__ void dmma(double (&d)[2], double a, double b) {      // d += a (8 x 4) b (4 x 8)

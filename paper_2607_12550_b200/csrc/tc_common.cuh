@@ -110,8 +110,8 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr, uint32_t
   return d;
 }
 // The k-th 16-element (32-byte) K slice of a K-major swizzled tile: the start-address field counts 16-byte units,
-// so the slice's descriptor is the tile's plus 2k.  Building descriptors once and stepping them keeps the single
-// MMA-issuing thread ahead of the tensor pipe (a full rebuild per MMA costs it ~100 cycles, more than the MMA).
+// so the slice's descriptor is the tile's plus 2k.  Built once and stepped: a full rebuild per MMA is more work than the 64 cycles
+// that an MMA of 128 x 128 x 16 takes.
 __device__ __forceinline__ uint64_t umma_desc_kslice(uint64_t tile_desc, int k) { return tile_desc + (uint64_t)(2 * k); }
 
 // Instruction descriptor: fp16 A and B, fp32 D, M x N tile, per-operand major (0 = K-major, 1 = MN-major).
@@ -119,9 +119,11 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N, int a_mn_maj
   return (1u << 4) | (0u << 7) | (0u << 10) | ((uint32_t)a_mn_major << 15) | ((uint32_t)b_mn_major << 16) |
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// The whole warp comes here, converged, and one elected lane issues (the same one each time, which the commit relies on).  An MMA
-// takes its operands from uniform registers: in code that one lane runs by itself every descriptor word has to be moved there
-// first, and the issuing thread was slower than the tensor core (about 110 cycles an MMA against 64).
+// The whole warp comes here, converged, and one elected lane issues (the same one each time, which the commit relies on).  On an SM
+// that does nothing else this form and umma_f16_lane both issue an MMA of 128 x 128 x 16 every 64 cycles, the tensor core's rate, and of
+// 128 x 256 x 16 every 128; the first sixteen take 79 against 92 each.  Which of them a kernel takes is a matter of what the rest of it
+// does, and measured at each: the token sweeps (62 -> 50 us a launch), the residual pass, the orthonormalisation and the per-item decode (534 -> 525 us)
+// take this one, the feature sweeps (30.8 -> 28.7 us) and the persistent decode the other.
 __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"

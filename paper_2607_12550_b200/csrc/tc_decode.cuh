@@ -23,10 +23,10 @@
 namespace jolt {
 namespace tc {
 
-// Two epilogue warpgroups, a producer warpgroup (TMA thread, MMA thread), 224 KB of shared memory, one CTA per SM.
+// Two epilogue warpgroups, a producer warpgroup (TMA thread, two MMA issuers), 224 KB of shared memory, one CTA per SM.
 // Any r_t <= 256: P region 64 KB, 4-stage U_T ring, one operand tile and one accumulator per warpgroup.  For
 // r_t <= 128 half of the P region is free and extends the ring to six stages (three U_T tiles in flight), and each
-// warpgroup owns TWO accumulators: the MMA thread issues the backbone of a tile two tiles before its rotation, so
+// warpgroup owns TWO accumulators: the backbone of a tile is issued two tiles before its rotation, so
 // backbones wait in TMEM instead of U_T tiles waiting in shared memory, and a warpgroup only waits for the eight
 // rotation MMAs of its tile.
 constexpr int DEC_H_BYTES = 32768;
@@ -739,9 +739,8 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_kernel(const __g
         }
       }
     } else if (role == NWG * 4 + 1) {
-      // ---------------- backbone MMA issuer.  Issuing an MMA costs its thread tens of cycles of dependent
-      // instructions, and a tile needs sixteen of them: the two halves of a tile's accumulation (backbone, rotation)
-      // are issued by two threads on different schedulers, ordered per accumulator through bBB.  The backbone thread
+      // ---------------- backbone MMA issuer.  The two halves of a tile's accumulation (backbone, rotation) are issued by two
+      // warps on different schedulers, ordered per accumulator through bBB, because they wait for different things.  The backbone's
       // runs ahead as far as free accumulators and landed U_T stages allow (two accumulators per warpgroup when
       // r_t <= 128), so backbones wait in TMEM instead of U_T tiles in shared memory, and a late U_T stage never
       // holds back a rotation whose operands are complete.
