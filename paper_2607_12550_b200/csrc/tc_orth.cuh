@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(OR_THREADS, 1) orth_gram_kernel(const OrthCell
 //   update   every living tile but the next diagonal block; its eight products are summed first and then subtracted
 // The order of the operations is that of a matrix in shared memory updated by FMAs, one rounding each (the matrix instruction is four
 // FMAs in the order of k, the reciprocal is correctly rounded), and so are the results, bit for bit.  Multiplying the panel by the explicit inverse
-// of the block instead is 5 us shorter at n = 138 but not as good: the residual of L L^T in units of 2^-53 of the diagonal, 1081 against 3.2
+// of the block instead is 6 us shorter at n = 138 but not as good: the residual of L L^T in units of 2^-53 of the diagonal, 1081 against 3.2
 // where neighbouring columns are close (n = 74), 7.6 against 4.1 on a graded matrix.
 // What bounds it: fp64 operations and their latency: the chain, 8 x (estimate, five FMAs, product, FMA) and the substitution, and
 // at n > 100 the products of the early panels.  The loops are short on purpose: nothing runs more than a few times, and with tiles in
