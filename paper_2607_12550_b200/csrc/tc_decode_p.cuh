@@ -321,10 +321,12 @@ __global__ void __launch_bounds__(DecLayout::THREADS, 1) decode_persistent_kerne
   auto bRready = [=](int b) { return sBar + 184 + 8 * b; };
   auto bBB = [=](int b) { return sBar + 216 + 8 * b; };           // backbone of the accumulator's tile complete
 
-  // The warp number as one value per warp (a shuffle) leaves the tile loops of 4 and 8 bits without spills, and adds some to the others:
-  // 32 layers x 8 heads x 4096 tokens at 2x 205.6 -> 203.1 us, keys rotated 276 -> 273; with it, 2 bits everywhere took 107 instead of
-  // 100 us (16 layers), one layer of 128 tokens 8.7 instead of 8.2.
-  const int warp = BITMASK == 272u ? warp_uniform() : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  // The warp number as one value per warp (a shuffle) leaves the tile loops of 4 and 8 bits without spills, and adds some to others:
+  // 32 layers x 8 heads x 4096 tokens at 2x 205.6 -> 203.1 us, keys rotated 276 -> 273, 8 bits alone (16 layers) 109.0 -> 107.8, fp32
+  // output 234.2 -> 232.5, short ones of these equal; with it, 2 bits everywhere took 107 instead of 100 us (16 layers), one layer of 128
+  // tokens 8.7 instead of 8.2 (generic).
+  constexpr bool UNIFORM = BITMASK == 0x110u || BITMASK == 0x100u || !TMA_ONLY;
+  const int warp = UNIFORM ? warp_uniform() : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int wg = warp >> 2;
   BBCell *sc_cell = (BBCell *)(smBar + 512);      // the epilogue's copy of the current cell's descriptor
 
